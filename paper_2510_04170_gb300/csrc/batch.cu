@@ -15,8 +15,8 @@
 // The autotuner picks, per sketch size (s, n), the QR configuration: FP64
 // panels with the FP64 trailing update, or the tensor-core (emulated FP64)
 // trailing update, each with the panel factorisation spread over at most 16,
-// 32, 64 or all SMs (fewer CTAs make the two grid barriers per column cheaper,
-// more CTAs share the panel's rows; shared memory bounds the rows per CTA).
+// 32, 64 or all SMs (fewer CTAs make the exchange per column cheaper, more CTAs
+// share the panel's rows; shared memory bounds the rows per CTA).
 // Each candidate factors the first 128 columns of a seeded random s x n
 // matrix (updating all n columns), timed with CUDA events after one warm-up;
 // the fastest is cached per (s, n) for the process.
@@ -111,7 +111,11 @@ rfm_status probe_qr(long long s, long long n, cudaStream_t st, QrChoice* out) {
     for (int c = 1; c < kCands; ++c)
       if (out->ms[c] < out->ms[arg]) arg = c;
     out->precision = arg < kCaps ? 0 : 2;
-    out->panel_cap = caps[arg % kCaps];
+    // The block factorisation chooses its CTAs by the row count, and its sums
+    // follow that choice: a cap is taken only where the probe shows a clear
+    // gain, so that a batch otherwise gives the bits of a stand-alone solve.
+    const int all = (arg / kCaps) * kCaps + kCaps - 1;
+    out->panel_cap = out->ms[arg] < 0.75 * out->ms[all] ? caps[arg % kCaps] : caps[kCaps - 1];
   }
   cudaStreamSynchronize(st);
   if (e0) cudaEventDestroy(e0);

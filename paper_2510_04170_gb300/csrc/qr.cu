@@ -2,23 +2,18 @@
 // the right preconditioner R.  Blocked right-looking Householder with the
 // compact-WY trailing update (Schreiber & Van Loan):
 //
-//   for each panel of NB columns:
-//     k_panel   (cooperative, one CTA per SM slice of rows): the panel's rows
-//               stay in shared memory; per column one bounded grid barrier
-//               combines the column norm below the pivot and the products of
-//               the unscaled column with the rest of the panel, from which
-//               every CTA forms v^T A (details at the kernel).  Reflector
-//               H = I - tau v v^T, v_0 = 1, beta = -sign(alpha) ||x||.  At the
-//               end T (NB x NB, upper) with T_jj = tau_j,
-//               T_{:j,j} = -tau_j T_{:j,:j} V_{:,:j}^T v_j.
-//     k_vta     W_z = V^T A_trail over a K-slice z (split K, deterministic)
-//     k_wt      W2 = T^T sum_z W_z
-//     k_update  A_trail -= V W2
-//   k_normalise: flip rows of R to a positive diagonal, floor pivots below
-//               1e-14 max_j R_jj (rank guard; flag raised).
+//   k_block     (cooperative) factors a block of up to 128 columns (32 when the
+//               trailing update is in FP64), one exchange between the CTAs per
+//               column.  Reflector H = I - tau v v^T, v_0 = 1,
+//               beta = -sign(alpha) ||x||.
+//   k_vta       W_z = V^T A_trail over a K-slice z (split K, deterministic)
+//   k_wt        W2 = T^T sum_z W_z, T the panel's compact-WY factor
+//   k_update    A_trail -= V W2
+//   k_diag, k_flip, k_floor: rows of R flipped to a positive diagonal, pivots
+//               below 1e-14 max_j R_jj floored (rank guard; flag raised).
 //
 // All sums are reduced in a fixed order, so repeated runs give identical bits.
-#include <cooperative_groups.h>
+#include <math.h>
 
 #include <algorithm>
 #include <mutex>
@@ -30,191 +25,400 @@ namespace {
 
 constexpr int NB = 32;
 
-struct PanelArgs {
+// ---------------------------------------------------------------------------
+// Cooperative block factorisation k_block.
+//
+// GB300's FP64 unit takes 64 cycles (31 ns) for a warp instruction, the same
+// for a dependent chain as for independent ones and for one lane as for 32
+// (measured).  What bounds a column of the factorisation is therefore the
+// number of FP64 warp instructions on one SM partition, plus one exchange
+// between the CTAs; the kernel is laid out to issue few of them:
+//  - 4 warps per CTA, one per SM partition; the lanes of a warp are the 32
+//    columns of the panel, so a row of the panel is one instruction and no
+//    reduction over lanes is needed.  A warp owns every fourth row.
+//  - the columns k < j already hold their reflectors u_k, so the same
+//    instruction that gives x^T a_k for the columns to the right (and
+//    sigma = x^T x in lane j) gives u_k^T x for the columns to the left: the
+//    panel's Gram comes with the reduction and needs no pass of its own.
+//  - H = I - gamma u u^T with the unscaled u = (alpha - beta, x) and
+//    gamma = 1 / (beta (beta - alpha)): the column is scaled once, at the end
+//    of the panel.  sqrt and the reciprocal are one third-order step
+//    (Householder's iteration) from an FP32 seed, 18 instructions where the
+//    library's sqrt and two divisions take 28 (0.86 us).
+//  - the CTAs exchange their 32 sums as 16-byte records {low, tag, high, tag}
+//    whose tag is the column's number: a reader polls the records themselves,
+//    so there is no fence, no counter and no second trip to L2.  Two slots
+//    alternate; a CTA can only be one exchange ahead of another.
+// Between the panels of a block, the block's remaining columns (in the same
+// shared-memory slab) are updated with W = V^T A, W2 = T^T W, A -= V W2: CTA c
+// sums column c of W over the CTAs and solves for its column of W2.
+//
+// Times per column at 12,288 rows: 16.5 us with one grid barrier and a
+// redundant butterfly reduction per column (k_panel, 32 columns per launch).
+constexpr int KB_THREADS = 128;
+constexpr int KB_SMEM = 227 * 1024;              // dynamic shared memory of a CTA
+constexpr int KB_MAXP = 256;                     // CTAs of one factorisation
+constexpr int KB_POLL = 19;                      // records in flight per lane and poll round
+constexpr int KB_SLOT = (KB_MAXP + 1) * NB * 2;  // 8-byte words of one exchange slot (row P: the pivot row)
+
+struct BlockArgs {
   double* A;
   long long lda;
   long long s;
   long long j0;
-  int nbw;           // columns in this panel (<= NB)
-  int P;             // CTAs (<= 256)
-  int chunk;         // rows per CTA
-  double* part;      // two buffers of [512][NB + 2] partials (row 511 of each: the pivot row)
-  double* gram;      // [P][NB*NB]
-  double* tau;       // [n]
-  double* T;         // [NB][NB] (row-major T[i][j])
-  unsigned int* bar;  // [2]: count, generation
+  int nb;              // columns of the block (<= 128)
+  int P;               // CTAs
+  int chunk;           // rows per CTA
+  unsigned long long* xch;  // [2][KB_SLOT] exchange records
+  double* part;        // [P][3 NB][NB] partial W of the in-block update
+  double* w2;          // [3 NB][NB]
+  double* tau;         // [n]
+  double* G;           // [NB][NB] of the last panel: G[p * NB + q] = tau_p v_q^T v_p for q < p, else 0
+  unsigned int* bar;   // arrival counter of the grid barriers
+  unsigned int bar0;   // its value before this launch
   unsigned int* err;
 };
 
-// Grid-wide barrier: an arrival counter bar[0] and a generation word
-// bar[BAR_GEN], on different 128-byte lines so that the CTAs polling the
-// generation do not contend with the arrivals' atomics.
-constexpr int BAR_GEN = 32;
+constexpr int KB_TRI = NB * (NB - 1) / 2;  // entries q < p of the panel's Gram
+__host__ __device__ constexpr int kb_tri(int p, int q) { return p * (p - 1) / 2 + q; }
+__host__ __device__ constexpr size_t kb_fixed_smem() { return (size_t)(KB_TRI + 13 * NB) * sizeof(double); }
 
-__device__ __forceinline__ void grid_barrier(unsigned int* bar, unsigned int nblocks, unsigned int* err) {
-  __threadfence();
+// Slab element (local row r, column c): 32-column groups with the column index
+// XORed by the row, so that both a row (lanes = columns) and a column (lanes =
+// rows) are free of bank conflicts.
+__device__ __forceinline__ int kb_at(int r, int c, int ld) { return r * ld + (c & ~31) + ((c ^ r) & 31); }
+
+struct KbWait {
+  int lim;             // polls of one wait; < 0: give up at once
+  unsigned int* err;
+  bool dead;           // a wait of this launch gave up: do not wait again
+  __device__ __forceinline__ bool spin(unsigned int& n) {  // false: give up
+    if (dead || lim < 0 || ++n > (unsigned int)lim) {
+      if (!dead) atomicExch(err, 1u);
+      dead = true;
+      return false;
+    }
+    if (n > (1u << 16)) __nanosleep(128);
+    return true;
+  }
+};
+
+// Arrivals of all CTAs up to the count `want` (the counter only grows).
+__device__ __forceinline__ void kb_barrier(unsigned int* bar, unsigned int want, KbWait& kw) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned int g = ld_acquire(bar + BAR_GEN);
-    const unsigned int arrived = atomicAdd(bar, 1u);
-    if (arrived == nblocks - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      st_release(bar + BAR_GEN, g + 1);
-    } else {
-      wait_flag(bar + BAR_GEN, g + 1, err, 32);
-    }
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned int n = 0;
+    while ((int)(ld_acquire(bar) - want) < 0)
+      if (!kw.spin(n)) break;
   }
   __syncthreads();
 }
 
-// Sum over the P CTAs of partial value idx (stride NB + 2 per CTA) in a fixed
-// order: each lane loads its CTAs' values (all loads issued before the adds),
-// then the lanes are combined by the warp's butterfly.  Every CTA obtains
-// bitwise the same result.
-__device__ __forceinline__ double sum_partials(const double* part, int P, int idx, int lane) {
-  double t[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const int q = lane + 32 * u;
-    t[u] = q < P ? __ldcg(part + q * (NB + 2) + idx) : 0.0;
-  }
-  double s = 0.0;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) s += t[u];
-  return warp_sum(s);
+__device__ __forceinline__ void kb_publish(unsigned long long* rec, double v, unsigned int tag) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long lo = (b & 0xffffffffull) | ((unsigned long long)tag << 32);
+  const unsigned long long hi = (b >> 32) | ((unsigned long long)tag << 32);
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(rec), "l"(lo), "l"(hi) : "memory");
+}
+__device__ __forceinline__ void kb_load(const unsigned long long* rec, unsigned long long& lo,
+                                        unsigned long long& hi) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(rec) : "memory");
+}
+__device__ __forceinline__ bool kb_ready(unsigned long long lo, unsigned long long hi, unsigned int tag) {
+  return (unsigned int)(lo >> 32) == tag && (unsigned int)(hi >> 32) == tag;
+}
+__device__ __forceinline__ double kb_value(unsigned long long lo, unsigned long long hi) {
+  return __longlong_as_double((long long)((lo & 0xffffffffull) | (hi << 32)));
 }
 
-// One grid-wide barrier per column.  Before it, every CTA contributes, for
-// its rows below the pivot row j, sigma = sum x_r^2 and p_k = sum x_r A_rk for
-// the remaining panel columns k (x = column j, not yet scaled); the CTA that
-// holds row j also publishes alpha = A_jj and the pivot row A_jk.  After it,
-// every CTA forms beta, tau, 1/(alpha - beta) and
-//     w_k = v^T A_k = A_jk + p_k / (alpha - beta)     (v_j = 1, v_r = x_r / (alpha - beta)),
-// the same quantities the two-barrier form obtains by reducing v^T A_k after
-// scaling.  The partials alternate between two buffers, so a CTA that runs
-// ahead into column j + 1 never overwrites values another CTA still reads.
-__global__ void __launch_bounds__(256) k_panel(PanelArgs a) {
-  extern __shared__ double sp[];  // [NB][chunk] column-major panel slice
-  __shared__ double sw[NB];       // w_k, then tau w_k
-  __shared__ double sv[NB + 2];   // reduced sigma and p_k
-  const int c = blockIdx.x;
+// norm = sqrt(alpha^2 + sigma) and gamma = 1 / (norm^2 + |alpha| norm) for
+// sigma > 0.  In the scaled variables m = t 2^-e in [1, 4) (e even), the
+// seeds are FP32 (2^-21) and one step of third order leaves ~2^-63; sqrt gets
+// one Newton correction.  Exponents near the ends of the range (and Inf, NaN)
+// take the library functions.
+__device__ __forceinline__ void kb_norm_gamma(double alpha, double sigma, double& nrm, double& gam) {
+  const double t = fma(alpha, alpha, sigma);
+  const int hi = __double2hiint(t), lo = __double2loint(t);
+  const int ex = ((hi >> 20) & 0x7FF) - 1023;
+  if (ex < -900 || ex > 900 || hi < 0) {
+    nrm = sqrt(t);
+    gam = 1.0 / fma(fabs(alpha), nrm, t);
+    return;
+  }
+  const int e = ex & ~1;
+  const int mh = hi - (e << 20);  // m = t 2^-e
+  const double m = __hiloint2double(mh, lo);
+  // FP32 value of m with its low bits cut off (integer operations only)
+  const float mf = __int_as_float(((mh >> 20) - 1023 + 127) << 23 | (mh & 0xFFFFF) << 3 | (int)((unsigned)lo >> 29));
+  const int yb = __float_as_int(rsqrtf(mf));
+  const double y0 = __hiloint2double((((yb >> 23) - 127 + 1023) << 20) | ((yb & 0x7FFFFF) >> 3), (int)((unsigned)(yb & 7) << 29));
+  const double h = m * y0;
+  const double r = fma(-h, y0, 1.0);
+  const double y = fma(y0, fma(r, 0.375, 0.5) * r, y0);  // 1 / sqrt(m)
+  double q = m * y;                                        // sqrt(m)
+  const double half_y = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));
+  q = fma(fma(-q, q, m), half_y, q);
+  const double back = __hiloint2double((1023 - (e >> 1)) << 20, 0);  // 2^(-e/2)
+  const double d = fma(fabs(alpha) * back, q, m);                    // in [1, 8)
+  const int dh = __double2hiint(d), dl = __double2loint(d);
+  const float df = __int_as_float(((dh >> 20) - 1023 + 127) << 23 | (dh & 0xFFFFF) << 3 | (int)((unsigned)dl >> 29));
+  const int gb = __float_as_int(__frcp_rn(df));
+  const double g0 = __hiloint2double((((gb >> 23) - 127 + 1023) << 20) | ((gb & 0x7FFFFF) >> 3), (int)((unsigned)(gb & 7) << 29));
+  const double w = fma(-d, g0, 1.0);
+  const double g = fma(g0, fma(w, w, w), g0);  // 1 / d
+  nrm = __hiloint2double(__double2hiint(q) + ((e >> 1) << 20), __double2loint(q));
+  gam = __hiloint2double(__double2hiint(g) - (e << 20), __double2loint(g));
+}
+
+__device__ __forceinline__ void kb_copy8(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
+  extern __shared__ __align__(16) double kb_sm[];
+  double* Gs = kb_sm;              // tau_p v_q^T v_p of the panel at kb_tri(p, q), q < p
+  double* wp = Gs + KB_TRI;       // [4][NB] the warps' partial sums
+  double* rs = wp + 4 * NB;        // [4][NB] the warps' shares of the sums over CTAs
+  double* pv = rs + 4 * NB;        // [NB] pivot row
+  double* dab = pv + NB;           // [NB] alpha - beta
+  double* gam = dab + NB;          // [NB] gamma
+  double* scl = gam + NB;          // [NB] 1 / (alpha - beta)
+  double* taus = scl + NB;         // [NB]
+  double* sl = kb_sm + (kb_fixed_smem() / sizeof(double));  // slab [rows][ld]
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int c = blockIdx.x, P = a.P;
   const long long rbeg = a.j0 + (long long)c * a.chunk;
   const long long rend = min(a.s, rbeg + a.chunk);
   const int nr = rbeg < rend ? (int)(rend - rbeg) : 0;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int chunk = a.chunk;
-  for (int jj = 0; jj < a.nbw; ++jj) {
-    const double* col = a.A + (size_t)(a.j0 + jj) * a.lda + rbeg;
-    for (int r = tid; r < nr; r += blockDim.x) sp[jj * chunk + r] = col[r];
+  const int np = (a.nb + NB - 1) / NB, ld = np * NB;
+  const int wl = (int)__ldcg(a.err + (SYNC_WAITLIM - SYNC_ERR));
+  KbWait kw{wl == 0 ? (1 << 22) : wl, a.err, __ldcg(a.err) != 0u};
+  if (wl < 0) {  // test setting: every wait gives up at once
+    if (tid == 0) atomicExch(a.err, 1u);
+    kw.dead = true;
   }
+  unsigned int barrier = a.bar0;
+  for (int cc = w; cc < ld; cc += 4) {
+    const double* col = a.A + (size_t)(a.j0 + cc) * a.lda + rbeg;
+    for (int r = lane; r < nr; r += 32) {
+      if (cc < a.nb) kb_copy8(sl + kb_at(r, cc, ld), col + r);
+      else sl[kb_at(r, cc, ld)] = 0.0;
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  for (int jj = 0; jj < a.nbw; ++jj) {
-    const long long j = a.j0 + jj;  // pivot row
-    double* v = sp + jj * chunk;
-    const int rest = a.nbw - jj - 1;
-    double* part = a.part + (size_t)(jj & 1) * 512 * (NB + 2);  // [P][NB + 2] this column's partials
-    double* piv = part + (size_t)511 * (NB + 2);                 // alpha, A_jk of the pivot row
-    // local partials: slot 0 sigma (kk = -1), slot 1 + kk p_k; one warp per slot
-    for (int kk = w - 1; kk < rest; kk += (blockDim.x >> 5)) {
-      const double* ck = kk < 0 ? v : sp + (jj + 1 + kk) * chunk;
+  for (int pi = 0; pi < np; ++pi) {
+    const int p0 = pi * NB, nbw = min(NB, a.nb - p0);
+    for (int jj = 0; jj < nbw; ++jj) {
+      const long long j = a.j0 + p0 + jj;  // pivot row and column
+      const unsigned int tag = (unsigned int)(j + 1);
+      unsigned long long* slot = a.xch + (size_t)(jj & 1) * KB_SLOT;
+      const int lr = j + 1 > rbeg ? (int)min((long long)nr, j + 1 - rbeg) : 0;  // rows below the pivot
+      const int rw = lr + ((w - lr) & 3);                                       // this warp's first one
       double acc = 0.0;
-      for (int r = lane; r < nr; r += 32)
-        if (rbeg + r > j) acc += v[r] * ck[r];
-      acc = warp_sum(acc);
-      if (lane == 0) part[c * (NB + 2) + 1 + kk] = acc;
-    }
-    if (j >= rbeg && j < rend && tid <= rest) piv[tid] = sp[(jj + tid) * chunk + (j - rbeg)];
-    grid_barrier(a.bar, a.P, a.err);
-    for (int idx = w; idx <= rest; idx += (blockDim.x >> 5)) {
-      const double sm = sum_partials(part, a.P, idx, lane);
-      if (lane == 0) sv[idx] = sm;
+#pragma unroll 4
+      for (int r = rw; r < nr; r += 4) acc = fma(sl[kb_at(r, p0 + jj, ld)], sl[kb_at(r, p0 + lane, ld)], acc);
+      wp[w * NB + lane] = acc;
+      __syncthreads();
+      if (w == 0) {
+        const double sm = (wp[lane] + wp[NB + lane]) + (wp[2 * NB + lane] + wp[3 * NB + lane]);
+        kb_publish(slot + ((size_t)c * NB + lane) * 2, sm, tag);
+      } else if (w == 1 && j >= rbeg && j < rend) {
+        kb_publish(slot + ((size_t)P * NB + lane) * 2, sl[kb_at((int)(j - rbeg), p0 + lane, ld)], tag);
+      }
+      // sum over the CTAs, warp w the CTAs w, w + 4, ... in increasing order;
+      // record P is the pivot row
+      double sum = 0.0;
+      for (int q0 = w; q0 <= P; q0 += 4 * KB_POLL) {
+        unsigned long long lo[KB_POLL], hi[KB_POLL];
+        unsigned int spins = 0;
+        for (;;) {
+          bool all = true;
+#pragma unroll
+          for (int i = 0; i < KB_POLL; ++i)
+            if (q0 + 4 * i <= P) kb_load(slot + ((size_t)(q0 + 4 * i) * NB + lane) * 2, lo[i], hi[i]);
+#pragma unroll
+          for (int i = 0; i < KB_POLL; ++i)
+            if (q0 + 4 * i <= P) all = all && kb_ready(lo[i], hi[i], tag);
+          if (__all_sync(0xffffffffu, all) || !__all_sync(0xffffffffu, kw.spin(spins))) break;
+        }
+#pragma unroll
+        for (int i = 0; i < KB_POLL; ++i) {
+          const int q = q0 + 4 * i;
+          if (q < P) sum += kb_value(lo[i], hi[i]);
+          else if (q == P) pv[lane] = kb_value(lo[i], hi[i]);
+        }
+      }
+      rs[w * NB + lane] = sum;
+      __syncthreads();
+      const double tot = (rs[lane] + rs[NB + lane]) + (rs[2 * NB + lane] + rs[3 * NB + lane]);
+      const double piv = pv[lane];
+      const double alpha = pv[jj];
+      const double sigma = __shfl_sync(0xffffffffu, tot, jj);
+      double dj = 0.0, gj = 0.0, beta = alpha;
+      if (sigma != 0.0) {
+        double nrm;
+        kb_norm_gamma(alpha, sigma, nrm, gj);
+        beta = alpha >= 0.0 ? -nrm : nrm;
+        dj = alpha - beta;
+      }
+      // u^T a_k for the columns to the right, u_k^T u for those to the left
+      const double wk = fma(dj, piv, tot);
+      const double f = lane > jj ? gj * wk : 0.0;
+      if (w == 0) {
+        if (lane < jj) Gs[kb_tri(jj, lane)] = wk;
+        if (lane == jj) {
+          dab[jj] = dj;
+          gam[jj] = gj;
+        }
+      }
+      if (jj < 16) {
+#pragma unroll 4
+        for (int r = rw; r < nr; r += 4) {
+          double* e = sl + kb_at(r, p0 + lane, ld);
+          *e = fma(-f, sl[kb_at(r, p0 + jj, ld)], *e);
+        }
+      } else {
+        // only columns 16 .. 31 are left: two rows per instruction
+        const int cl = 16 + (lane & 15);
+        const double fh = __shfl_sync(0xffffffffu, f, cl);
+#pragma unroll 4
+        for (int r = rw; r < nr; r += 8) {
+          const int rr = r + 4 * (lane >> 4);
+          if (rr < nr) {
+            double* e = sl + kb_at(rr, p0 + cl, ld);
+            const double x = sl[kb_at(rr, p0 + jj, ld)];
+            if (cl > jj) *e = fma(-fh, x, *e);
+          }
+        }
+      }
+      if (j >= rbeg && j < rend && w == ((int)(j - rbeg) & 3)) {  // the pivot row itself
+        double* e = sl + kb_at((int)(j - rbeg), p0 + lane, ld);
+        if (lane > jj) *e = fma(-f, dj, *e);
+        if (lane == jj) *e = beta;
+      }
+      __syncwarp();
     }
     __syncthreads();
-    const double sigma = sv[0], alpha = __ldcg(piv);
-    double tau = 0.0, beta = alpha, scale = 0.0;
-    if (sigma != 0.0) {
-      const double nrm = sqrt(alpha * alpha + sigma);
-      beta = alpha >= 0.0 ? -nrm : nrm;
-      tau = (beta - alpha) / beta;
-      scale = 1.0 / (alpha - beta);
+    if (w == 0) {
+      const double d = lane < nbw ? dab[lane] : 0.0;
+      const bool on = d != 0.0;
+      scl[lane] = on ? 1.0 / d : 0.0;
+      taus[lane] = on ? gam[lane] * (d * d) : 0.0;
+      if (c == 0 && lane < nbw) a.tau[a.j0 + p0 + lane] = taus[lane];
     }
-    if (tid < rest) sw[tid] = tau * (__ldcg(piv + 1 + tid) + scale * sv[1 + tid]);  // tau w_k
-    // v_r = x_r / (alpha - beta) below the pivot, v_j = 1
-    if (tau != 0.0)
-      for (int r = tid; r < nr; r += blockDim.x)
-        if (rbeg + r > j) v[r] *= scale;
     __syncthreads();
-    if (tau != 0.0) {
-      for (int kk = 0; kk < rest; ++kk) {
-        const double f = sw[kk];
-        double* ck = sp + (jj + 1 + kk) * chunk;
-        for (int r = tid; r < nr; r += blockDim.x) {
-          const long long gr = rbeg + r;
-          if (gr >= j) ck[r] -= (gr == j ? 1.0 : v[r]) * f;
+    for (int idx = tid; idx < NB * NB; idx += KB_THREADS) {
+      const int p = idx / NB, q = idx % NB;
+      double g = 0.0;
+      if (q < p && p < nbw) {
+        g = Gs[kb_tri(p, q)] * scl[q] * scl[p] * taus[p];
+        Gs[kb_tri(p, q)] = g;
+      }
+      if (c == 0) a.G[idx] = g;
+    }
+    // R on and above the diagonal and v below to global memory; the slab keeps
+    // v with its unit diagonal and zeros above
+    for (int cc = w; cc < nbw; cc += 4) {
+      const long long pr = a.j0 + p0 + cc;  // this column's pivot row
+      double* col = a.A + (size_t)pr * a.lda + rbeg;
+      const double sc = scl[cc];
+      for (int r = lane; r < nr; r += 32) {
+        double* e = sl + kb_at(r, p0 + cc, ld);
+        const long long gr = rbeg + r;
+        const double v = gr > pr ? *e * sc : *e;
+        col[r] = v;
+        *e = gr > pr ? v : (gr == pr ? 1.0 : 0.0);
+      }
+    }
+    __syncthreads();
+    const int ng = np - 1 - pi;  // column groups to the right in the block
+    if (ng == 0) break;
+    // W = V^T A: lanes are the columns of a group, warp w takes p = 8 w .. 8 w + 7
+    {
+      double acc[3][8];
+#pragma unroll
+      for (int g = 0; g < 3; ++g)
+#pragma unroll
+        for (int p = 0; p < 8; ++p) acc[g][p] = 0.0;
+      const long long first = a.j0 + p0;
+      for (int r = first > rbeg ? (int)min((long long)nr, first - rbeg) : 0; r < nr; ++r) {
+        double av[3];
+#pragma unroll
+        for (int g = 0; g < 3; ++g) av[g] = g < ng ? sl[kb_at(r, p0 + NB * (g + 1) + lane, ld)] : 0.0;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const double v = sl[kb_at(r, p0 + 8 * w + p, ld)];
+#pragma unroll
+          for (int g = 0; g < 3; ++g)
+            if (g < ng) acc[g][p] = fma(v, av[g], acc[g][p]);
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < 3; ++g)
+        if (g < ng) {
+          double* out = a.part + ((size_t)c * 3 * NB + g * NB + lane) * NB + 8 * w;
+#pragma unroll
+          for (int p = 0; p < 8; p += 2)
+            __stcg(reinterpret_cast<double2*>(out + p), make_double2(acc[g][p], acc[g][p + 1]));
+        }
+    }
+    barrier += P;
+    kb_barrier(a.bar, barrier, kw);
+    for (int col = c; col < ng * NB; col += P) {
+      double sum = 0.0;
+      for (int q0 = w; q0 < P; q0 += 4 * KB_POLL) {
+        double t[KB_POLL];
+#pragma unroll
+        for (int i = 0; i < KB_POLL; ++i) {
+          const int q = q0 + 4 * i;
+          t[i] = q < P ? __ldcg(a.part + ((size_t)q * 3 * NB + col) * NB + lane) : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < KB_POLL; ++i)
+          if (q0 + 4 * i < P) sum += t[i];
+      }
+      rs[w * NB + lane] = sum;
+      __syncthreads();
+      if (w == 0) {
+        // W2 = T^T W from T^-1 = diag(1 / tau) + strict upper part of V^T V:
+        // y_p = tau_p w_p - sum_{q<p} (tau_p v_q^T v_p) y_q
+        double x = ((rs[lane] + rs[NB + lane]) + (rs[2 * NB + lane] + rs[3 * NB + lane])) * taus[lane];
+        for (int q = 0; q < nbw; ++q) {
+          const double y = __shfl_sync(0xffffffffu, x, q);
+          if (lane > q && lane < nbw) x = fma(-Gs[kb_tri(lane, q)], y, x);
+        }
+        __stcg(a.w2 + (size_t)col * NB + lane, x);
+      }
+      __syncthreads();
+    }
+    barrier += P;
+    kb_barrier(a.bar, barrier, kw);
+    // A -= V W2: a lane keeps its column of W2
+    {
+      const long long first = a.j0 + p0;
+      const int lr = first > rbeg ? (int)min((long long)nr, first - rbeg) : 0;
+      for (int g = 0; g < ng; ++g) {
+        double y[NB];
+        const double* src = a.w2 + (size_t)(g * NB + lane) * NB;
+#pragma unroll
+        for (int p = 0; p < NB; p += 2) {
+          const double2 t = __ldcg(reinterpret_cast<const double2*>(src + p));
+          y[p] = t.x;
+          y[p + 1] = t.y;
+        }
+        for (int r = lr + ((w - lr) & 3); r < nr; r += 4) {
+          double* e = sl + kb_at(r, p0 + NB * (g + 1) + lane, ld);
+          double x = *e;
+#pragma unroll
+          for (int p = 0; p < NB; ++p) x = fma(-sl[kb_at(r, p0 + p, ld)], y[p], x);
+          *e = x;
         }
       }
     }
     __syncthreads();
-    if (tid == 0 && j >= rbeg && j < rend) v[j - rbeg] = beta;
-    if (c == 0 && tid == 0) a.tau[j] = tau;
-    __syncthreads();
-  }
-  // partial Gram V^T V of this CTA's rows (v_j = 1 on the pivot, 0 above)
-  for (int pq = tid; pq < a.nbw * a.nbw; pq += blockDim.x) {
-    const int p = pq / a.nbw, q = pq % a.nbw;
-    double acc = 0.0;
-    if (p <= q) {
-      for (int r = 0; r < nr; ++r) {
-        const long long gr = rbeg + r;
-        const double vp = gr < a.j0 + p ? 0.0 : (gr == a.j0 + p ? 1.0 : sp[p * chunk + r]);
-        const double vq = gr < a.j0 + q ? 0.0 : (gr == a.j0 + q ? 1.0 : sp[q * chunk + r]);
-        acc += vp * vq;
-      }
-    }
-    a.gram[(size_t)c * NB * NB + pq] = acc;
-  }
-  // write the panel back (R entries on and above the diagonal, v below)
-  for (int jj = 0; jj < a.nbw; ++jj) {
-    double* col = a.A + (size_t)(a.j0 + jj) * a.lda + rbeg;
-    for (int r = tid; r < nr; r += blockDim.x) col[r] = sp[jj * chunk + r];
-  }
-  grid_barrier(a.bar, a.P, a.err);
-  if (c == 0) {
-    __shared__ double G[NB][NB + 1];
-    __shared__ double Ts[NB][NB + 1];
-    for (int pq = tid; pq < a.nbw * a.nbw; pq += blockDim.x) {
-      // sum over CTAs in increasing order, eight loads in flight
-      double s = 0.0;
-      int q = 0;
-      for (; q + 8 <= a.P; q += 8) {
-        double t[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) t[u] = __ldcg(a.gram + (size_t)(q + u) * NB * NB + pq);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) s += t[u];
-      }
-      for (; q < a.P; ++q) s += __ldcg(a.gram + (size_t)q * NB * NB + pq);
-      G[pq / a.nbw][pq % a.nbw] = s;
-    }
-    for (int pq = tid; pq < NB * (NB + 1); pq += blockDim.x) Ts[pq / (NB + 1)][pq % (NB + 1)] = 0.0;
-    __syncthreads();
-    // T column by column (compact WY: T[:j, j] = -tau_j T[:j, :j] G[:j, j]); rows in parallel
-    for (int jj = 0; jj < a.nbw; ++jj) {
-      const double tj = __ldcg(a.tau + a.j0 + jj);
-      if (tid < jj) {
-        double s = 0.0;
-        for (int l = tid; l < jj; ++l) s += Ts[tid][l] * G[l][jj];
-        Ts[tid][jj] = -tj * s;
-      } else if (tid == jj) {
-        Ts[jj][jj] = tj;
-      }
-      __syncthreads();
-    }
-    for (int pq = tid; pq < NB * NB; pq += blockDim.x) {
-      const int p = pq / NB, q = pq % NB;
-      a.T[pq] = (p < a.nbw && q < a.nbw) ? Ts[p][q] : 0.0;
-    }
   }
 }
 
@@ -226,7 +430,7 @@ __device__ __forceinline__ double vval(const double* A, long long lda, long long
   return A[(size_t)(j0 + p) * lda + gr];
 }
 
-// Wp[z][p][col] = sum_{r in K-slice z} v_p(r) A[r, j1 + col]
+// Wp[z][col][p] = sum_{r in K-slice z} v_p(r) A[r, j1 + col]
 __global__ void __launch_bounds__(256) k_vta(const double* __restrict__ A, long long lda, long long s, long long j0,
                                              int nbw, long long j1, long long nt, long long kchunk,
                                              double* __restrict__ Wp) {
@@ -267,26 +471,38 @@ __global__ void __launch_bounds__(256) k_vta(const double* __restrict__ A, long 
     for (int q = 0; q < 4; ++q) {
       const long long gc = col0 + cx + 16 * q;
       const int p = ay + 16 * h;
-      if (gc < nt) Wp[((size_t)z * NB + p) * nt + gc] = acc[h][q];
+      if (gc < nt) Wp[((size_t)z * nt + gc) * NB + p] = acc[h][q];
     }
 }
 
-// W2[p][col] = sum_q T[q][p] sum_z Wp[z][q][col]
-__global__ void k_wt(const double* __restrict__ Wp, int nz, const double* __restrict__ T, int nbw, long long nt,
-                     double* __restrict__ W2) {
-  const long long col = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+// W2 = T^T sum_z Wp[z], one warp per column, lanes = p.  T is not formed: with
+// T^-1 = diag(1 / tau) + strict upper part of V^T V the column is a forward
+// substitution, y_p = tau_p w_p - sum_{q<p} G_pq y_q with G_pq = tau_p v_q^T v_p.
+// Both the sum over z and the substitution are chains of FP64 instructions of
+// 31 ns; one column per warp leaves them short and all columns independent.
+// (The form with one thread per column and T^T W took 120 us at 12,288 rows.)
+__global__ void __launch_bounds__(128) k_wt(const double* __restrict__ Wp, int nz, const double* __restrict__ G,
+                                            const double* __restrict__ tau, int nbw, long long nt,
+                                            double* __restrict__ W2) {
+  const int lane = threadIdx.x & 31;
+  const long long col = blockIdx.x * 4LL + (threadIdx.x >> 5);
   if (col >= nt) return;
-  double wv[NB];
-  for (int q = 0; q < NB; ++q) {
-    double s = 0.0;
-    for (int z = 0; z < nz; ++z) s += Wp[((size_t)z * NB + q) * nt + col];
-    wv[q] = s;
+  double x = 0.0;
+  for (int z0 = 0; z0 < nz; z0 += 8) {
+    double t[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = z0 + u < nz ? Wp[((size_t)(z0 + u) * nt + col) * NB + lane] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (z0 + u < nz) x += t[u];
   }
-  for (int p = 0; p < NB; ++p) {
-    double s = 0.0;
-    for (int q = 0; q <= p && q < nbw; ++q) s += T[q * NB + p] * wv[q];
-    W2[(size_t)p * nt + col] = p < nbw ? s : 0.0;
-  }
+  x = lane < nbw ? x * tau[lane] : 0.0;
+  double g[NB];
+#pragma unroll
+  for (int q = 0; q < NB; ++q) g[q] = G[lane * NB + q];  // 0 for q >= lane
+#pragma unroll
+  for (int q = 0; q < NB; ++q) x = fma(-g[q], __shfl_sync(0xffffffffu, x, q), x);
+  W2[(size_t)lane * nt + col] = x;
 }
 
 // A[r, j1 + col] -= sum_p v_p(r) W2[p][col] for r in [j0, s)
@@ -373,10 +589,11 @@ __global__ void k_floor(double* __restrict__ A, long long lda, long long n, unsi
 }
 
 struct QrScratch {
-  double* part;
-  double* gram;
+  unsigned long long* xch;  // exchange records of k_block
+  double* part;             // its partial products of the in-block update
+  double* bw2;              // and their W2
   double* tau;
-  double* T;
+  double* G;
   double* Wp;
   double* W2;
   double* dg;
@@ -384,10 +601,16 @@ struct QrScratch {
 
 }  // namespace
 
+// Doubles of the panel scratch: exchange records, in-block partials and W2 of
+// k_block, tau, G, and the split-K partials, W2 and diagonal of the trailing update.
+__host__ __device__ constexpr long long qr_scratch_len(long long n) {
+  return 2LL * KB_SLOT + (long long)KB_MAXP * 3 * NB * NB + 3LL * NB * NB + n + NB * NB + 64LL * NB * n + NB * n + n +
+         64;
+}
+
 long long rfm_householder_scratch(long long s, long long n) {
-  const long long P = 1024;
-  const long long maxz = 64;
-  return P * (NB + 2) + P * NB * NB + n + NB * NB + maxz * NB * n + NB * n + n + 64;
+  (void)s;
+  return qr_scratch_len(n);
 }
 
 namespace {
@@ -395,18 +618,19 @@ namespace {
 QrScratch carve(double* scratch, long long n) {
   QrScratch q;
   double* w = scratch;
-  q.part = w; w += 1024 * (NB + 2);
-  q.gram = w; w += 1024LL * NB * NB;
-  q.tau = w; w += n;
-  q.T = w; w += NB * NB;
+  q.xch = reinterpret_cast<unsigned long long*>(w); w += 2LL * KB_SLOT;
+  q.part = w; w += (long long)KB_MAXP * 3 * NB * NB;
+  q.bw2 = w; w += 3LL * NB * NB;
+  q.G = w; w += NB * NB;
   q.Wp = w; w += 64LL * NB * n;
   q.W2 = w; w += (long long)NB * n;
+  q.tau = w; w += n;
   q.dg = w;
   return q;
 }
 
 rfm_status qr_init_device() {
-  const cudaError_t attr = rfm_smem_attr((const void*)k_panel, 200 * 1024);  // once per device
+  const cudaError_t attr = rfm_smem_attr((const void*)k_block, KB_SMEM);  // once per device
   if (attr != cudaSuccess || rfm_num_sms() == 0) {
     rfm_set_error("householder: device set-up failed");
     return RFM_ECUDA;
@@ -414,55 +638,105 @@ rfm_status qr_init_device() {
   return RFM_OK;
 }
 
-// Householder factorisation of columns [c0, c1) (rows c0..s) in NB-wide
-// panels; the FP64 compact-WY update of each panel is applied to the columns
-// up to cend (cend >= c1).
-rfm_status factor_range(double* A, long long s, long long lda, long long c0, long long c1, long long cend,
-                        cudaStream_t st, const QrScratch& q, unsigned int* sync, int panel_cap) {
-  unsigned int* bar = sync + SYNC_BAR;
-  unsigned int* err = sync + SYNC_ERR;
+// Rows of k_block's slab for np 32-column groups.
+long long kb_max_rows(int np) { return (long long)((KB_SMEM - kb_fixed_smem()) / (NB * np * sizeof(double))); }
+
+// Widest block (32 .. 128 columns) that k_block can hold in shared memory for
+// `rows` rows on all SMs.
+int kb_width(long long rows) {
+  const long long per = (rows + rfm_num_sms() - 1) / rfm_num_sms();
+  for (int np = 4; np > 1; --np)
+    if (per <= kb_max_rows(np)) return np * NB;
+  return NB;
+}
+
+// State of one factorisation's exchange: barrier arrivals so far.
+struct KbState {
+  unsigned int arrived = 0;
+};
+
+rfm_status kb_begin(const QrScratch& q, unsigned int* sync, cudaStream_t st) {
+  // tags and barrier count of an earlier factorisation must not be mistaken for this one's
+  RFM_CUDA(cudaMemsetAsync(q.xch, 0, 2LL * KB_SLOT * sizeof(unsigned long long), st));
+  RFM_CUDA(cudaMemsetAsync(sync + SYNC_BAR, 0, sizeof(unsigned int), st));
+  return RFM_OK;
+}
+
+// Factors columns [c0, c0 + nb) (rows c0..s) in place, nb <= kb_width.
+rfm_status factor_block(double* A, long long s, long long lda, long long c0, int nb, cudaStream_t st,
+                        const QrScratch& q, unsigned int* sync, int panel_cap, KbState* ks) {
+  const long long rows = s - c0;
+  const int np = (nb + NB - 1) / NB;
   const int nsm = rfm_num_sms();
-  for (long long j0 = c0; j0 < c1; j0 += NB) {
-    const int nbw = (int)std::min<long long>(NB, c1 - j0);
-    const long long rows = s - j0;
-    // rows per CTA: at least 64, at most what fits in 200 KB of shared memory
-    const long long maxchunk = (200LL * 1024) / (NB * (long long)sizeof(double));
-    const long long cap = panel_cap > 0 ? std::min(panel_cap, nsm) : nsm;
-    long long P = std::min<long long>(std::min<long long>((rows + 63) / 64, cap), 256);  // k_panel sums <= 256 partials
-    if (P < 1) P = 1;
-    long long chunk = (rows + P - 1) / P;
-    if (chunk > maxchunk && cap < nsm) {  // the cap would overflow shared memory: take the fewest CTAs that fit
-      P = std::min<long long>((rows + maxchunk - 1) / maxchunk, nsm);
-      chunk = (rows + P - 1) / P;
-    }
-    if (chunk > maxchunk) {
+  // In 31 ns instructions a 32-column panel costs rows / (2 P) a column for its
+  // products and updates, P / 4 for the sum over P CTAs and, with columns to
+  // the right in the block, rows / P a column for their update: least at
+  // P^2 = 2 rows (one panel) or 6 rows (a block of four).
+  const double opt = sqrt((np > 1 ? 6.0 : 2.0) * (double)rows);
+  const long long cap = std::min<long long>(panel_cap > 0 ? std::min(panel_cap, nsm) : nsm, KB_MAXP);
+  long long P = std::max<long long>(1, std::min<long long>((long long)opt, cap));
+  long long chunk = (rows + P - 1) / P;
+  const long long most = kb_max_rows(np);
+  if (chunk > most) {  // a cap would overflow shared memory: take the fewest CTAs that fit
+    chunk = most;
+    P = (rows + most - 1) / most;
+    if (P > std::min(nsm, KB_MAXP)) {
       rfm_set_error("householder: sketch too tall for the panel kernel");
       return RFM_EINVAL;
     }
-    PanelArgs a;
-    a.A = A; a.lda = lda; a.s = s; a.j0 = j0; a.nbw = nbw; a.P = (int)P; a.chunk = (int)chunk;
-    a.part = q.part; a.gram = q.gram; a.tau = q.tau; a.T = q.T; a.bar = bar; a.err = err;
-    void* args[] = {&a};
-    const size_t smem = (size_t)NB * chunk * sizeof(double);
-    {
-      ProfScope ps(PF_QR_PANEL, st);
-      RFM_CUDA(cudaLaunchCooperativeKernel((const void*)k_panel, dim3((unsigned)P), dim3(256), args, smem, st));
-      rfm_count_launch();
-    }
+    chunk = (rows + P - 1) / P;
+  }
+  P = (rows + chunk - 1) / chunk;  // no CTA without rows
+  BlockArgs a;
+  a.A = A; a.lda = lda; a.s = s; a.j0 = c0; a.nb = nb; a.P = (int)P; a.chunk = (int)chunk;
+  a.xch = q.xch; a.part = q.part; a.w2 = q.bw2; a.tau = q.tau; a.G = q.G;
+  a.bar = sync + SYNC_BAR; a.bar0 = ks->arrived; a.err = sync + SYNC_ERR;
+  ks->arrived += 2u * (unsigned)(np - 1) * (unsigned)P;
+  void* args[] = {&a};
+  const size_t smem = kb_fixed_smem() + (size_t)NB * np * chunk * sizeof(double);
+  ProfScope ps(PF_QR_PANEL, st);
+  RFM_CUDA(cudaLaunchCooperativeKernel((const void*)k_block, dim3((unsigned)P), dim3(KB_THREADS), args, smem, st));
+  rfm_count_launch();
+  return RFM_OK;
+}
+
+// Householder factorisation of columns [c0, c1) (rows c0..s); the reflectors
+// are applied in FP64 to the columns up to cend (cend >= c1).  Without columns
+// past c1 the blocks are as wide as shared memory allows (k_block updates
+// inside them); with them, 32 columns at a time.
+rfm_status factor_range(double* A, long long s, long long lda, long long c0, long long c1, long long cend,
+                        cudaStream_t st, const QrScratch& q, unsigned int* sync, int panel_cap, KbState* ks) {
+  const int nsm = rfm_num_sms();
+  if (cend == c1 && kb_width(s - c0) >= c1 - c0)
+    return factor_block(A, s, lda, c0, (int)(c1 - c0), st, q, sync, panel_cap, ks);
+  for (long long j0 = c0; j0 < c1; j0 += NB) {
+    const int nbw = (int)std::min<long long>(NB, c1 - j0);
+    const long long rows = s - j0;
+    RFM_TRY(factor_block(A, s, lda, j0, nbw, st, q, sync, panel_cap, ks));
     const long long j1 = j0 + nbw;
     const long long nt = cend - j1;
     if (nt <= 0) continue;
     const long long ctiles = (nt + 63) / 64;
-    long long nz = (2LL * nsm + ctiles - 1) / ctiles;
-    nz = std::max<long long>(1, std::min<long long>(nz, std::min<long long>(64, (rows + 255) / 256)));
-    const long long kchunk = (rows + nz - 1) / nz;
+    // K slices of whole 32-row steps: the count that leaves the fewest steps on
+    // the busiest SM (FP64 bound, so co-resident CTAs only share the unit)
+    const long long steps = (rows + 31) / 32;
+    long long nz = 1, best = -1;
+    for (long long z = 1; z <= std::min<long long>(64, steps); ++z) {
+      const long long per = (steps + z - 1) / z, zz = (steps + per - 1) / per;
+      const long long cost = ((ctiles * zz + nsm - 1) / nsm) * per * 64 + zz;  // + k_wt's sum over slices
+      if (best < 0 || cost < best) {
+        best = cost;
+        nz = zz;
+      }
+    }
+    const long long kchunk = (steps + nz - 1) / nz * 32;
     nz = (rows + kchunk - 1) / kchunk;
     {
       ProfScope ps(PF_QR_VTA, st);
       rfm_prof_work(PF_QR_VTA, 2.0 * nbw * (double)nt * (double)rows);  // FP64 flops
       k_vta<<<dim3((unsigned)ctiles, (unsigned)nz), 256, 0, st>>>(A, lda, s, j0, nbw, j1, nt, kchunk, q.Wp);
       RFM_CHECK_LAUNCH();
-      k_wt<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>(q.Wp, (int)nz, q.T, nbw, nt, q.W2);
+      k_wt<<<(unsigned)((nt + 3) / 4), 128, 0, st>>>(q.Wp, (int)nz, q.G, q.tau + j0, nbw, nt, q.W2);
       RFM_CHECK_LAUNCH();
     }
     ProfScope psu(PF_QR_UPDATE, st);
@@ -512,9 +786,10 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
   }
   RFM_TRY(qr_init_device());
   const QrScratch q = carve(scratch, n);
-  RFM_CUDA(cudaMemsetAsync(sync + SYNC_BAR, 0, 2 * sizeof(unsigned int), st));
+  KbState ks;
+  RFM_TRY(kb_begin(q, sync, st));
   const long long c1 = ncols < 0 ? n : std::min<long long>(n, ((ncols + NB - 1) / NB) * NB);
-  RFM_TRY(factor_range(A, s, lda, 0, c1, n, st, q, sync, panel_cap));
+  RFM_TRY(factor_range(A, s, lda, 0, c1, n, st, q, sync, panel_cap, &ks));
   return finish_r(A, n, lda, st, q, sync, rank_flag_host);
 }
 
@@ -526,7 +801,7 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
 // front through their own pool (where a cudaMalloc fails or implicitly
 // synchronises the device and stalls other streams), or loops with fixed
 // latency budgets.  The QR scratch lives in file-scope device arrays of fixed
-// size (17.2 MB of scratch + 16 KB of barrier words per GPU that loads the
+// size (15.1 MB of scratch + 16 KB of barrier words per GPU that loads the
 // library, held until the process exits), sized for n <= 512 columns.
 // Every call shares these arrays and they keep the last call's contents;
 // calls that overlap on the GPU (two streams, or two host threads) race on
@@ -535,9 +810,7 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
 #define RFM_NOALLOC_MAX_DEVICES 64
 
 namespace {
-constexpr long long kNoallocScratch = 1024LL * (NB + 2) + 1024LL * NB * NB + RFM_NOALLOC_MAX_N + NB * NB +
-                                      64LL * NB * RFM_NOALLOC_MAX_N + (long long)NB * RFM_NOALLOC_MAX_N +
-                                      RFM_NOALLOC_MAX_N + 64;
+constexpr long long kNoallocScratch = qr_scratch_len(RFM_NOALLOC_MAX_N);
 }  // namespace
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocScratch];
@@ -647,27 +920,37 @@ namespace {
 constexpr int QB = 128;
 constexpr int QDIG = 8;
 
-// T from G and tau, column by column.  One CTA of QB threads; T is kept in
-// dynamic shared memory (QB x (QB+1) doubles).
-__global__ void k_block_t(const double* __restrict__ G, const double* __restrict__ tau, int nbw,
-                          double* __restrict__ T) {
-  extern __shared__ double Ts[];  // [QB][QB + 1]
-  for (int idx = threadIdx.x; idx < QB * (QB + 1); idx += blockDim.x) Ts[idx] = 0.0;
-  __syncthreads();
-  const int i = threadIdx.x;
-  for (int j = 0; j < nbw; ++j) {
-    const double tj = tau[j];
-    double v = 0.0;
-    if (i < j) {
-      for (int l = i; l < j; ++l) v += Ts[i * (QB + 1) + l] * G[l * QB + j];
-      v = -tj * v;
-    }
-    __syncthreads();
-    if (i < j) Ts[i * (QB + 1) + j] = v;
-    if (i == j) Ts[j * (QB + 1) + j] = tj;
-    __syncthreads();
+// T from G and tau: T^-1 = diag(1 / tau) + strict upper part of G, so column j
+// of T is a back substitution, t_j = tau_j, t_i = -tau_i sum_{l>i} G_il t_l (no
+// division; tau_i = 0 gives a zero row).  One warp per column, lane L holding
+// rows L, L + 32, ..: the columns are independent, and a step is one shuffle
+// and at most four FP64 instructions.  (Column after column on one CTA, whose
+// FP64 unit had to do all of it, took 447 us for 128 columns.)
+__global__ void __launch_bounds__(128) k_block_t(const double* __restrict__ G, const double* __restrict__ tau,
+                                                 int nbw, double* __restrict__ T) {
+  const int lane = threadIdx.x & 31;
+  const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
+  double t[QB / 32], tu[QB / 32];
+#pragma unroll
+  for (int u = 0; u < QB / 32; ++u) {
+    const int i = lane + 32 * u;
+    t[u] = i == j && j < nbw ? 1.0 : 0.0;  // e_j, then the right-hand side less the solved part
+    tu[u] = i < nbw ? tau[i] : 0.0;
   }
-  for (int idx = threadIdx.x; idx < QB * QB; idx += blockDim.x) T[idx] = Ts[(idx / QB) * (QB + 1) + idx % QB];
+#pragma unroll
+  for (int h = QB / 32 - 1; h >= 0; --h)  // row l = 32 h + ll is held in t[h]
+    for (int l = min(min(j, nbw - 1), 32 * h + 31); l >= 32 * h; --l) {
+      if (lane == (l & 31)) t[h] *= tu[h];
+      const double y = __shfl_sync(0xffffffffu, t[h], l & 31);
+#pragma unroll
+      for (int u = 0; u <= h; ++u)
+        if (u < h || lane < (l & 31)) t[u] = fma(-G[(size_t)l * QB + lane + 32 * u], y, t[u]);
+    }
+#pragma unroll
+  for (int u = 0; u < QB / 32; ++u) {
+    const int i = lane + 32 * u;
+    T[(size_t)i * QB + j] = i <= j && j < nbw ? t[u] : 0.0;
+  }
 }
 
 
@@ -697,11 +980,6 @@ rfm_status rfm_householder_emulated(double* A, long long s, long long n, long lo
     return RFM_EINVAL;
   }
   RFM_TRY(qr_init_device());
-  const cudaError_t t_attr = rfm_smem_attr((const void*)k_block_t, (int)(QB * (QB + 1) * sizeof(double)));
-  if (t_attr != cudaSuccess) {
-    rfm_set_error("householder: k_block_t shared-memory attribute");
-    return RFM_ECUDA;
-  }
   const QrScratch q = carve(scratch, n);
   char* w = static_cast<char*>(emu);
   auto take = [&](long long bytes) {
@@ -723,14 +1001,15 @@ rfm_status rfm_householder_emulated(double* A, long long s, long long n, long lo
   int* e_v = reinterpret_cast<int*>(take(4LL * s));
   int* e_w2 = reinterpret_cast<int*>(take(4LL * n));
   unsigned int* err = sync + SYNC_ERR;
-  RFM_CUDA(cudaMemsetAsync(sync + SYNC_BAR, 0, 2 * sizeof(unsigned int), st));
+  KbState ks;
+  RFM_TRY(kb_begin(q, sync, st));
   const long long cstop = ncols < 0 ? n : std::min<long long>(n, ncols);
   for (long long J0 = 0; J0 < cstop; J0 += QB) {
     const long long c1 = std::min<long long>(n, J0 + QB);
     const int nbw = (int)(c1 - J0);
     const long long rows = s - J0;
     const long long nt = n - c1;
-    RFM_TRY(factor_range(A, s, lda, J0, c1, c1, st, q, sync, panel_cap));
+    RFM_TRY(factor_range(A, s, lda, J0, c1, c1, st, q, sync, panel_cap, &ks));
     if (nt <= 0) break;
     {
       // One emulated product gives the block's Gram and V^T A_t: its B operand
@@ -746,7 +1025,7 @@ rfm_status rfm_householder_emulated(double* A, long long s, long long n, long lo
                                       st));
       RFM_TRY(rfm_oz_gemm_part(d_vt, QDIG, e_vt, d_at, QDIG, e_at, nbw, QB + nt, rows, QDIG + 1, Wm, QB, 0, err, st,
                                part, part_elems));
-      k_block_t<<<1, QB, QB * (QB + 1) * sizeof(double), st>>>(Wm, q.tau + J0, nbw, T);
+      k_block_t<<<QB / 4, 128, 0, st>>>(Wm, q.tau + J0, nbw, T);
       RFM_CHECK_LAUNCH();
       // W2 = T^T W on the emulated GEMM as well (M = K = 128, N = nt): the
       // digit buffers of V^T and of W2 are free at this point of the stream.
