@@ -45,21 +45,29 @@ constexpr int NB = 32;
 //    of the panel.  sqrt and the reciprocal are one third-order step
 //    (Householder's iteration) from an FP32 seed, 18 instructions where the
 //    library's sqrt and two divisions take 28 (0.86 us).
-//  - the CTAs exchange their 32 sums as 16-byte records {low, tag, high, tag}
-//    whose tag is the column's number: a reader polls the records themselves,
-//    so there is no fence, no counter and no second trip to L2.  Two slots
-//    alternate; a CTA can only be one exchange ahead of another.
+//  - the 32 sums are first combined in clusters of four CTAs (each rank sums
+//    eight columns of the 16 warps, through distributed shared memory and one
+//    cluster barrier, 0.2 us), then between the clusters as 16-byte records
+//    {low, tag, high, tag} whose tag is the column's number: a reader polls the
+//    records themselves, so there is no fence, no counter and no second trip to
+//    L2.  Two slots alternate; a CTA can only be one exchange ahead of another.
+//    (With a record per CTA every CTA read 78 KB per column, which is L2 bound,
+//    and added 38 records per warp.)  Four is the largest cluster that still
+//    puts a CTA on 144 of the 152 SMs (eight: 120).
 // Between the panels of a block, the block's remaining columns (in the same
 // shared-memory slab) are updated with W = V^T A, W2 = T^T W, A -= V W2: CTA c
 // sums column c of W over the CTAs and solves for its column of W2.
 //
-// Times per column at 12,288 rows: 16.5 us with one grid barrier and a
-// redundant butterfly reduction per column (k_panel, 32 columns per launch).
+// Per column at 12,288 rows: 16.5 us with one grid barrier and a redundant
+// butterfly reduction per column (the former panel kernel), now 5.2 us (0.95
+// products, 0.4 cluster barrier, 0.25 publish, 1.7 poll and sums, 1.05 scalars,
+// 0.8 update); a 128-column block with its in-block updates 3.7 -> 0.94 ms.
 constexpr int KB_THREADS = 128;
 constexpr int KB_SMEM = 227 * 1024;              // dynamic shared memory of a CTA
+constexpr int KB_CL = 4;                         // CTAs of a cluster
 constexpr int KB_MAXP = 256;                     // CTAs of one factorisation
-constexpr int KB_POLL = 19;                      // records in flight per lane and poll round
-constexpr int KB_SLOT = (KB_MAXP + 1) * NB * 2;  // 8-byte words of one exchange slot (row P: the pivot row)
+constexpr int KB_POLL = 10;                      // records in flight per lane and poll round
+constexpr int KB_SLOT = (KB_MAXP / KB_CL + 1) * NB * 2;  // 8-byte words of an exchange slot (last record: the pivot row)
 
 struct BlockArgs {
   double* A;
@@ -67,11 +75,11 @@ struct BlockArgs {
   long long s;
   long long j0;
   int nb;              // columns of the block (<= 128)
-  int P;               // CTAs
+  int P;               // CTAs (a multiple of KB_CL)
   int chunk;           // rows per CTA
   unsigned long long* xch;  // [2][KB_SLOT] exchange records
   double* part;        // [P][3 NB][NB] partial W of the in-block update
-  double* w2;          // [3 NB][NB]
+  double* w2;          // [NB][3 NB]
   double* tau;         // [n]
   double* G;           // [NB][NB] of the last panel: G[p * NB + q] = tau_p v_q^T v_p for q < p, else 0
   unsigned int* bar;   // arrival counter of the grid barriers
@@ -115,6 +123,18 @@ __device__ __forceinline__ void kb_barrier(unsigned int* bar, unsigned int want,
   __syncthreads();
 }
 
+// Store to the same shared-memory variable of rank `rank` of the cluster.
+__device__ __forceinline__ void kb_store_cluster(double* p, int rank, double v) {
+  asm volatile(
+      "{\n .reg .b32 r;\n mapa.shared::cluster.u32 r, %0, %1;\n st.shared::cluster.f64 [r], %2;\n}\n" ::"r"(
+          (unsigned)__cvta_generic_to_shared(p)),
+      "r"(rank), "d"(v)
+      : "memory");
+}
+__device__ __forceinline__ void kb_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ void kb_publish(unsigned long long* rec, double v, unsigned int tag) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   const unsigned long long lo = (b & 0xffffffffull) | ((unsigned long long)tag << 32);
@@ -131,6 +151,9 @@ __device__ __forceinline__ bool kb_ready(unsigned long long lo, unsigned long lo
 __device__ __forceinline__ double kb_value(unsigned long long lo, unsigned long long hi) {
   return __longlong_as_double((long long)((lo & 0xffffffffull) | (hi << 32)));
 }
+
+// x != 0 (true for NaN) without an FP64 compare.
+__device__ __forceinline__ bool kb_nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 
 // norm = sqrt(alpha^2 + sigma) and gamma = 1 / (norm^2 + |alpha| norm) for
 // sigma > 0.  In the scaled variables m = t 2^-e in [1, 4) (e even), the
@@ -176,10 +199,57 @@ __device__ __forceinline__ void kb_copy8(double* dst, const double* src) {
                : "memory");
 }
 
+// In-block W = V^T A of a CTA's rows: lanes are the columns of a group, warp w
+// takes p = 8 w .. 8 w + 7, NG groups of columns follow the panel at p0.
+template <int NG>
+__device__ __forceinline__ void kb_wpart(const double* sl, int ld, int p0, int r0, int nr, int w, int lane,
+                                         double* out) {
+  double acc[NG][8];
+#pragma unroll
+  for (int g = 0; g < NG; ++g)
+#pragma unroll
+    for (int p = 0; p < 8; ++p) acc[g][p] = 0.0;
+#pragma unroll 2
+  for (int r = r0; r < nr; ++r) {
+    double av[NG], v[8];
+#pragma unroll
+    for (int g = 0; g < NG; ++g) av[g] = sl[kb_at(r, p0 + NB * (g + 1) + lane, ld)];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) v[p] = sl[kb_at(r, p0 + 8 * w + p, ld)];
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+      for (int g = 0; g < NG; ++g) acc[g][p] = fma(v[p], av[g], acc[g][p]);
+  }
+#pragma unroll
+  for (int g = 0; g < NG; ++g)
+#pragma unroll
+    for (int p = 0; p < 8; p += 2)
+      __stcg(reinterpret_cast<double2*>(out + (g * NB + lane) * NB + 8 * w + p),
+             make_double2(acc[g][p], acc[g][p + 1]));
+}
+
+// In-block A -= V W2 of a CTA's rows for the column group at pc: a lane keeps
+// its column of W2.
+__device__ __forceinline__ void kb_wupdate(double* sl, int ld, int p0, int pc, int r0, int nr, int w, int lane,
+                                           const double* w2) {
+  double y[NB];
+#pragma unroll
+  for (int p = 0; p < NB; ++p) y[p] = __ldcg(w2 + p * (3 * NB) + lane);
+  for (int r = r0 + ((w - r0) & 3); r < nr; r += 4) {
+    double* e = sl + kb_at(r, pc + lane, ld);
+    const double* v = sl + r * ld + p0;
+    double x = *e;
+#pragma unroll
+    for (int p = 0; p < NB; ++p) x = fma(-v[(p ^ r) & 31], y[p], x);
+    *e = x;
+  }
+}
+
 __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
   extern __shared__ __align__(16) double kb_sm[];
   double* Gs = kb_sm;              // tau_p v_q^T v_p of the panel at kb_tri(p, q), q < p
-  double* wp = Gs + KB_TRI;       // [4][NB] the warps' partial sums
+  double* wp = Gs + KB_TRI;        // [4][4][8] partial sums of this rank's 8 columns, by CTA and warp of the cluster
   double* rs = wp + 4 * NB;        // [4][NB] the warps' shares of the sums over CTAs
   double* pv = rs + 4 * NB;        // [NB] pivot row
   double* dab = pv + NB;           // [NB] alpha - beta
@@ -189,6 +259,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
   double* sl = kb_sm + (kb_fixed_smem() / sizeof(double));  // slab [rows][ld]
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int c = blockIdx.x, P = a.P;
+  const int rank = c % KB_CL, cl = c / KB_CL, ncl = P / KB_CL;
   const long long rbeg = a.j0 + (long long)c * a.chunk;
   const long long rend = min(a.s, rbeg + a.chunk);
   const int nr = rbeg < rend ? (int)(rend - rbeg) : 0;
@@ -208,7 +279,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
+  kb_cluster_sync();  // all ranks run: their shared memory may be written
   for (int pi = 0; pi < np; ++pi) {
     const int p0 = pi * NB, nbw = min(NB, a.nb - p0);
     for (int jj = 0; jj < nbw; ++jj) {
@@ -218,37 +289,51 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
       const int lr = j + 1 > rbeg ? (int)min((long long)nr, j + 1 - rbeg) : 0;  // rows below the pivot
       const int rw = lr + ((w - lr) & 3);                                       // this warp's first one
       double acc = 0.0;
+      if (rw < nr) {  // the next row's loads go ahead of a row's instruction
+        const int last = nr - 1 - ((nr - 1 - rw) & 3);
+        double x = sl[kb_at(rw, p0 + jj, ld)], e = sl[kb_at(rw, p0 + lane, ld)];
 #pragma unroll 4
-      for (int r = rw; r < nr; r += 4) acc = fma(sl[kb_at(r, p0 + jj, ld)], sl[kb_at(r, p0 + lane, ld)], acc);
-      wp[w * NB + lane] = acc;
-      __syncthreads();
-      if (w == 0) {
-        const double sm = (wp[lane] + wp[NB + lane]) + (wp[2 * NB + lane] + wp[3 * NB + lane]);
-        kb_publish(slot + ((size_t)c * NB + lane) * 2, sm, tag);
-      } else if (w == 1 && j >= rbeg && j < rend) {
-        kb_publish(slot + ((size_t)P * NB + lane) * 2, sl[kb_at((int)(j - rbeg), p0 + lane, ld)], tag);
+        for (int r = rw; r < last; r += 4) {
+          const double xn = sl[kb_at(r + 4, p0 + jj, ld)], en = sl[kb_at(r + 4, p0 + lane, ld)];
+          acc = fma(x, e, acc);
+          x = xn;
+          e = en;
+        }
+        acc = fma(x, e, acc);
       }
-      // sum over the CTAs, warp w the CTAs w, w + 4, ... in increasing order;
-      // record P is the pivot row
+      kb_store_cluster(wp + (rank * 4 + w) * 8 + (lane & 7), lane >> 3, acc);
+      kb_cluster_sync();
+      if (w == 0) {
+        const double* x = wp + (lane >> 3) * 32 + (lane & 7);
+        double sm = (x[0] + x[8]) + (x[16] + x[24]);
+        sm += __shfl_xor_sync(0xffffffffu, sm, 8);
+        sm += __shfl_xor_sync(0xffffffffu, sm, 16);
+        if (lane < 8) kb_publish(slot + ((size_t)cl * NB + rank * 8 + lane) * 2, sm, tag);
+      } else if (w == 1 && j >= rbeg && j < rend) {
+        kb_publish(slot + ((size_t)ncl * NB + lane) * 2, sl[kb_at((int)(j - rbeg), p0 + lane, ld)], tag);
+      }
+      // sum over the clusters, warp w the clusters w, w + 4, ... in increasing
+      // order; record ncl is the pivot row.  A complete record of this cluster
+      // also says that all its ranks have read wp.
       double sum = 0.0;
-      for (int q0 = w; q0 <= P; q0 += 4 * KB_POLL) {
+      for (int q0 = w; q0 <= ncl; q0 += 4 * KB_POLL) {
         unsigned long long lo[KB_POLL], hi[KB_POLL];
         unsigned int spins = 0;
         for (;;) {
           bool all = true;
 #pragma unroll
           for (int i = 0; i < KB_POLL; ++i)
-            if (q0 + 4 * i <= P) kb_load(slot + ((size_t)(q0 + 4 * i) * NB + lane) * 2, lo[i], hi[i]);
+            if (q0 + 4 * i <= ncl) kb_load(slot + ((size_t)(q0 + 4 * i) * NB + lane) * 2, lo[i], hi[i]);
 #pragma unroll
           for (int i = 0; i < KB_POLL; ++i)
-            if (q0 + 4 * i <= P) all = all && kb_ready(lo[i], hi[i], tag);
+            if (q0 + 4 * i <= ncl) all = all && kb_ready(lo[i], hi[i], tag);
           if (__all_sync(0xffffffffu, all) || !__all_sync(0xffffffffu, kw.spin(spins))) break;
         }
 #pragma unroll
         for (int i = 0; i < KB_POLL; ++i) {
           const int q = q0 + 4 * i;
-          if (q < P) sum += kb_value(lo[i], hi[i]);
-          else if (q == P) pv[lane] = kb_value(lo[i], hi[i]);
+          if (q < ncl) sum += kb_value(lo[i], hi[i]);
+          else if (q == ncl) pv[lane] = kb_value(lo[i], hi[i]);
         }
       }
       rs[w * NB + lane] = sum;
@@ -258,10 +343,10 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
       const double alpha = pv[jj];
       const double sigma = __shfl_sync(0xffffffffu, tot, jj);
       double dj = 0.0, gj = 0.0, beta = alpha;
-      if (sigma != 0.0) {
+      if (kb_nonzero(sigma)) {
         double nrm;
         kb_norm_gamma(alpha, sigma, nrm, gj);
-        beta = alpha >= 0.0 ? -nrm : nrm;
+        beta = __double2hiint(alpha) < 0 && kb_nonzero(alpha) ? nrm : -nrm;
         dj = alpha - beta;
       }
       // u^T a_k for the columns to the right, u_k^T u for those to the left
@@ -275,24 +360,42 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
         }
       }
       if (jj < 16) {
+        if (rw < nr) {
+          const int last = nr - 1 - ((nr - 1 - rw) & 3);
+          double x = sl[kb_at(rw, p0 + jj, ld)], e = sl[kb_at(rw, p0 + lane, ld)];
 #pragma unroll 4
-        for (int r = rw; r < nr; r += 4) {
-          double* e = sl + kb_at(r, p0 + lane, ld);
-          *e = fma(-f, sl[kb_at(r, p0 + jj, ld)], *e);
+          for (int r = rw; r < last; r += 4) {
+            const double xn = sl[kb_at(r + 4, p0 + jj, ld)], en = sl[kb_at(r + 4, p0 + lane, ld)];
+            sl[kb_at(r, p0 + lane, ld)] = fma(-f, x, e);
+            x = xn;
+            e = en;
+          }
+          sl[kb_at(last, p0 + lane, ld)] = fma(-f, x, e);
         }
       } else {
         // only columns 16 .. 31 are left: two rows per instruction
-        const int cl = 16 + (lane & 15);
-        const double fh = __shfl_sync(0xffffffffu, f, cl);
-#pragma unroll 4
-        for (int r = rw; r < nr; r += 8) {
-          const int rr = r + 4 * (lane >> 4);
-          if (rr < nr) {
-            double* e = sl + kb_at(rr, p0 + cl, ld);
-            const double x = sl[kb_at(rr, p0 + jj, ld)];
-            if (cl > jj) *e = fma(-fh, x, *e);
+        const int ch = 16 + (lane & 15);
+        const double fh = __shfl_sync(0xffffffffu, f, ch);
+        int r = rw + 4 * (lane >> 4);
+        for (; r + 24 < nr; r += 32) {
+          double x[4], e[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            x[u] = sl[kb_at(r + 8 * u, p0 + jj, ld)];
+            e[u] = sl[kb_at(r + 8 * u, p0 + ch, ld)];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            e[u] = fma(-fh, x[u], e[u]);
+            if (ch > jj) sl[kb_at(r + 8 * u, p0 + ch, ld)] = e[u];
           }
         }
+        for (; r < nr; r += 8) {
+          double* e = sl + kb_at(r, p0 + ch, ld);
+          const double x = fma(-fh, sl[kb_at(r, p0 + jj, ld)], *e);
+          if (ch > jj) *e = x;
+        }
+        __syncwarp();
       }
       if (j >= rbeg && j < rend && w == ((int)(j - rbeg) & 3)) {  // the pivot row itself
         double* e = sl + kb_at((int)(j - rbeg), p0 + lane, ld);
@@ -335,36 +438,12 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
     }
     __syncthreads();
     const int ng = np - 1 - pi;  // column groups to the right in the block
-    if (ng == 0) break;
-    // W = V^T A: lanes are the columns of a group, warp w takes p = 8 w .. 8 w + 7
-    {
-      double acc[3][8];
-#pragma unroll
-      for (int g = 0; g < 3; ++g)
-#pragma unroll
-        for (int p = 0; p < 8; ++p) acc[g][p] = 0.0;
-      const long long first = a.j0 + p0;
-      for (int r = first > rbeg ? (int)min((long long)nr, first - rbeg) : 0; r < nr; ++r) {
-        double av[3];
-#pragma unroll
-        for (int g = 0; g < 3; ++g) av[g] = g < ng ? sl[kb_at(r, p0 + NB * (g + 1) + lane, ld)] : 0.0;
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-          const double v = sl[kb_at(r, p0 + 8 * w + p, ld)];
-#pragma unroll
-          for (int g = 0; g < 3; ++g)
-            if (g < ng) acc[g][p] = fma(v, av[g], acc[g][p]);
-        }
-      }
-#pragma unroll
-      for (int g = 0; g < 3; ++g)
-        if (g < ng) {
-          double* out = a.part + ((size_t)c * 3 * NB + g * NB + lane) * NB + 8 * w;
-#pragma unroll
-          for (int p = 0; p < 8; p += 2)
-            __stcg(reinterpret_cast<double2*>(out + p), make_double2(acc[g][p], acc[g][p + 1]));
-        }
-    }
+    if (ng == 0) break;  // the last cluster barrier came after the last remote store
+    const long long first = a.j0 + p0;
+    const int lv = first > rbeg ? (int)min((long long)nr, first - rbeg) : 0;  // rows before are zero in V
+    if (ng == 3) kb_wpart<3>(sl, ld, p0, lv, nr, w, lane, a.part + (size_t)c * 3 * NB * NB);
+    else if (ng == 2) kb_wpart<2>(sl, ld, p0, lv, nr, w, lane, a.part + (size_t)c * 3 * NB * NB);
+    else kb_wpart<1>(sl, ld, p0, lv, nr, w, lane, a.part + (size_t)c * 3 * NB * NB);
     barrier += P;
     kb_barrier(a.bar, barrier, kw);
     for (int col = c; col < ng * NB; col += P) {
@@ -390,34 +469,13 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
           const double y = __shfl_sync(0xffffffffu, x, q);
           if (lane > q && lane < nbw) x = fma(-Gs[kb_tri(lane, q)], y, x);
         }
-        __stcg(a.w2 + (size_t)col * NB + lane, x);
+        __stcg(a.w2 + lane * (3 * NB) + col, x);
       }
       __syncthreads();
     }
     barrier += P;
     kb_barrier(a.bar, barrier, kw);
-    // A -= V W2: a lane keeps its column of W2
-    {
-      const long long first = a.j0 + p0;
-      const int lr = first > rbeg ? (int)min((long long)nr, first - rbeg) : 0;
-      for (int g = 0; g < ng; ++g) {
-        double y[NB];
-        const double* src = a.w2 + (size_t)(g * NB + lane) * NB;
-#pragma unroll
-        for (int p = 0; p < NB; p += 2) {
-          const double2 t = __ldcg(reinterpret_cast<const double2*>(src + p));
-          y[p] = t.x;
-          y[p + 1] = t.y;
-        }
-        for (int r = lr + ((w - lr) & 3); r < nr; r += 4) {
-          double* e = sl + kb_at(r, p0 + NB * (g + 1) + lane, ld);
-          double x = *e;
-#pragma unroll
-          for (int p = 0; p < NB; ++p) x = fma(-sl[kb_at(r, p0 + p, ld)], y[p], x);
-          *e = x;
-        }
-      }
-    }
+    for (int g = 0; g < ng; ++g) kb_wupdate(sl, ld, p0, p0 + NB * (g + 1), lv, nr, w, lane, a.w2 + g * NB);
     __syncthreads();
   }
 }
@@ -638,13 +696,40 @@ rfm_status qr_init_device() {
   return RFM_OK;
 }
 
+// CTAs of k_block that can be resident together with the largest slab (whole
+// clusters; depends on how the device's SMs are grouped), per device; 0 on failure.
+int kb_max_ctas() {
+  static std::mutex mu;
+  static int cached[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  if (cached[dev] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = KB_CL;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(KB_CL);
+    cfg.blockDim = dim3(KB_THREADS);
+    cfg.dynamicSmemBytes = KB_SMEM;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_block, &cfg) != cudaSuccess) return 0;
+    cached[dev] = std::min(n * KB_CL, KB_MAXP);
+  }
+  return cached[dev];
+}
+
 // Rows of k_block's slab for np 32-column groups.
 long long kb_max_rows(int np) { return (long long)((KB_SMEM - kb_fixed_smem()) / (NB * np * sizeof(double))); }
 
 // Widest block (32 .. 128 columns) that k_block can hold in shared memory for
 // `rows` rows on all SMs.
 int kb_width(long long rows) {
-  const long long per = (rows + rfm_num_sms() - 1) / rfm_num_sms();
+  const long long ctas = std::max(1, kb_max_ctas());
+  const long long per = (rows + ctas - 1) / ctas;
   for (int np = 4; np > 1; --np)
     if (per <= kb_max_rows(np)) return np * NB;
   return NB;
@@ -667,36 +752,48 @@ rfm_status factor_block(double* A, long long s, long long lda, long long c0, int
                         const QrScratch& q, unsigned int* sync, int panel_cap, KbState* ks) {
   const long long rows = s - c0;
   const int np = (nb + NB - 1) / NB;
-  const int nsm = rfm_num_sms();
-  // In 31 ns instructions a 32-column panel costs rows / (2 P) a column for its
-  // products and updates, P / 4 for the sum over P CTAs and, with columns to
-  // the right in the block, rows / P a column for their update: least at
-  // P^2 = 2 rows (one panel) or 6 rows (a block of four).
-  const double opt = sqrt((np > 1 ? 6.0 : 2.0) * (double)rows);
-  const long long cap = std::min<long long>(panel_cap > 0 ? std::min(panel_cap, nsm) : nsm, KB_MAXP);
-  long long P = std::max<long long>(1, std::min<long long>((long long)opt, cap));
-  long long chunk = (rows + P - 1) / P;
-  const long long most = kb_max_rows(np);
-  if (chunk > most) {  // a cap would overflow shared memory: take the fewest CTAs that fit
-    chunk = most;
-    P = (rows + most - 1) / most;
-    if (P > std::min(nsm, KB_MAXP)) {
-      rfm_set_error("householder: sketch too tall for the panel kernel");
-      return RFM_EINVAL;
-    }
-    chunk = (rows + P - 1) / P;
+  const int ctas = kb_max_ctas();
+  if (ctas < KB_CL) {
+    rfm_set_error("householder: no cluster of the panel kernel fits on the device");
+    return RFM_ECUDA;
   }
-  P = (rows + chunk - 1) / chunk;  // no CTA without rows
+  // In 31 ns instructions a 32-column panel costs rows / (2 P) a column for its
+  // products and updates, P / 16 for the sum over the clusters of P CTAs and,
+  // with columns to the right in the block, rows / P a column for their update:
+  // least at P^2 = 8 rows (one panel) or 24 rows (a block of four).
+  const double opt = sqrt((np > 1 ? 24.0 : 8.0) * (double)rows);
+  const long long cap = panel_cap > 0 ? std::min(panel_cap, ctas) : ctas;
+  auto whole = [](long long v) { return std::max<long long>(KB_CL, v / KB_CL * KB_CL); };
+  long long P = whole(std::min<long long>((long long)opt, cap));
+  const long long most = kb_max_rows(np);
+  if ((rows + P - 1) / P > most)  // a cap would overflow shared memory: take the fewest clusters that fit
+    P = ((rows + most - 1) / most + KB_CL - 1) / KB_CL * KB_CL;
+  const long long chunk = (rows + P - 1) / P;
+  if (P > ctas || chunk > most) {
+    rfm_set_error("householder: sketch too tall for the panel kernel");
+    return RFM_EINVAL;
+  }
   BlockArgs a;
   a.A = A; a.lda = lda; a.s = s; a.j0 = c0; a.nb = nb; a.P = (int)P; a.chunk = (int)chunk;
   a.xch = q.xch; a.part = q.part; a.w2 = q.bw2; a.tau = q.tau; a.G = q.G;
   a.bar = sync + SYNC_BAR; a.bar0 = ks->arrived; a.err = sync + SYNC_ERR;
   ks->arrived += 2u * (unsigned)(np - 1) * (unsigned)P;
-  void* args[] = {&a};
-  const size_t smem = kb_fixed_smem() + (size_t)NB * np * chunk * sizeof(double);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: they wait on each other's records
+  at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = KB_CL;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)P);
+  cfg.blockDim = dim3(KB_THREADS);
+  cfg.dynamicSmemBytes = kb_fixed_smem() + (size_t)NB * np * chunk * sizeof(double);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   ProfScope ps(PF_QR_PANEL, st);
-  RFM_CUDA(cudaLaunchCooperativeKernel((const void*)k_block, dim3((unsigned)P), dim3(KB_THREADS), args, smem, st));
-  rfm_count_launch();
+  RFM_CUDA(cudaLaunchKernelEx(&cfg, k_block, a));
+  RFM_CHECK_LAUNCH();
   return RFM_OK;
 }
 
