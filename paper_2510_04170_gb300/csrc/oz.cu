@@ -90,10 +90,12 @@ __device__ __forceinline__ unsigned long long gtimer() {
 }
 // Bounded wait for completion of the phase with the given parity: gives up
 // after kWaitNs of wall time and records `code` in *err.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsigned* err, unsigned code) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsigned* err, unsigned code,
+                                          unsigned pause_ns = 0) {
   if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = gtimer();
   for (unsigned i = 1;; ++i) {
+    if (pause_ns) __nanosleep(pause_ns);
     if (mbar_try(bar, parity)) return true;
     if ((i & 255) == 0 && gtimer() - t0 > kWaitNs) break;
   }
@@ -117,7 +119,7 @@ __device__ __forceinline__ uint64_t umma_desc(const void* smem_tile) {
   return d;
 }
 // kind::f16 instruction descriptor: bf16 A and B (K-major), f32 accumulate,
-// M=128, N = 64 w (w = 1, 2 or 4 consecutive B digit tiles).
+// M=128, N = 64 w (w = 1 .. 4 consecutive B digit tiles).
 __host__ __device__ constexpr uint32_t idesc_n(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
@@ -137,36 +139,44 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {  // completed by tmem_wait
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+// The loaded registers pass through the wait, so no use can move above it.
+__device__ __forceinline__ void tmem_wait(uint32_t* a, uint32_t* b) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                 "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+               :
+               : "memory");
 }
 
-// Levels l0 .. l0+3 of 8 columns (levels >= nlev read as 0) combined exactly,
-// L_l0 2^(3 BETA) + L_(l0+1) 2^(2 BETA) + L_(l0+2) 2^BETA + L_(l0+3), and
-// added to acc[0..7].  (Eighteen warps leave 96 registers a thread, which the
-// accumulators largely fill, so one level is loaded per wait.)
-__device__ __forceinline__ void tmem_levels4(uint32_t cbase, int l0, int nlev, long long* acc) {
-  float v[8];
-  long long I[8];
+// Levels l and l + 1 of 8 columns (levels >= nlev are 0), times 2^SH and 2^(SH -
+// BETA), added to acc[0..7].  |L_l| <= 512 (2 2^13 + (l - 1) 2^12) for digits of
+// magnitude 2^7 (the top one) and 2^6, so L_l 2^BETA + L_(l+1) fits in 32 bits
+// up to l = 4 and one 32-bit and one wide multiply-add serve two levels; the
+// last pair (WIDE) takes two wide ones.  (Shifting and adding every level in
+// 64 bits made the drain of a 128 x 64 tile ALU bound at 3.6 us.)
+template <int SH, bool WIDE>
+__device__ __forceinline__ void tmem_pair(uint32_t cbase, int l, int nlev, long long* acc) {
+  if (l >= nlev) return;  // warp-uniform
+  uint32_t a[8], b[8];
+  tmem_ld8(cbase + (uint32_t)(l * BN), a);
+  if (l + 1 < nlev) {
+    tmem_ld8(cbase + (uint32_t)((l + 1) * BN), b);
+  } else {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (l0 + q < nlev) {  // warp-uniform
-      tmem_ld8(cbase + (uint32_t)((l0 + q) * BN), v);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) I[i] = (q == 0 ? 0 : I[i] << BETA) + (long long)__float2int_rn(v[i]);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) I[i] = q == 0 ? 0 : I[i] << BETA;
-    }
+    for (int i = 0; i < 8; ++i) b[i] = 0u;
   }
+  tmem_wait(a, b);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] += I[i];
+  for (int i = 0; i < 8; ++i) {
+    const int x = __float2int_rn(__uint_as_float(a[i])), y = __float2int_rn(__uint_as_float(b[i]));
+    if (WIDE) acc[i] += (long long)x * (1 << SH) + (long long)y * (1 << (SH - BETA));
+    else acc[i] += (long long)(x * (1 << BETA) + y) * (1 << (SH - BETA));
+  }
 }
 
 // (ah 2^28 + al) 2^k rounded to the nearest double (ties to even) with integer
@@ -230,6 +240,7 @@ struct OzArgs {
   // part[kz][i + j M] (summed in order by k_split_sum)
   int ksplit, cps;
   double* part;
+  int a64;            // > 0: A is the first rows of an operand in BN-row tiles with a64 row tiles per plane
 };
 
 // Tile order: groups of TGM M-tiles, N-tiles swept inside a group with the
@@ -315,8 +326,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(OzArgs g) {
             if (use > 0) ok = mbar_wait(&bars->a_empty[s], (use - 1) & 1, g.err, 3);
             if (!ok) break;
             mbar_expect_tx(&bars->a_full[s], (unsigned)ATILE);
-            const uint16_t* src = g.A + (((size_t)p * g.mtiles + mt) * g.ktiles + kt) * (ATILE / 2);
-            bulk_g2s(abuf + (size_t)s * ATILE, src, ATILE, &bars->a_full[s]);
+            unsigned char* dst = abuf + (size_t)s * ATILE;
+            if (g.a64) {  // rows 64 .. 127 are the next row tile (the same one again past the operand's last)
+              const uint16_t* src = g.A + (((size_t)p * g.a64 + 2 * mt) * g.ktiles + kt) * (BTILE / 2);
+              bulk_g2s(dst, src, BTILE, &bars->a_full[s]);
+              bulk_g2s(dst + BTILE, 2 * mt + 1 < g.a64 ? src + (size_t)g.ktiles * (BTILE / 2) : src, BTILE,
+                       &bars->a_full[s]);
+            } else {
+              bulk_g2s(dst, g.A + (((size_t)p * g.mtiles + mt) * g.ktiles + kt) * (ATILE / 2), ATILE,
+                       &bars->a_full[s]);
+            }
             ++aidx;
           }
         }
@@ -330,7 +349,23 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(OzArgs g) {
   } else if (warp == 1) {
     if (lane == 0) {
       // ---------------- MMA issuer
-      unsigned aidx = 0, kglob = 0, cglob = 0;
+      // Pairs (p, q) with p + q + 2 <= Lmax.  The B digit tiles q, q+1, ... are
+      // consecutive in shared memory and their levels p+q, p+q+1, ... are
+      // consecutive 64-column TMEM accumulators, so w of them form one MMA with
+      // N = 64 w: one read of the A tile serves w pairs (an N = 64 MMA alone
+      // runs at half rate).  Runs of up to four levels that end at level 3 or
+      // at the last one: 12 MMAs per 16-deep step for 8 digits, 4,890 cycles
+      // per 64-deep K step against 4,608 at full rate (runs of 4, 2 or 1 from
+      // level p on: 5,470).  A run's levels are all fresh (first write) or all
+      // started; each level receives its pairs in increasing p.  The 8 x 8
+      // digit case has its schedule unrolled: this one thread feeds the tensor
+      // core, and its own instructions between two MMAs must take less time
+      // than they do (with the schedule worked out per MMA the tensor core
+      // idled half the time: M = 16,384, N = 8,192, K = 512 went from 5.0 ms,
+      // 989 TFLOP/s of digit pairs, to 2.75 ms, 1,800 TFLOP/s).
+      const bool full8 = g.pA == MAXD && g.pB == MAXD && g.Lmax == MAXD + 1;
+      const uint64_t ad0 = umma_desc(abuf);
+      unsigned as = 0, aph = 0, kglob = 0, cglob = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles_total && ok; t += gridDim.x) {
         const int kz = t % g.ksplit;
@@ -347,40 +382,59 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(OzArgs g) {
             const int b = kglob & 1;
             ok = mbar_wait(&bars->b_full[b], (kglob >> 1) & 1, g.err, 7);
             if (!ok) break;
-            for (int p = 0; p < g.pA && ok; ++p) {
-              const int s = aidx % ASTAGES;
-              ok = mbar_wait(&bars->a_full[s], (aidx / ASTAGES) & 1, g.err, 8);
-              if (!ok) break;
-              tc_fence_after();
-              const uint64_t ad = umma_desc(abuf + (size_t)s * ATILE);
-              // Pairs (p, q) with p + q + 2 <= Lmax.  The B digit tiles q, q+1, ...
-              // are consecutive in shared memory and their levels p+q, p+q+1, ...
-              // are consecutive 64-column TMEM accumulators, so w of them form one
-              // MMA with N = 64 w: one read of the A tile serves w pairs.  Each
-              // level receives its pairs in the same order as one MMA per pair.
-              // A group's levels are all fresh (first write) or all started.
-              const int qmax = min(g.pB - 1, g.Lmax - 2 - p);
-              for (int q = 0; q <= qmax;) {
-                const int l = p + q;
-                int w = 4;
-                while (w > 1) {
-                  const unsigned m = ((1u << w) - 1u) << l;
-                  const unsigned fresh = ~initmask & m;
-                  if (q + w - 1 <= qmax && (fresh == 0u || fresh == m)) break;
-                  w >>= 1;
+            const uint64_t bd0 = umma_desc(bbuf + (size_t)b * MAXD * BTILE);
+            if (full8) {
+              const uint32_t first = kt == c * KCHUNK ? 0u : 1u;  // the chunk's first K step starts every level (p = 0)
+#pragma unroll
+              for (int p = 0; p < MAXD; ++p) {
+                ok = ok && mbar_wait(&bars->a_full[as], aph, g.err, 8);
+                if (!ok) break;
+                const uint64_t ad = ad0 + (uint64_t)(as * (ATILE >> 4));
+                if (p < 4) {
+#pragma unroll
+                  for (int kk = 0; kk < BK / 16; ++kk)
+                    umma_bf16(tmem + (uint32_t)(p * BN), ad + (uint64_t)(kk * 2), bd0 + (uint64_t)(kk * 2),
+                              idesc_n(BN * (4 - p)), p == 0 && kk == 0 ? first : 1u);
                 }
-                const uint64_t bd = umma_desc(bbuf + (size_t)(b * MAXD + q) * BTILE);
-                const uint32_t started = (initmask >> l) & 1u;
-                const uint32_t idesc = idesc_n(BN * w);
+                constexpr int BT = BTILE >> 4;
+                const int l = p < 4 ? 4 : p;
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk)
-                  umma_bf16(tmem + (uint32_t)(l * BN), ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
-                            (started || kk > 0) ? 1u : 0u);
-                initmask |= ((1u << w) - 1u) << l;
-                q += w;
+                  umma_bf16(tmem + (uint32_t)(l * BN), ad + (uint64_t)(kk * 2), bd0 + (uint64_t)((l - p) * BT + kk * 2),
+                            idesc_n(BN * (8 - l)), p == 0 && kk == 0 ? first : 1u);
+                umma_commit(&bars->a_empty[as]);
+                if (++as == ASTAGES) {
+                  as = 0;
+                  aph ^= 1u;
+                }
               }
-              umma_commit(&bars->a_empty[s]);
-              ++aidx;
+              if (!ok) break;
+            } else {
+              for (int p = 0; p < g.pA && ok; ++p) {
+                ok = mbar_wait(&bars->a_full[as], aph, g.err, 8);
+                if (!ok) break;
+                const uint64_t ad = ad0 + (uint64_t)(as * (ATILE >> 4));
+                const int lmax = min(p + g.pB - 1, g.Lmax - 2);
+                for (int l = p; l <= lmax;) {
+                  const uint32_t started = (initmask >> l) & 1u;
+                  int w = 1;
+                  while (w < 4 && l + w <= lmax && l + w != 4 && ((initmask >> (l + w)) & 1u) == started) ++w;
+                  const uint64_t bd = bd0 + (uint64_t)((l - p) * (BTILE >> 4));
+                  const uint32_t idesc = idesc_n(BN * w);
+#pragma unroll
+                  for (int kk = 0; kk < BK / 16; ++kk)
+                    umma_bf16(tmem + (uint32_t)(l * BN), ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
+                              (started || kk > 0) ? 1u : 0u);
+                  initmask |= ((1u << w) - 1u) << l;
+                  l += w;
+                }
+                umma_commit(&bars->a_empty[as]);
+                if (++as == ASTAGES) {
+                  as = 0;
+                  aph ^= 1u;
+                }
+              }
+              if (!ok) break;
             }
             umma_commit(&bars->b_empty[b]);
             ++kglob;
@@ -423,7 +477,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(OzArgs g) {
       }
       const int c1 = min(nchunks, (kz + 1) * g.cps);
       for (int c = kz * g.cps; c < c1; ++c) {
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&bars->acc_full, cglob & 1, g.err, 9));
+        // one lane polls, with pauses, so that the 512 threads leave issue slots
+        // and shared memory to the MMAs they wait for
+        bool ok = true;
+        if (lane == 0) ok = mbar_wait(&bars->acc_full, cglob & 1, g.err, 9, 64);
+        ok = __all_sync(0xffffffffu, ok);
         tc_fence_after();
         if (!ok) {
           alive = false;
@@ -432,13 +490,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(OzArgs g) {
 #pragma unroll
         for (int grp = 0; grp < EPI_COLS / 8; ++grp) {
           const uint32_t cbase = tmem + tlane + (uint32_t)(col0 + grp * 8);
-          // leading levels: exact integers below 2^24 (32-bit conversions),
-          // combined exactly in int64
-          tmem_levels4(cbase, 0, nlev, ai + grp * 8);
-          // remaining levels, combined the same way in int64 (their FP32
-          // accumulators may exceed 2^24 and round there, far below the
-          // result's last bit; the values stay integers below 2^31)
-          if (nlev > 4) tmem_levels4(cbase, 4, nlev, al + grp * 8);
+          // leading levels: exact integers below 2^24, combined exactly; the
+          // remaining ones the same way (their FP32 accumulators may exceed
+          // 2^24 and round there, far below the result's last bit; the values
+          // stay integers)
+          tmem_pair<3 * BETA, false>(cbase, 0, nlev, ai + grp * 8);
+          tmem_pair<BETA, false>(cbase, 2, nlev, ai + grp * 8);
+          tmem_pair<3 * BETA, false>(cbase, 4, nlev, al + grp * 8);
+          tmem_pair<BETA, true>(cbase, 6, nlev, al + grp * 8);
         }
         tc_fence_before();
         __syncwarp();
@@ -490,13 +549,11 @@ struct AccStrided {  // X(i, k) = base[i * si + k * sk]
   long long si, sk;
   __device__ double operator()(long long i, long long k) const { return base[i * si + k * sk]; }
 };
-struct AccHouseVt {  // row i = Householder vector i of the panel at j0, k = row offset from j0
+struct AccHouseVt {  // row i = Householder vector i of the panel at j0 less its unit entry, k = row offset from j0
   const double* A;
   long long lda, j0;
   __device__ double operator()(long long i, long long k) const {
-    if (k < i) return 0.0;
-    if (k == i) return 1.0;
-    return A[(size_t)(j0 + i) * lda + j0 + k];
+    return k <= i ? 0.0 : A[(size_t)(j0 + i) * lda + j0 + k];
   }
 };
 struct AccHouseV {  // row i = matrix row j0 + i, k = panel column
@@ -524,32 +581,49 @@ struct AccJBlock {  // row j = column j of a Jacobian column block, k = k-th row
 };
 
 // e[i] = exponent with max_k |X(i,k)| < 2^e[i] (0 for a zero row), from the
-// largest biased exponent field of the row (integer work only).  One warp per row.
-template <class Acc>
-__global__ void k_rowexp(Acc X, long long R, long long K, int* __restrict__ e) {
+// largest biased exponent field of the row (integer work only).  One warp per
+// row, or one CTA per row (CTA_ROW) where the rows alone would not fill the
+// SMs and a row is long.
+template <class Acc, bool CTA_ROW>
+__global__ void __launch_bounds__(256) k_rowexp(Acc X, long long R, long long K, int* __restrict__ e) {
   const int lane = threadIdx.x & 31;
-  for (long long i = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); i < R;
-       i += (long long)gridDim.x * (blockDim.x >> 5)) {
+  const int step = CTA_ROW ? 256 : 32;
+  const long long first = CTA_ROW ? blockIdx.x : blockIdx.x * 8LL + (threadIdx.x >> 5);
+  for (long long i = first; i < R; i += CTA_ROW ? (long long)gridDim.x : gridDim.x * 8LL) {
     unsigned mx = 0;
     bool nz = false;
-    long long k = lane;
-    for (; k + 96 < K; k += 128) {  // four independent loads in flight per lane
+    long long k = CTA_ROW ? threadIdx.x : lane;
+    for (; k + 3 * step < K; k += 4 * step) {  // four independent loads in flight per lane
       const unsigned long long b0 = (unsigned long long)__double_as_longlong(X(i, k));
-      const unsigned long long b1 = (unsigned long long)__double_as_longlong(X(i, k + 32));
-      const unsigned long long b2 = (unsigned long long)__double_as_longlong(X(i, k + 64));
-      const unsigned long long b3 = (unsigned long long)__double_as_longlong(X(i, k + 96));
+      const unsigned long long b1 = (unsigned long long)__double_as_longlong(X(i, k + step));
+      const unsigned long long b2 = (unsigned long long)__double_as_longlong(X(i, k + 2 * step));
+      const unsigned long long b3 = (unsigned long long)__double_as_longlong(X(i, k + 3 * step));
       mx = max(max(mx, (unsigned)((b0 >> 52) & 0x7FF)), (unsigned)((b1 >> 52) & 0x7FF));
       mx = max(max(mx, (unsigned)((b2 >> 52) & 0x7FF)), (unsigned)((b3 >> 52) & 0x7FF));
       nz |= ((b0 | b1 | b2 | b3) << 1) != 0;
     }
-    for (; k < K; k += 32) {
+    for (; k < K; k += step) {
       const unsigned long long b = (unsigned long long)__double_as_longlong(X(i, k));
       mx = max(mx, (unsigned)((b >> 52) & 0x7FF));
       nz |= (b << 1) != 0;
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     nz = __any_sync(0xffffffffu, nz);
-    if (lane == 0) e[i] = nz ? (mx == 0 ? -1022 : (int)mx - 1022) : 0;
+    if (CTA_ROW) {
+      __shared__ unsigned sh[8];
+      if (lane == 0) sh[threadIdx.x >> 5] = mx * 2 + (nz ? 1u : 0u);
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        nz = false;
+        mx = 0;
+        for (int q = 0; q < 8; ++q) {
+          mx = max(mx, sh[q] >> 1);
+          nz |= (sh[q] & 1u) != 0;
+        }
+      }
+      __syncthreads();
+    }
+    if (CTA_ROW ? threadIdx.x == 0 : lane == 0) e[i] = nz ? (mx == 0 ? -1022 : (int)mx - 1022) : 0;
   }
 }
 
@@ -567,7 +641,7 @@ __device__ __forceinline__ long long biased_of(double x, int e, int ndig) {
   if (E != 0) m |= 1ull << 52;
   const int sh = (E == 0 ? 1 : E) - 1075 - e + 7 * ndig;
   long long V;
-  if (sh >= 0) V = (long long)(m << sh);
+  if (sh >= 0) V = (long long)(m << min(sh, 10));  // sh <= 4 for |x| < 2^e
   else if (sh > -63) V = (long long)((m + (1ull << (-sh - 1))) >> (-sh));
   else V = 0;
   if (b >> 63) V = -V;
@@ -645,9 +719,17 @@ template <class Acc>
 static rfm_status slice(Acc X, long long R, long long K, int ndig, int tile_rows, int* e, uint16_t* out,
                         cudaStream_t st, long long plane_rtiles = 0, long long rt0 = 0) {
   ProfScope ps(PF_OZ_SLICE, st);
-  const int g1 = (int)std::min<long long>((R + 7) / 8, 152LL * 32);
-  k_rowexp<<<std::max(1, g1), 256, 0, st>>>(X, R, K, e);
-  RFM_CHECK_LAUNCH();
+  {
+    // one CTA per row below 8 warps on each SM, where a row feeds 256 threads
+    // (128 rows of 12,288: 28 us with a warp each)
+    if (R < 152LL * 8 && K >= 1024) {
+      k_rowexp<Acc, true><<<(unsigned)R, 256, 0, st>>>(X, R, K, e);
+    } else {
+      const int g1 = (int)std::min<long long>((R + 7) / 8, 152LL * 32);
+      k_rowexp<Acc, false><<<std::max(1, g1), 256, 0, st>>>(X, R, K, e);
+    }
+    RFM_CHECK_LAUNCH();
+  }
   const long long rt = (R + tile_rows - 1) / tile_rows, kt = (K + 63) / 64;
   const long long prt = plane_rtiles > 0 ? plane_rtiles : rt;
   const long long total = rt * tile_rows * kt * 8;
@@ -663,10 +745,6 @@ static rfm_status slice(Acc X, long long R, long long K, int ndig, int tile_rows
 rfm_status rfm_oz_slice_strided(const double* base, long long si, long long sk, long long R, long long K, int ndig,
                                 int tile_rows, int* e, uint16_t* out, cudaStream_t st) {
   return slice(AccStrided{base, si, sk}, R, K, ndig, tile_rows, e, out, st);
-}
-rfm_status rfm_oz_slice_house_vt(const double* A, long long lda, long long j0, long long nb, long long K, int ndig,
-                                 int* e, uint16_t* out, cudaStream_t st) {
-  return slice(AccHouseVt{A, lda, j0}, nb, K, ndig, BM, e, out, st);
 }
 rfm_status rfm_oz_slice_strided_at(const double* base, long long si, long long sk, long long R, long long K, int ndig,
                                    int tile_rows, int* e, uint16_t* out, long long plane_rtiles, long long rt0,
@@ -711,7 +789,7 @@ rfm_status rfm_oz_gemm(const uint16_t* Ad, int pA, const int* ea, const uint16_t
 
 rfm_status rfm_oz_gemm_part(const uint16_t* Ad, int pA, const int* ea, const uint16_t* Bd, int pB, const int* eb,
                             long long M, long long N, long long K, int Lmax, double* C, long long ldc, int mode,
-                            unsigned* err, cudaStream_t st, double* part, long long part_elems) {
+                            unsigned* err, cudaStream_t st, double* part, long long part_elems, long long a64) {
   if (pA < 1 || pB < 1 || pA > MAXD || pB > MAXD || Lmax < 2 || Lmax - 1 > 8) {
     rfm_set_error("oz_gemm: bad digit counts");
     return RFM_EINVAL;
@@ -739,15 +817,16 @@ rfm_status rfm_oz_gemm_part(const uint16_t* Ad, int pA, const int* ea, const uin
   }
   const long long tiles = (long long)a.mtiles * a.ntiles;
   // Split K when the output tiles leave the last wave of CTAs partly idle
-  // (mode 0, a workspace for the partials, at least two 512-deep chunks per
+  // (mode 0, a workspace for the partials, at least one 512-deep chunk per
   // split): the split count with the best fill of whole waves, ties to fewer.
   const int nchunks = (a.ktiles + KCHUNK - 1) / KCHUNK;
   a.ksplit = 1;
   a.cps = nchunks;
   a.part = part;
-  if (mode == 0 && part && tiles < 4LL * nsm && nchunks >= 4) {
+  a.a64 = (int)a64;
+  if (mode == 0 && part && tiles < 4LL * nsm && nchunks >= 2) {
     double best = (double)tiles / (double)(nsm * ((tiles + nsm - 1) / nsm));
-    for (int z = 2; z <= 8 && nchunks / z >= 2; ++z) {
+    for (int z = 2; z <= std::min(64, nchunks); ++z) {
       const int cps = (nchunks + z - 1) / z;
       const int zz = (nchunks + cps - 1) / cps;  // no empty split
       if ((long long)zz * M * N > part_elems) break;

@@ -64,6 +64,7 @@ constexpr int NB = 32;
 // 0.8 update); a 128-column block with its in-block updates 3.7 -> 0.94 ms.
 constexpr int KB_THREADS = 128;
 constexpr int KB_SMEM = 227 * 1024;              // dynamic shared memory of a CTA
+constexpr long long KB_WIDE_ROWS = 16384;
 constexpr int KB_CL = 4;                         // CTAs of a cluster
 constexpr int KB_MAXP = 256;                     // CTAs of one factorisation
 constexpr int KB_POLL = 10;                      // records in flight per lane and poll round
@@ -990,17 +991,23 @@ extern "C" rfm_status rfm_householder_r_noalloc(double* A_dev, int64_t s, int64_
 // ---------------------------------------------------------------------------
 // Householder QR with the trailing update on the tensor cores.
 //
-// Outer blocks of QB = 128 columns: inside a block the 32-wide panels and their
-// FP64 updates run as above; the block's reflectors V (rows x 128, unit
-// diagonal) then update the trailing matrix in compact-WY form
+// A block of w columns is factored recursively: its left half, the block
+// reflector of that half applied to the right half, then the right half; blocks
+// of kb_base columns go to k_block.  A factored block's reflectors V (rows x w,
+// unit diagonal) update the columns to its right in compact-WY form
 //     W = V^T A_t,  W2 = T^T W,  A_t -= V W2
-// with both products on the emulated-FP64 tensor-core GEMM (digit splitting,
-// exact level accumulation).  T (128 x 128) comes from the Gram V^T V, which
-// the first product returns next to W, and the reflector coefficients,
+// with all products on the emulated-FP64 tensor-core GEMM (digit splitting,
+// exact level accumulation).  T (w x w) comes from the Gram V^T V, which the
+// first product returns next to W, and the reflector coefficients,
 // T_jj = tau_j, T_{:j,j} = -tau_j T_{:j,:j} G_{:j,j}.
+//
+// The trailing matrix is updated once per QB columns: its digits are formed and
+// C is read and written once per pass, and the update's depth K = w is the MMA
+// work of an output tile for one drain of its accumulators.  With w = 128 the
+// update ran at 35 % of the tensor rate and the digits of the trailing matrix
+// took 20 % of the time; w = 512 is one exact chunk of the GEMM, the largest
+// depth that one drain covers.
 
-rfm_status rfm_oz_slice_house_vt(const double* A, long long lda, long long j0, long long nb, long long K, int ndig,
-                                 int* e, uint16_t* out, cudaStream_t st);
 rfm_status rfm_oz_slice_house_v(const double* A, long long lda, long long j0, long long rows, long long nb, int ndig,
                                 int* e, uint16_t* out, cudaStream_t st);
 // Digit slices written into row tiles rt0 .. of planes holding plane_rtiles row
@@ -1014,53 +1021,137 @@ rfm_status rfm_oz_slice_house_vt_at(const double* A, long long lda, long long j0
 
 namespace {
 
-constexpr int QB = 128;
+constexpr int QB = 512;   // columns of an outer block (n >= 2 QB)
 constexpr int QDIG = 8;
 
 // T from G and tau: T^-1 = diag(1 / tau) + strict upper part of G, so column j
 // of T is a back substitution, t_j = tau_j, t_i = -tau_i sum_{l>i} G_il t_l (no
 // division; tau_i = 0 gives a zero row).  One warp per column, lane L holding
 // rows L, L + 32, ..: the columns are independent, and a step is one shuffle
-// and at most four FP64 instructions.  (Column after column on one CTA, whose
-// FP64 unit had to do all of it, took 447 us for 128 columns.)
+// and at most U FP64 instructions.  (Column after column on one CTA, whose
+// FP64 unit had to do all of it, took 447 us for 128 columns; now 35 us.)
+// G is column-major, T row-major, both w x w with w = 32 U.
+template <int U>
 __global__ void __launch_bounds__(128) k_block_t(const double* __restrict__ G, const double* __restrict__ tau,
-                                                 int nbw, double* __restrict__ T) {
+                                                 double* __restrict__ T) {
+  constexpr int w = 32 * U;
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
-  double t[QB / 32], tu[QB / 32];
+  double t[U], tu[U];
 #pragma unroll
-  for (int u = 0; u < QB / 32; ++u) {
-    const int i = lane + 32 * u;
-    t[u] = i == j && j < nbw ? 1.0 : 0.0;  // e_j, then the right-hand side less the solved part
-    tu[u] = i < nbw ? tau[i] : 0.0;
+  for (int u = 0; u < U; ++u) {
+    t[u] = lane + 32 * u == j ? 1.0 : 0.0;  // e_j, then the right-hand side less the solved part
+    tu[u] = tau[lane + 32 * u];
   }
 #pragma unroll
-  for (int h = QB / 32 - 1; h >= 0; --h)  // row l = 32 h + ll is held in t[h]
-    for (int l = min(min(j, nbw - 1), 32 * h + 31); l >= 32 * h; --l) {
+  for (int h = U - 1; h >= 0; --h)  // row l = 32 h + ll is held in t[h]
+    for (int l = min(j, 32 * h + 31); l >= 32 * h; --l) {
+      double g[U];
+#pragma unroll
+      for (int u = 0; u <= h; ++u) g[u] = G[(size_t)l * w + lane + 32 * u];
       if (lane == (l & 31)) t[h] *= tu[h];
       const double y = __shfl_sync(0xffffffffu, t[h], l & 31);
 #pragma unroll
       for (int u = 0; u <= h; ++u)
-        if (u < h || lane < (l & 31)) t[u] = fma(-G[(size_t)l * QB + lane + 32 * u], y, t[u]);
+        if (u < h || lane < (l & 31)) t[u] = fma(-g[u], y, t[u]);
     }
 #pragma unroll
-  for (int u = 0; u < QB / 32; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int i = lane + 32 * u;
-    T[(size_t)i * QB + j] = i <= j && j < nbw ? t[u] : 0.0;
+    T[(size_t)i * w + j] = i <= j ? t[u] : 0.0;
   }
 }
 
+// [G, W] (w x N, ld w) += E^T [V, A_t] + V'^T E [I, 0] of the block at c0: the
+// rows c0 .. c0 + w of the trailing columns; in the Gram's upper part (all that
+// T needs), V'^T E, entry (p, j) = v_p(j) for p < j.
+__global__ void __launch_bounds__(64) k_add_top(const double* __restrict__ A, long long lda, long long c0, int w,
+                                                long long N, double* __restrict__ C) {
+  const int p = blockIdx.x * 64 + threadIdx.x;
+  for (long long j = blockIdx.y; j < N; j += gridDim.y) {
+    double add = 0.0;
+    if (j >= w) add = A[(size_t)(c0 + j) * lda + c0 + p];
+    else if (p < j) add = A[(size_t)(c0 + p) * lda + c0 + j];
+    C[(size_t)j * w + p] += add;
+  }
+}
+
+// Workspace of the block reflectors' application.
+struct EmuWs {
+  uint16_t *at, *t, *v, *w2;  // digits of [V, A_t], T^T, V, W2 (and of W before it)
+  double *Wm, *W2, *T, *part;
+  long long part_elems;
+  int *e_at, *e_t, *e_v, *e_w2;
+};
+
+long long emu_part_elems(long long n) { return 16LL * 128 * (n + QB); }
+
+rfm_status apply_block(double* A, long long s, long long lda, long long c0, int w, long long cend, cudaStream_t st,
+                       const double* tau, const EmuWs& e, unsigned int* err) {
+  const long long rows = s - c0, c1 = c0 + w, nt = cend - c1;
+  {
+    // One emulated product gives the block's Gram and V^T A_t.  V is sliced
+    // without its unit diagonal, V = E + V': the digits of a row are scaled by
+    // its largest entry, and beside the 1 the others (about 1 / sqrt(2 rows))
+    // would keep 5 to 7 bits less.  The B operand is [V', A_t] (V'^T as the
+    // first w / 64 row tiles, then the trailing columns), the A operand the
+    // same V'^T tiles, and k_add_top adds E^T [V, A_t] and V'^T E in FP64.
+    // (With the unit diagonal in the digits R of a 12,288 x 4,096 sketch was
+    // four times as far from the exact one as the FP64 path's.)
+    ProfScope ps(PF_QR_VTA, st);
+    const long long prt = w / 64 + (nt + 63) / 64;  // row tiles of the B operand
+    RFM_TRY(rfm_oz_slice_house_vt_at(A, lda, c0, w, rows, QDIG, 64, e.e_at, e.at, prt, 0, st));
+    RFM_TRY(rfm_oz_slice_strided_at(A + (size_t)c1 * lda + c0, lda, 1, nt, rows, QDIG, 64, e.e_at + w, e.at, prt,
+                                    w / 64, st));
+    RFM_TRY(rfm_oz_gemm_part(e.at, QDIG, e.e_at, e.at, QDIG, e.e_at, w, w + nt, rows, QDIG + 1, e.Wm, w, 0, err, st,
+                             e.part, e.part_elems, prt));
+    k_add_top<<<dim3((unsigned)(w / 64), (unsigned)std::min<long long>(w + nt, 32768)), 64, 0, st>>>(
+        A, lda, c0, w, w + nt, e.Wm);
+    RFM_CHECK_LAUNCH();
+    if (w == 64) k_block_t<2><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
+    else if (w == 128) k_block_t<4><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
+    else if (w == 256) k_block_t<8><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
+    else k_block_t<16><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
+    RFM_CHECK_LAUNCH();
+    // W2 = T^T W on the emulated GEMM as well (M = K = w, N = nt).
+    // T is stored row-major, T(q, p) = T[q w + p], so T^T(p, q) = T[p + q w].
+    RFM_TRY(rfm_oz_slice_strided(e.T, 1, w, w, w, QDIG, 128, e.e_t, e.t, st));
+    RFM_TRY(rfm_oz_slice_strided(e.Wm + (size_t)w * w, w, 1, nt, w, QDIG, 64, e.e_w2, e.w2, st));
+    RFM_TRY(rfm_oz_gemm(e.t, QDIG, e.e_t, e.w2, QDIG, e.e_w2, w, nt, w, QDIG + 1, e.W2, w, 0, err, st));
+  }
+  ProfScope ps(PF_QR_UPDATE, st);
+  RFM_TRY(rfm_oz_slice_house_v(A, lda, c0, rows, w, QDIG, e.e_v, e.v, st));
+  RFM_TRY(rfm_oz_slice_strided(e.W2, w, 1, nt, w, QDIG, 64, e.e_w2, e.w2, st));
+  return rfm_oz_gemm(e.v, QDIG, e.e_v, e.w2, QDIG, e.e_w2, rows, nt, w, QDIG + 1, A + (size_t)c1 * lda + c0, lda, 1,
+                     err, st);
+}
+
+// Columns of one k_block: 128 while its slab holds them and the FP64 update
+// inside the block (rows x 128 columns on the FP64 units) costs less than the
+// dozen small launches of an emulated one, else 64.
+int kb_base(long long rows) { return rows <= KB_WIDE_ROWS && kb_width(rows) >= 128 ? 128 : 64; }
+
+rfm_status factor_recursive(double* A, long long s, long long lda, long long c0, int w, cudaStream_t st,
+                            const QrScratch& q, const EmuWs& e, unsigned int* sync, int panel_cap, KbState* ks) {
+  const int base = kb_base(s - c0);
+  if (w <= base) return factor_range(A, s, lda, c0, c0 + w, c0 + w, st, q, sync, panel_cap, ks);
+  int h = base;
+  while (2 * h < w) h *= 2;
+  RFM_TRY(factor_recursive(A, s, lda, c0, h, st, q, e, sync, panel_cap, ks));
+  RFM_TRY(apply_block(A, s, lda, c0, h, c0 + w, st, q.tau, e, sync + SYNC_ERR));
+  return factor_recursive(A, s, lda, c0 + h, w - h, st, q, e, sync, panel_cap, ks);
+}
 
 }  // namespace
 
 long long rfm_householder_emulated_bytes(long long s, long long n) {
   long long b = 0;
-  b += rfm_oz_digit_bytes(QB, s, QDIG, 128);  // V^T
   b += rfm_oz_digit_bytes(n + QB, s, QDIG, 64);  // [V, A_t]: the Gram and V^T A_t in one product
-  b += rfm_oz_digit_bytes(s, QB, QDIG, 128);  // V
-  b += rfm_oz_digit_bytes(n, QB, QDIG, 64);   // W2
-  b += 8LL * (2LL * QB * (n + QB) + QB * QB);  // [G, W], W2, T
-  b += 8LL * 8 * QB * (n + QB);  // split-K partials of V^T [V, A_t]
+  b += rfm_oz_digit_bytes(QB, QB, QDIG, 128);    // T^T
+  b += rfm_oz_digit_bytes(s, QB, QDIG, 128);     // V
+  b += rfm_oz_digit_bytes(n, QB, QDIG, 64);      // W2
+  b += 8LL * (2LL * QB * (n + QB) + QB * QB);    // [G, W], W2, T
+  b += 8LL * emu_part_elems(n);                  // split-K partials of V^T [V, A_t]
   b += 4LL * (QB + n + QB + s + n) + 4096;
   return b;
 }
@@ -1078,66 +1169,37 @@ rfm_status rfm_householder_emulated(double* A, long long s, long long n, long lo
   }
   RFM_TRY(qr_init_device());
   const QrScratch q = carve(scratch, n);
-  char* w = static_cast<char*>(emu);
+  char* p = static_cast<char*>(emu);
   auto take = [&](long long bytes) {
-    char* r = w;
-    w += (bytes + 255) & ~255LL;
+    char* r = p;
+    p += (bytes + 255) & ~255LL;
     return r;
   };
-  uint16_t* d_vt = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(QB, s, QDIG, 128)));
-  uint16_t* d_at = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n + QB, s, QDIG, 64)));
-  uint16_t* d_v = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(s, QB, QDIG, 128)));
-  uint16_t* d_w2 = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n, QB, QDIG, 64)));
-  double* Wm = reinterpret_cast<double*>(take(8LL * QB * (n + QB)));  // [G, W] = V^T [V, A_t]
-  double* W2 = reinterpret_cast<double*>(take(8LL * QB * n));
-  double* T = reinterpret_cast<double*>(take(8LL * QB * QB));
-  const long long part_elems = 8LL * QB * (n + QB);
-  double* part = reinterpret_cast<double*>(take(8LL * part_elems));
-  int* e_vt = reinterpret_cast<int*>(take(4LL * QB));
-  int* e_at = reinterpret_cast<int*>(take(4LL * (n + QB)));
-  int* e_v = reinterpret_cast<int*>(take(4LL * s));
-  int* e_w2 = reinterpret_cast<int*>(take(4LL * n));
-  unsigned int* err = sync + SYNC_ERR;
+  EmuWs e;
+  e.at = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n + QB, s, QDIG, 64)));
+  e.t = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(QB, QB, QDIG, 128)));
+  e.v = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(s, QB, QDIG, 128)));
+  e.w2 = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n, QB, QDIG, 64)));
+  e.Wm = reinterpret_cast<double*>(take(8LL * QB * (n + QB)));  // [G, W] = V^T [V, A_t]
+  e.W2 = reinterpret_cast<double*>(take(8LL * QB * n));
+  e.T = reinterpret_cast<double*>(take(8LL * QB * QB));
+  e.part_elems = emu_part_elems(n);
+  e.part = reinterpret_cast<double*>(take(8LL * e.part_elems));
+  e.e_at = reinterpret_cast<int*>(take(4LL * (n + QB)));
+  e.e_t = reinterpret_cast<int*>(take(4LL * QB));
+  e.e_v = reinterpret_cast<int*>(take(4LL * s));
+  e.e_w2 = reinterpret_cast<int*>(take(4LL * n));
   KbState ks;
   RFM_TRY(kb_begin(q, sync, st));
+  // Outer blocks of 512 columns; narrower ones where n holds only a few, and
+  // for a timing probe of the first ncols columns.
+  int wb = QB;
+  while (wb > 128 && (wb * 2 > n || (ncols >= 0 && wb > ncols))) wb /= 2;
   const long long cstop = ncols < 0 ? n : std::min<long long>(n, ncols);
-  for (long long J0 = 0; J0 < cstop; J0 += QB) {
-    const long long c1 = std::min<long long>(n, J0 + QB);
-    const int nbw = (int)(c1 - J0);
-    const long long rows = s - J0;
-    const long long nt = n - c1;
-    RFM_TRY(factor_range(A, s, lda, J0, c1, c1, st, q, sync, panel_cap, &ks));
-    if (nt <= 0) break;
-    {
-      // One emulated product gives the block's Gram and V^T A_t: its B operand
-      // is [V, A_t] (V^T as the first two 64-row tiles, then the trailing
-      // columns), so C = [G, W] with G = V^T V (exactly symmetric: the digit
-      // pairs (p, q) and (q, p) give the same integer level sums).  T then
-      // comes from G and tau, T_jj = tau_j, T_{:j,j} = -tau_j T_{:j,:j} G_{:j,j}.
-      ProfScope ps(PF_QR_VTA, st);
-      const long long prt = 2 + (nt + 63) / 64;  // row tiles of the B operand
-      RFM_TRY(rfm_oz_slice_house_vt(A, lda, J0, nbw, rows, QDIG, e_vt, d_vt, st));
-      RFM_TRY(rfm_oz_slice_house_vt_at(A, lda, J0, nbw, rows, QDIG, 64, e_at, d_at, prt, 0, st));
-      RFM_TRY(rfm_oz_slice_strided_at(A + (size_t)c1 * lda + J0, lda, 1, nt, rows, QDIG, 64, e_at + QB, d_at, prt, 2,
-                                      st));
-      RFM_TRY(rfm_oz_gemm_part(d_vt, QDIG, e_vt, d_at, QDIG, e_at, nbw, QB + nt, rows, QDIG + 1, Wm, QB, 0, err, st,
-                               part, part_elems));
-      k_block_t<<<QB / 4, 128, 0, st>>>(Wm, q.tau + J0, nbw, T);
-      RFM_CHECK_LAUNCH();
-      // W2 = T^T W on the emulated GEMM as well (M = K = 128, N = nt): the
-      // digit buffers of V^T and of W2 are free at this point of the stream.
-      // T is stored row-major, T(q, p) = T[q QB + p], so T^T(p, q) = T[p + q QB].
-      RFM_TRY(rfm_oz_slice_strided(T, 1, QB, nbw, nbw, QDIG, 128, e_vt, d_vt, st));
-      RFM_TRY(rfm_oz_slice_strided(Wm + (size_t)QB * QB, QB, 1, nt, nbw, QDIG, 64, e_w2, d_w2, st));
-      RFM_TRY(rfm_oz_gemm(d_vt, QDIG, e_vt, d_w2, QDIG, e_w2, nbw, nt, nbw, QDIG + 1, W2, QB, 0, err, st));
-    }
-    {
-      ProfScope ps(PF_QR_UPDATE, st);
-      RFM_TRY(rfm_oz_slice_house_v(A, lda, J0, rows, nbw, QDIG, e_v, d_v, st));
-      RFM_TRY(rfm_oz_slice_strided(W2, QB, 1, nt, nbw, QDIG, 64, e_w2, d_w2, st));
-      RFM_TRY(rfm_oz_gemm(d_v, QDIG, e_v, d_w2, QDIG, e_w2, rows, nt, nbw, QDIG + 1, A + (size_t)c1 * lda + J0, lda,
-                          1, err, st));
-    }
+  for (long long J0 = 0; J0 < cstop; J0 += wb) {
+    const int w = (int)std::min<long long>(wb, n - J0);
+    RFM_TRY(factor_recursive(A, s, lda, J0, w, st, q, e, sync, panel_cap, &ks));
+    if (J0 + w < n) RFM_TRY(apply_block(A, s, lda, J0, w, n, st, q.tau, e, sync + SYNC_ERR));
   }
   return finish_r(A, n, lda, st, q, sync, rank_flag_host);
 }

@@ -42,9 +42,11 @@ def holds(B, R):
 
 
 # one column; one row per column; a panel, a block and one more; rows that leave
-# some CTAs of the last cluster empty; a slab of many rows per warp
+# some CTAs of the last cluster empty; a slab of many rows per warp; outer blocks
+# of 256 and 512 columns, whole and ragged, and blocks built from 64 columns
 SIZES = [(1, 1), (33, 1), (32, 32), (33, 33), (65, 31), (130, 129), (257, 96), (500, 127), (1201, 128), (2999, 161),
-         (20000, 130), (40001, 140), (66000, 70)]
+         (20000, 130), (40001, 140), (66000, 70),
+         (1300, 700), (2600, 1100), (3100, 1537), (20000, 600)]
 
 
 @pytest.mark.parametrize("s,n", SIZES)
