@@ -45,36 +45,45 @@ __device__ __forceinline__ double bf16_bits_to_double(uint16_t h) {
 }
 
 // Gaussian sketch entries rounded to the grid 2^-4: (rint(16 z0), rint(16 z1))
-// for the Box-Muller pair z0 = r cos(t), z1 = r sin(t), r = sqrt(-2 log(1-u1)),
-// t = 2 pi u2, identical to evaluating Box-Muller in FP64 and rounding.
-// The pair is evaluated in FP32 (w = 1 - u1 is formed exactly in FP64 first);
-// with r >= 0.01 the FP32 error of 16 z is below 2.5e-4 (logf 1 ulp, sinf/cosf
-// 2 ulp, sqrtf correctly rounded, inputs rounded once), so an FP32 result more
-// than 1e-3 away from a rounding tie decides the same integer; only the rest
-// (about 0.2%) is recomputed in FP64.  For r < 0.01, |16 z| < 0.17 and the
-// integer is 0 either way.
-__device__ __forceinline__ void gauss_pair_q16(const uint32_t c[4], float* d0, float* d1) {
+// for the Box-Muller pair z0 = r cos(t), z1 = r sin(t), r = sqrt(-2 log(w)),
+// w = 1 - u1, t = 2 pi u2, by definition evaluated in FP64 and then rounded.
+__device__ __forceinline__ void gauss_pair_q16_exact(const uint32_t c[4], float* d0, float* d1) {
   const double u1 = uniform53(c[0], c[1]);
   const double u2 = uniform53(c[2], c[3]);
   const double w = 1.0 - u1;  // exact
-  const float rf = sqrtf(-2.0f * logf((float)w));
-  float sf, cf;
-  sincosf(6.2831853f * (float)u2, &sf, &cf);
-  const float t0 = 16.0f * (rf * cf), t1 = 16.0f * (rf * sf);
-  const float q0 = rintf(t0), q1 = rintf(t1);
-  if (rf < 0.01f) {
-    *d0 = 0.0f;
-    *d1 = 0.0f;
-    return;
-  }
-  const bool safe = fabsf(fabsf(t0 - q0) - 0.5f) > 1e-3f && fabsf(fabsf(t1 - q1) - 0.5f) > 1e-3f;
-  if (safe) {
-    *d0 = q0;
-    *d1 = q1;
-    return;
-  }
   const double rad = sqrt(-2.0 * log(w));
   const double th = 6.283185307179586 * u2;
   *d0 = (float)rint(16.0 * (rad * cos(th)));
   *d1 = (float)rint(16.0 * (rad * sin(th)));
+}
+
+// The same integers from FP32 with the hardware's log2, square root, sine and
+// cosine; false where 16 z lies too near a rounding tie to be sure (0.2 % of
+// the pairs) or w is below 2^-12.  No FP64 instruction (31 ns each on GB300).
+// Errors of 16 z: w from its top 32 bits, 2^-20 relative or less; log2 2^-22
+// absolute on [0.5, 2], 2 ulp elsewhere, so L = r^2 is within 5e-7 (L <= 1.4) or
+// 4e-7 L, and 16 r within 8 dL / r <= 4e-4 for r >= 0.01; sine and cosine on
+// [-pi, pi] within 6e-7 and their argument within 4e-7, times 16 r <= 66 (w >=
+// 2^-12): 7e-5 where the first term is below 4e-5.  Below 5e-4 in all.  For r <
+// 0.01 the computed r^2 is off by 5e-7 at most, |16 z| < 0.2 and both are 0.
+__device__ __forceinline__ bool gauss_pair_q16_fast(const uint32_t c[4], float* d0, float* d1) {
+  const uint32_t wt = ~(((c[0] >> 5) << 5) | (c[1] >> 27));  // top 32 bits of 2^53 - (53 bits of u1), less one unit
+  const float w = fmaf((float)wt, 0x1p-32f, 0x1p-33f);
+  const float L = -1.3862944f * __log2f(w);
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(L, 0.0f)));
+  const uint32_t a = ((c[2] >> 5) << 5) | (c[3] >> 27);  // top 32 bits of u2
+  const float x = (float)(int)(a ^ 0x80000000u) * 1.4629180792671596e-9f;  // 2 pi (u2 - 1/2)
+  const float r16 = -16.0f * r;  // cos(t) = -cos(x), sin(t) = -sin(x)
+  const float t0 = r16 * __cosf(x), t1 = r16 * __sinf(x);
+  const float q0 = rintf(t0), q1 = rintf(t1);
+  const bool zero = r < 0.01f;
+  *d0 = zero ? 0.0f : q0;
+  *d1 = zero ? 0.0f : q1;
+  const bool safe = fabsf(fabsf(t0 - q0) - 0.5f) > 5e-4f && fabsf(fabsf(t1 - q1) - 0.5f) > 5e-4f;
+  return wt >= (1u << 20) && (zero || safe);
+}
+
+__device__ __forceinline__ void gauss_pair_q16(const uint32_t c[4], float* d0, float* d1) {
+  if (!gauss_pair_q16_fast(c, d0, d1)) gauss_pair_q16_exact(c, d0, d1);
 }

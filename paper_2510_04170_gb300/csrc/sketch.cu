@@ -203,36 +203,95 @@ __global__ void __launch_bounds__(256) k_gauss_gemm(const uint16_t* __restrict__
 // Digit tiles of S for the split product (one digit per entry: d = rint(16 z),
 // so S = d * 2^(3 - 7) with exponent 3), for every column block b: tiles
 // [s/128][ktiles_b] starting at tile toff[b], K index = position in the block's
-// row list.  Threads run along K so each warp writes within 128-byte rows.
-__global__ void k_gauss_digits(long long s, long long totK, const int* __restrict__ colptr, int G,
-                               const int* __restrict__ colrows, const long long* __restrict__ toff, uint32_t kJ,
-                               uint32_t key0, uint32_t key1, uint16_t* __restrict__ out) {
-  const long long half = s / 2;
-  const long long total = half * totK;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long g = t % totK, q = t / totK;
-    int lo = 0, hi = G - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) / 2;
-      if (colptr[mid] <= g) lo = mid; else hi = mid - 1;
-    }
-    const int b = lo;
-    const long long k = g - colptr[b];
-    const long long kt_b = (colptr[b + 1] - colptr[b] + 63) / 64;
-    const unsigned i = (unsigned)colrows[g] & 0x7fffffffu;
-    uint32_t c[4] = {2u, i, (uint32_t)q, kJ};
+// row list; zeros past the block's rows and past s.
+//
+// A CTA forms a tile of 128 x 64 entries in shared memory (thread = one K index
+// and every fourth pair of sketch rows) and writes it as 16-byte chunks.  The
+// pairs that FP32 cannot decide are queued and recomputed in FP64 once a full
+// set of threads has one each: a warp pays for the FP64 path (about 150
+// instructions of 31 ns) whenever one of its lanes takes it, and with the path
+// inline 12 % of the warps did, which was most of the kernel's time.
+constexpr int GD_THREADS = 256;
+constexpr int GD_QUEUE = 2048;
+
+struct GdPlace {
+  int b;
+  long long mt, kt, K;
+};
+__device__ __forceinline__ GdPlace gd_place(long long tile, const int* colptr, int G, const long long* toff) {
+  int lo = 0, hi = G - 1;
+  while (lo < hi) {  // the last block that starts at or before the tile (empty blocks own none)
+    const int mid = (lo + hi + 1) / 2;
+    if (toff[mid] <= tile) lo = mid; else hi = mid - 1;
+  }
+  GdPlace p;
+  p.b = lo;
+  p.K = colptr[lo + 1] - colptr[lo];
+  const long long kts = (p.K + 63) / 64, rel = tile - toff[lo];
+  p.mt = rel / kts;
+  p.kt = rel - p.mt * kts;
+  return p;
+}
+
+__global__ void __launch_bounds__(GD_THREADS) k_gauss_digits(long long s, const int* __restrict__ colptr, int G,
+                                                             const int* __restrict__ colrows,
+                                                             const long long* __restrict__ toff, uint32_t kJ,
+                                                             uint32_t key0, uint32_t key1,
+                                                             uint16_t* __restrict__ out) {
+  __shared__ uint4 tile_s[128 * 64 * 2 / 16];
+  __shared__ unsigned long long queue[GD_QUEUE];  // tile * 4096 + pair * 64 + k
+  __shared__ int queued;
+  uint16_t* ts = reinterpret_cast<uint16_t*>(tile_s);
+  const int tid = threadIdx.x, k64 = tid & 63;
+  const long long half = s / 2, tiles = toff[G];
+  if (tid == 0) queued = 0;
+  __syncthreads();
+  // one queued pair again in FP64, straight into its tile in global memory
+  auto redo = [&](unsigned long long ent) {
+    const long long tile = (long long)(ent >> 12);
+    const int pr = (int)(ent >> 6) & 63, k = (int)ent & 63;
+    const GdPlace p = gd_place(tile, colptr, G, toff);
+    uint32_t c[4] = {2u, (uint32_t)colrows[colptr[p.b] + p.kt * 64 + k] & 0x7fffffffu, (uint32_t)(p.mt * 64 + pr), kJ};
     philox4x32_10(c, key0, key1);
     float d0, d1;
-    gauss_pair_q16(c, &d0, &d1);
-    const long long r = 2 * q;
-    const long long mt = r >> 7;
-    const int rr = (int)(r & 127);
-    const long long tile = toff[b] + mt * kt_b + (k >> 6);
+    gauss_pair_q16_exact(c, &d0, &d1);
     uint16_t* base = out + (size_t)tile * (128 * 64);
-    const int k64 = (int)(k & 63);
-    base[rfm_swz128(rr, k64) >> 1] = (uint16_t)(__float_as_uint(d0) >> 16);
-    base[rfm_swz128(rr + 1, k64) >> 1] = (uint16_t)(__float_as_uint(d1) >> 16);
+    base[rfm_swz128(2 * pr, k) >> 1] = (uint16_t)(__float_as_uint(d0) >> 16);
+    base[rfm_swz128(2 * pr + 1, k) >> 1] = (uint16_t)(__float_as_uint(d1) >> 16);
+  };
+  for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const GdPlace p = gd_place(tile, colptr, G, toff);
+    const bool kin = p.kt * 64 + k64 < p.K;
+    const uint32_t i = kin ? (uint32_t)colrows[colptr[p.b] + p.kt * 64 + k64] & 0x7fffffffu : 0u;
+#pragma unroll 4
+    for (int u = 0; u < 16; ++u) {
+      const int pr = (tid >> 6) + 4 * u;
+      const long long q = p.mt * 64 + pr;
+      float d0 = 0.0f, d1 = 0.0f;
+      if (kin && q < half) {
+        uint32_t c[4] = {2u, i, (uint32_t)q, kJ};
+        philox4x32_10(c, key0, key1);
+        if (!gauss_pair_q16_fast(c, &d0, &d1)) {
+          const int at = atomicAdd(&queued, 1);
+          if (at < GD_QUEUE) queue[at] = ((unsigned long long)tile << 12) | (unsigned)(pr << 6 | k64);
+          else gauss_pair_q16_exact(c, &d0, &d1);
+        }
+      }
+      ts[rfm_swz128(2 * pr, k64) >> 1] = (uint16_t)(__float_as_uint(d0) >> 16);
+      ts[rfm_swz128(2 * pr + 1, k64) >> 1] = (uint16_t)(__float_as_uint(d1) >> 16);
+    }
+    __syncthreads();
+    uint4* dst = reinterpret_cast<uint4*>(out + (size_t)tile * (128 * 64));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) dst[tid + GD_THREADS * u] = tile_s[tid + GD_THREADS * u];
+    __syncthreads();  // the tile is written; ts and the queue may change again
+    const int nq = min(queued, GD_QUEUE);
+    if (nq >= GD_THREADS || tile + gridDim.x >= tiles) {
+      for (int at = tid; at < nq; at += GD_THREADS) redo(queue[at]);
+      __syncthreads();
+      if (tid == 0) queued = 0;
+      __syncthreads();
+    }
   }
 }
 
@@ -321,10 +380,8 @@ rfm_status rfm_launch_gauss_sketch_tc(rfm_problem* p, long long s, int kJ) {
   int* ej = p->oz_e + s;
   {
     ProfScope ps(PF_SKETCH_GEN, p->stream);
-    RFM_CUDA(cudaMemsetAsync(p->sdig, 0, (size_t)sbytes, p->stream));
-    const long long totK = p->colptr_h[G];
-    k_gauss_digits<<<152 * 16, 256, 0, p->stream>>>(s, totK, p->colptr, G, p->colrows, p->oz_toff, (uint32_t)kJ, k0, k1,
-                                                   p->sdig);
+    k_gauss_digits<<<(unsigned)std::max<long long>(1, std::min<long long>(toff[G], 152LL * 8)), GD_THREADS, 0, p->stream>>>(
+        s, p->colptr, G, p->colrows, p->oz_toff, (uint32_t)kJ, k0, k1, p->sdig);
     RFM_CHECK_LAUNCH();
     k_fill_int<<<64, 256, 0, p->stream>>>(es, s, 3);
     RFM_CHECK_LAUNCH();
