@@ -939,6 +939,7 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->mu, muh.size()));
     TRYA(dalloc(&p->sig, sgh.size()));
     TRYA(dalloc(&p->feat, 4 * nfeat));
+    TRYA(dalloc(&p->slopes, 4 * nfeat));
     TRYA(dalloc(&p->segs, segs.size()));
     TRYA(dalloc(&p->pts, 4 * p->m));
     TRYA(dalloc(&p->rmeta, p->m));
@@ -1003,7 +1004,7 @@ rfm_status rfm_problem_destroy(rfm_problem* p) {
   if (!p) return RFM_OK;
   if (p->stream) cudaStreamSynchronize(p->stream);
   else cudaDeviceSynchronize();
-  void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
+  void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slopes, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
                   p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->work,
                   p->red, p->sync, p->sdig, p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch,
                   p->trsv_acc, p->dinv};

@@ -41,6 +41,7 @@ struct rfm_problem {
   double* mu = nullptr;     // [G][4]
   double* sig = nullptr;    // [G][4]
   double* feat = nullptr;   // [G*fields*M][4]
+  double* slopes = nullptr; // [G*fields*M][4]: k_b / sigma_b and the sum of their squares
   RowSeg* segs = nullptr;
   int nseg = 0;
   bool explicit_rows = false;  // geometry with masked grids: points and row metadata built on the host
