@@ -52,7 +52,7 @@ __global__ void k_features(double* __restrict__ feat, long long nfeat, int d, do
 // feature: the derivatives of phi_j are t, 1 - t^2 and these factors.  Formed
 // once per problem: an FP64 division takes some nine FP64 instructions of 31 ns
 // on GB300, and three per feature and row were a third of the assembly's time
-// (124,416 rows of 512 features: 10.8 -> 6.9 ms with the table).
+// (124,416 rows of 512 features: 10.8 -> 6.8 ms with the table).
 __global__ void k_feature_slopes(const double* __restrict__ feat, const double* __restrict__ sig, long long nfeat,
                                  int per_sub, int d, double* __restrict__ ks) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;

@@ -1,12 +1,12 @@
 // Matrix-vector kernels of the LSQR inner solve on J R^{-1} (Alg. 1 steps 3-4).
 //
-//  * k_jmv:   y = s1 * J x + s2 * y.  One warp per row; a row is W contiguous
-//             doubles of its primary block (and W more of the secondary block
-//             for interface rows), read once, coalesced.
-//  * k_jtmv:  y = J^T x.  One CTA per (column block, 64-column chunk); the
-//             rows touching the block are walked in a fixed order and the
-//             eight warps' partial sums are combined in a fixed order, so the
-//             result is deterministic.
+//  * k_jmv:   y = s1 * J x + s2 * y.  One warp per four rows; a row is W
+//             contiguous doubles of its primary block (and W more of the
+//             secondary block for interface rows), read once, coalesced.
+//  * k_jtmv:  y = J^T x.  One CTA per (column block, 64-column chunk, slice of
+//             the block's rows); the rows are walked in a fixed order and the
+//             eight warps' and the slices' partial sums are combined in a fixed
+//             order, so the result is deterministic.
 //  * k_trsv_chain: x = R^{-1} b or x = R^{-T} b for the upper-triangular
 //             preconditioner R (column-major, leading dimension ldr), in one
 //             cooperative launch: one chain CTA solves the 64 x 64 diagonal
@@ -29,6 +29,13 @@ namespace {
 
 constexpr int TB = 64;  // triangular block
 
+// Four rows per warp: an FP64 warp instruction takes 31 ns on GB300 whatever it
+// does, so the reduction over the lanes (five additions a row) counts beside the
+// W / 32 products; reducing four rows together takes six additions for all.
+// FP64 bound: 124,416 rows of 512 take 110 us at two FMAs per clock and SM
+// (one row per warp: 178 us, four: 147).
+constexpr int JMV_ROWS = 4;
+
 __global__ void __launch_bounds__(256) k_jmv(const double* __restrict__ Jp, const double* __restrict__ Js,
                                              const int4* __restrict__ meta, long long m, long long m_int, int W,
                                              const double* __restrict__ x, double s1, double s2,
@@ -38,40 +45,89 @@ __global__ void __launch_bounds__(256) k_jmv(const double* __restrict__ Jp, cons
   if (s2dev) s2 *= s2dev[0];
   const int lane = threadIdx.x & 31;
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long i = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); i < m; i += nwarps) {
-    const int4 mt = meta[i];
-    const double* row = Jp + (size_t)i * W;
-    const double* xb = x + (size_t)mt.y * W;
-    double acc = 0.0;
-    for (int j = lane; j < W; j += 32) acc += row[j] * xb[j];
-    if ((mt.x & 0xF) == 1) {
-      const double* row2 = Js + (size_t)(i - m_int) * W;
-      const double* xb2 = x + (size_t)mt.z * W;
-      for (int j = lane; j < W; j += 32) acc += row2[j] * xb2[j];
+  for (long long i0 = (blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5)) * JMV_ROWS; i0 < m;
+       i0 += nwarps * JMV_ROWS) {
+    const double *row[JMV_ROWS], *xb[JMV_ROWS];
+    double acc[JMV_ROWS];
+#pragma unroll
+    for (int r = 0; r < JMV_ROWS; ++r) {
+      const long long i = min(i0 + r, m - 1);
+      row[r] = Jp + (size_t)i * W;
+      xb[r] = x + (size_t)meta[i].y * W;
+      acc[r] = 0.0;
     }
-    acc = warp_sum(acc);
-    if (lane == 0) y[i] = s2 == 0.0 ? s1 * acc : s1 * acc + s2 * y[i];
+#pragma unroll 2
+    for (int j = lane; j < W; j += 32) {
+      double v[JMV_ROWS], xv[JMV_ROWS];
+#pragma unroll
+      for (int r = 0; r < JMV_ROWS; ++r) {
+        v[r] = __ldcs(row[r] + j);
+        xv[r] = xb[r][j];
+      }
+#pragma unroll
+      for (int r = 0; r < JMV_ROWS; ++r) acc[r] += v[r] * xv[r];
+    }
+    if (i0 + JMV_ROWS > m_int) {
+#pragma unroll
+      for (int r = 0; r < JMV_ROWS; ++r) {
+        const long long i = min(i0 + r, m - 1);
+        const int4 mt = meta[i];
+        if ((mt.x & 0xF) == 1) {
+          const double* row2 = Js + (size_t)(i - m_int) * W;
+          const double* xb2 = x + (size_t)mt.z * W;
+          for (int j = lane; j < W; j += 32) acc[r] += row2[j] * xb2[j];
+        }
+      }
+    }
+    // lanes with bit 4 set keep rows 2, 3, bit 3 picks the odd row of the pair
+    {
+      const bool hi = lane & 16, odd = lane & 8;
+      const double a0 = (hi ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, hi ? acc[0] : acc[2], 16);
+      const double a1 = (hi ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, hi ? acc[1] : acc[3], 16);
+      double a = (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      const long long i = i0 + (hi ? 2 : 0) + (odd ? 1 : 0);
+      if ((lane & 7) == 0 && i < m) y[i] = s2 == 0.0 ? s1 * a : s1 * a + s2 * y[i];
+    }
   }
 }
 
+// Slice z of the rows of column block b; with more than one slice the partial
+// sums go to part[z][n] and k_jtmv_sum adds them.  Four rows' loads are in flight
+// per warp.
 __global__ void __launch_bounds__(256) k_jtmv(const double* __restrict__ Jp, const double* __restrict__ Js,
                                               const int* __restrict__ colptr, const int* __restrict__ colrows,
                                               long long m_int, int W, const double* __restrict__ x,
-                                              const int* __restrict__ skip, double* __restrict__ y) {
+                                              const int* __restrict__ skip, double* __restrict__ y, long long n) {
   if (skip && *skip) return;
   const int b = blockIdx.x;
   const int c0 = blockIdx.y * 64;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int ca = c0 + lane, cb = c0 + 32 + lane;
   double acc0 = 0.0, acc1 = 0.0;
-  const int beg = colptr[b], end = colptr[b + 1];
-  for (int t = beg + w; t < end; t += 8) {
-    const unsigned int ent = (unsigned int)colrows[t];
-    const long long r = ent & 0x7fffffffu;
-    const double* row = (ent >> 31) ? Js + (size_t)(r - m_int) * W : Jp + (size_t)r * W;
-    const double xr = x[r];
-    if (ca < W) acc0 += row[ca] * xr;
-    if (cb < W) acc1 += row[cb] * xr;
+  const int all = colptr[b + 1] - colptr[b];
+  const int per = (all + (int)gridDim.z - 1) / (int)gridDim.z;
+  const int beg = colptr[b] + min(all, per * (int)blockIdx.z), end = colptr[b] + min(all, per * ((int)blockIdx.z + 1));
+  const bool ina = ca < W, inb = cb < W;
+  for (int t = beg + w; t < end; t += 32) {
+    double v0[4], v1[4], xr[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool in = t + 8 * u < end;
+      const unsigned int ent = in ? (unsigned int)colrows[t + 8 * u] : 0u;
+      const long long r = ent & 0x7fffffffu;
+      const double* row = (ent >> 31) ? Js + (size_t)(r - m_int) * W : Jp + (size_t)r * W;
+      xr[u] = in ? x[r] : 0.0;
+      v0[u] = in && ina ? __ldcs(row + ca) : 0.0;
+      v1[u] = in && inb ? __ldcs(row + cb) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + 8 * u < end) {
+        acc0 += v0[u] * xr[u];
+        acc1 += v1[u] * xr[u];
+      }
   }
   __shared__ double sh[8][64];
   sh[w][lane] = acc0;
@@ -82,8 +138,18 @@ __global__ void __launch_bounds__(256) k_jtmv(const double* __restrict__ Jp, con
 #pragma unroll
     for (int k = 0; k < 8; ++k) s += sh[k][threadIdx.x];
     const int col = c0 + threadIdx.x;
-    if (col < W) y[(size_t)b * W + col] = s;
+    if (col < W) y[(size_t)blockIdx.z * n + (size_t)b * W + col] = s;
   }
+}
+
+__global__ void k_jtmv_sum(const double* __restrict__ part, int Z, long long n, const int* __restrict__ skip,
+                           double* __restrict__ y) {
+  if (skip && *skip) return;
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double s = 0.0;
+  for (int z = 0; z < Z; ++z) s += part[(size_t)z * n + i];
+  y[i] = s;
 }
 
 // x = R^{-1} b (TRANS = 0) or R^{-T} b (TRANS = 1).
@@ -737,7 +803,7 @@ rfm_status rfm_dot(cudaStream_t st, const double* x, const double* y, long long 
 rfm_status rfm_launch_jmv(rfm_problem* p, const double* x, double* y) {
   ProfScope ps(PF_JMV, p->stream);
   rfm_prof_work(PF_JMV, 8.0 * ((double)(p->m + p->m_iface) * p->W + p->m + p->n));
-  long long g = (p->m + 7) / 8;
+  long long g = (p->m + 8 * JMV_ROWS - 1) / (8 * JMV_ROWS);
   if (g > 152 * 64) g = 152 * 64;
   k_jmv<<<(int)g, 256, 0, p->stream>>>(p->Jp, p->Js, p->rmeta, p->m, p->m_int, p->W, x, 1.0, 0.0, nullptr, p->skip,
                                        y);
@@ -749,19 +815,45 @@ rfm_status rfm_launch_jmv_axpby(rfm_problem* p, const double* x, double s1, doub
                                 const double* s2dev) {
   ProfScope ps(PF_JMV, p->stream);
   rfm_prof_work(PF_JMV, 8.0 * ((double)(p->m + p->m_iface) * p->W + 2.0 * p->m + p->n));
-  long long g = (p->m + 7) / 8;
+  long long g = (p->m + 8 * JMV_ROWS - 1) / (8 * JMV_ROWS);
   if (g > 152 * 64) g = 152 * 64;
   k_jmv<<<(int)g, 256, 0, p->stream>>>(p->Jp, p->Js, p->rmeta, p->m, p->m_int, p->W, x, s1, s2, s2dev, p->skip, y);
   RFM_CHECK_LAUNCH();
   return RFM_OK;
 }
 
+// Slices of every column block's rows: the count with the least work on the
+// busiest SM (about 16 CTAs of an SM run at once), at most JT_SLICES and at
+// least 128 rows each on average.  One slice per block left 16 CTAs for 15,552
+// rows of 8 blocks of 128 (60 us; 10 with 19 slices, and 2 for their sum).
+static int jtmv_slices(const rfm_problem* p) {
+  const int nsm = std::max(1, rfm_num_sms());
+  const long long tiles = (long long)p->G * ((p->W + 63) / 64);
+  const long long rows = (p->m + p->m_iface) / std::max(1, p->G);
+  int best = 1;
+  double cost = 0.0;
+  for (int z = 1; z <= JT_SLICES && (z == 1 || rows / z >= 128); ++z) {
+    const double c = (double)((tiles * z + nsm - 1) / nsm) / z + 0.01 * z;  // + the slices' sum
+    if (z == 1 || c < cost) {
+      cost = c;
+      best = z;
+    }
+  }
+  return best;
+}
+
 rfm_status rfm_launch_jtmv(rfm_problem* p, const double* x, double* y) {
-  dim3 grid(p->G, (p->W + 63) / 64);
+  const int Z = p->jt_part ? jtmv_slices(p) : 1;
+  dim3 grid(p->G, (p->W + 63) / 64, Z);
   ProfScope ps(PF_JTMV, p->stream);
   rfm_prof_work(PF_JTMV, 8.0 * ((double)(p->m + p->m_iface) * p->W + p->m + p->n));
-  k_jtmv<<<grid, 256, 0, p->stream>>>(p->Jp, p->Js, p->colptr, p->colrows, p->m_int, p->W, x, p->skip, y);
+  k_jtmv<<<grid, 256, 0, p->stream>>>(p->Jp, p->Js, p->colptr, p->colrows, p->m_int, p->W, x, p->skip,
+                                      Z > 1 ? p->jt_part : y, p->n);
   RFM_CHECK_LAUNCH();
+  if (Z > 1) {
+    k_jtmv_sum<<<(unsigned)((p->n + 255) / 256), 256, 0, p->stream>>>(p->jt_part, Z, p->n, p->skip, y);
+    RFM_CHECK_LAUNCH();
+  }
   return RFM_OK;
 }
 

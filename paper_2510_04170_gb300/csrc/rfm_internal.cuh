@@ -14,6 +14,7 @@
 
 #define RFM_MAX_FIELDS 2
 #define RFM_MAX_WIDTH 2048
+#define JT_SLICES 32
 
 // One run of rows that share a point grid (Sec. 5): an interior grid of a
 // subdomain, or a face grid on an interface or a boundary face.
@@ -98,6 +99,7 @@ struct rfm_problem {
   long long lsqr_graph_launches = 0;  // kernels per chunk (launch accounting)
   bool lsqr_eager = false;        // graph capture failed once: replay the chunk's kernels eagerly
   int qr_panel_cap = 0;           // most CTAs per panel factorisation (0: one per SM)
+  double* jt_part = nullptr;      // [JT_SLICES][n] partial sums of J^T x
   double* trsv_acc = nullptr;     // [ceil(n/64)][64] partial sums of the triangular solve's helpers
   double* dinv = nullptr;         // [ceil(n/64)][64 x 64] inverses of R's diagonal blocks (column-major)
   const double* dinv_of = nullptr;  // the R that dinv was computed from (nullptr: stale)
