@@ -954,7 +954,8 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->hsign, p->m));
     TRYA(dalloc(&p->red, 4096));
     TRYA(dalloc(&p->jt_part, (size_t)JT_SLICES * p->n));
-    TRYA(dalloc(&p->trsv_acc, (size_t)((p->n + 63) / 64) * 64));
+    TRYA(dalloc(&p->trsv_rec, (size_t)((p->n + 63) / 64) * 64 * 4));
+    TRYA(dalloc(&p->chain_tiles, (size_t)rfm_trsv_tiles_len(p->n)));
     TRYA(dalloc(&p->dinv, (size_t)((p->n + 63) / 64) * 64 * 64));
     TRYA(dalloc(&p->sync, RFM_SYNC_WORDS));
     p->work_cap = vec_stride(p) * WV_COUNT;
@@ -982,7 +983,9 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
       CPY(p->rmeta, ball_meta.data(), ball_meta.size());
     }
 #undef CPY
-    if (cudaMemsetAsync(p->sync, 0, RFM_SYNC_WORDS * sizeof(unsigned int), s0) != cudaSuccess) {
+    if (cudaMemsetAsync(p->sync, 0, RFM_SYNC_WORDS * sizeof(unsigned int), s0) != cudaSuccess ||
+        cudaMemsetAsync(p->trsv_rec, 0, (size_t)((p->n + 63) / 64) * 64 * 4 * sizeof(unsigned long long), s0) !=
+            cudaSuccess) {
       st = RFM_ECUDA;
       goto fail;
     }
@@ -1008,7 +1011,7 @@ rfm_status rfm_problem_destroy(rfm_problem* p) {
   void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slopes, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
                   p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->work,
                   p->red, p->sync, p->sdig, p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch,
-                  p->jt_part, p->trsv_acc, p->dinv};
+                  p->jt_part, p->trsv_rec, p->dinv, p->chain_tiles};
   drop_lsqr_graph(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   for (void* b : bufs) dfree(b);

@@ -9,11 +9,10 @@
 //             order, so the result is deterministic.
 //  * k_trsv_chain: x = R^{-1} b or x = R^{-T} b for the upper-triangular
 //             preconditioner R (column-major, leading dimension ldr), in one
-//             cooperative launch: one chain CTA solves the 64 x 64 diagonal
-//             blocks in dependency order from tiles it prefetched into shared
-//             memory, and helper CTAs stream the rest of R once, each adding
-//             the contributions of published blocks to the blocks it owns
-//             (details at the kernel).
+//             cooperative launch: a cluster of four CTAs solves the 64-row
+//             blocks in dependency order, and helper CTAs stream the rest of R
+//             once, each adding the contributions of published blocks to the
+//             blocks it owns (details at the kernel).
 //  * k_trsv:  the same solve for sizes with more blocks than the helpers can
 //             own: 64-row blocks are claimed through a ticket counter in
 //             dependency order, each block waits (bounded) on the per-block
@@ -22,6 +21,7 @@
 //             one warp and publishes its part of x with a release flag.
 //  * k_partial_* / k_finish_*: deterministic two-stage norms and dots.
 #include <algorithm>
+#include <mutex>
 
 #include "rfm_internal.cuh"
 
@@ -263,67 +263,39 @@ __global__ void __launch_bounds__(256) k_trsv(const double* __restrict__ R, long
 }
 
 // ---------------------------------------------------------------------------
-// Triangular solve as one chain CTA plus helper CTAs (cooperative launch, all
-// CTAs co-resident).  The 64-row blocks are solved in dependency order
-// t = 0, 1, ... (block nblk-1-t for R^{-1}, block t for R^{-T}).  The chain
-// CTA solves the diagonal blocks one after another, with the inverse Z_k of
-// each 64 x 64 diagonal block, computed once per factorisation
-// (k_trsv_dinv): x_k = Z_k (b_k - sum_j R_kj x_j), two dense products and no
-// dependent substitution.  It holds Z_k and the tiles coupling block k to the
-// two blocks solved just before (order distance 1 and 2) in shared memory
-// (cp.async, issued ahead), so its step reads no global memory except the
-// right-hand side and one partial sum.  The helper CTAs add the
-// contributions of all earlier blocks (distance >= 3) as soon as each block
-// is published: helper h owns the targets t = 3 + (h - 1) + H m, streams
-// their tiles of R (each read once), and publishes each target's partial sum
-// three steps before the chain needs it.  All sums are in a fixed order, so
-// results are deterministic.  Waits are bounded (wait_flag).
-constexpr int TLD = TB + 2;            // leading dimension of a shared-memory tile (doubles; 16-byte rows)
-constexpr int TTILE = TB * TLD;        // doubles per shared-memory tile
-constexpr int CHAIN_NEAR = 3;          // the chain applies distances 1 .. CHAIN_NEAR-1 itself
+// Triangular solve by a chain cluster and helper CTAs (cooperative launch, all
+// CTAs co-resident).  The 64-row blocks are solved in dependency order t = 0,
+// 1, ... (block k = nblk-1-t for R^{-1}, block t for R^{-T}).  With Z_k the
+// inverse of the diagonal block (k_trsv_dinv, once per factorisation) and C_d
+// the couplings of block k to the blocks solved d = 1 .. CHAIN_D steps before,
+//     y_t = (b_k - s_t) - sum_d C_d x_{t-d},    x_t = Z_k y_t,
+// where s_t, the contributions of all earlier blocks, comes from a helper: it
+// owns the targets t = h + H m, adds each published block's part and publishes
+// the sum after its last one.
+//
+// What bounds a step is again FP64 instruction issue (31 ns per warp instruction
+// and SM partition) and the exchanges: the four CTAs take 16 rows each, a thread
+// 8 columns of one row, so a product is 8 instructions per warp, the sum over
+// columns one shuffle and four shared-memory partials, and y_t and x_t go to all
+// four CTAs through distributed shared memory with one cluster barrier each (0.2
+// us).  Only C_1 and Z_k wait for the step before; their tiles and the others are
+// read from a copy in the threads' order (k_trsv_pack), two steps ahead.  One
+// chain CTA that did both products alone took 3.7 to 4.6 us per step, this takes
+// 2.1 (n = 4,096: 239 / 295 -> 135 us for R^{-1} / R^{-T}); from n = 16,384 on the
+// helpers' FP64 work bounds it (n = 32,768: 2.55 / 2.89 -> 1.84 / 1.78 ms, with
+// n^2 / 2 products worth 0.93 ms).  CHAIN_D = 2 gives a helper two to three steps
+// between a block's publication and the chain's need of its sum; 3 measured the
+// same.  (Z_k C_d formed once,
+// which would leave one exchange per step, lost digits where Z_k is
+// ill-conditioned: LSQR on a cond(R) = 1e9 problem took 44 steps for 41.)
+//
+// Published values are records {low, tag, high, tag} (rec_publish) whose tag is
+// the solve's epoch, polled directly; nothing is reset between solves.  All sums
+// are in a fixed order, so results are deterministic.  Waits are bounded.
+constexpr int CHAIN_CL = 4;            // CTAs of the chain cluster (16 rows each)
+constexpr int CHAIN_D = 2;             // distances 1 .. CHAIN_D are the chain's
 constexpr int HMAXT = 4;               // targets per helper CTA
-
-__host__ __device__ constexpr size_t chain_smem_bytes() {
-  return (size_t)(2 * 3 * TTILE + 3 * TB + TB + 2 * TB + 2 * TB) * sizeof(double);
-}
-
-__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async16(double* dst, const double* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Tile of R with row block a and column block b into shared memory,
-// column-major with leading dimension TLD: T[cc * TLD + rr] = R(a*64 + rr, b*64 + cc).
-// Entries outside the n x n triangle's index range are zero.
-__device__ __forceinline__ void load_tile(double* T, const double* __restrict__ R, long long ldr, int n, int a,
-                                          int b, int first, int stride) {
-  // pairs of rows: one 16-byte copy when both lie inside (R's leading
-  // dimension and row offsets are even, so the source is 16-byte aligned)
-  const bool even = (ldr & 1) == 0;
-  for (int idx = first; idx < TB * TB / 2; idx += stride) {
-    const int rr = (idx & (TB / 2 - 1)) * 2, cc = idx >> 5;
-    const int gr = a * TB + rr, gc = b * TB + cc;
-    double* dst = T + cc * TLD + rr;
-    const double* src = R + (size_t)gc * ldr + gr;
-    if (gc < n && gr + 1 < n && even) {
-      cp_async16(dst, src);
-    } else {
-      if (gc < n && gr < n) cp_async8(dst, src);
-      else dst[0] = 0.0;
-      if (gc < n && gr + 1 < n) cp_async8(dst + 1, src + 1);
-      else dst[1] = 0.0;
-    }
-  }
-}
+constexpr int ZLD = TB + 1;            // leading dimension of a tile in shared memory
 
 template <int TRANS>
 __device__ __forceinline__ int chain_block(int t, int nblk) { return TRANS == 0 ? nblk - 1 - t : t; }
@@ -331,29 +303,34 @@ __device__ __forceinline__ int chain_block(int t, int nblk) { return TRANS == 0 
 // Inverse of each 64 x 64 diagonal block of R, block k stored column-major at
 // Z + k * 4096: Z[k][c * 64 + r] = (R_kk^{-1})(r, c).  Entries below the
 // diagonal and, in a ragged last block, rows and columns past n are zero.
-// Column c solves R_kk z = e_c by back substitution (one warp per column,
-// rows on the lanes, IEEE division by each pivot).
-__global__ void __launch_bounds__(256) k_trsv_dinv(const double* __restrict__ R, long long ldr, int n,
+// Column c solves R_kk z = e_c by back substitution (one warp per column, rows
+// on the lanes) with the pivots' reciprocals; four CTAs share a block's columns,
+// as the FP64 units of one SM would take 50 us for them.
+__global__ void __launch_bounds__(128) k_trsv_dinv(const double* __restrict__ R, long long ldr, int n,
                                                    double* __restrict__ Z) {
-  __shared__ double D[TB * TLD];
+  __shared__ double D[TB * ZLD];
+  __shared__ double rec[TB];
   const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int r0 = k * TB, rows = min(TB, n - r0);
   for (int idx = tid; idx < TB * TB; idx += blockDim.x) {
     const int r = idx & (TB - 1), c = idx >> 6;
-    D[c * TLD + r] = (r <= c && c < rows) ? R[(size_t)(r0 + c) * ldr + r0 + r] : 0.0;
+    D[c * ZLD + r] = (r <= c && c < rows) ? R[(size_t)(r0 + c) * ldr + r0 + r] : 0.0;
   }
   __syncthreads();
+  if (tid < TB) rec[tid] = tid < rows ? 1.0 / D[tid * ZLD + tid] : 0.0;
+  __syncthreads();
   double* out = Z + (size_t)k * TB * TB;
-  for (int j = w; j < TB; j += 8) {
+  for (int jj = 0; jj < TB / 16; ++jj) {
+    const int j = blockIdx.y + 4 * (w + 4 * jj);  // columns spread over CTAs and warps
     double acc0 = lane == j ? 1.0 : 0.0, acc1 = lane + 32 == j ? 1.0 : 0.0;
     double z0 = 0.0, z1 = 0.0;
     if (j < rows) {
       for (int i = j; i >= 0; --i) {
-        const double zi = __shfl_sync(0xffffffffu, i < 32 ? acc0 : acc1, i & 31) / D[i * TLD + i];
+        const double zi = __shfl_sync(0xffffffffu, i < 32 ? acc0 : acc1, i & 31) * rec[i];
         if (i < 32 && lane == i) z0 = zi;
         if (i >= 32 && lane == i - 32) z1 = zi;
-        if (lane < i) acc0 -= D[i * TLD + lane] * zi;
-        if (lane + 32 < i) acc1 -= D[i * TLD + lane + 32] * zi;
+        if (lane < i) acc0 -= D[i * ZLD + lane] * zi;
+        if (i > 32 && lane + 32 < i) acc1 -= D[i * ZLD + lane + 32] * zi;
       }
     }
     out[j * TB + lane] = z0;
@@ -361,395 +338,330 @@ __global__ void __launch_bounds__(256) k_trsv_dinv(const double* __restrict__ R,
   }
 }
 
-// A helper's partial sum is published by overwriting this value, which the
-// chain polls for: a signalling NaN with a fixed payload, which no
-// arithmetic result has (operations on NaN return the canonical quiet NaN).
-constexpr unsigned long long ACC_EMPTY = 0x7FF4A5A5A5A5A5A5ull;
-__device__ __forceinline__ void st_relaxed_f64(double* p, double v) {
-  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_relaxed_b64(const double* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
+// Offset of entry (r, c) of a tile in the order the chain's threads read it:
+// rank r / 16, then the thread's i-th column, warp, lane.
+__device__ __forceinline__ int pack_at(int r, int c) {
+  return (((r >> 4) * 8 + (c & 7)) * 4 + (c >> 4)) * 32 + (((c >> 3) & 1) << 4 | (r & 15));
 }
 
-// Before each chain launch: the progress counter at 0 and every helper
-// partial sum at ACC_EMPTY.
-__global__ void k_trsv_chain_prep(unsigned int* __restrict__ prog, double* __restrict__ accbuf, int count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) *prog = 0u;
-  if (i < count) reinterpret_cast<unsigned long long*>(accbuf)[i] = ACC_EMPTY;
+// Tiles of the chain, P[dir][k][d]: d = 0 the inverse (dir 0 Z_k, dir 1 Z_k^T),
+// d >= 1 the couplings (dir 0 R_{k,k+d}, dir 1 R_{k-d,k}^T); zero where the
+// neighbour does not exist or past n.
+__global__ void __launch_bounds__(256) k_trsv_pack(const double* __restrict__ R, long long ldr, int n, int nblk,
+                                                   const double* __restrict__ Z, double* __restrict__ P) {
+  __shared__ double t[TB * ZLD];
+  const int k = blockIdx.x, d = blockIdx.y, dir = blockIdx.z, tid = threadIdx.x;
+  const int j = dir == 0 ? k + d : k - d;  // column block (dir 0) or row block (dir 1) of the coupling
+  double* out = P + (((size_t)dir * nblk + k) * (CHAIN_D + 1) + d) * TB * TB;
+  for (int idx = tid; idx < TB * TB; idx += 256) {
+    const int lo = idx & (TB - 1), hi = idx >> 6;  // row and column of the tile as stored
+    double v = 0.0;
+    if (d == 0) {
+      v = Z[(size_t)k * TB * TB + idx];
+    } else if (j >= 0 && j < nblk) {
+      const int gr = (dir == 0 ? k : j) * TB + lo, gc = (dir == 0 ? j : k) * TB + hi;
+      if (gr < n && gc < n) v = R[(size_t)gc * ldr + gr];
+    }
+    t[dir == 0 ? hi * ZLD + lo : lo * ZLD + hi] = v;  // t[c * ZLD + r]
+  }
+  __syncthreads();
+  for (int idx = tid; idx < TB * TB; idx += 256) {
+    const int lane = idx & 31, w = (idx >> 5) & 3, i = (idx >> 7) & 7, q = idx >> 10;
+    const int r = q * 16 + (lane & 15), c = w * 16 + (lane >> 4) * 8 + i;
+    out[pack_at(r, c)] = t[c * ZLD + r];
+  }
 }
 
 struct ChainArgs {
   const double* R;
-  const double* Z;            // inverses of the diagonal blocks (k_trsv_dinv)
+  const double* P;            // the chain's tiles of this direction (k_trsv_pack)
   long long ldr;
   int n, nblk, H;
   const double* rhs;
   double* x;
-  double* accbuf;             // [nblk][64] helper partial sums, ACC_EMPTY until published
-  unsigned int* prog;         // number of blocks the chain has published (reset by k_trsv_chain_prep)
+  unsigned long long* hrec;   // [nblk][64] records of the helpers' sums
+  unsigned long long* xrec;   // [nblk][64] records of x
+  const unsigned int* epoch;  // tag of this solve (k_trsv_prep)
   unsigned int* err;
   const int* skip;
 };
 
+// The chain: ranks 0-3 of cluster 0.  Warps 0-3 take a step's critical path,
+// C_1 x_{t-1} and Z_k y_t; warps 4-7 meanwhile form the rest of the next step's
+// right-hand side (C_2, the helper's sum), one warp of each group per SM
+// partition, so that this product fills the FP64 units while the critical warps
+// wait for an exchange.  Two cluster barriers a step: B (y_t is spread) and A
+// (x_t is spread and the next right-hand side is ready).
 template <int TRANS>
-__global__ void __launch_bounds__(256, 1) k_trsv_chain(ChainArgs a) {
-  if (a.skip && *a.skip) return;
-  extern __shared__ __align__(16) double csm[];
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int nblk = a.nblk, n = a.n;
-  const int wlim = (int)__ldcg(a.err + (SYNC_WAITLIM - SYNC_ERR));
-  const unsigned int wlimit = wlim == 0 ? (1u << 22) : (unsigned int)wlim;
-  if (blockIdx.x == 0) {
-    // ------------------------------------------------------------ chain
-    // Warps 0-3 take step t's critical path: y = base_t - C1_t x_{t-1}, then
-    // x_t = Z_k y, two threads per row (each a fixed half of the terms), with
-    // base_t = b_k - (helper sum) - (distance-2 sum) prepared one step ahead.
-    // Warps 4-7 meanwhile publish x_{t-1}, issue the copies of Z and C1 for
-    // step t + 2, form the distance-2 sum of step t + 1 (C2_{t+1} x_{t-1},
-    // with C2_{t+1} fetched into registers one step earlier), fetch C2_{t+2},
-    // acquire the helpers' sum of step t + 1 and form base_{t+1}.
-    double* Zb = csm;                          // [3] inverse diagonal tiles
-    double* C1b = Zb + 3 * TTILE;              // [3] coupling to the previous block
-    double* xh = C1b + 3 * TTILE;              // x of the last three steps [3][64]
-    double* ys = xh + 3 * TB;                  // [64] right-hand side of the diagonal block
-    double* base = ys + TB;                    // [2][64]
-    double* d2p = base + 2 * TB;               // [2][64] halves of the distance-2 sum
-    const bool crit = w < 4;
-    const int ct = crit ? tid : tid - 128;     // thread index within its group of 128
-    const int r = ct >> 1, hh = ct & 1;        // row and half (critical path)
-    const int q64 = ct & 63, qh = ct >> 6;     // distance-2 layout
-    // Term i (0..31) of half hh: the column index of a tile row.  The order
-    // keeps a warp's shared-memory reads on distinct banks: T[term * TLD + r]
-    // for TRANS 0, T[r * TLD + term] for TRANS 1.
-    auto term = [&](int i) { return TRANS == 0 ? (i & 3) + 8 * (i >> 2) + 4 * hh : 2 * i + hh; };
-    auto tile_dot = [&](const double* T, const double* v, int i0, int i1) {
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      for (int i = i0; i < i1; i += 4) {
-        const int y0 = term(i), y1 = term(i + 1), y2 = term(i + 2), y3 = term(i + 3);
-        if (TRANS == 0) {
-          s0 += T[y0 * TLD + r] * v[y0];
-          s1 += T[y1 * TLD + r] * v[y1];
-          s2 += T[y2 * TLD + r] * v[y2];
-          s3 += T[y3 * TLD + r] * v[y3];
-        } else {
-          s0 += T[r * TLD + y0] * v[y0];
-          s1 += T[r * TLD + y1] * v[y1];
-          s2 += T[r * TLD + y2] * v[y2];
-          s3 += T[r * TLD + y3] * v[y3];
-        }
-      }
-      const double s = (s0 + s1) + (s2 + s3);
-      return s + __shfl_xor_sync(0xffffffffu, s, 1);
-    };
-    auto issue_zc1 = [&](int tt) {             // Z_tt and C1_tt
-      const int k = chain_block<TRANS>(tt, nblk);
-      const double* src = a.Z + (size_t)k * TB * TB;
-      double* dst = Zb + (tt % 3) * TTILE;
-      for (int idx = ct; idx < TB * TB / 2; idx += 128) {
-        const int rr = (idx & (TB / 2 - 1)) * 2, cc = idx >> 5;
-        cp_async16(dst + cc * TLD + rr, src + cc * TB + rr);
-      }
-      if (tt >= 1) {
-        const int j = chain_block<TRANS>(tt - 1, nblk);
-        if (TRANS == 0) load_tile(C1b + (tt % 3) * TTILE, a.R, a.ldr, n, k, j, ct, 128);
-        else load_tile(C1b + (tt % 3) * TTILE, a.R, a.ldr, n, j, k, ct, 128);
-      }
-    };
-    // C2_tt in registers: thread (q64, qh) holds the 32 entries of output
-    // row q64 of block k against the source rows 32 qh .. 32 qh + 31 of
-    // block j.  TRANS 0: R(k*64 + q64, j*64 + 32 qh + i), one column of R per
-    // entry, the lanes of a warp on consecutive rows; TRANS 1 (the coupling
-    // of R^T): R(j*64 + 32 qh + i, k*64 + q64), 32 consecutive entries of one
-    // column of R per thread.
-    double c2v[32];
-    auto fetch_c2 = [&](int tt) {
-      const int k = chain_block<TRANS>(tt, nblk), j = chain_block<TRANS>(tt - 2, nblk);
-      const int go = k * TB + q64, gs = j * TB + 32 * qh;  // output index, first source index
+__device__ __forceinline__ void trsv_chain(const ChainArgs& a, unsigned int tag, RecWait& wait, double* sm) {
+  double* xs = sm;                 // [4][64] x of the last steps, all rows
+  double* ys = xs + 4 * TB;        // [64] y, all rows
+  double* part = ys + TB;          // [3][4][16] the warps' partial sums: y, x, next right-hand side
+  double* hs = part + 3 * 4 * 16;  // [2][16] this rank's rows of b - s - C_2 x, steps alternating
+  const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 3;
+  const bool crit = tid < 128;
+  const int rank = blockIdx.x, nblk = a.nblk, n = a.n;
+  const int c0 = (w * 2 + (lane >> 4)) * 8;  // this thread's columns
+  // tile d of step t
+  auto fetch = [&](double (&q)[8], int t, int d) {
+    if (t >= nblk) return;
+    const double* src = a.P + ((size_t)chain_block<TRANS>(t, nblk) * (CHAIN_D + 1) + d) * TB * TB +
+                        (rank * 8 * 4 + w) * 32 + lane;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const bool ok = go < n && gs + i < n;
-        if (TRANS == 0) c2v[i] = ok ? __ldg(a.R + (size_t)(gs + i) * a.ldr + go) : 0.0;
-        else c2v[i] = ok ? __ldg(a.R + (size_t)go * a.ldr + gs + i) : 0.0;
-      }
-    };
-    // the half qh of C2 x_{t-2} for output q64, into d2p[2][64]
-    auto dist2 = [&](const double* xv) {
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    for (int i = 0; i < 8; ++i) q[i] = __ldg(src + i * 128);
+  };
+  auto dot8 = [&](const double (&q)[8], const double* v, double acc) {
 #pragma unroll
-      for (int i = 0; i < 32; i += 4) {
-        s0 += c2v[i] * xv[32 * qh + i];
-        s1 += c2v[i + 1] * xv[32 * qh + i + 1];
-        s2 += c2v[i + 2] * xv[32 * qh + i + 2];
-        s3 += c2v[i + 3] * xv[32 * qh + i + 3];
-      }
-      d2p[qh * TB + q64] = (s0 + s1) + (s2 + s3);
-    };
-    // x = Z y with the triangle balanced over the threads: rows g and 63 - g
-    // share four threads (s = ct & 3), whose terms are the positions p = s,
-    // s + 4, ... of the pair's 65 terms (row A = g first, then row B = 63 - g).
-    const int zg = ct >> 2, zs = ct & 3;
-    const int zA = zg, zB = TB - 1 - zg;
-    const int znA = TRANS == 0 ? TB - zg : zg + 1;  // terms of row A
-    auto zdot = [&](const double* Zt, const double* yv, double& xa, double& xb) {
-      double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
-#pragma unroll
-      for (int i = 0; i < 17; ++i) {
-        const int pos = zs + 4 * i;
-        if (pos > TB) break;  // 65 terms per pair
-        const bool inA = pos < znA;
-        // column of the term: TRANS 0 row A columns g .. 63, row B 63-g .. 63;
-        // TRANS 1 row A columns 0 .. g, row B 0 .. 63-g
-        const int c = TRANS == 0 ? (inA ? zg + pos : pos - 1) : (inA ? pos : pos - znA);
-        const int row = inA ? zA : zB;
-        const double zv = TRANS == 0 ? Zt[c * TLD + row] : Zt[row * TLD + c];
-        const double prod = zv * yv[c];
-        if (inA) {
-          if (i & 1) a1 += prod; else a0 += prod;
-        } else {
-          if (i & 1) b1 += prod; else b0 += prod;
-        }
-      }
-      double sa = a0 + a1, sb = b0 + b1;
-      sa += __shfl_xor_sync(0xffffffffu, sa, 1);
-      sb += __shfl_xor_sync(0xffffffffu, sb, 1);
-      sa += __shfl_xor_sync(0xffffffffu, sa, 2);
-      sb += __shfl_xor_sync(0xffffffffu, sb, 2);
-      xa = sa;
-      xb = sb;
-    };
-    if (!crit) {
-      issue_zc1(0);
-      cp_async_commit();
-      if (nblk > 1) issue_zc1(1);
-      cp_async_commit();
-      if (ct < TB) {
-        const int r0 = chain_block<TRANS>(0, nblk) * TB;
-        base[ct] = r0 + ct < n ? a.rhs[r0 + ct] : 0.0;
-      }
-      cp_async_wait1();
+    for (int i = 0; i < 8; i += 2) {
+      const double2 t = *reinterpret_cast<const double2*>(v + c0 + i);
+      acc = fma(q[i], t.x, acc);
+      acc = fma(q[i + 1], t.y, acc);
     }
-    __syncthreads();
-    for (int t = 0; t < nblk; ++t) {
-      if (crit) {
-        const int k = chain_block<TRANS>(t, nblk);
-        const int r0 = k * TB, rows = min(TB, n - r0);
-        const double bs = base[(t & 1) * TB + r];
-        const double p = t >= 1 ? tile_dot(C1b + (t % 3) * TTILE, xh + ((t + 2) % 3) * TB, 0, 32) : 0.0;
-        if (hh == 0) ys[r] = bs - p;
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        double xa, xb;
-        zdot(Zb + (t % 3) * TTILE, ys, xa, xb);
-        if (zs == 0) {
-          xh[(t % 3) * TB + zA] = xa;
-          if (zA < rows) a.x[r0 + zA] = xa;
-        } else if (zs == 1) {
-          xh[(t % 3) * TB + zB] = xb;
-          if (zB < rows) a.x[r0 + zB] = xb;
+    return acc;
+  };
+  // this thread's part of a row summed over its warp's columns, then the warps'
+  auto row_part = [&](double acc, double* p) {
+    acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+    if (lane < 16) p[w * 16 + lane] = acc;
+    __syncwarp();
+    if (crit) asm volatile("bar.sync 1, 128;" ::: "memory");
+    else asm volatile("bar.sync 2, 128;" ::: "memory");
+  };
+  auto row_sum = [&](const double* p) {
+    const int r = lane & 15;
+    return (p[r] + p[16 + r]) + (p[32 + r] + p[48 + r]);
+  };
+  // row r of this rank to every rank: lanes 0-15 write to ranks 0, 1, lanes 16-31 to ranks 2, 3
+  auto spread = [&](double* v, double val) {
+    double* dst = v + rank * 16 + (lane & 15);
+    st_cluster(dst, (lane >> 4) * 2, val);
+    st_cluster(dst, (lane >> 4) * 2 + 1, val);
+  };
+  double m[2][2][8];
+  if (crit) {
+    for (int i = tid; i < 4 * TB; i += 128) xs[i] = 0.0;
+    fetch(m[0][0], 0, 0);
+    fetch(m[0][1], 0, 1);
+    fetch(m[1][0], 1, 0);
+    fetch(m[1][1], 1, 1);
+    cluster_arrive();
+    auto step = [&](double (&q)[2][8], int t) {
+      const int k = chain_block<TRANS>(t, nblk);
+      cluster_wait();  // A: x_{t-1} and hs of this step
+      row_part(dot8(q[1], xs + ((t - 1) & 3) * TB, 0.0), part);
+      if (w == 0) spread(ys, hs[(t & 1) * 16 + (lane & 15)] - row_sum(part));
+      cluster_arrive();
+      cluster_wait();  // B: y_t
+      row_part(dot8(q[0], ys, 0.0), part + 64);
+      if (w == 0) {
+        const double xv = row_sum(part + 64);
+        spread(xs + (t & 3) * TB, xv);
+        if (lane < 16) {
+          const int gi = k * TB + rank * 16 + lane;
+          rec_publish(a.xrec + (size_t)gi * 2, xv, tag);
+          if (gi < n) a.x[gi] = xv;
         }
-      } else {
-        const bool more = t + 1 < nblk;
-        const int r1 = more ? chain_block<TRANS>(t + 1, nblk) * TB : 0;
-        const double rb = more && ct < TB && r1 + ct < n ? a.rhs[r1 + ct] : 0.0;
-        if (ct == 96 && t >= 1) {  // blocks 0 .. t-1 are in a.x (barrier at the end of step t-1)
-          __threadfence();
-          st_release(a.prog, (unsigned int)t);
-        }
-        if (t + 2 < nblk) issue_zc1(t + 2);
-        cp_async_commit();
-        if (more) {
-          if (t + 1 >= 2) {
-            dist2(xh + ((t + 2) % 3) * TB);
-          } else if (ct < TB) {
-            d2p[ct] = 0.0;
-            d2p[TB + ct] = 0.0;
-          }
-          if (t + 2 < nblk) fetch_c2(t + 2);
-        }
-        // the helpers' sum of step t + 1: poll the entry until it is published
-        double acc = 0.0;
-        if (more && ct < TB && t + 1 >= CHAIN_NEAR) {
-          const double* src = a.accbuf + (size_t)r1 + ct;
-          unsigned long long v = ld_relaxed_b64(src);
+      }
+      cluster_arrive();
+      fetch(q[0], t + 2, 0);
+      fetch(q[1], t + 2, 1);
+    };
+    for (int t = 0; t < nblk; t += 2) {
+      step(m[0], t);
+      if (t + 1 < nblk) step(m[1], t + 1);
+    }
+  } else {
+    // b - s - C_2 x_{t-2} of step t into hs
+    auto prepare = [&](double (&q)[8], int t) {
+      const int gi = t < nblk ? chain_block<TRANS>(t, nblk) * TB + rank * 16 + lane : 0;
+      const bool own = w == 0 && lane < 16 && t < nblk;
+      const bool summed = own && t > CHAIN_D;
+      const unsigned long long* rec = a.hrec + (size_t)gi * 2;
+      unsigned long long lo = 0, hi = 0;
+      if (summed) rec_load(rec, lo, hi);
+      double v = own && gi < n ? a.rhs[gi] : 0.0;
+      row_part(dot8(q, xs + ((t - 2) & 3) * TB, 0.0), part + 128);
+      if (w == 0) {
+        const double near = row_sum(part + 128);
+        if (summed) {
           unsigned int spins = 0;
-          while (v == ACC_EMPTY) {
-            if (wlim < 0 || ++spins > wlimit) {
-              atomicExch(a.err, 1u);
-              v = 0ull;
-              break;
-            }
-            if (spins > (1u << 16)) __nanosleep(128);
-            v = ld_relaxed_b64(src);
-          }
-          acc = __longlong_as_double((long long)v);
+          while (!rec_ready(lo, hi, tag) && wait.spin(spins)) rec_load(rec, lo, hi);
+          v -= rec_value(lo, hi);
         }
-        asm volatile("bar.sync 2, 128;" ::: "memory");
-        if (more && ct < TB) base[((t + 1) & 1) * TB + ct] = (rb - acc) - (d2p[ct] + d2p[TB + ct]);
-        cp_async_wait1();  // Z_{t+1} and C1_{t+1}
+        if (own) hs[(t & 1) * 16 + lane] = v - near;
       }
-      __syncthreads();
+      fetch(q, t + 2, 2);
+    };
+    if (w == 0 && lane < 16) {
+      const int gi = chain_block<TRANS>(0, nblk) * TB + rank * 16 + lane;
+      hs[lane] = gi < n ? a.rhs[gi] : 0.0;
     }
-    if (!crit && ct == 96) {
-      __threadfence();
-      st_release(a.prog, (unsigned int)nblk);
+    fetch(m[1][0], 1, 2);
+    fetch(m[0][0], 2, 2);
+    cluster_arrive();
+    auto step = [&](double (&q)[8], int t) {
+      cluster_wait();    // A: x_{t-1}
+      cluster_arrive();  // B needs nothing of these warps
+      if (t + 1 < nblk) prepare(q, t + 1);
+      cluster_wait();
+      cluster_arrive();
+    };
+    for (int t = 0; t < nblk; t += 2) {
+      step(m[1][0], t);
+      if (t + 1 < nblk) step(m[0][0], t + 1);
     }
-    cp_async_wait0();
-    return;
   }
-  // -------------------------------------------------------------- helper
-  const int h = blockIdx.x - 1;
-  int tg[HMAXT], nt = 0;
+  cluster_wait();  // no rank leaves before the last remote store has landed
+}
+
+// Helper h: its targets t = h + H m, m < NT.
+template <int TRANS, int NT>
+__device__ __forceinline__ void trsv_helper(const ChainArgs& a, unsigned int tag, RecWait& wait, double* sm) {
+  double* xs = sm;                   // [2][64] x of the source block
+  double* sred = xs + 2 * TB;        // [8][64]
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int nblk = a.nblk, n = a.n, h = blockIdx.x - CHAIN_CL;
+  int tg[NT], nt = 0;
 #pragma unroll
-  for (int m = 0; m < HMAXT; ++m) {
-    const int t = CHAIN_NEAR + h + a.H * m;
+  for (int m = 0; m < NT; ++m) {
+    const int t = h + a.H * m;
     tg[m] = t < nblk ? t : -1;
     if (t < nblk) nt = m + 1;
   }
   if (nt == 0) return;
-  const int tmax = tg[nt - 1];
-  double* sred = csm;                    // [8][64]
-  __shared__ unsigned int seen_s;        // progress counter as last read
-  double pa[HMAXT][2];   // TRANS 0: partial sums of target rows lane, lane+32 over this warp's sources
-  double ptp[HMAXT][8];  // TRANS 1: partial sums of target rows w + 8 q over this lane's sources
+  const int tmax = h + a.H * (nt - 1);
+  double pa[NT][2];   // TRANS 0: partial sums of target rows lane, lane+32 over this warp's sources
+  double ptp[NT][8];  // TRANS 1: partial sums of target rows w + 8 q over this lane's sources
 #pragma unroll
-  for (int m = 0; m < HMAXT; ++m) {
+  for (int m = 0; m < NT; ++m) {
     pa[m][0] = pa[m][1] = 0.0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) ptp[m][q] = 0.0;
   }
-  unsigned int seen = 0;
-  for (int u = 0; u + CHAIN_NEAR <= tmax; ++u) {
-    const int j = chain_block<TRANS>(u, nblk);
-    const int c0 = j * TB;
-    // this step's tile entries into registers first (they do not depend on
-    // x): TRANS 0 rows lane, lane+32 of R(k, j), columns w + 8 q; TRANS 1
-    // rows w + 8 q of R(j, k) (columns of block k), read along j's rows
-    double tv[HMAXT][16];
-#pragma unroll
-    for (int m = 0; m < HMAXT; ++m) {
-      const bool live = m < nt && tg[m] >= u + CHAIN_NEAR;
-      const int k = live ? chain_block<TRANS>(tg[m], nblk) : 0;
-      const int r0 = k * TB;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int y = w + 8 * q;
-        if (TRANS == 0) {  // R(r0 + lane (+32), c0 + y)
-          const bool ok = live && c0 + y < n;
-          const double* col = a.R + (size_t)(c0 + y) * a.ldr + r0;
-          tv[m][2 * q] = ok && r0 + lane < n ? __ldg(col + lane) : 0.0;
-          tv[m][2 * q + 1] = ok && r0 + lane + 32 < n ? __ldg(col + lane + 32) : 0.0;
-        } else {           // R(c0 + lane (+32), r0 + y): target row y
-          const bool ok = live && r0 + y < n;
-          const double* col = a.R + (size_t)(r0 + y) * a.ldr + c0;
-          tv[m][2 * q] = ok ? __ldg(col + lane) : 0.0;
-          tv[m][2 * q + 1] = ok ? __ldg(col + lane + 32) : 0.0;
-        }
-      }
-    }
-    // block u published?  (the counter only grows; read it again only when needed)
-    if (seen < (unsigned int)(u + 1)) {
-      if (tid == 0) {
-        unsigned int v = ld_acquire(a.prog), spins = 0;
-        while (v < (unsigned int)(u + 1)) {
-          if (wlim < 0 || ++spins > wlimit) {
-            atomicExch(a.err, 1u);
-            v = (unsigned int)(u + 1);
-            break;
-          }
-          if (spins > (1u << 16)) __nanosleep(128);
-          v = ld_acquire(a.prog);
-        }
-        seen_s = v;
-      }
+  // the sum of target m's partial sums, published
+  auto finish = [&](int m, const double (&p2)[2], const double (&p8)[8]) {
+    unsigned long long* out = a.hrec + (size_t)chain_block<TRANS>(tg[m], nblk) * TB * 2;
+    if (TRANS == 0) {
+      sred[w * TB + lane] = p2[0];
+      sred[w * TB + lane + 32] = p2[1];
       __syncthreads();
-      seen = seen_s;
+      if (tid < TB) {
+        double sum = sred[tid];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) sum += sred[q * TB + tid];
+        rec_publish(out + 2 * tid, sum, tag);
+      }
+      __syncthreads();  // sred is rewritten by the next target
+    } else {
+      // sum of p8[q] over the lanes, lane q (< 8) ends with entry q
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = p8[q];
+#pragma unroll
+      for (int o = 4; o >= 1; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < o; ++q) {
+          const double send = up ? v[q] : v[q + o];
+          const double keep = up ? v[q + o] : v[q];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+      if (lane < 8) rec_publish(out + 2 * (w + 8 * lane), v[0], tag);
     }
+  };
+  // tile entries of (source u, target m): TRANS 0 rows lane, lane+32 of R(k, j),
+  // columns w + 8 q; TRANS 1 rows w + 8 q of R(j, k) (columns of block k), read
+  // along j's rows
+  auto load_tile = [&](double (&tv)[16], int u, int t) {
+    const bool live = t >= u + CHAIN_D + 1;
+    const int j = chain_block<TRANS>(u, nblk), k = live ? chain_block<TRANS>(t, nblk) : 0;
+    const int c0 = j * TB, r0 = k * TB;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int y = w + 8 * q;
+      if (TRANS == 0) {  // R(r0 + lane (+32), c0 + y)
+        const bool ok = live && c0 + y < n;
+        const double* col = a.R + (size_t)(c0 + y) * a.ldr + r0;
+        tv[2 * q] = ok && r0 + lane < n ? __ldg(col + lane) : 0.0;
+        tv[2 * q + 1] = ok && r0 + lane + 32 < n ? __ldg(col + lane + 32) : 0.0;
+      } else {           // R(c0 + lane (+32), r0 + y): target row y
+        const bool ok = live && r0 + y < n;
+        const double* col = a.R + (size_t)(r0 + y) * a.ldr + c0;
+        tv[2 * q] = ok ? __ldg(col + lane) : 0.0;
+        tv[2 * q + 1] = ok ? __ldg(col + lane + 32) : 0.0;
+      }
+    }
+  };
+  // x_u by records: threads 0-63 load theirs for the next source ahead
+  unsigned long long xlo = 0, xhi = 0;
+  auto load_x = [&](int u) {
+    if (tid < TB && u < nblk) rec_load(a.xrec + ((size_t)chain_block<TRANS>(u, nblk) * TB + tid) * 2, xlo, xhi);
+  };
+  const int last = tmax - CHAIN_D - 1;  // last source of the last target
+  double t[NT][16];
+  auto source = [&](int u) {
+    double* xb = xs + (u & 1) * TB;
+    if (tid < TB) {
+      unsigned int spins = 0;
+      while (!rec_ready(xlo, xhi, tag) && wait.spin(spins)) load_x(u);
+      xb[tid] = rec_value(xlo, xhi);
+    }
+    __syncthreads();
+    load_x(u + 1);
     double xv[8], z0 = 0.0, z1 = 0.0;
     if (TRANS == 0) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int y = w + 8 * q;
-        xv[q] = c0 + y < n ? __ldcg(a.x + c0 + y) : 0.0;
-      }
+      for (int q = 0; q < 8; ++q) xv[q] = xb[w + 8 * q];
     } else {
-      z0 = __ldcg(a.x + c0 + lane);
-      z1 = __ldcg(a.x + c0 + lane + 32);
+      z0 = xb[lane];
+      z1 = xb[lane + 32];
     }
-    // The target due now (its last helper source) first, then published;
-    // then the targets still live.  Slots past their target (or empty) do no
-    // arithmetic.
+    // the targets in the order they are due (the first live one may be due now)
 #pragma unroll
-    for (int m = 0; m < HMAXT; ++m) {
-      if (!(m < nt && tg[m] == u + CHAIN_NEAR)) continue;
+    for (int m = 0; m < NT; ++m) {
+      if (!(m < nt && tg[m] >= u + CHAIN_D + 1)) continue;
       if (TRANS == 0) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          pa[m][0] += tv[m][2 * q] * xv[q];
-          pa[m][1] += tv[m][2 * q + 1] * xv[q];
+          pa[m][0] += t[m][2 * q] * xv[q];
+          pa[m][1] += t[m][2 * q + 1] * xv[q];
         }
       } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) ptp[m][q] = fma(tv[m][2 * q + 1], z1, fma(tv[m][2 * q], z0, ptp[m][q]));
+        for (int q = 0; q < 8; ++q) ptp[m][q] = fma(t[m][2 * q + 1], z1, fma(t[m][2 * q], z0, ptp[m][q]));
       }
-      const int k = chain_block<TRANS>(tg[m], nblk);
-      double* out = a.accbuf + (size_t)k * TB;
-      if (TRANS == 0) {
-        sred[w * TB + lane] = pa[m][0];
-        sred[w * TB + lane + 32] = pa[m][1];
-        __syncthreads();
-        if (w == 0) {
-          for (int hh = 0; hh < 2; ++hh) {
-            double sm = 0.0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) sm += sred[q * TB + lane + 32 * hh];
-            st_relaxed_f64(out + lane + 32 * hh, sm);
-          }
-        }
-      } else {
-        // sum of ptp[m][q] over the lanes, lane q (< 8) ends with entry q
-        double v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = ptp[m][q];
-#pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) {
-          const bool up = (lane & o) != 0;
-#pragma unroll
-          for (int q = 0; q < o; ++q) {
-            const double send = up ? v[q] : v[q + o];
-            const double keep = up ? v[q + o] : v[q];
-            v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-          }
-        }
-        // lanes L and L ^ 8, L ^ 16, L ^ 24 hold partial sums of entry L & 7
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
-        if (lane < 8) st_relaxed_f64(out + w + 8 * lane, v[0]);
-      }
-      __syncthreads();  // sred is rewritten by the next publication
+      if (tg[m] == u + CHAIN_D + 1) finish(m, pa[m], ptp[m]);
+      else load_tile(t[m], u + 1, tg[m]);  // in flight during the other targets and the wait for x_{u+1}
     }
+  };
+  load_x(0);
 #pragma unroll
-    for (int m = 0; m < HMAXT; ++m) {
-      if (!(m < nt && tg[m] > u + CHAIN_NEAR)) continue;
-      if (TRANS == 0) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          pa[m][0] += tv[m][2 * q] * xv[q];
-          pa[m][1] += tv[m][2 * q + 1] * xv[q];
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) ptp[m][q] = fma(tv[m][2 * q + 1], z1, fma(tv[m][2 * q], z0, ptp[m][q]));
-      }
-    }
+  for (int m = 0; m < NT; ++m)
+    if (m < nt) load_tile(t[m], 0, tg[m]);
+  for (int u = 0; u <= last; ++u) source(u);
+}
+
+constexpr size_t chain_smem_bytes() { return (size_t)(2 * TB + 8 * TB) * sizeof(double); }
+
+template <int TRANS, int NT>
+__global__ void __launch_bounds__(256, 1) k_trsv_chain(ChainArgs a) {
+  if (a.skip && *a.skip) return;
+  extern __shared__ __align__(16) double csm[];
+  const unsigned int tag = *a.epoch;  // set by k_trsv_prep, which ran before this launch
+  RecWait wait(a.err, threadIdx.x);
+  if (blockIdx.x < CHAIN_CL) {
+    trsv_chain<TRANS>(a, tag, wait, csm);
+  } else {
+    trsv_helper<TRANS, NT>(a, tag, wait, csm);
   }
 }
 
-// Next epoch for the block flags (never 0, the initial flag value) and a fresh
-// ticket counter; runs before every k_trsv so that replays of a captured graph
-// see a new epoch each time.
+// Next epoch for the block flags and record tags (never 0, their initial value)
+// and a fresh ticket counter; runs before every solve so that replays of a
+// captured graph see a new epoch each time.
 __global__ void k_trsv_prep(unsigned int* __restrict__ epoch, unsigned int* __restrict__ ticket) {
   unsigned int e = *epoch + 1u;
   *epoch = e == 0u ? 1u : e;
@@ -825,7 +737,7 @@ rfm_status rfm_launch_jmv_axpby(rfm_problem* p, const double* x, double s1, doub
 // Slices of every column block's rows: the count with the least work on the
 // busiest SM (about 16 CTAs of an SM run at once), at most JT_SLICES and at
 // least 128 rows each on average.  One slice per block left 16 CTAs for 15,552
-// rows of 8 blocks of 128 (60 us; 10 with 19 slices, and 2 for their sum).
+// rows of 8 blocks of 128 (60 us; 10 with 9 slices, and 2 for their sum).
 static int jtmv_slices(const rfm_problem* p) {
   const int nsm = std::max(1, rfm_num_sms());
   const long long tiles = (long long)p->G * ((p->W + 63) / 64);
@@ -859,12 +771,60 @@ rfm_status rfm_launch_jtmv(rfm_problem* p, const double* x, double* y) {
 
 rfm_status rfm_trsv_prepare(rfm_problem* p) {
   if (!p->dinv || !p->R) return RFM_OK;
-  const int n = (int)p->n;
-  k_trsv_dinv<<<(n + TB - 1) / TB, 256, 0, p->stream>>>(p->R, p->ldr, n, p->dinv);
+  const int n = (int)p->n, nblk = (n + TB - 1) / TB;
+  k_trsv_dinv<<<dim3(nblk, 4), 128, 0, p->stream>>>(p->R, p->ldr, n, p->dinv);
+  RFM_CHECK_LAUNCH();
+  k_trsv_pack<<<dim3(nblk, CHAIN_D + 1, 2), 256, 0, p->stream>>>(p->R, p->ldr, n, nblk, p->dinv, p->chain_tiles);
   RFM_CHECK_LAUNCH();
   p->dinv_of = p->R;
   return RFM_OK;
 }
+
+long long rfm_trsv_tiles_len(long long n) { return 2LL * ((n + TB - 1) / TB) * (CHAIN_D + 1) * TB * TB; }
+
+namespace {
+using ChainKernel = void (*)(ChainArgs);
+ChainKernel chain_kernel(int trans, int nt) {
+  static const ChainKernel k[2][3] = {{k_trsv_chain<0, 1>, k_trsv_chain<0, 2>, k_trsv_chain<0, HMAXT>},
+                                      {k_trsv_chain<1, 1>, k_trsv_chain<1, 2>, k_trsv_chain<1, HMAXT>}};
+  return k[trans ? 1 : 0][nt == 1 ? 0 : nt == 2 ? 1 : 2];
+}
+
+// CTAs of the chain kernels that are resident together (whole clusters), per
+// device; 0 on failure.
+int chain_max_ctas() {
+  static std::mutex mu;
+  static int cached[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  if (cached[dev] == 0) {
+    int least = 1 << 30;
+    for (int trans = 0; trans < 2; ++trans)
+      for (int nt : {1, 2, HMAXT}) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CHAIN_CL;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(CHAIN_CL);
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = chain_smem_bytes();
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int c = 0;
+        const ChainKernel fn = chain_kernel(trans, nt);
+        if (rfm_smem_attr((const void*)fn, (int)chain_smem_bytes()) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&c, fn, &cfg) != cudaSuccess)
+          return 0;
+        least = std::min(least, c * CHAIN_CL);
+      }
+    // one CTA per SM: two would share the FP64 units the chain depends on
+    cached[dev] = std::min(least, rfm_num_sms() / CHAIN_CL * CHAIN_CL);
+  }
+  return cached[dev];
+}
+}  // namespace
 
 rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x) {
   const int n = (int)p->n;
@@ -876,35 +836,33 @@ rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x
   if (p->dinv && p->dinv_of != p->R) RFM_TRY(rfm_trsv_prepare(p));
   ProfScope ps(PF_TRSV, p->stream);
   rfm_prof_work(PF_TRSV, 8.0 * (double)n * (n + 1) / 2 + 16.0 * n);  // R read once, b and x
-  // chain + helpers when every target past distance 2 has a helper slot
-  const int nsm = rfm_num_sms();
-  const int H = nblk > CHAIN_NEAR ? std::min(nsm - 1, nblk - CHAIN_NEAR) : 0;
-  if (p->trsv_acc && p->dinv && nsm > 1 && nblk - CHAIN_NEAR <= HMAXT * H) {
-    k_trsv_chain_prep<<<(nblk * TB + 255) / 256, 256, 0, p->stream>>>(p->sync + SYNC_TICKET, p->trsv_acc, nblk * TB);
-    RFM_CHECK_LAUNCH();
+  k_trsv_prep<<<1, 1, 0, p->stream>>>(p->sync + SYNC_EPOCH, p->sync + SYNC_TICKET);
+  RFM_CHECK_LAUNCH();
+  // chain + helpers when every block has a helper slot
+  const int H = std::min(chain_max_ctas() - CHAIN_CL, (nblk + CHAIN_CL - 1) / CHAIN_CL * CHAIN_CL);
+  if (p->trsv_rec && p->dinv && p->chain_tiles && H > 0 && nblk <= HMAXT * H) {
     ChainArgs a;
-    a.R = p->R; a.Z = p->dinv; a.ldr = p->ldr; a.n = n; a.nblk = nblk; a.H = H; a.rhs = b; a.x = x;
-    a.accbuf = p->trsv_acc; a.prog = p->sync + SYNC_TICKET;
-    a.err = p->sync + SYNC_ERR; a.skip = p->skip;
-    const void* fn = trans == 0 ? (const void*)k_trsv_chain<0> : (const void*)k_trsv_chain<1>;
-    RFM_CUDA(rfm_smem_attr(fn, (int)chain_smem_bytes()));
+    a.R = p->R; a.P = p->chain_tiles + (trans ? rfm_trsv_tiles_len(n) / 2 : 0);
+    a.ldr = p->ldr; a.n = n; a.nblk = nblk; a.H = H; a.rhs = b; a.x = x;
+    a.hrec = p->trsv_rec; a.xrec = p->trsv_rec + (size_t)nblk * TB * 2;
+    a.epoch = p->sync + SYNC_EPOCH; a.err = p->sync + SYNC_ERR; a.skip = p->skip;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(1 + H));
+    cfg.gridDim = dim3((unsigned)(CHAIN_CL + H));
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = chain_smem_bytes();
     cfg.stream = p->stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: helpers and the chain wait on each other
     attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = CHAIN_CL;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (trans == 0) RFM_CUDA(cudaLaunchKernelEx(&cfg, k_trsv_chain<0>, a));
-    else RFM_CUDA(cudaLaunchKernelEx(&cfg, k_trsv_chain<1>, a));
+    cfg.numAttrs = 2;
+    RFM_CUDA(cudaLaunchKernelEx(&cfg, chain_kernel(trans, (nblk + H - 1) / H), a));
     RFM_CHECK_LAUNCH();
     return RFM_OK;
   }
-  k_trsv_prep<<<1, 1, 0, p->stream>>>(p->sync + SYNC_EPOCH, p->sync + SYNC_TICKET);
-  RFM_CHECK_LAUNCH();
   if (trans == 0)
     k_trsv<0><<<nblk, 256, 0, p->stream>>>(p->R, p->ldr, n, b, x, p->sync + SYNC_FLAGS, p->sync + SYNC_EPOCH,
                                            p->sync + SYNC_TICKET, p->sync + SYNC_ERR, p->skip);

@@ -97,23 +97,8 @@ __host__ __device__ constexpr size_t kb_fixed_smem() { return (size_t)(KB_TRI + 
 // rows) are free of bank conflicts.
 __device__ __forceinline__ int kb_at(int r, int c, int ld) { return r * ld + (c & ~31) + ((c ^ r) & 31); }
 
-struct KbWait {
-  int lim;             // polls of one wait; < 0: give up at once
-  unsigned int* err;
-  bool dead;           // a wait of this launch gave up: do not wait again
-  __device__ __forceinline__ bool spin(unsigned int& n) {  // false: give up
-    if (dead || lim < 0 || ++n > (unsigned int)lim) {
-      if (!dead) atomicExch(err, 1u);
-      dead = true;
-      return false;
-    }
-    if (n > (1u << 16)) __nanosleep(128);
-    return true;
-  }
-};
-
 // Arrivals of all CTAs up to the count `want` (the counter only grows).
-__device__ __forceinline__ void kb_barrier(unsigned int* bar, unsigned int want, KbWait& kw) {
+__device__ __forceinline__ void kb_barrier(unsigned int* bar, unsigned int want, RecWait& kw) {
   __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
@@ -122,35 +107,6 @@ __device__ __forceinline__ void kb_barrier(unsigned int* bar, unsigned int want,
       if (!kw.spin(n)) break;
   }
   __syncthreads();
-}
-
-// Store to the same shared-memory variable of rank `rank` of the cluster.
-__device__ __forceinline__ void kb_store_cluster(double* p, int rank, double v) {
-  asm volatile(
-      "{\n .reg .b32 r;\n mapa.shared::cluster.u32 r, %0, %1;\n st.shared::cluster.f64 [r], %2;\n}\n" ::"r"(
-          (unsigned)__cvta_generic_to_shared(p)),
-      "r"(rank), "d"(v)
-      : "memory");
-}
-__device__ __forceinline__ void kb_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void kb_publish(unsigned long long* rec, double v, unsigned int tag) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const unsigned long long lo = (b & 0xffffffffull) | ((unsigned long long)tag << 32);
-  const unsigned long long hi = (b >> 32) | ((unsigned long long)tag << 32);
-  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(rec), "l"(lo), "l"(hi) : "memory");
-}
-__device__ __forceinline__ void kb_load(const unsigned long long* rec, unsigned long long& lo,
-                                        unsigned long long& hi) {
-  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(rec) : "memory");
-}
-__device__ __forceinline__ bool kb_ready(unsigned long long lo, unsigned long long hi, unsigned int tag) {
-  return (unsigned int)(lo >> 32) == tag && (unsigned int)(hi >> 32) == tag;
-}
-__device__ __forceinline__ double kb_value(unsigned long long lo, unsigned long long hi) {
-  return __longlong_as_double((long long)((lo & 0xffffffffull) | (hi << 32)));
 }
 
 // x != 0 (true for NaN) without an FP64 compare.
@@ -265,12 +221,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
   const long long rend = min(a.s, rbeg + a.chunk);
   const int nr = rbeg < rend ? (int)(rend - rbeg) : 0;
   const int np = (a.nb + NB - 1) / NB, ld = np * NB;
-  const int wl = (int)__ldcg(a.err + (SYNC_WAITLIM - SYNC_ERR));
-  KbWait kw{wl == 0 ? (1 << 22) : wl, a.err, __ldcg(a.err) != 0u};
-  if (wl < 0) {  // test setting: every wait gives up at once
-    if (tid == 0) atomicExch(a.err, 1u);
-    kw.dead = true;
-  }
+  RecWait kw(a.err, tid);
   unsigned int barrier = a.bar0;
   for (int cc = w; cc < ld; cc += 4) {
     const double* col = a.A + (size_t)(a.j0 + cc) * a.lda + rbeg;
@@ -280,7 +231,8 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
-  kb_cluster_sync();  // all ranks run: their shared memory may be written
+  cluster_arrive();
+  cluster_wait();  // all ranks run: their shared memory may be written
   for (int pi = 0; pi < np; ++pi) {
     const int p0 = pi * NB, nbw = min(NB, a.nb - p0);
     for (int jj = 0; jj < nbw; ++jj) {
@@ -302,16 +254,17 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
         }
         acc = fma(x, e, acc);
       }
-      kb_store_cluster(wp + (rank * 4 + w) * 8 + (lane & 7), lane >> 3, acc);
-      kb_cluster_sync();
+      st_cluster(wp + (rank * 4 + w) * 8 + (lane & 7), lane >> 3, acc);
+      cluster_arrive();
+      cluster_wait();
       if (w == 0) {
         const double* x = wp + (lane >> 3) * 32 + (lane & 7);
         double sm = (x[0] + x[8]) + (x[16] + x[24]);
         sm += __shfl_xor_sync(0xffffffffu, sm, 8);
         sm += __shfl_xor_sync(0xffffffffu, sm, 16);
-        if (lane < 8) kb_publish(slot + ((size_t)cl * NB + rank * 8 + lane) * 2, sm, tag);
+        if (lane < 8) rec_publish(slot + ((size_t)cl * NB + rank * 8 + lane) * 2, sm, tag);
       } else if (w == 1 && j >= rbeg && j < rend) {
-        kb_publish(slot + ((size_t)ncl * NB + lane) * 2, sl[kb_at((int)(j - rbeg), p0 + lane, ld)], tag);
+        rec_publish(slot + ((size_t)ncl * NB + lane) * 2, sl[kb_at((int)(j - rbeg), p0 + lane, ld)], tag);
       }
       // sum over the clusters, warp w the clusters w, w + 4, ... in increasing
       // order; record ncl is the pivot row.  A complete record of this cluster
@@ -324,17 +277,17 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
           bool all = true;
 #pragma unroll
           for (int i = 0; i < KB_POLL; ++i)
-            if (q0 + 4 * i <= ncl) kb_load(slot + ((size_t)(q0 + 4 * i) * NB + lane) * 2, lo[i], hi[i]);
+            if (q0 + 4 * i <= ncl) rec_load(slot + ((size_t)(q0 + 4 * i) * NB + lane) * 2, lo[i], hi[i]);
 #pragma unroll
           for (int i = 0; i < KB_POLL; ++i)
-            if (q0 + 4 * i <= ncl) all = all && kb_ready(lo[i], hi[i], tag);
+            if (q0 + 4 * i <= ncl) all = all && rec_ready(lo[i], hi[i], tag);
           if (__all_sync(0xffffffffu, all) || !__all_sync(0xffffffffu, kw.spin(spins))) break;
         }
 #pragma unroll
         for (int i = 0; i < KB_POLL; ++i) {
           const int q = q0 + 4 * i;
-          if (q < ncl) sum += kb_value(lo[i], hi[i]);
-          else if (q == ncl) pv[lane] = kb_value(lo[i], hi[i]);
+          if (q < ncl) sum += rec_value(lo[i], hi[i]);
+          else if (q == ncl) pv[lane] = rec_value(lo[i], hi[i]);
         }
       }
       rs[w * NB + lane] = sum;

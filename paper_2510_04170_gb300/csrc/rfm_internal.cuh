@@ -100,7 +100,8 @@ struct rfm_problem {
   bool lsqr_eager = false;        // graph capture failed once: replay the chunk's kernels eagerly
   int qr_panel_cap = 0;           // most CTAs per panel factorisation (0: one per SM)
   double* jt_part = nullptr;      // [JT_SLICES][n] partial sums of J^T x
-  double* trsv_acc = nullptr;     // [ceil(n/64)][64] partial sums of the triangular solve's helpers
+  unsigned long long* trsv_rec = nullptr;  // [2][ceil(n/64)][64] 16-byte records: the triangular solve's sums and x
+  double* chain_tiles = nullptr;  // dinv and R's near off-diagonal blocks in the chain's order (rfm_trsv_tiles_len)
   double* dinv = nullptr;         // [ceil(n/64)][64 x 64] inverses of R's diagonal blocks (column-major)
   const double* dinv_of = nullptr;  // the R that dinv was computed from (nullptr: stale)
   // per-problem QR scratch (FP64 panel buffers)
@@ -175,6 +176,7 @@ rfm_status rfm_launch_jmv(rfm_problem* p, const double* x, double* y);
 rfm_status rfm_launch_jtmv(rfm_problem* p, const double* x, double* y);
 rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x);
 rfm_status rfm_trsv_prepare(rfm_problem* p);  // inverts R's diagonal blocks (after every change of R)
+long long rfm_trsv_tiles_len(long long n);    // doubles of rfm_problem::chain_tiles
 rfm_status rfm_launch_count_sketch(rfm_problem* p, long long s, int kJ);
 rfm_status rfm_launch_gauss_sketch(rfm_problem* p, long long s, int kJ);
 rfm_status rfm_launch_gauss_sketch_tc(rfm_problem* p, long long s, int kJ);
@@ -268,6 +270,71 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* flag, unsigned int
     else if (spins > (1u << 16)) __nanosleep(128);
   }
   return true;
+}
+// Values exchanged between CTAs as 16-byte records {low 32 bits, tag, high 32
+// bits, tag}: each 8-byte half is written and read whole, so a reader that finds
+// its tag in both has the value.  Readers poll the records themselves: no fence,
+// no counter, no second trip to L2.
+__device__ __forceinline__ void rec_publish(unsigned long long* rec, double v, unsigned int tag) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long lo = (b & 0xffffffffull) | ((unsigned long long)tag << 32);
+  const unsigned long long hi = (b >> 32) | ((unsigned long long)tag << 32);
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(rec), "l"(lo), "l"(hi) : "memory");
+}
+__device__ __forceinline__ void rec_load(const unsigned long long* rec, unsigned long long& lo,
+                                         unsigned long long& hi) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(rec) : "memory");
+}
+__device__ __forceinline__ bool rec_ready(unsigned long long lo, unsigned long long hi, unsigned int tag) {
+  return (unsigned int)(lo >> 32) == tag && (unsigned int)(hi >> 32) == tag;
+}
+__device__ __forceinline__ double rec_value(unsigned long long lo, unsigned long long hi) {
+  return __longlong_as_double((long long)((lo & 0xffffffffull) | (hi << 32)));
+}
+
+// Bound of a thread's waits in one launch: `spin` counts a poll of one wait and
+// says whether to go on.  `err` and the limit are as for wait_flag; once a wait
+// of this thread gave up, or an earlier kernel's did, no later one waits.
+struct RecWait {
+  int lim;             // polls of one wait
+  unsigned int* err;
+  bool dead;
+  __device__ __forceinline__ RecWait(unsigned int* e, int tid) : err(e), dead(__ldcg(e) != 0u) {
+    const int wl = (int)__ldcg(e + (SYNC_WAITLIM - SYNC_ERR));
+    lim = wl == 0 ? (1 << 22) : wl;
+    if (wl < 0) {  // test setting: every wait gives up at once
+      if (tid == 0) atomicExch(e, 1u);
+      dead = true;
+    }
+  }
+  __device__ __forceinline__ bool spin(unsigned int& n) {  // false: give up
+    if (dead || ++n > (unsigned int)lim) {
+      if (!dead) atomicExch(err, 1u);
+      dead = true;
+      return false;
+    }
+    if (n > (1u << 16)) __nanosleep(128);
+    return true;
+  }
+};
+
+// Store to the same shared-memory variable of rank `rank` of the cluster.
+__device__ __forceinline__ void st_cluster(double* p, int rank, double v) {
+  asm volatile(
+      "{\n .reg .b32 r;\n mapa.shared::cluster.u32 r, %0, %1;\n st.shared::cluster.f64 [r], %2;\n}\n" ::"r"(
+          (unsigned)__cvta_generic_to_shared(p)),
+      "r"(rank), "d"(v)
+      : "memory");
+}
+// Barrier of all threads of the cluster that have not exited: stores before the
+// arrival are seen after the wait.
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 #endif
 
