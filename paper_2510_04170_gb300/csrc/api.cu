@@ -55,7 +55,11 @@ __global__ void k_sub(double* __restrict__ y, const double* __restrict__ a, cons
 // iterations, and the convergence flag *done makes the iteration's kernels
 // return at once, so a fixed chunk of iterations can be replayed as one graph.
 enum LsqrSlot {
-  LS_ALPHA, LS_RHOBAR, LS_PHIBAR, LS_SUMSQ, LS_DD, LS_NORMB, LS_ETA, LS_CONLIM, LS_LIMIT, LS_ITN, LS_ISTOP, LS_SLOTS
+  LS_ALPHA, LS_RHOBAR, LS_PHIBAR, LS_SUMSQ, LS_DD, LS_NORMB, LS_ETA, LS_CONLIM, LS_LIMIT, LS_ITN, LS_ISTOP,
+  LS_AB,                      // alpha / beta: u is kept as beta u
+  LS_RHO, LS_PHI, LS_TR,      // this iteration's rotation: rho, phi, theta / rho,
+  LS_C, LS_NRHOBAR, LS_NPHIBAR,  // c and the next rhobar and phibar
+  LS_SLOTS
 };
 
 struct Rot {
@@ -92,86 +96,127 @@ __global__ void k_lsqr_init(double* __restrict__ st, const double* __restrict__ 
   st[LS_LIMIT] = limit;
   st[LS_ITN] = 0.0;
   st[LS_ISTOP] = 7.0;
+  st[LS_AB] = alpha;  // u_1 is normalised
   *done = (beta > 0.0 && alpha > 0.0 && limit > 0.0) ? 0 : 1;
   if (!(beta > 0.0 && alpha > 0.0)) st[LS_ISTOP] = 0.0;
 }
 
-// y = a x + b y with b = bscale * bdev[0]
-__global__ void k_axpby_dev(double* __restrict__ y, const double* __restrict__ x, long long n, double a,
-                            const double* __restrict__ bdev, double bscale, const int* __restrict__ skip) {
-  if (*skip) return;
-  const double b = bscale * bdev[0];
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = a * x[i] + b * y[i];
-}
-
-// LSQR update with the old w: dk = w / rho; x += phi dk; w = v - (theta/rho) w;
-// partial sums of ||dk||^2 and ||x||^2 per block.  Every block derives the
-// rotation from the same device scalars.
-__global__ void k_lsqr_update(double* __restrict__ x, double* __restrict__ w, const double* __restrict__ v, long long n,
-                              const double* __restrict__ lst, const double* __restrict__ sc,
-                              double* __restrict__ partial, const int* __restrict__ skip) {
-  if (*skip) return;
-  const Rot r = lsqr_rot(lst, sc);
-  const double rho = r.rho, phi = r.phi, theta = r.theta;
-  double sd = 0.0, sx = 0.0;
-  const double tr = theta / rho;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const double dk = w[i] / rho;
-    const double xi = x[i] + phi * dk;
-    x[i] = xi;
-    w[i] = v[i] - tr * w[i];
-    sd += dk * dk;
-    sx += xi * xi;
-  }
-  __shared__ double sh[2][32];
-  sd = warp_sum(sd);
-  sx = warp_sum(sx);
-  if ((threadIdx.x & 31) == 0) {
-    sh[0][threadIdx.x >> 5] = sd;
-    sh[1][threadIdx.x >> 5] = sx;
+// Sums over a grid without a second launch: every block leaves its K sums in
+// partial[K * block ..], and the block that finds all others done (an arrival
+// counter, back at zero for the next use) adds them, thread t the blocks t, t +
+// 256, .. and then a fixed tree, so the result does not depend on which block it
+// is.  Returns true in thread 0 of that block, with the sums.
+template <int K>
+__device__ __forceinline__ bool grid_sums(double (&v)[K], double* __restrict__ partial, unsigned int* __restrict__ count) {
+  __shared__ double sh[K][8];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto block_sum = [&] {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      v[k] = warp_sum(v[k]);
+      if (lane == 0) sh[k][w] = v[k];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        v[k] = sh[k][0];
+        for (int q = 1; q < 8; ++q) v[k] += sh[k][q];
+      }
+  };
+  block_sum();
+  if (gridDim.x == 1) return threadIdx.x == 0;
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) __stcg(partial + K * blockIdx.x + k, v[k]);
+    __threadfence();
+    last = atomicInc(count, gridDim.x - 1) == gridDim.x - 1;
   }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double a = threadIdx.x < (blockDim.x >> 5) ? sh[0][threadIdx.x] : 0.0;
-    double b = threadIdx.x < (blockDim.x >> 5) ? sh[1][threadIdx.x] : 0.0;
-    a = warp_sum(a);
-    b = warp_sum(b);
-    if (threadIdx.x == 0) {
-      partial[2 * blockIdx.x] = a;
-      partial[2 * blockIdx.x + 1] = b;
-    }
+  if (!last) return false;
+  __threadfence();
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    v[k] = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) v[k] += __ldcg(partial + K * i + k);
+  }
+  block_sum();
+  return threadIdx.x == 0;
+}
+
+// sc[0] = ||u||
+__global__ void __launch_bounds__(256) k_lsqr_beta(const double* __restrict__ u, long long m, double* __restrict__ sc,
+                                                   double* __restrict__ partial, unsigned int* __restrict__ count,
+                                                   const int* __restrict__ skip) {
+  if (*skip) return;
+  double v[1] = {0.0};
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < m; i += gridDim.x * 256LL) v[0] += u[i] * u[i];
+  if (grid_sums<1>(v, partial, count)) sc[0] = sqrt(v[0]);
+}
+
+// v = t / beta - beta v (t = R^-T J^T of the unscaled u), sc[1] = ||v||, and the
+// iteration's rotation.
+__global__ void __launch_bounds__(256) k_lsqr_alpha(double* __restrict__ v, const double* __restrict__ t, long long n,
+                                                    double* __restrict__ st, double* __restrict__ sc,
+                                                    double* __restrict__ partial, unsigned int* __restrict__ count,
+                                                    const int* __restrict__ skip) {
+  if (*skip) return;
+  const double beta = sc[0], inv = beta != 0.0 ? 1.0 / beta : 1.0;
+  double q[1] = {0.0};
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
+    const double x = t[i] * inv - beta * v[i];
+    v[i] = x;
+    q[0] += x * x;
+  }
+  if (grid_sums<1>(q, partial, count)) {
+    sc[1] = sqrt(q[0]);
+    const Rot r = lsqr_rot(st, sc);
+    st[LS_RHO] = r.rho;
+    st[LS_PHI] = r.phi;
+    st[LS_TR] = r.theta / r.rho;
+    st[LS_C] = r.c;
+    st[LS_NRHOBAR] = r.rhobar;
+    st[LS_NPHIBAR] = r.phibar;
+    st[LS_AB] = sc[1] * inv;
   }
 }
 
-// End of an LSQR iteration (one warp): reduces ||dk||^2 and ||x||^2, advances
-// the state and applies the stopping tests (istop 1: ||r|| small, 2: ||A^T r||
-// small, 3: cond(A) above conlim, 7: iteration limit).
-__global__ void k_lsqr_finish(const double* __restrict__ partial, int np, double* __restrict__ st,
-                              const double* __restrict__ sc, int* __restrict__ done) {
+// LSQR update: v = v / alpha; with the old w: dk = w / rho; x += phi dk;
+// w = v - (theta/rho) w; then, with ||dk||^2 and ||x||^2, the end of the
+// iteration: advances the state and applies the stopping tests (istop 1: ||r||
+// small, 2: ||A^T r|| small, 3: cond(A) above conlim, 7: iteration limit).
+__global__ void __launch_bounds__(256) k_lsqr_update(double* __restrict__ x, double* __restrict__ w,
+                                                     double* __restrict__ v, long long n, double* __restrict__ st,
+                                                     const double* __restrict__ sc, double* __restrict__ partial,
+                                                     unsigned int* __restrict__ count, int* __restrict__ done) {
   if (*done) return;
-  double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < np; i += 32) {
-    a += partial[2 * i];
-    b += partial[2 * i + 1];
+  const double rho = st[LS_RHO], phi = st[LS_PHI], tr = st[LS_TR], alpha = sc[1];
+  double sums[2] = {0.0, 0.0};
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
+    const double vi = alpha != 0.0 ? v[i] / alpha : v[i];
+    const double dk = w[i] / rho;
+    const double xi = x[i] + phi * dk;
+    v[i] = vi;
+    x[i] = xi;
+    w[i] = vi - tr * w[i];
+    sums[0] += dk * dk;
+    sums[1] += xi * xi;
   }
-  a = warp_sum(a);
-  b = warp_sum(b);
-  if (threadIdx.x != 0) return;
-  const Rot r = lsqr_rot(st, sc);
-  const double beta = sc[0], alpha = sc[1];
+  if (!grid_sums<2>(sums, partial, count)) return;
+  const double beta = sc[0], phibar = st[LS_NPHIBAR];
   st[LS_SUMSQ] += st[LS_ALPHA] * st[LS_ALPHA] + beta * beta;  // ||B_k||_F^2: alpha_i with beta_{i+1}
   st[LS_ALPHA] = alpha;
-  st[LS_RHOBAR] = r.rhobar;
-  st[LS_PHIBAR] = r.phibar;
-  st[LS_DD] += a;
+  st[LS_RHOBAR] = st[LS_NRHOBAR];
+  st[LS_PHIBAR] = phibar;
+  st[LS_DD] += sums[0];
   st[LS_ITN] += 1.0;
   const double eta = st[LS_ETA];
-  const double normx = sqrt(b);
+  const double normx = sqrt(sums[1]);
   const double normA = sqrt(st[LS_SUMSQ]);
   const double condA = normA * sqrt(st[LS_DD]);
-  const double normr = r.phibar;
-  const double normar = r.phibar * alpha * fabs(r.c);
+  const double normr = phibar;
+  const double normar = phibar * alpha * fabs(st[LS_C]);
   int istop = 7;
   if (normr <= eta * st[LS_NORMB] + eta * normA * normx) istop = 1;
   else if (normar <= eta * normA * normr) istop = 2;
@@ -192,6 +237,9 @@ int vgrid(long long n) {
   long long g = (n + 255) / 256;
   return (int)std::max<long long>(1, std::min<long long>(g, kVecBlocks));
 }
+
+// Blocks of a kernel that ends in grid_sums: few, as the last one adds their sums.
+int sum_grid(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 511) / 512, kVecBlocks)); }
 
 // ---------------------------------------------------------------- helpers
 template <class T>
@@ -539,7 +587,10 @@ struct LsqrOut {
 
 constexpr int kLsqrChunk = 16;  // iterations per replayed graph
 
-// One chunk of kLsqrChunk iterations, every kernel guarded by the done flag.
+// One chunk of kLsqrChunk iterations, every kernel guarded by the done flag.  Norms,
+// scalings and the scalar recurrences ride in three vector kernels (beta; alpha and
+// the rotation; the update and the stopping tests): as twelve launches of their own
+// they took 30 of 105 us per iteration at n = 1,024.
 rfm_status lsqr_chunk(rfm_problem* p, double* lst, int* done) {
   const long long m = p->m, n = p->n;
   cudaStream_t st = p->stream;
@@ -550,24 +601,19 @@ rfm_status lsqr_chunk(rfm_problem* p, double* lst, int* done) {
   double* tn = wv(p, WV_TN);
   double* tn2 = wv(p, WV_TN2);
   double* sc = p->red + 1024;
+  unsigned int* count = p->sync + SYNC_COUNT;
   for (int it = 0; it < kLsqrChunk; ++it) {
-    // beta u = J R^{-1} v - alpha u
+    // u holds beta u: the new one is J R^{-1} v - alpha u
     RFM_TRY(rfm_launch_trsv(p, 0, v, tn));
-    RFM_TRY(rfm_launch_jmv_axpby(p, tn, 1.0, -1.0, u, lst + LS_ALPHA));
-    RFM_TRY(rfm_norm2(st, u, m, p->red, sc));
-    k_scale_by<<<vgrid(m), 256, 0, st>>>(u, m, sc, 1, done);
+    RFM_TRY(rfm_launch_jmv_axpby(p, tn, 1.0, -1.0, u, lst + LS_AB));
+    k_lsqr_beta<<<sum_grid(m), 256, 0, st>>>(u, m, sc, p->red, count, done);
     RFM_CHECK_LAUNCH();
     // alpha v = R^{-T} J^T u - beta v
     RFM_TRY(rfm_launch_jtmv(p, u, tn));
     RFM_TRY(rfm_launch_trsv(p, 1, tn, tn2));
-    k_axpby_dev<<<vgrid(n), 256, 0, st>>>(v, tn2, n, 1.0, sc, -1.0, done);
+    k_lsqr_alpha<<<sum_grid(n), 256, 0, st>>>(v, tn2, n, lst, sc, p->red, count, done);
     RFM_CHECK_LAUNCH();
-    RFM_TRY(rfm_norm2(st, v, n, p->red, sc + 1));
-    k_scale_by<<<vgrid(n), 256, 0, st>>>(v, n, sc + 1, 1, done);
-    RFM_CHECK_LAUNCH();
-    k_lsqr_update<<<kVecBlocks, 256, 0, st>>>(x, w, v, n, lst, sc, p->red, done);
-    RFM_CHECK_LAUNCH();
-    k_lsqr_finish<<<1, 32, 0, st>>>(p->red, kVecBlocks, lst, sc, done);
+    k_lsqr_update<<<sum_grid(n), 256, 0, st>>>(x, w, v, n, lst, sc, p->red, count, done);
     RFM_CHECK_LAUNCH();
   }
   return RFM_OK;

@@ -381,7 +381,7 @@ struct ChainArgs {
   double* x;
   unsigned long long* hrec;   // [nblk][64] records of the helpers' sums
   unsigned long long* xrec;   // [nblk][64] records of x
-  const unsigned int* epoch;  // tag of this solve (k_trsv_prep)
+  unsigned int* epoch;        // solves so far; this one's tag is the next number
   unsigned int* err;
   const int* skip;
 };
@@ -650,18 +650,21 @@ template <int TRANS, int NT>
 __global__ void __launch_bounds__(256, 1) k_trsv_chain(ChainArgs a) {
   if (a.skip && *a.skip) return;
   extern __shared__ __align__(16) double csm[];
-  const unsigned int tag = *a.epoch;  // set by k_trsv_prep, which ran before this launch
+  unsigned int tag = __ldcg(a.epoch) + 1u;
+  if (tag == 0u) tag = 1u;  // 0 is the records' initial tag
   RecWait wait(a.err, threadIdx.x);
   if (blockIdx.x < CHAIN_CL) {
     trsv_chain<TRANS>(a, tag, wait, csm);
+    // every helper whose records the chain used has read the epoch; the others use no tag
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.epoch = tag;
   } else {
     trsv_helper<TRANS, NT>(a, tag, wait, csm);
   }
 }
 
-// Next epoch for the block flags and record tags (never 0, their initial value)
-// and a fresh ticket counter; runs before every solve so that replays of a
-// captured graph see a new epoch each time.
+// Next epoch for the block flags (never 0, their initial value) and a fresh ticket
+// counter; runs before every k_trsv so that replays of a captured graph see a new
+// epoch each time.
 __global__ void k_trsv_prep(unsigned int* __restrict__ epoch, unsigned int* __restrict__ ticket) {
   unsigned int e = *epoch + 1u;
   *epoch = e == 0u ? 1u : e;
@@ -836,8 +839,6 @@ rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x
   if (p->dinv && p->dinv_of != p->R) RFM_TRY(rfm_trsv_prepare(p));
   ProfScope ps(PF_TRSV, p->stream);
   rfm_prof_work(PF_TRSV, 8.0 * (double)n * (n + 1) / 2 + 16.0 * n);  // R read once, b and x
-  k_trsv_prep<<<1, 1, 0, p->stream>>>(p->sync + SYNC_EPOCH, p->sync + SYNC_TICKET);
-  RFM_CHECK_LAUNCH();
   // chain + helpers when every block has a helper slot
   const int H = std::min(chain_max_ctas() - CHAIN_CL, (nblk + CHAIN_CL - 1) / CHAIN_CL * CHAIN_CL);
   if (p->trsv_rec && p->dinv && p->chain_tiles && H > 0 && nblk <= HMAXT * H) {
@@ -863,6 +864,8 @@ rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x
     RFM_CHECK_LAUNCH();
     return RFM_OK;
   }
+  k_trsv_prep<<<1, 1, 0, p->stream>>>(p->sync + SYNC_EPOCH, p->sync + SYNC_TICKET);
+  RFM_CHECK_LAUNCH();
   if (trans == 0)
     k_trsv<0><<<nblk, 256, 0, p->stream>>>(p->R, p->ldr, n, b, x, p->sync + SYNC_FLAGS, p->sync + SYNC_EPOCH,
                                            p->sync + SYNC_TICKET, p->sync + SYNC_ERR, p->skip);

@@ -220,6 +220,7 @@ rfm_status rfm_dot(cudaStream_t st, const double* x, const double* y, long long 
 #define SYNC_EPOCH 9
 #define SYNC_LSQR_DONE 10
 #define SYNC_WAITLIM 11
+#define SYNC_COUNT 12
 #define SYNC_BAR 16
 #define SYNC_FLAGS 64
 
