@@ -760,8 +760,6 @@ rfm_status lsqr(rfm_problem* p, const double* b, double eta, double conlim, long
 }
 
 // ---------------------------------------------------------------- line search
-const double kGold = 0.6180339887498949;  // (sqrt(5) - 1) / 2
-
 rfm_status linesearch(rfm_problem* p, const double* c, const double* dvec, double f0, double* alpha_out,
                       double* fbest_out) {
   double* P0 = wv(p, WV_P0);
@@ -770,52 +768,12 @@ rfm_status linesearch(rfm_problem* p, const double* c, const double* dvec, doubl
   double* V = wv(p, WV_VV);
   RFM_TRY(rfm_launch_ls_precompute(p, c, dvec, P0, P1, U, V));
   double* sc = p->red + 1024 + 8;
-  auto phi = [&](double a, double* out) -> rfm_status {
-    RFM_TRY(rfm_launch_ls_eval(p, P0, P1, U, V, a, sc));
-    return read_scalars(p, sc, 1, out);
-  };
-  double a = 0.0, b = 1.0;
-  double x1 = b - kGold * (b - a), x2 = a + kGold * (b - a);
-  double f1, f2;
-  RFM_TRY(phi(x1, &f1));
-  RFM_TRY(phi(x2, &f2));
-  std::vector<std::pair<double, double>> pts = {{x1, f1}, {x2, f2}};
-  while (b - a > 1e-3) {
-    if (f1 < f2) {
-      b = x2;
-      x2 = x1;
-      f2 = f1;
-      x1 = b - kGold * (b - a);
-      RFM_TRY(phi(x1, &f1));
-      pts.push_back({x1, f1});
-    } else {
-      a = x1;
-      x1 = x2;
-      f1 = f2;
-      x2 = a + kGold * (b - a);
-      RFM_TRY(phi(x2, &f2));
-      pts.push_back({x2, f2});
-    }
-  }
-  double fone;
-  RFM_TRY(phi(1.0, &fone));
-  pts.push_back({1.0, fone});
-  double fmin = pts[0].second;
-  for (auto& q : pts) fmin = std::min(fmin, q.second);
-  double best = -1.0, fbest = 0.0;
-  for (auto& q : pts)
-    if (q.second <= fmin * (1.0 + 1e-12) && q.first > best) best = q.first;
-  fbest = INFINITY;
-  for (auto& q : pts)
-    if (q.first == best) fbest = std::min(fbest, q.second);
-  if (!(fbest < f0)) {
-    *alpha_out = 0.0;
-    *fbest_out = f0;
-  } else {
-    *alpha_out = best;
-    *fbest_out = fbest;
-  }
-  return RFM_OK;
+  RFM_TRY(rfm_launch_ls_search(p, P0, P1, U, V, f0, sc));
+  double got[2];
+  RFM_TRY(read_scalars(p, sc, 2, got));
+  *alpha_out = got[0];
+  *fbest_out = got[1];
+  return check_timeout(p);
 }
 
 long long sketch_rows_for(const rfm_problem* p, const rfm_solve_opts* o) {
@@ -999,6 +957,7 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->hbuck, p->m));
     TRYA(dalloc(&p->hsign, p->m));
     TRYA(dalloc(&p->red, 4096));
+    TRYA(dalloc(&p->ls_rec, 2 * LS_BLOCKS * 2));
     TRYA(dalloc(&p->jt_part, (size_t)JT_SLICES * p->n));
     TRYA(dalloc(&p->trsv_rec, (size_t)((p->n + 63) / 64) * 64 * 4));
     TRYA(dalloc(&p->chain_tiles, (size_t)rfm_trsv_tiles_len(p->n)));
@@ -1031,7 +990,8 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
 #undef CPY
     if (cudaMemsetAsync(p->sync, 0, RFM_SYNC_WORDS * sizeof(unsigned int), s0) != cudaSuccess ||
         cudaMemsetAsync(p->trsv_rec, 0, (size_t)((p->n + 63) / 64) * 64 * 4 * sizeof(unsigned long long), s0) !=
-            cudaSuccess) {
+            cudaSuccess ||
+        cudaMemsetAsync(p->ls_rec, 0, 2 * LS_BLOCKS * 2 * sizeof(unsigned long long), s0) != cudaSuccess) {
       st = RFM_ECUDA;
       goto fail;
     }
@@ -1057,7 +1017,7 @@ rfm_status rfm_problem_destroy(rfm_problem* p) {
   void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slopes, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
                   p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->work,
                   p->red, p->sync, p->sdig, p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch,
-                  p->jt_part, p->trsv_rec, p->dinv, p->chain_tiles};
+                  p->ls_rec, p->jt_part, p->trsv_rec, p->dinv, p->chain_tiles};
   drop_lsqr_graph(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   for (void* b : bufs) dfree(b);
@@ -1290,6 +1250,7 @@ rfm_status rfm_linesearch(rfm_problem* p, const double* c_dev, const double* d_d
                           double* fbest_host) {
   if (!p || !p->have_j || !c_dev || !d_dev) return RFM_EINVAL;
   double a = 0, fb = 0;
+  RFM_TRY(clear_err(p));
   RFM_TRY(linesearch(p, c_dev, d_dev, f0, &a, &fb));
   if (alpha_host) *alpha_host = a;
   if (fbest_host) *fbest_host = fb;

@@ -9,15 +9,17 @@
 //                epilogue.  One warp per row: the tanh features of the row's
 //                subdomain are evaluated once, staged in shared memory, and
 //                the warp writes the scaled row (W contiguous doubles).
-//  * k_ls_pre / k_ls_eval: the golden-section objective
-//                phi(alpha) = ||W F(c + alpha d)|| (Alg. 1 step 5) in O(m) per
-//                alpha after one pass that splits every row into its linear
-//                part and the field values entering the nonlinearity.
+//  * k_ls_search: the golden-section search on phi(alpha) = ||W F(c + alpha d)||
+//                (Alg. 1 step 5), O(m) per alpha after one pass (MODE_LS) that
+//                splits every row into its linear part and the field values
+//                entering the nonlinearity.
 //  * k_eval:     u_n(x) on the owning subdomain (Eq. 2.7, indicator PoU).
 //
 // Features: phi = tanh(z), z = sum_b k_b (x_b - mu_b)/sigma_b + b;
 //   d phi/dx_b = (1 - t^2) k_b/sigma_b,  d^2 phi/dx_b^2 = -2 t (1 - t^2) (k_b/sigma_b)^2.
 #include <math.h>
+
+#include <algorithm>
 
 #include "philox.cuh"
 #include "rfm_internal.cuh"
@@ -595,45 +597,128 @@ __global__ void __launch_bounds__(128) k_assemble(PdeConst pc, const double* __r
   }
 }
 
-// phi(alpha)^2 partial sums: sum_i (lambda_i (P0 + alpha P1 + N_f(U + alpha V)))^2.
-__global__ void k_ls_eval(PdeConst pc, const int4* __restrict__ meta, const double* __restrict__ lam,
-                          const double* __restrict__ P0, const double* __restrict__ P1,
-                          const double* __restrict__ U, const double* __restrict__ V, long long m,
-                          double alpha, double* __restrict__ partial) {
+// Golden-section search on phi(alpha) = ||lambda (P0 + alpha P1 + N_f(U + alpha
+// V))|| over [0, 1] (Alg. 1 step 5), all 18 evaluations in one cooperative launch:
+// an evaluation reads a few vectors of m entries (1 to 10 us), and as a kernel,
+// its finish, a copy and a synchronisation each it took 25 us.  Every CTA leaves
+// its partial sum of an evaluation as a record tagged with the evaluation's
+// number and adds all CTAs' records in the same order, so every CTA takes the
+// same decisions; CTA 0 writes (alpha, phi) to out.  The bracket's arithmetic is
+// rounded operation by operation.
+constexpr int LS_EVALS = 32;  // more than the search makes
+
+struct LsArgs {
+  PdeConst pc;
+  const int4* meta;
+  const double *lam, *P0, *P1, *U, *V;
+  long long m;
+  double f0;
+  unsigned long long* rec;  // [LS_BLOCKS] records, twice (evaluations alternate)
+  unsigned int* epoch;      // evaluations made so far by this problem's searches
+  unsigned int* err;
+  double* out;              // alpha, phi
+};
+
+__device__ __forceinline__ double ls_phi(const LsArgs& a, double alpha, unsigned int tag, RecWait& wait,
+                                         double* sh) {
   double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
-    double val = P0[i] + alpha * P1[i];
-    const int kind = meta[i].x & 0xF;
-    if (kind == 0 && pc.kind >= 4) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.m; i += (long long)gridDim.x * blockDim.x) {
+    double val = a.P0[i] + alpha * a.P1[i];
+    const int code = a.meta[i].x, kind = code & 0xF;
+    if (kind == 0 && a.pc.kind >= 4) {
       double q[10], C[10];
 #pragma unroll
-      for (int k = 0; k < 10; ++k) q[k] = U[i * 10 + k] + alpha * V[i * 10 + k];
-      val += jet_residual(pc, q, C);
+      for (int k = 0; k < 10; ++k) q[k] = a.U[i * 10 + k] + alpha * a.V[i * 10 + k];
+      val += jet_residual(a.pc, q, C);
     } else if (kind == 0) {
-      const int f = (meta[i].x >> 4) & 0xF;
+      const int f = (code >> 4) & 0xF;
       double u[2] = {0, 0}, coef[2];
-      for (int ff = 0; ff < pc.fields; ++ff) u[ff] = U[i * pc.fields + ff] + alpha * V[i * pc.fields + ff];
-      val += nonlinear(pc, f, u, coef);
+      for (int ff = 0; ff < a.pc.fields; ++ff) u[ff] = a.U[i * a.pc.fields + ff] + alpha * a.V[i * a.pc.fields + ff];
+      val += nonlinear(a.pc, f, u, coef);
     }
-    const double r = lam[i] * val;
+    const double r = a.lam[i] * val;
     acc += r * r;
   }
-  __shared__ double sh[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  if (lane == 0) sh[w] = acc;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
+  if (w == 0) {
+    unsigned long long* rec = a.rec + (size_t)(tag & 1u) * LS_BLOCKS * 2;
+    double v = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
     v = warp_sum(v);
-    if (threadIdx.x == 0) partial[blockIdx.x] = v;
+    if (lane == 0) rec_publish(rec + 2 * blockIdx.x, v, tag);
+    double s = 0.0;
+    for (int q = lane; q < (int)gridDim.x; q += 32) {
+      unsigned long long lo, hi;
+      unsigned int spins = 0;
+      rec_load(rec + 2 * q, lo, hi);
+      while (!rec_ready(lo, hi, tag) && wait.spin(spins)) rec_load(rec + 2 * q, lo, hi);
+      s += rec_value(lo, hi);
+    }
+    __syncwarp();
+    s = warp_sum(s);
+    if (lane == 0) sh[32] = sqrt(s);
   }
+  __syncthreads();
+  const double phi = sh[32];
+  __syncthreads();
+  return phi;
 }
 
-__global__ void k_sum_sqrt(const double* __restrict__ partial, int np, double* __restrict__ out) {
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < np; i += 32) acc += partial[i];
-  acc = warp_sum(acc);
-  if (threadIdx.x == 0) out[0] = sqrt(acc);
+__global__ void __launch_bounds__(256, 2) k_ls_search(LsArgs a) {
+  __shared__ double sh[34];
+  __shared__ double px[LS_EVALS], pf[LS_EVALS];
+  const double gold = 0.6180339887498949;  // (sqrt(5) - 1) / 2
+  const unsigned int base = __ldcg(a.epoch);
+  RecWait wait(a.err, threadIdx.x);
+  int evals = 0;
+  auto phi = [&](double alpha) {
+    unsigned int tag = base + 1u + (unsigned int)evals;
+    const double f = ls_phi(a, alpha, tag, wait, sh);
+    if (threadIdx.x == 0) {
+      px[evals] = alpha;
+      pf[evals] = f;
+    }
+    ++evals;
+    return f;
+  };
+  auto lower = [&](double lo, double hi) { return __dsub_rn(hi, __dmul_rn(gold, __dsub_rn(hi, lo))); };
+  auto upper = [&](double lo, double hi) { return __dadd_rn(lo, __dmul_rn(gold, __dsub_rn(hi, lo))); };
+  double lo = 0.0, hi = 1.0;
+  double x1 = lower(lo, hi), x2 = upper(lo, hi);
+  double f1 = phi(x1), f2 = phi(x2);
+  while (__dsub_rn(hi, lo) > 1e-3 && evals < LS_EVALS - 1) {
+    if (f1 < f2) {
+      hi = x2;
+      x2 = x1;
+      f2 = f1;
+      x1 = lower(lo, hi);
+      f1 = phi(x1);
+    } else {
+      lo = x1;
+      x1 = x2;
+      f1 = f2;
+      x2 = upper(lo, hi);
+      f2 = phi(x2);
+    }
+  }
+  phi(1.0);
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  // the largest alpha among the evaluations within 1e-12 of the smallest phi
+  double fmin = pf[0];
+  for (int k = 1; k < evals; ++k)
+    if (pf[k] < fmin) fmin = pf[k];
+  double best = -1.0, fbest = INFINITY;
+  for (int k = 0; k < evals; ++k)
+    if (pf[k] <= fmin * (1.0 + 1e-12) && px[k] > best) best = px[k];
+  for (int k = 0; k < evals; ++k)
+    if (px[k] == best && pf[k] < fbest) fbest = pf[k];
+  const bool down = fbest < a.f0;
+  a.out[0] = down ? best : 0.0;
+  a.out[1] = down ? fbest : a.f0;
+  // every other CTA has read the epoch: this one has seen its records
+  *a.epoch = base + (unsigned int)evals;
 }
 
 // u_n(x) at query points: one warp per point, lanes over features.
@@ -776,14 +861,16 @@ rfm_status rfm_launch_ls_precompute(rfm_problem* p, const double* c, const doubl
   return RFM_OK;
 }
 
-rfm_status rfm_launch_ls_eval(rfm_problem* p, const double* P0, const double* P1, const double* U, const double* V,
-                              double alpha, double* out_dev) {
-  PdeConst pc = make_pc(p);
-  const int nb = 304;
+rfm_status rfm_launch_ls_search(rfm_problem* p, const double* P0, const double* P1, const double* U, const double* V,
+                                double f0, double* out_dev) {
+  LsArgs a;
+  a.pc = make_pc(p);
+  a.meta = p->rmeta; a.lam = p->lam; a.P0 = P0; a.P1 = P1; a.U = U; a.V = V; a.m = p->m; a.f0 = f0;
+  a.rec = p->ls_rec; a.epoch = p->sync + SYNC_LS_EPOCH; a.err = p->sync + SYNC_ERR; a.out = out_dev;
+  const int nb = std::min(LS_BLOCKS, 2 * std::max(1, rfm_num_sms()));  // two per SM: all must be resident
+  void* args[] = {&a};
   ProfScope ps(PF_LS_EVAL, p->stream);
-  k_ls_eval<<<nb, 256, 0, p->stream>>>(pc, p->rmeta, p->lam, P0, P1, U, V, p->m, alpha, p->red);
-  RFM_CHECK_LAUNCH();
-  k_sum_sqrt<<<1, 32, 0, p->stream>>>(p->red, nb, out_dev);
+  RFM_CUDA(cudaLaunchCooperativeKernel((const void*)k_ls_search, dim3((unsigned)nb), dim3(256), args, 0, p->stream));
   RFM_CHECK_LAUNCH();
   return RFM_OK;
 }

@@ -15,6 +15,7 @@
 #define RFM_MAX_FIELDS 2
 #define RFM_MAX_WIDTH 2048
 #define JT_SLICES 32
+#define LS_BLOCKS 304
 
 // One run of rows that share a point grid (Sec. 5): an interior grid of a
 // subdomain, or a face grid on an interface or a boundary face.
@@ -99,6 +100,7 @@ struct rfm_problem {
   long long lsqr_graph_launches = 0;  // kernels per chunk (launch accounting)
   bool lsqr_eager = false;        // graph capture failed once: replay the chunk's kernels eagerly
   int qr_panel_cap = 0;           // most CTAs per panel factorisation (0: one per SM)
+  unsigned long long* ls_rec = nullptr;  // [2][LS_BLOCKS] 16-byte records of the line search
   double* jt_part = nullptr;      // [JT_SLICES][n] partial sums of J^T x
   unsigned long long* trsv_rec = nullptr;  // [2][ceil(n/64)][64] 16-byte records: the triangular solve's sums and x
   double* chain_tiles = nullptr;  // dinv and R's near off-diagonal blocks in the chain's order (rfm_trsv_tiles_len)
@@ -167,8 +169,9 @@ rfm_status rfm_launch_assemble(rfm_problem* p, const double* c, double cscale, b
                                const double* lam_in, double* Fout);
 rfm_status rfm_launch_ls_precompute(rfm_problem* p, const double* c, const double* dvec, double* P0,
                                     double* P1, double* U, double* V);
-rfm_status rfm_launch_ls_eval(rfm_problem* p, const double* P0, const double* P1, const double* U,
-                              const double* V, double alpha, double* out_dev);
+// alpha and phi(alpha) of the golden-section search to out_dev[0..1]
+rfm_status rfm_launch_ls_search(rfm_problem* p, const double* P0, const double* P1, const double* U, const double* V,
+                                double f0, double* out_dev);
 rfm_status rfm_launch_eval(const rfm_problem* p, const double* c, const double* pts, long long npts,
                            double* u);
 rfm_status rfm_launch_phi_values(const rfm_problem* p, const double* pts, long long npts, float scale, float* Phi);
@@ -221,6 +224,7 @@ rfm_status rfm_dot(cudaStream_t st, const double* x, const double* y, long long 
 #define SYNC_LSQR_DONE 10
 #define SYNC_WAITLIM 11
 #define SYNC_COUNT 12
+#define SYNC_LS_EPOCH 13
 #define SYNC_BAR 16
 #define SYNC_FLAGS 64
 
