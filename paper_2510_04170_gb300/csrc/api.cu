@@ -943,7 +943,6 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->mu, muh.size()));
     TRYA(dalloc(&p->sig, sgh.size()));
     TRYA(dalloc(&p->feat, 4 * nfeat));
-    TRYA(dalloc(&p->slopes, 4 * nfeat));
     TRYA(dalloc(&p->segs, segs.size()));
     TRYA(dalloc(&p->pts, 4 * p->m));
     TRYA(dalloc(&p->rmeta, p->m));
@@ -957,10 +956,15 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->hbuck, p->m));
     TRYA(dalloc(&p->hsign, p->m));
     TRYA(dalloc(&p->red, 4096));
-    TRYA(dalloc(&p->ls_rec, 2 * LS_BLOCKS * 2));
-    TRYA(dalloc(&p->jt_part, (size_t)JT_SLICES * p->n));
-    TRYA(dalloc(&p->trsv_rec, (size_t)((p->n + 63) / 64) * 64 * 4));
-    TRYA(dalloc(&p->chain_tiles, (size_t)rfm_trsv_tiles_len(p->n)));
+    // one allocation for the smaller solver buffers; the records, which start at
+    // zero, come first
+    const long long nrec = 2 * LS_BLOCKS * 2 + (p->n + 63) / 64 * 64 * 4;
+    TRYA(dalloc(&p->slab, (size_t)(nrec + 4 * nfeat + JT_SLICES * p->n + rfm_trsv_tiles_len(p->n))));
+    p->ls_rec = reinterpret_cast<unsigned long long*>(p->slab);
+    p->trsv_rec = p->ls_rec + 2 * LS_BLOCKS * 2;
+    p->slopes = p->slab + nrec;
+    p->jt_part = p->slopes + 4 * nfeat;
+    p->chain_tiles = p->jt_part + JT_SLICES * p->n;
     TRYA(dalloc(&p->dinv, (size_t)((p->n + 63) / 64) * 64 * 64));
     TRYA(dalloc(&p->sync, RFM_SYNC_WORDS));
     p->work_cap = vec_stride(p) * WV_COUNT;
@@ -989,9 +993,7 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     }
 #undef CPY
     if (cudaMemsetAsync(p->sync, 0, RFM_SYNC_WORDS * sizeof(unsigned int), s0) != cudaSuccess ||
-        cudaMemsetAsync(p->trsv_rec, 0, (size_t)((p->n + 63) / 64) * 64 * 4 * sizeof(unsigned long long), s0) !=
-            cudaSuccess ||
-        cudaMemsetAsync(p->ls_rec, 0, 2 * LS_BLOCKS * 2 * sizeof(unsigned long long), s0) != cudaSuccess) {
+        cudaMemsetAsync(p->slab, 0, (size_t)nrec * sizeof(double), s0) != cudaSuccess) {
       st = RFM_ECUDA;
       goto fail;
     }
@@ -1014,10 +1016,10 @@ rfm_status rfm_problem_destroy(rfm_problem* p) {
   if (!p) return RFM_OK;
   if (p->stream) cudaStreamSynchronize(p->stream);
   else cudaDeviceSynchronize();
-  void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slopes, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
+  void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slab, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
                   p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->work,
                   p->red, p->sync, p->sdig, p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch,
-                  p->ls_rec, p->jt_part, p->trsv_rec, p->dinv, p->chain_tiles};
+                  p->dinv};
   drop_lsqr_graph(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   for (void* b : bufs) dfree(b);

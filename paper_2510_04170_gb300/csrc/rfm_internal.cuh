@@ -42,6 +42,7 @@ struct rfm_problem {
   double* X = nullptr;      // breakpoints [3][nmaxbp]
   double* mu = nullptr;     // [G][4]
   double* sig = nullptr;    // [G][4]
+  double* slab = nullptr;   // allocation of slopes, jt_part, ls_rec, trsv_rec and chain_tiles
   double* feat = nullptr;   // [G*fields*M][4]
   double* slopes = nullptr; // [G*fields*M][4]: k_b / sigma_b and the sum of their squares
   RowSeg* segs = nullptr;
