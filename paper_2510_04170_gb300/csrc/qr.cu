@@ -45,6 +45,12 @@ constexpr int NB = 32;
 //    of the panel.  sqrt and the reciprocal are one third-order step
 //    (Householder's iteration) from an FP32 seed, 18 instructions where the
 //    library's sqrt and two divisions take 28 (0.86 us).
+//  - a column's reflector is applied to the next column at once and to the others
+//    while the next column's exchange is on its way.  The next column's products
+//    are then taken with a_k still lacking that reflector f_k u, and
+//    x^T (a_k - f_k u) = x^T a_k - f_k x^T u is formed after the sum, x^T u being
+//    the Gram entry in its lane.  The error against ||x|| ||a_k|| is that of the
+//    step before, so the sum of all steps' errors is the same.
 //  - the 32 sums are first combined in clusters of four CTAs (each rank sums
 //    eight columns of the 16 warps, through distributed shared memory and one
 //    cluster barrier, 0.2 us), then between the clusters as 16-byte records
@@ -59,9 +65,12 @@ constexpr int NB = 32;
 // sums column c of W over the CTAs and solves for its column of W2.
 //
 // Per column at 12,288 rows: 16.5 us with one grid barrier and a redundant
-// butterfly reduction per column (the former panel kernel), now 5.2 us (0.95
+// butterfly reduction per column (the former panel kernel), then 5.2 us (0.95
 // products, 0.4 cluster barrier, 0.25 publish, 1.7 poll and sums, 1.05 scalars,
-// 0.8 update); a 128-column block with its in-block updates 3.7 -> 0.94 ms.
+// 0.8 update).  The poll leaves the FP64 pipes idle, so only the next column is
+// updated at once; a reflector's other columns follow while the next column's
+// records are on their way.  A 128-column block with its in-block updates: 3.7
+// -> 0.94 ms, with the deferred updates 0.87 ms.
 constexpr int KB_THREADS = 128;
 constexpr int KB_SMEM = 227 * 1024;              // dynamic shared memory of a CTA
 constexpr long long KB_WIDE_ROWS = 16384;
@@ -204,6 +213,51 @@ __device__ __forceinline__ void kb_wupdate(double* sl, int ld, int p0, int pc, i
   }
 }
 
+// A_rk -= f_k u_r for this warp's rows r >= r0 of the panel at p0, u its column jj,
+// f the lanes' factors (0 up to column jj + 1, which is up to date).
+__device__ __forceinline__ void kb_apply(double* sl, int ld, int p0, int jj, double f, int r0, int nr, int w,
+                                         int lane) {
+  const int rw = r0 + ((w - r0) & 3);
+  if (jj < 15) {
+    if (rw < nr) {
+      const int last = nr - 1 - ((nr - 1 - rw) & 3);
+      double x = sl[kb_at(rw, p0 + jj, ld)], e = sl[kb_at(rw, p0 + lane, ld)];
+#pragma unroll 4
+      for (int r = rw; r < last; r += 4) {
+        const double xn = sl[kb_at(r + 4, p0 + jj, ld)], en = sl[kb_at(r + 4, p0 + lane, ld)];
+        sl[kb_at(r, p0 + lane, ld)] = fma(-f, x, e);
+        x = xn;
+        e = en;
+      }
+      sl[kb_at(last, p0 + lane, ld)] = fma(-f, x, e);
+    }
+  } else {
+    // only columns 17 .. 31 are left: two rows per instruction
+    const int ch = 16 + (lane & 15);
+    const double fh = __shfl_sync(0xffffffffu, f, ch);
+    int r = rw + 4 * (lane >> 4);
+    for (; r + 24 < nr; r += 32) {
+      double x[4], e[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        x[u] = sl[kb_at(r + 8 * u, p0 + jj, ld)];
+        e[u] = sl[kb_at(r + 8 * u, p0 + ch, ld)];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        e[u] = fma(-fh, x[u], e[u]);
+        if (ch > jj + 1) sl[kb_at(r + 8 * u, p0 + ch, ld)] = e[u];
+      }
+    }
+    for (; r < nr; r += 8) {
+      double* e = sl + kb_at(r, p0 + ch, ld);
+      const double x = fma(-fh, sl[kb_at(r, p0 + jj, ld)], *e);
+      if (ch > jj + 1) *e = x;
+    }
+  }
+  __syncwarp();
+}
+
 __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
   extern __shared__ __align__(16) double kb_sm[];
   double* Gs = kb_sm;              // tau_p v_q^T v_p of the panel at kb_tri(p, q), q < p
@@ -236,6 +290,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
   cluster_wait();  // all ranks run: their shared memory may be written
   for (int pi = 0; pi < np; ++pi) {
     const int p0 = pi * NB, nbw = min(NB, a.nb - p0);
+    double fprev = 0.0;  // factors of the previous column's reflector that columns past jj still lack
     for (int jj = 0; jj < nbw; ++jj) {
       const long long j = a.j0 + p0 + jj;  // pivot row and column
       const unsigned int tag = (unsigned int)(j + 1);
@@ -265,7 +320,15 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
         sm += __shfl_xor_sync(0xffffffffu, sm, 16);
         if (lane < 8) rec_publish(slot + ((size_t)cl * NB + rank * 8 + lane) * 2, sm, tag);
       } else if (w == 1 && j >= rbeg && j < rend) {
-        rec_publish(slot + ((size_t)ncl * NB + lane) * 2, sl[kb_at((int)(j - rbeg), p0 + lane, ld)], tag);
+        const int r = (int)(j - rbeg);
+        double v = sl[kb_at(r, p0 + lane, ld)];
+        if (jj > 0) v = fma(-fprev, sl[kb_at(r, p0 + jj - 1, ld)], v);
+        rec_publish(slot + ((size_t)ncl * NB + lane) * 2, v, tag);
+      }
+      // meanwhile the previous column's reflector on the columns past jj
+      if (jj > 0) {
+        if (j >= rbeg && j < rend) __syncthreads();  // warp 1 has read the pivot row
+        kb_apply(sl, ld, p0, jj - 1, fprev, j > rbeg ? (int)min((long long)nr, j - rbeg) : 0, nr, w, lane);
       }
       // sum over the clusters, warp w the clusters w, w + 4, ... in increasing
       // order; record ncl is the pivot row.  A complete record of this cluster
@@ -293,7 +356,8 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
       }
       rs[w * NB + lane] = sum;
       __syncthreads();
-      const double tot = (rs[lane] + rs[NB + lane]) + (rs[2 * NB + lane] + rs[3 * NB + lane]);
+      double tot = (rs[lane] + rs[NB + lane]) + (rs[2 * NB + lane] + rs[3 * NB + lane]);
+      if (jj > 0) tot = fma(-fprev, __shfl_sync(0xffffffffu, tot, jj - 1), tot);
       const double piv = pv[lane];
       const double alpha = pv[jj];
       const double sigma = __shfl_sync(0xffffffffu, tot, jj);
@@ -314,44 +378,15 @@ __global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
           gam[jj] = gj;
         }
       }
-      if (jj < 16) {
-        if (rw < nr) {
-          const int last = nr - 1 - ((nr - 1 - rw) & 3);
-          double x = sl[kb_at(rw, p0 + jj, ld)], e = sl[kb_at(rw, p0 + lane, ld)];
-#pragma unroll 4
-          for (int r = rw; r < last; r += 4) {
-            const double xn = sl[kb_at(r + 4, p0 + jj, ld)], en = sl[kb_at(r + 4, p0 + lane, ld)];
-            sl[kb_at(r, p0 + lane, ld)] = fma(-f, x, e);
-            x = xn;
-            e = en;
-          }
-          sl[kb_at(last, p0 + lane, ld)] = fma(-f, x, e);
+      // the next column only (lanes are rows); the others wait for the next exchange
+      if (jj + 1 < NB) {
+        const double f1 = __shfl_sync(0xffffffffu, f, jj + 1);
+        for (int r = rw + 4 * lane; r < nr; r += 128) {
+          double* e = sl + kb_at(r, p0 + jj + 1, ld);
+          *e = fma(-f1, sl[kb_at(r, p0 + jj, ld)], *e);
         }
-      } else {
-        // only columns 16 .. 31 are left: two rows per instruction
-        const int ch = 16 + (lane & 15);
-        const double fh = __shfl_sync(0xffffffffu, f, ch);
-        int r = rw + 4 * (lane >> 4);
-        for (; r + 24 < nr; r += 32) {
-          double x[4], e[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            x[u] = sl[kb_at(r + 8 * u, p0 + jj, ld)];
-            e[u] = sl[kb_at(r + 8 * u, p0 + ch, ld)];
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            e[u] = fma(-fh, x[u], e[u]);
-            if (ch > jj) sl[kb_at(r + 8 * u, p0 + ch, ld)] = e[u];
-          }
-        }
-        for (; r < nr; r += 8) {
-          double* e = sl + kb_at(r, p0 + ch, ld);
-          const double x = fma(-fh, sl[kb_at(r, p0 + jj, ld)], *e);
-          if (ch > jj) *e = x;
-        }
-        __syncwarp();
       }
+      fprev = lane > jj + 1 ? f : 0.0;
       if (j >= rbeg && j < rend && w == ((int)(j - rbeg) & 3)) {  // the pivot row itself
         double* e = sl + kb_at((int)(j - rbeg), p0 + lane, ld);
         if (lane > jj) *e = fma(-f, dj, *e);
