@@ -647,8 +647,9 @@ __device__ __forceinline__ void trsv_helper(const ChainArgs& a, unsigned int tag
 constexpr size_t chain_smem_bytes() { return (size_t)(2 * TB + 8 * TB) * sizeof(double); }
 
 template <int TRANS, int NT>
-__global__ void __launch_bounds__(256, 1) k_trsv_chain(ChainArgs a) {
+__global__ void __cluster_dims__(CHAIN_CL, 1, 1) __launch_bounds__(256, 1) k_trsv_chain(ChainArgs a) {
   if (a.skip && *a.skip) return;
+  if (!in_cluster(CHAIN_CL, a.err)) return;
   extern __shared__ __align__(16) double csm[];
   unsigned int tag = __ldcg(a.epoch) + 1u;
   if (tag == 0u) tag = 1u;  // 0 is the records' initial tag
@@ -806,15 +807,9 @@ int chain_max_ctas() {
     for (int trans = 0; trans < 2; ++trans)
       for (int nt : {1, 2, HMAXT}) {
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = CHAIN_CL;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(CHAIN_CL);
         cfg.blockDim = dim3(256);
         cfg.dynamicSmemBytes = chain_smem_bytes();
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
         int c = 0;
         const ChainKernel fn = chain_kernel(trans, nt);
         if (rfm_smem_attr((const void*)fn, (int)chain_smem_bytes()) != cudaSuccess ||
@@ -852,14 +847,11 @@ rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = chain_smem_bytes();
     cfg.stream = p->stream;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: helpers and the chain wait on each other
     attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = CHAIN_CL;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     RFM_CUDA(cudaLaunchKernelEx(&cfg, chain_kernel(trans, (nblk + H - 1) / H), a));
     RFM_CHECK_LAUNCH();
     return RFM_OK;

@@ -258,7 +258,8 @@ __device__ __forceinline__ void kb_apply(double* sl, int ld, int p0, int jj, dou
   __syncwarp();
 }
 
-__global__ void __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
+__global__ void __cluster_dims__(KB_CL, 1, 1) __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
+  if (!in_cluster(KB_CL, a.err)) return;
   extern __shared__ __align__(16) double kb_sm[];
   double* Gs = kb_sm;              // tau_p v_q^T v_p of the panel at kb_tri(p, q), q < p
   double* wp = Gs + KB_TRI;        // [4][4][8] partial sums of this rank's 8 columns, by CTA and warp of the cluster
@@ -702,15 +703,9 @@ int kb_max_ctas() {
   std::lock_guard<std::mutex> lk(mu);
   if (cached[dev] == 0) {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = KB_CL;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(KB_CL);
     cfg.blockDim = dim3(KB_THREADS);
     cfg.dynamicSmemBytes = KB_SMEM;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k_block, &cfg) != cudaSuccess) return 0;
     cached[dev] = std::min(n * KB_CL, KB_MAXP);
@@ -775,18 +770,15 @@ rfm_status factor_block(double* A, long long s, long long lda, long long c0, int
   a.bar = sync + SYNC_BAR; a.bar0 = ks->arrived; a.err = sync + SYNC_ERR;
   ks->arrived += 2u * (unsigned)(np - 1) * (unsigned)P;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: they wait on each other's records
   at[0].val.cooperative = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = KB_CL;
-  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)P);
   cfg.blockDim = dim3(KB_THREADS);
   cfg.dynamicSmemBytes = kb_fixed_smem() + (size_t)NB * np * chunk * sizeof(double);
   cfg.stream = st;
   cfg.attrs = at;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = 1;
   ProfScope ps(PF_QR_PANEL, st);
   RFM_CUDA(cudaLaunchKernelEx(&cfg, k_block, a));
   RFM_CHECK_LAUNCH();

@@ -332,6 +332,16 @@ __device__ __forceinline__ void st_cluster(double* p, int rank, double v) {
       "r"(rank), "d"(v)
       : "memory");
 }
+// Whether the CTA runs in a cluster of n, whose peers' shared memory it may write;
+// otherwise the error word is set and the kernel returns before its first remote
+// store.  The cluster's size is an attribute of the kernels themselves, so no
+// launch path (a profiler's replay, say) can leave it out.
+__device__ __forceinline__ bool in_cluster(unsigned int n, unsigned int* err) {
+  unsigned int size;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+  if (size != n && threadIdx.x == 0) atomicExch(err, 1u);
+  return size == n;
+}
 // Barrier of all threads of the cluster that have not exited: stores before the
 // arrival are seen after the wait.
 __device__ __forceinline__ void cluster_arrive() {
