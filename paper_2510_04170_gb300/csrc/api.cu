@@ -1,9 +1,8 @@
 // C ABI of librfm: problem set-up, the individual hot-path steps and the IPN /
 // AMIPN drivers (Alg. 1, Alg. 2 of arXiv 2510.04170).  All numerical work runs
 // in kernels (here and in assemble.cu, sketch.cu, qr.cu, oz.cu, krylov.cu);
-// LSQR's scalar recurrences run on the device too.  The host code sequences
-// launches and evaluates the golden-section bracket and the Newton stopping
-// tests.
+// LSQR's scalar recurrences and the golden-section search run on the device too.
+// The host code sequences launches and evaluates the Newton stopping tests.
 #include <math.h>
 #include <string.h>
 
