@@ -180,9 +180,9 @@ rfm_status rfm_sketch(rfm_problem* p, int kind, int64_t s, int kJ, double* B_dev
  * F_i = (operator row) - rhs_i. */
 rfm_status rfm_set_rhs(rfm_problem* p, const double* rhs_dev);
 
-/* Limit on the device-side polls of the bounded flag waits (the grid barriers
- * of the QR panel factorisation and the block flags of the triangular solves)
- * of this problem: 0 restores the default (2^22 polls), a positive count sets
+/* Limit on the device-side polls of the bounded waits (the exchanges of the QR
+ * block factorisation, of the triangular solves and of the line search) of this
+ * problem: 0 restores the default (2^22 polls), a positive count sets
  * that many, a negative value makes every such wait give up at once (for
  * testing the RFM_ETIMEOUT path).  A wait that gives up sets the problem's
  * error word; the call reports RFM_ETIMEOUT and its result is invalid, and
