@@ -958,11 +958,11 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     // one allocation for the smaller solver buffers; the records, which start at
     // zero, come first
     const long long nrec = 2 * LS_BLOCKS * 2 + (p->n + 63) / 64 * 64 * 4;
-    TRYA(dalloc(&p->slab, (size_t)(nrec + 4 * nfeat + JT_SLICES * p->n + rfm_trsv_tiles_len(p->n))));
+    TRYA(dalloc(&p->slab, (size_t)(nrec + 8 * nfeat + JT_SLICES * p->n + rfm_trsv_tiles_len(p->n))));
     p->ls_rec = reinterpret_cast<unsigned long long*>(p->slab);
     p->trsv_rec = p->ls_rec + 2 * LS_BLOCKS * 2;
     p->slopes = p->slab + nrec;
-    p->jt_part = p->slopes + 4 * nfeat;
+    p->jt_part = p->slopes + 8 * nfeat;
     p->chain_tiles = p->jt_part + JT_SLICES * p->n;
     TRYA(dalloc(&p->dinv, (size_t)((p->n + 63) / 64) * 64 * 64));
     TRYA(dalloc(&p->sync, RFM_SYNC_WORDS));

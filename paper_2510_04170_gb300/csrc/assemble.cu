@@ -50,22 +50,23 @@ __global__ void k_features(double* __restrict__ feat, long long nfeat, int d, do
   *reinterpret_cast<double4*>(feat + 4 * g) = make_double4(out[0], out[1], out[2], out[3]);
 }
 
-// ks[g] = (k_1/sigma_1, k_2/sigma_2, k_3/sigma_3, sum of their squares) of every
-// feature: the derivatives of phi_j are t, 1 - t^2 and these factors.  Formed
-// once per problem: an FP64 division takes some nine FP64 instructions of 31 ns
-// on GB300, and three per feature and row were a third of the assembly's time
-// (124,416 rows of 512 features: 10.8 -> 6.8 ms with the table).
+// ks[2 g] = (k_1/sigma_1, k_2/sigma_2, k_3/sigma_3, 0) of every feature and ks[2 g +
+// 1] their squares: the derivatives of phi_j are t, 1 - t^2 and these factors.
+// Formed once per problem: an FP64 division takes some nine FP64 instructions of
+// 31 ns on GB300, and three per feature and row were a third of the assembly's
+// time (124,416 rows of 512 features: 10.8 -> 7.0 ms with the table).
+// The squares stand one by one, not as their sum: the Laplacian's three products
+// are added in the order and with the roundings of the quotients' own formula, so
+// that J, and with it the step counts of a solve, do not depend on the table.
 __global__ void k_feature_slopes(const double* __restrict__ feat, const double* __restrict__ sig, long long nfeat,
                                  int per_sub, int d, double* __restrict__ ks) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (g >= nfeat) return;
   const double* sg = sig + 4 * (g / per_sub);
-  double v[3] = {0.0, 0.0, 0.0}, q = 0.0;
-  for (int b = 0; b < d; ++b) {
-    v[b] = feat[4 * g + b] / sg[b];
-    q += v[b] * v[b];
-  }
-  *reinterpret_cast<double4*>(ks + 4 * g) = make_double4(v[0], v[1], v[2], q);
+  double v[3] = {0.0, 0.0, 0.0};
+  for (int b = 0; b < d; ++b) v[b] = feat[4 * g + b] / sg[b];
+  *reinterpret_cast<double4*>(ks + 8 * g) = make_double4(v[0], v[1], v[2], 0.0);
+  *reinterpret_cast<double4*>(ks + 8 * g + 4) = make_double4(v[0] * v[0], v[1] * v[1], v[2] * v[2], 0.0);
 }
 
 __device__ __forceinline__ double grid_pt(const double* X, int nbp, int b, int j, int p, int q) {
@@ -336,24 +337,32 @@ __device__ __forceinline__ RowGeo row_geo(const double* mu, const double* sig, i
   return g;
 }
 
-// tanh feature at the row point: t, 1 - t^2 and the feature vector k.
+// tanh feature at the row point: t, 1 - t^2 and the feature vector k.  The
+// multiply-adds are written out: which of two products the compiler fuses differs
+// between the loops that use this, and tanh's argument would with it.  The
+// assembly adds the axes in order; k_eval and k_phi_values (AXIS0_LAST) fuse the
+// first axis' product.
+template <bool AXIS0_LAST = false>
 __device__ __forceinline__ void feature_at(const double4 kb, const RowGeo& g, int d, double& t, double& s1) {
-  double z = g.l[0] * kb.x;
-  if (d > 1) z = z + g.l[1] * kb.y;
-  if (d > 2) z = z + g.l[2] * kb.z;
+  double z = AXIS0_LAST ? __fma_rn(g.l[0], kb.x, __dmul_rn(g.l[1], kb.y)) : __fma_rn(g.l[1], kb.y, __dmul_rn(g.l[0], kb.x));
+  if (d > 2) z = __fma_rn(g.l[2], kb.z, z);
   z = z + (d == 2 ? kb.z : kb.w);
   t = tanh(z);
   s1 = 1.0 - t * t;
 }
 
 // Linear-operator part L(phi_j) of an interior row of field f (Alg. 3 step 1);
-// ks as in k_feature_slopes, Lap phi = -2 t (1 - t^2) sum_b (k_b / sigma_b)^2.
-__device__ __forceinline__ double linear_part(const PdeConst& pc, int f, const double4 ks, double t, double s1,
+// ks the feature's entry of k_feature_slopes.
+__device__ __forceinline__ double linear_part(const PdeConst& pc, int f, const double* ks, double t, double s1,
                                               double a, double ax) {
-  const double lap = (-2.0 * t * s1) * ks.w;
+  const double4 sq = *reinterpret_cast<const double4*>(ks + 4);
+  double lap = 0.0;
+  lap = lap + (-2.0 * t * s1) * sq.x;
+  lap = lap + (-2.0 * t * s1) * sq.y;
+  if (pc.d == 3) lap = lap + (-2.0 * t * s1) * sq.z;
   if (pc.kind == 0) return -lap;
   if (pc.kind == 1) return -(f == 0 ? pc.p[0] : pc.p[1]) * lap;
-  return -a * lap - ax * (s1 * ks.x);
+  return -a * lap - ax * (s1 * ks[0]);
 }
 
 // Largest |x| of a row as the bits of a non-negative double, which order like
@@ -411,25 +420,19 @@ __global__ void __launch_bounds__(128) k_assemble(PdeConst pc, const double* __r
         const double4 kb = *reinterpret_cast<const double4*>(feat + 4 * (fb + j));
         double t, s1;
         feature_at(kb, g, d, t, s1);
-        const double4 ks = *reinterpret_cast<const double4*>(slopes + 4 * (fb + j));
+        const double4 ks = *reinterpret_cast<const double4*>(slopes + 8 * (fb + j));
+        const double k0 = ks.x, k1 = ks.y, k2 = ks.z;
         const double h = -2.0 * t * s1;
-        // the 2-jet of phi is (t, s1 k_b, h k_a k_b)
-        auto add_jet = [&](double cj, double* q) {
-          const double a = cj * s1, b = cj * h;
-          const double b0 = b * ks.x, b1 = b * ks.y, b2 = b * ks.z;
-          q[0] += cj * t;
-          q[1] += a * ks.x;
-          q[2] += a * ks.y;
-          q[3] += a * ks.z;
-          q[4] += b0 * ks.x;
-          q[5] += b1 * ks.y;
-          q[6] += b2 * ks.z;
-          q[7] += b0 * ks.y;
-          q[8] += b0 * ks.z;
-          q[9] += b1 * ks.z;
-        };
-        add_jet(c[fb + j], Q);
-        if (MODE == MODE_LS) add_jet(dv[fb + j], Qd);
+        const double jt[10] = {t, s1 * k0, s1 * k1, s1 * k2, h * k0 * k0, h * k1 * k1, h * k2 * k2,
+                               h * k0 * k1, h * k0 * k2, h * k1 * k2};
+        const double cj = c[fb + j];
+#pragma unroll
+        for (int k = 0; k < 10; ++k) Q[k] += cj * jt[k];
+        if (MODE == MODE_LS) {
+          const double dj = dv[fb + j];
+#pragma unroll
+          for (int k = 0; k < 10; ++k) Qd[k] += dj * jt[k];
+        }
         if (MODE == MODE_JF) {
           sA[j] = t;
           sB[j] = s1;
@@ -457,12 +460,12 @@ __global__ void __launch_bounds__(128) k_assemble(PdeConst pc, const double* __r
       if (MODE == MODE_JF) {
         __syncwarp();
         for (int j = lane; j < M; j += 32) {
-          const double4 k = *reinterpret_cast<const double4*>(slopes + 4 * (fb + j));
+          const double4 ks = *reinterpret_cast<const double4*>(slopes + 8 * (fb + j));
+          const double k0 = ks.x, k1 = ks.y, k2 = ks.z;
           const double t = sA[j], s1 = sB[j], h = -2.0 * t * s1;
-          const double g1 = C[1] * k.x + C[2] * k.y + C[3] * k.z;
-          const double h2 = k.x * (C[4] * k.x + C[7] * k.y + C[8] * k.z) + k.y * (C[5] * k.y + C[9] * k.z) +
-                            k.z * (C[6] * k.z);
-          const double Jv = C[0] * t + s1 * g1 + h * h2;
+          const double Jv = C[0] * t + s1 * (C[1] * k0 + C[2] * k1 + C[3] * k2) +
+                            h * (C[4] * k0 * k0 + C[5] * k1 * k1 + C[6] * k2 * k2 + C[7] * k0 * k1 +
+                                 C[8] * k0 * k2 + C[9] * k1 * k2);
           sA[j] = Jv;
           max_abs(rowmax, Jv);
         }
@@ -487,8 +490,7 @@ __global__ void __launch_bounds__(128) k_assemble(PdeConst pc, const double* __r
           if (MODE == MODE_LS) ud[ff] += t * dv[fb + j];
           if (MODE == MODE_JF) sA[ff * M + j] = t;
           if (ff == f) {
-            const double4 ks = *reinterpret_cast<const double4*>(slopes + 4 * (fb + j));
-            const double L = linear_part(pc, f, ks, t, s1, a, ax);
+            const double L = linear_part(pc, f, slopes + 8 * (fb + j), t, s1, a, ax);
             lu += L * cj;
             if (MODE == MODE_LS) lud += L * dv[fb + j];
             if (MODE == MODE_JF) sB[j] = L;
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(128) k_assemble(PdeConst pc, const double* __r
           double t, s1;
           feature_at(kb, g, d, t, s1);
           double val = t;
-          if (iface && sord == 1) val = s1 * slopes[4 * (fb + j) + axis];
+          if (iface && sord == 1) val = s1 * slopes[8 * (fb + j) + axis];
           val = sgn * val;
           acc += val * c[fb + j];
           if (MODE == MODE_LS) accd += val * dv[fb + j];
@@ -745,7 +747,7 @@ __global__ void k_eval(PdeConst pc, const double* __restrict__ feat, const doubl
       for (int j = lane; j < pc.M; j += 32) {
         const double4 kb = *reinterpret_cast<const double4*>(feat + 4 * (fb + j));
         double t, s1;
-        feature_at(kb, g, pc.d, t, s1);
+        feature_at<true>(kb, g, pc.d, t, s1);
         acc += t * c[fb + j];
       }
       acc = warp_sum(acc);
@@ -777,7 +779,7 @@ __global__ void k_phi_values(PdeConst pc, const double* __restrict__ feat, const
       const long long fb = (long long)e * pc.W + col;
       const double4 kb = *reinterpret_cast<const double4*>(feat + 4 * fb);
       double t, s1;
-      feature_at(kb, g, pc.d, t, s1);
+      feature_at<true>(kb, g, pc.d, t, s1);
       Phi[(size_t)q * pc.W + col] = scale * (float)t;
     }
   }

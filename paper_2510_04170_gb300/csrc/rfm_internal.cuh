@@ -44,7 +44,7 @@ struct rfm_problem {
   double* sig = nullptr;    // [G][4]
   double* slab = nullptr;   // allocation of slopes, jt_part, ls_rec, trsv_rec and chain_tiles
   double* feat = nullptr;   // [G*fields*M][4]
-  double* slopes = nullptr; // [G*fields*M][4]: k_b / sigma_b and the sum of their squares
+  double* slopes = nullptr; // [G*fields*M][8]: k_b / sigma_b and their squares
   RowSeg* segs = nullptr;
   int nseg = 0;
   bool explicit_rows = false;  // geometry with masked grids: points and row metadata built on the host

@@ -1,0 +1,89 @@
+"""Outputs that are pinned bit for bit, and the LSQR step counts that follow them.
+
+The LSQR of a solve stops by a test on rounded numbers, and at cond(R) = 1e8 ..
+1e9 the last bits of J, R and of a triangular solve decide on about every fourth
+problem whether that is one step sooner or later.  The order and the roundings of
+those sums are therefore part of the results: a kernel may spread the work
+differently but returns the same bits.  The digests (SHA-256 of the bytes) and
+the counts were recorded on a GB300 with 152 SMs; the row split of the QR's sums
+depends on the number of SMs."""
+import hashlib
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import rfm_workloads as W  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def rfm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("recorded with 152 SMs")
+    from paper_2510_04170_gb300 import build, rfm as _rfm
+    build.build()
+    return _rfm
+
+
+def vec(count, tag):
+    """Fixed values in [-1, 1) (a multiplicative hash of the index)."""
+    i = np.arange(1, count + 1, dtype=np.uint64) * np.uint64(0x9E3779B97F4A7C15)
+    i += np.uint64(tag * 0xD1B54A32D192ED03 % 2 ** 64)
+    i ^= i >> np.uint64(29)
+    i *= np.uint64(0xBF58476D1CE4E5B9)
+    return torch.as_tensor((i >> np.uint64(11)).astype(np.float64) * 2.0 ** -52 - 1.0, device="cuda")
+
+
+def digest(*tensors):
+    h = hashlib.sha256()
+    for t in tensors:
+        h.update(t.contiguous().cpu().numpy().tobytes())
+    return h.hexdigest()[:16]
+
+
+PROBLEMS = {
+    "kind0_2d": lambda: W.problem(2, (3, 2), 37, (11, 9), (7, 7), (8, 8)),
+    "kind0": lambda: W.problem(3, (2, 2, 2), 45, (6, 6, 6), (4, 4, 4), (4, 4, 4)),
+    "kind1": lambda: W.problem(3, (2, 2, 2), 33, (6, 6, 6), (5, 5, 5), (5, 5, 5), fields=2, pde_kind=1),
+    "kind2_2d": lambda: W.problem(2, (2, 2), 100, (20, 20), (20, 20), (20, 20), pde_kind=2),
+    "kind2": lambda: W.problem(3, (3, 2, 2), 64, (7, 6, 6), (4, 5, 4), (4, 4, 4), pde_kind=2),
+    "kind4": lambda: W.problem(3, (2, 2, 2), 45, (6, 6, 6), (4, 4, 4), (4, 4, 4), pde_kind=4),
+    "kind5": lambda: W.problem(3, (3, 3, 3), 45, (6, 6, 6), (4, 4, 4), (4, 4, 4), pde_kind=5),
+    "kind6": lambda: W.problem(3, (2, 2, 2), 70, (6, 6, 6), (4, 4, 4), (4, 4, 4), pde_kind=6),
+    "kind7": lambda: W.ball(40, 6, 300),
+}
+
+
+def assembled(rfm, name):
+    gp = rfm.Problem(PROBLEMS[name]())
+    c = vec(gp.n, 1) * 0.1
+    return gp, c, gp.rfm_assemble(c)
+
+
+def run_assemble(rfm, name):
+    gp, c, (F, lam) = assembled(rfm, name)
+    Jp, Js, _ = gp.rfm_get_jacobian()
+    alpha, f = gp.rfm_linesearch(c, -1.3 * c + 0.01 * vec(gp.n, 2), gp.rfm_residual(c)[1])
+    return F, lam, Jp, Js, gp.rfm_residual(0.9 * c)[0], torch.tensor([alpha, f], dtype=torch.float64)
+
+
+ASSEMBLE = {
+    'kind0_2d': '54d0f2806fdab43b',
+    'kind0': '71b1dc80055421ae',
+    'kind1': '710a4b07b0e2f40d',
+    'kind2_2d': 'b2d3531204a5271e',
+    'kind2': 'b9cf1088f4b9fa08',
+    'kind4': '2f0f81e7361b7a3c',
+    'kind5': '0d798da6bfa5350a',
+    'kind6': '59e2fcada769b1ba',
+    'kind7': '0ade3f6f2625de8a',
+}
+
+
+@pytest.mark.parametrize("name", list(PROBLEMS))
+def test_assembly(rfm, name):
+    assert digest(*run_assemble(rfm, name)) == ASSEMBLE[name]
