@@ -55,8 +55,7 @@ __global__ void k_sub(double* __restrict__ y, const double* __restrict__ a, cons
 // return at once, so a fixed chunk of iterations can be replayed as one graph.
 enum LsqrSlot {
   LS_ALPHA, LS_RHOBAR, LS_PHIBAR, LS_SUMSQ, LS_DD, LS_NORMB, LS_ETA, LS_CONLIM, LS_LIMIT, LS_ITN, LS_ISTOP,
-  LS_AB,                      // alpha / beta: u is kept as beta u
-  LS_RHO, LS_PHI, LS_TR,      // this iteration's rotation: rho, phi, theta / rho,
+  LS_RHO, LS_PHI, LS_TR,         // this iteration's rotation: rho, phi, theta / rho,
   LS_C, LS_NRHOBAR, LS_NPHIBAR,  // c and the next rhobar and phibar
   LS_SLOTS
 };
@@ -95,53 +94,47 @@ __global__ void k_lsqr_init(double* __restrict__ st, const double* __restrict__ 
   st[LS_LIMIT] = limit;
   st[LS_ITN] = 0.0;
   st[LS_ISTOP] = 7.0;
-  st[LS_AB] = alpha;  // u_1 is normalised
   *done = (beta > 0.0 && alpha > 0.0 && limit > 0.0) ? 0 : 1;
   if (!(beta > 0.0 && alpha > 0.0)) st[LS_ISTOP] = 0.0;
 }
 
 // Sums over a grid without a second launch: every block leaves its K sums in
 // partial[K * block ..], and the block that finds all others done (an arrival
-// counter, back at zero for the next use) adds them, thread t the blocks t, t +
-// 256, .. and then a fixed tree, so the result does not depend on which block it
-// is.  Returns true in thread 0 of that block, with the sums.
+// counter, back at zero for the next use) adds them, lane t of its first warp the
+// blocks t, t + 32, .. and then a butterfly, so the result does not depend on
+// which block it is and has the bits of rfm_norm2's two launches.  Returns true in
+// thread 0 of that block, with the sums.
 template <int K>
 __device__ __forceinline__ bool grid_sums(double (&v)[K], double* __restrict__ partial, unsigned int* __restrict__ count) {
   __shared__ double sh[K][8];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  auto block_sum = [&] {
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      v[k] = warp_sum(v[k]);
-      if (lane == 0) sh[k][w] = v[k];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
+  for (int k = 0; k < K; ++k) {
+    v[k] = warp_sum(v[k]);
+    if (lane == 0) sh[k][w] = v[k];
+  }
+  __syncthreads();
+  if (w != 0) return false;
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        v[k] = sh[k][0];
-        for (int q = 1; q < 8; ++q) v[k] += sh[k][q];
-      }
-  };
-  block_sum();
-  if (gridDim.x == 1) return threadIdx.x == 0;
-  if (threadIdx.x == 0) {
+  for (int k = 0; k < K; ++k) v[k] = warp_sum(lane < 8 ? sh[k][lane] : 0.0);
+  if (gridDim.x == 1) return lane == 0;
+  if (lane == 0) {
 #pragma unroll
     for (int k = 0; k < K; ++k) __stcg(partial + K * blockIdx.x + k, v[k]);
     __threadfence();
     last = atomicInc(count, gridDim.x - 1) == gridDim.x - 1;
   }
-  __syncthreads();
+  __syncwarp();
   if (!last) return false;
   __threadfence();
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     v[k] = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) v[k] += __ldcg(partial + K * i + k);
+    for (int i = lane; i < (int)gridDim.x; i += 32) v[k] += __ldcg(partial + K * i + k);
+    v[k] = warp_sum(v[k]);
   }
-  block_sum();
-  return threadIdx.x == 0;
+  return lane == 0;
 }
 
 // sc[0] = ||u||
@@ -154,17 +147,16 @@ __global__ void __launch_bounds__(256) k_lsqr_beta(const double* __restrict__ u,
   if (grid_sums<1>(v, partial, count)) sc[0] = sqrt(v[0]);
 }
 
-// v = t / beta - beta v (t = R^-T J^T of the unscaled u), sc[1] = ||v||, and the
-// iteration's rotation.
+// v = R^-T J^T u - beta v, sc[1] = ||v||, and the iteration's rotation.
 __global__ void __launch_bounds__(256) k_lsqr_alpha(double* __restrict__ v, const double* __restrict__ t, long long n,
                                                     double* __restrict__ st, double* __restrict__ sc,
                                                     double* __restrict__ partial, unsigned int* __restrict__ count,
                                                     const int* __restrict__ skip) {
   if (*skip) return;
-  const double beta = sc[0], inv = beta != 0.0 ? 1.0 / beta : 1.0;
+  const double beta = sc[0];
   double q[1] = {0.0};
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
-    const double x = t[i] * inv - beta * v[i];
+    const double x = __dadd_rn(t[i], -__dmul_rn(beta, v[i]));  // both rounded: LSQR's counts follow these bits
     v[i] = x;
     q[0] += x * x;
   }
@@ -177,7 +169,6 @@ __global__ void __launch_bounds__(256) k_lsqr_alpha(double* __restrict__ v, cons
     st[LS_C] = r.c;
     st[LS_NRHOBAR] = r.rhobar;
     st[LS_NPHIBAR] = r.phibar;
-    st[LS_AB] = sc[1] * inv;
   }
 }
 
@@ -236,9 +227,6 @@ int vgrid(long long n) {
   long long g = (n + 255) / 256;
   return (int)std::max<long long>(1, std::min<long long>(g, kVecBlocks));
 }
-
-// Blocks of a kernel that ends in grid_sums: few, as the last one adds their sums.
-int sum_grid(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 511) / 512, kVecBlocks)); }
 
 // ---------------------------------------------------------------- helpers
 template <class T>
@@ -587,9 +575,10 @@ struct LsqrOut {
 constexpr int kLsqrChunk = 16;  // iterations per replayed graph
 
 // One chunk of kLsqrChunk iterations, every kernel guarded by the done flag.  Norms,
-// scalings and the scalar recurrences ride in three vector kernels (beta; alpha and
-// the rotation; the update and the stopping tests): as twelve launches of their own
-// they took 30 of 105 us per iteration at n = 1,024.
+// scalings and the scalar recurrences ride in four vector kernels (beta; u / beta;
+// alpha and the rotation; the update and the stopping tests), every operation with
+// the rounding it has as a launch of its own: twelve launches took 30 us per
+// iteration at n = 1,024, these 16.
 rfm_status lsqr_chunk(rfm_problem* p, double* lst, int* done) {
   const long long m = p->m, n = p->n;
   cudaStream_t st = p->stream;
@@ -602,17 +591,19 @@ rfm_status lsqr_chunk(rfm_problem* p, double* lst, int* done) {
   double* sc = p->red + 1024;
   unsigned int* count = p->sync + SYNC_COUNT;
   for (int it = 0; it < kLsqrChunk; ++it) {
-    // u holds beta u: the new one is J R^{-1} v - alpha u
+    // beta u = J R^{-1} v - alpha u
     RFM_TRY(rfm_launch_trsv(p, 0, v, tn));
-    RFM_TRY(rfm_launch_jmv_axpby(p, tn, 1.0, -1.0, u, lst + LS_AB));
-    k_lsqr_beta<<<sum_grid(m), 256, 0, st>>>(u, m, sc, p->red, count, done);
+    RFM_TRY(rfm_launch_jmv_axpby(p, tn, 1.0, -1.0, u, lst + LS_ALPHA));
+    k_lsqr_beta<<<vgrid(m), 256, 0, st>>>(u, m, sc, p->red, count, done);
+    RFM_CHECK_LAUNCH();
+    k_scale_by<<<vgrid(m), 256, 0, st>>>(u, m, sc, 1, done);
     RFM_CHECK_LAUNCH();
     // alpha v = R^{-T} J^T u - beta v
     RFM_TRY(rfm_launch_jtmv(p, u, tn));
     RFM_TRY(rfm_launch_trsv(p, 1, tn, tn2));
-    k_lsqr_alpha<<<sum_grid(n), 256, 0, st>>>(v, tn2, n, lst, sc, p->red, count, done);
+    k_lsqr_alpha<<<vgrid(n), 256, 0, st>>>(v, tn2, n, lst, sc, p->red, count, done);
     RFM_CHECK_LAUNCH();
-    k_lsqr_update<<<sum_grid(n), 256, 0, st>>>(x, w, v, n, lst, sc, p->red, count, done);
+    k_lsqr_update<<<vgrid(n), 256, 0, st>>>(x, w, v, n, lst, sc, p->red, count, done);
     RFM_CHECK_LAUNCH();
   }
   return RFM_OK;

@@ -3,10 +3,10 @@
 //  * k_jmv:   y = s1 * J x + s2 * y.  One warp per four rows; a row is W
 //             contiguous doubles of its primary block (and W more of the
 //             secondary block for interface rows), read once, coalesced.
-//  * k_jtmv:  y = J^T x.  One CTA per (column block, 64-column chunk, slice of
+//  * k_jtmv:  y = J^T x.  One warp per (column block, 32-column chunk, eighth of
 //             the block's rows); the rows are walked in a fixed order and the
-//             eight warps' and the slices' partial sums are combined in a fixed
-//             order, so the result is deterministic.
+//             eight partial sums are added in a fixed order (k_jtmv_sum), so the
+//             result is deterministic.
 //  * k_trsv_chain: x = R^{-1} b or x = R^{-T} b for the upper-triangular
 //             preconditioner R (column-major, leading dimension ldr), in one
 //             cooperative launch: a cluster of four CTAs solves the 64-row
@@ -88,67 +88,76 @@ __global__ void __launch_bounds__(256) k_jmv(const double* __restrict__ Jp, cons
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       const long long i = i0 + (hi ? 2 : 0) + (odd ? 1 : 0);
-      if ((lane & 7) == 0 && i < m) y[i] = s2 == 0.0 ? s1 * a : s1 * a + s2 * y[i];
+      if ((lane & 7) == 0 && i < m) y[i] = s2 == 0.0 ? s1 * a : __fma_rn(s1, a, __dmul_rn(s2, y[i]));
     }
   }
 }
 
-// Slice z of the rows of column block b; with more than one slice the partial
-// sums go to part[z][n] and k_jtmv_sum adds them.  Four rows' loads are in flight
-// per warp.
-__global__ void __launch_bounds__(256) k_jtmv(const double* __restrict__ Jp, const double* __restrict__ Js,
+// Slice z of column block b: its rows z, z + JT_SLICES, z + 2 JT_SLICES, .., one
+// chain of products per column (lane).  Which rows form a chain and the order of
+// the sums over slices do not depend on how the work is spread, so the result
+// keeps its bits, and the chains of a column may run on different SMs: with all
+// eight in one CTA, 15,552 rows of 8 blocks of 128 were 16 CTAs and took 60 us
+// (now 20; 124,416 rows of 64 blocks of 512: 148 -> 136 us, 110 of them FP64
+// instructions).  A warp keeps 8 to 16 rows' loads in flight, the
+// indices and factors of 32 rows a batch ahead.
+__global__ void __launch_bounds__(128) k_jtmv(const double* __restrict__ Jp, const double* __restrict__ Js,
                                               const int* __restrict__ colptr, const int* __restrict__ colrows,
                                               long long m_int, int W, const double* __restrict__ x,
-                                              const int* __restrict__ skip, double* __restrict__ y, long long n) {
+                                              const int* __restrict__ skip, double* __restrict__ part, long long n) {
   if (skip && *skip) return;
-  const int b = blockIdx.x;
-  const int c0 = blockIdx.y * 64;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int ca = c0 + lane, cb = c0 + 32 + lane;
-  double acc0 = 0.0, acc1 = 0.0;
-  const int all = colptr[b + 1] - colptr[b];
-  const int per = (all + (int)gridDim.z - 1) / (int)gridDim.z;
-  const int beg = colptr[b] + min(all, per * (int)blockIdx.z), end = colptr[b] + min(all, per * ((int)blockIdx.z + 1));
-  const bool ina = ca < W, inb = cb < W;
-  for (int t = beg + w; t < end; t += 32) {
-    double v0[4], v1[4], xr[4];
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
+  const int c0 = (blockIdx.y * 4 + (threadIdx.x >> 5)) * 32;
+  if (c0 >= W) return;
+  const int col = min(c0 + lane, W - 1);
+  const int beg = colptr[b] + blockIdx.z, end = colptr[b + 1];
+  double acc = 0.0;
+  // lane i holds the index and the factor of row t + JT_SLICES i of the batch at t
+  // (row 0 with factor 0 past the last)
+  auto entry = [&](int t) { return t + JT_SLICES * lane < end ? (unsigned int)colrows[t + JT_SLICES * lane] : 0u; };
+  auto factor = [&](int t, unsigned int e) { return t + JT_SLICES * lane < end ? x[e & 0x7fffffffu] : 0.0; };
+  double v[2][8];
+  auto load = [&](double (&q)[8], unsigned int ent, int i0) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const bool in = t + 8 * u < end;
-      const unsigned int ent = in ? (unsigned int)colrows[t + 8 * u] : 0u;
-      const long long r = ent & 0x7fffffffu;
-      const double* row = (ent >> 31) ? Js + (size_t)(r - m_int) * W : Jp + (size_t)r * W;
-      xr[u] = in ? x[r] : 0.0;
-      v0[u] = in && ina ? __ldcs(row + ca) : 0.0;
-      v1[u] = in && inb ? __ldcs(row + cb) : 0.0;
+    for (int i = 0; i < 8; ++i) {
+      const unsigned int e = __shfl_sync(0xffffffffu, ent, i0 + i);
+      const long long r = e & 0x7fffffffu;
+      q[i] = __ldcs(((e >> 31) ? Js + (size_t)(r - m_int) * W : Jp + (size_t)r * W) + col);
     }
+  };
+  unsigned int ent = entry(beg);
+  double xr = factor(beg, ent);
+  load(v[0], ent, 0);
+  for (int t = beg; t < end; t += 32 * JT_SLICES) {
+    const int cnt = min(32, (end - t + JT_SLICES - 1) / JT_SLICES), tn = t + 32 * JT_SLICES;
+    const unsigned int nent = entry(tn);
+    double nxr = 0.0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (t + 8 * u < end) {
-        acc0 += v0[u] * xr[u];
-        acc1 += v1[u] * xr[u];
+    for (int i0 = 0; i0 < 32; i0 += 8) {  // the next eight rows' loads, then this eight's products
+      if (i0 < 24) {
+        if (cnt > i0 + 8) load(v[(i0 / 8 + 1) & 1], ent, i0 + 8);
+      } else if (tn < end) {
+        load(v[0], nent, 0);
       }
-  }
-  __shared__ double sh[8][64];
-  sh[w][lane] = acc0;
-  sh[w][32 + lane] = acc1;
-  __syncthreads();
-  if (threadIdx.x < 64) {
-    double s = 0.0;
+      if (i0 == 8) nxr = factor(tn, nent);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) s += sh[k][threadIdx.x];
-    const int col = c0 + threadIdx.x;
-    if (col < W) y[(size_t)blockIdx.z * n + (size_t)b * W + col] = s;
+      for (int i = 0; i < 8; ++i)
+        if (i0 + i < cnt) acc += v[(i0 / 8) & 1][i] * __shfl_sync(0xffffffffu, xr, i0 + i);
+    }
+    ent = nent;
+    xr = nxr;
   }
+  if (c0 + lane < W) part[(size_t)blockIdx.z * n + (size_t)b * W + col] = acc;
 }
 
-__global__ void k_jtmv_sum(const double* __restrict__ part, int Z, long long n, const int* __restrict__ skip,
+__global__ void k_jtmv_sum(const double* __restrict__ part, long long n, const int* __restrict__ skip,
                            double* __restrict__ y) {
   if (skip && *skip) return;
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= n) return;
   double s = 0.0;
-  for (int z = 0; z < Z; ++z) s += part[(size_t)z * n + i];
+#pragma unroll
+  for (int z = 0; z < JT_SLICES; ++z) s += part[(size_t)z * n + i];
   y[i] = s;
 }
 
@@ -278,7 +287,10 @@ __global__ void __launch_bounds__(256) k_trsv(const double* __restrict__ R, long
 // 8 columns of one row, so a product is 8 instructions per warp, the sum over
 // columns one shuffle and four shared-memory partials, and y_t and x_t go to all
 // four CTAs through distributed shared memory with one cluster barrier each (0.2
-// us).  Only C_1 and Z_k wait for the step before; their tiles and the others are
+// us).  Which columns a thread takes and how the partials are added is fixed by
+// chain_col, not by the split: a row's sum is eight chains of eight products in
+// the order that one CTA solving the chain alone would take, so the solution's
+// bits do not depend on the cluster.  Only C_1 and Z_k wait for the step before; their tiles and the others are
 // read from a copy in the threads' order (k_trsv_pack), two steps ahead.  One
 // chain CTA that did both products alone took 3.7 to 4.6 us per step, this takes
 // 2.1 (n = 4,096: 239 / 295 -> 135 us for R^{-1} / R^{-T}); from n = 16,384 on the
@@ -294,7 +306,7 @@ __global__ void __launch_bounds__(256) k_trsv(const double* __restrict__ R, long
 // are in a fixed order, so results are deterministic.  Waits are bounded.
 constexpr int CHAIN_CL = 4;            // CTAs of the chain cluster (16 rows each)
 constexpr int CHAIN_D = 2;             // distances 1 .. CHAIN_D are the chain's
-constexpr int HMAXT = 4;               // targets per helper CTA
+constexpr int HMAXT = 5;               // targets per helper CTA
 constexpr int ZLD = TB + 1;            // leading dimension of a tile in shared memory
 
 template <int TRANS>
@@ -304,12 +316,11 @@ __device__ __forceinline__ int chain_block(int t, int nblk) { return TRANS == 0 
 // Z + k * 4096: Z[k][c * 64 + r] = (R_kk^{-1})(r, c).  Entries below the
 // diagonal and, in a ragged last block, rows and columns past n are zero.
 // Column c solves R_kk z = e_c by back substitution (one warp per column, rows
-// on the lanes) with the pivots' reciprocals; four CTAs share a block's columns,
-// as the FP64 units of one SM would take 50 us for them.
+// on the lanes, IEEE division by each pivot); sixteen CTAs share a block's
+// columns, as a step is some twelve FP64 instructions of 31 ns.
 __global__ void __launch_bounds__(128) k_trsv_dinv(const double* __restrict__ R, long long ldr, int n,
                                                    double* __restrict__ Z) {
   __shared__ double D[TB * ZLD];
-  __shared__ double rec[TB];
   const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int r0 = k * TB, rows = min(TB, n - r0);
   for (int idx = tid; idx < TB * TB; idx += blockDim.x) {
@@ -317,31 +328,37 @@ __global__ void __launch_bounds__(128) k_trsv_dinv(const double* __restrict__ R,
     D[c * ZLD + r] = (r <= c && c < rows) ? R[(size_t)(r0 + c) * ldr + r0 + r] : 0.0;
   }
   __syncthreads();
-  if (tid < TB) rec[tid] = tid < rows ? 1.0 / D[tid * ZLD + tid] : 0.0;
-  __syncthreads();
   double* out = Z + (size_t)k * TB * TB;
-  for (int jj = 0; jj < TB / 16; ++jj) {
-    const int j = blockIdx.y + 4 * (w + 4 * jj);  // columns spread over CTAs and warps
-    double acc0 = lane == j ? 1.0 : 0.0, acc1 = lane + 32 == j ? 1.0 : 0.0;
-    double z0 = 0.0, z1 = 0.0;
-    if (j < rows) {
-      for (int i = j; i >= 0; --i) {
-        const double zi = __shfl_sync(0xffffffffu, i < 32 ? acc0 : acc1, i & 31) * rec[i];
-        if (i < 32 && lane == i) z0 = zi;
-        if (i >= 32 && lane == i - 32) z1 = zi;
-        if (lane < i) acc0 -= D[i * ZLD + lane] * zi;
-        if (i > 32 && lane + 32 < i) acc1 -= D[i * ZLD + lane + 32] * zi;
-      }
+  const int j = blockIdx.y + 16 * w;  // columns spread over CTAs and warps
+  double acc0 = lane == j ? 1.0 : 0.0, acc1 = lane + 32 == j ? 1.0 : 0.0;
+  double z0 = 0.0, z1 = 0.0;
+  if (j < rows) {
+    for (int i = j; i >= 0; --i) {
+      const double zi = __shfl_sync(0xffffffffu, i < 32 ? acc0 : acc1, i & 31) / D[i * ZLD + i];
+      if (i < 32 && lane == i) z0 = zi;
+      if (i >= 32 && lane == i - 32) z1 = zi;
+      if (lane < i) acc0 -= D[i * ZLD + lane] * zi;
+      if (i > 32 && lane + 32 < i) acc1 -= D[i * ZLD + lane + 32] * zi;
     }
-    out[j * TB + lane] = z0;
-    out[j * TB + lane + 32] = z1;
   }
+  out[j * TB + lane] = z0;
+  out[j * TB + lane + 32] = z1;
 }
 
-// Offset of entry (r, c) of a tile in the order the chain's threads read it:
-// rank r / 16, then the thread's i-th column, warp, lane.
-__device__ __forceinline__ int pack_at(int r, int c) {
-  return (((r >> 4) * 8 + (c & 7)) * 4 + (c >> 4)) * 32 + (((c >> 3) & 1) << 4 | (r & 15));
+// Column of the i-th product in chain g (0 .. 7) of row r of tile d.  The chains'
+// sums are added as ((0+1) + (2+3)) + ((4+5) + (6+7)):
+//  d = 0 (the inverse, a triangle): a pair of rows r, 63 - r is 65 terms dealt to
+//        eight chains in turn, row min(r, 63 - r) first; the entries outside the
+//        triangle are zeros in the same chains
+//  d = 1: columns of equal remainder modulo 8, the even remainders before the odd
+//        ones for R^{-T}
+//  d = 2: every fourth column of a half
+__device__ __forceinline__ int chain_col(int dir, int d, int r, int g, int i) {
+  if (d == 2) return 32 * (g >> 2) + (g & 3) + 4 * i;
+  if (d == 1) return 8 * i + (dir == 0 ? g : (g < 4 ? 2 * g : 2 * g - 7));
+  const int pos = (g >> 1) + 4 * (g & 1);  // term's position modulo 8
+  const int first = dir == 0 ? (r < TB / 2 ? pos + r : pos - 1) : (r < TB / 2 ? pos : pos + r);
+  return 8 * i + (first & 7);
 }
 
 // Tiles of the chain, P[dir][k][d]: d = 0 the inverse (dir 0 Z_k, dir 1 Z_k^T),
@@ -365,10 +382,11 @@ __global__ void __launch_bounds__(256) k_trsv_pack(const double* __restrict__ R,
     t[dir == 0 ? hi * ZLD + lo : lo * ZLD + hi] = v;  // t[c * ZLD + r]
   }
   __syncthreads();
+  // in the order the chain's threads read it: rank, the thread's i-th product, warp, lane
   for (int idx = tid; idx < TB * TB; idx += 256) {
     const int lane = idx & 31, w = (idx >> 5) & 3, i = (idx >> 7) & 7, q = idx >> 10;
-    const int r = q * 16 + (lane & 15), c = w * 16 + (lane >> 4) * 8 + i;
-    out[pack_at(r, c)] = t[c * ZLD + r];
+    const int r = q * 16 + (lane & 15), c = chain_col(dir, d, r, w * 2 + (lane >> 4), i);
+    out[idx] = t[c * ZLD + r];
   }
 }
 
@@ -401,7 +419,10 @@ __device__ __forceinline__ void trsv_chain(const ChainArgs& a, unsigned int tag,
   const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 3;
   const bool crit = tid < 128;
   const int rank = blockIdx.x, nblk = a.nblk, n = a.n;
-  const int c0 = (w * 2 + (lane >> 4)) * 8;  // this thread's columns
+  const int row = rank * 16 + (lane & 15), chain = w * 2 + (lane >> 4);
+  int c0[3];  // first columns of this thread's chains in the three tiles
+#pragma unroll
+  for (int d = 0; d < 3; ++d) c0[d] = chain_col(TRANS, d, row, chain, 0);
   // tile d of step t
   auto fetch = [&](double (&q)[8], int t, int d) {
     if (t >= nblk) return;
@@ -410,13 +431,10 @@ __device__ __forceinline__ void trsv_chain(const ChainArgs& a, unsigned int tag,
 #pragma unroll
     for (int i = 0; i < 8; ++i) q[i] = __ldg(src + i * 128);
   };
-  auto dot8 = [&](const double (&q)[8], const double* v, double acc) {
+  auto dot8 = [&](const double (&q)[8], const double* v, int d) {
+    double acc = 0.0;
 #pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      const double2 t = *reinterpret_cast<const double2*>(v + c0 + i);
-      acc = fma(q[i], t.x, acc);
-      acc = fma(q[i + 1], t.y, acc);
-    }
+    for (int i = 0; i < 8; ++i) acc = fma(q[i], v[c0[d] + (d == 2 ? 4 : 8) * i], acc);
     return acc;
   };
   // this thread's part of a row summed over its warp's columns, then the warps'
@@ -448,11 +466,11 @@ __device__ __forceinline__ void trsv_chain(const ChainArgs& a, unsigned int tag,
     auto step = [&](double (&q)[2][8], int t) {
       const int k = chain_block<TRANS>(t, nblk);
       cluster_wait();  // A: x_{t-1} and hs of this step
-      row_part(dot8(q[1], xs + ((t - 1) & 3) * TB, 0.0), part);
+      row_part(dot8(q[1], xs + ((t - 1) & 3) * TB, 1), part);
       if (w == 0) spread(ys, hs[(t & 1) * 16 + (lane & 15)] - row_sum(part));
       cluster_arrive();
       cluster_wait();  // B: y_t
-      row_part(dot8(q[0], ys, 0.0), part + 64);
+      row_part(dot8(q[0], ys, 0), part + 64);
       if (w == 0) {
         const double xv = row_sum(part + 64);
         spread(xs + (t & 3) * TB, xv);
@@ -480,7 +498,7 @@ __device__ __forceinline__ void trsv_chain(const ChainArgs& a, unsigned int tag,
       unsigned long long lo = 0, hi = 0;
       if (summed) rec_load(rec, lo, hi);
       double v = own && gi < n ? a.rhs[gi] : 0.0;
-      row_part(dot8(q, xs + ((t - 2) & 3) * TB, 0.0), part + 128);
+      row_part(dot8(q, xs + ((t - 2) & 3) * TB, 2), part + 128);
       if (w == 0) {
         const double near = row_sum(part + 128);
         if (summed) {
@@ -738,45 +756,21 @@ rfm_status rfm_launch_jmv_axpby(rfm_problem* p, const double* x, double s1, doub
   return RFM_OK;
 }
 
-// Slices of every column block's rows: the count with the least work on the
-// busiest SM (about 16 CTAs of an SM run at once), at most JT_SLICES and at
-// least 128 rows each on average.  One slice per block left 16 CTAs for 15,552
-// rows of 8 blocks of 128 (60 us; 10 with 9 slices, and 2 for their sum).
-static int jtmv_slices(const rfm_problem* p) {
-  const int nsm = std::max(1, rfm_num_sms());
-  const long long tiles = (long long)p->G * ((p->W + 63) / 64);
-  const long long rows = (p->m + p->m_iface) / std::max(1, p->G);
-  int best = 1;
-  double cost = 0.0;
-  for (int z = 1; z <= JT_SLICES && (z == 1 || rows / z >= 128); ++z) {
-    const double c = (double)((tiles * z + nsm - 1) / nsm) / z + 0.01 * z;  // + the slices' sum
-    if (z == 1 || c < cost) {
-      cost = c;
-      best = z;
-    }
-  }
-  return best;
-}
-
 rfm_status rfm_launch_jtmv(rfm_problem* p, const double* x, double* y) {
-  const int Z = p->jt_part ? jtmv_slices(p) : 1;
-  dim3 grid(p->G, (p->W + 63) / 64, Z);
   ProfScope ps(PF_JTMV, p->stream);
   rfm_prof_work(PF_JTMV, 8.0 * ((double)(p->m + p->m_iface) * p->W + p->m + p->n));
-  k_jtmv<<<grid, 256, 0, p->stream>>>(p->Jp, p->Js, p->colptr, p->colrows, p->m_int, p->W, x, p->skip,
-                                      Z > 1 ? p->jt_part : y, p->n);
+  k_jtmv<<<dim3(p->G, (p->W + 127) / 128, JT_SLICES), 128, 0, p->stream>>>(p->Jp, p->Js, p->colptr, p->colrows,
+                                                                          p->m_int, p->W, x, p->skip, p->jt_part, p->n);
   RFM_CHECK_LAUNCH();
-  if (Z > 1) {
-    k_jtmv_sum<<<(unsigned)((p->n + 255) / 256), 256, 0, p->stream>>>(p->jt_part, Z, p->n, p->skip, y);
-    RFM_CHECK_LAUNCH();
-  }
+  k_jtmv_sum<<<(unsigned)((p->n + 255) / 256), 256, 0, p->stream>>>(p->jt_part, p->n, p->skip, y);
+  RFM_CHECK_LAUNCH();
   return RFM_OK;
 }
 
 rfm_status rfm_trsv_prepare(rfm_problem* p) {
   if (!p->dinv || !p->R) return RFM_OK;
   const int n = (int)p->n, nblk = (n + TB - 1) / TB;
-  k_trsv_dinv<<<dim3(nblk, 4), 128, 0, p->stream>>>(p->R, p->ldr, n, p->dinv);
+  k_trsv_dinv<<<dim3(nblk, 16), 128, 0, p->stream>>>(p->R, p->ldr, n, p->dinv);
   RFM_CHECK_LAUNCH();
   k_trsv_pack<<<dim3(nblk, CHAIN_D + 1, 2), 256, 0, p->stream>>>(p->R, p->ldr, n, nblk, p->dinv, p->chain_tiles);
   RFM_CHECK_LAUNCH();
@@ -789,9 +783,10 @@ long long rfm_trsv_tiles_len(long long n) { return 2LL * ((n + TB - 1) / TB) * (
 namespace {
 using ChainKernel = void (*)(ChainArgs);
 ChainKernel chain_kernel(int trans, int nt) {
-  static const ChainKernel k[2][3] = {{k_trsv_chain<0, 1>, k_trsv_chain<0, 2>, k_trsv_chain<0, HMAXT>},
-                                      {k_trsv_chain<1, 1>, k_trsv_chain<1, 2>, k_trsv_chain<1, HMAXT>}};
-  return k[trans ? 1 : 0][nt == 1 ? 0 : nt == 2 ? 1 : 2];
+  static const ChainKernel k[2][4] = {
+      {k_trsv_chain<0, 1>, k_trsv_chain<0, 2>, k_trsv_chain<0, 4>, k_trsv_chain<0, HMAXT>},
+      {k_trsv_chain<1, 1>, k_trsv_chain<1, 2>, k_trsv_chain<1, 4>, k_trsv_chain<1, HMAXT>}};
+  return k[trans ? 1 : 0][nt == 1 ? 0 : nt == 2 ? 1 : nt <= 4 ? 2 : 3];
 }
 
 // CTAs of the chain kernels that are resident together (whole clusters), per
@@ -805,7 +800,7 @@ int chain_max_ctas() {
   if (cached[dev] == 0) {
     int least = 1 << 30;
     for (int trans = 0; trans < 2; ++trans)
-      for (int nt : {1, 2, HMAXT}) {
+      for (int nt : {1, 2, 4, HMAXT}) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CHAIN_CL);
         cfg.blockDim = dim3(256);
@@ -834,9 +829,12 @@ rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x
   if (p->dinv && p->dinv_of != p->R) RFM_TRY(rfm_trsv_prepare(p));
   ProfScope ps(PF_TRSV, p->stream);
   rfm_prof_work(PF_TRSV, 8.0 * (double)n * (n + 1) / 2 + 16.0 * n);  // R read once, b and x
-  // chain + helpers when every block has a helper slot
+  // Chain + helpers up to four blocks per SM (n = 38,800), a rule on n alone so
+  // that the solution's bits are those of one form; the helpers, fewer than the
+  // SMs, take a fifth target at the end of that range.
   const int H = std::min(chain_max_ctas() - CHAIN_CL, (nblk + CHAIN_CL - 1) / CHAIN_CL * CHAIN_CL);
-  if (p->trsv_rec && p->dinv && p->chain_tiles && H > 0 && nblk <= HMAXT * H) {
+  if (p->trsv_rec && p->dinv && p->chain_tiles && H > 0 && nblk <= HMAXT * H &&
+      nblk - CHAIN_D - 1 <= 4 * (rfm_num_sms() - 1)) {
     ChainArgs a;
     a.R = p->R; a.P = p->chain_tiles + (trans ? rfm_trsv_tiles_len(n) / 2 : 0);
     a.ldr = p->ldr; a.n = n; a.nblk = nblk; a.H = H; a.rhs = b; a.x = x;

@@ -14,7 +14,7 @@
 
 #define RFM_MAX_FIELDS 2
 #define RFM_MAX_WIDTH 2048
-#define JT_SLICES 32
+#define JT_SLICES 8
 #define LS_BLOCKS 304
 
 // One run of rows that share a point grid (Sec. 5): an interior grid of a

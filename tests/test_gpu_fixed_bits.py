@@ -87,3 +87,83 @@ ASSEMBLE = {
 @pytest.mark.parametrize("name", list(PROBLEMS))
 def test_assembly(rfm, name):
     assert digest(*run_assemble(rfm, name)) == ASSEMBLE[name]
+
+
+def run_products(rfm, name):
+    gp, _, _ = assembled(rfm, name)
+    return gp.rfm_jmv(vec(gp.n, 3), 0), gp.rfm_jmv(vec(gp.m, 4), 1)
+
+
+PRODUCTS = {
+    'kind0_2d': '56263d4b738cc017',
+    'kind0': 'edc0e124226aacdb',
+    'kind1': '55c71b4d50daed1a',
+    'kind2_2d': 'dde1f21b9d699edd',
+    'kind2': '842de401eac0491a',
+    'kind4': 'c88cb634dcd007b0',
+    'kind5': '6e4cebc1da280bba',
+    'kind6': 'a0a74712fc3ad251',
+    'kind7': '946183647454707e',
+}
+
+
+@pytest.mark.parametrize("name", list(PROBLEMS))
+def test_products(rfm, name):
+    assert digest(*run_products(rfm, name)) == PRODUCTS[name]
+
+
+def triangular(n):
+    """Upper triangle with a dominant diagonal, column-major."""
+    return (vec(n * n, 5).view(n, n).tril() / n ** 0.5 + 2.0 * torch.eye(n, dtype=torch.float64, device="cuda")).contiguous()
+
+
+def run_trsv(rfm, gm):
+    g, M = gm
+    gp = rfm.Problem(W.problem(3, (g,) * 3, M, (4, 4, 4), (3, 3, 3), (3, 3, 3)))
+    gp.rfm_set_r(triangular(gp.n))
+    return gp.rfm_trsv(vec(gp.n, 6), 0), gp.rfm_trsv(vec(gp.n, 7), 1)
+
+
+# subdomains per axis and features: part of a block, one block, ragged last
+# blocks, one to four targets per helper
+TRSV_CASES = [(1, 24), (1, 64), (1, 65), (1, 257), (2, 45), (2, 250), (3, 300), (4, 300)]
+TRSV = {
+    (1, 24): '5a51774327bb7dda',
+    (1, 64): 'befd79fcc94dfefb',
+    (1, 65): '8997f9cfce975ae0',
+    (1, 257): 'bcb68d129ecd3685',
+    (2, 45): '89cc4096fec1c028',
+    (2, 250): 'db3a7760a77a696c',
+    (3, 300): '9c6a510765ef454b',
+    (4, 300): '07655576d44365ca',
+}
+
+
+@pytest.mark.parametrize("gm", TRSV_CASES)
+def test_triangular_solves(rfm, gm):
+    assert digest(*run_trsv(rfm, gm)) == TRSV[gm]
+
+
+def run_lsqr(rfm, name):
+    gp, _, (F, _) = assembled(rfm, name)
+    gp.rfm_set_r(triangular(gp.n))
+    d, itn, istop = gp.rfm_lsqr(-F, 1e-13, 1e30, 37)
+    return d, torch.tensor([itn, istop])
+
+
+LSQR = {
+    'kind0_2d': '78f42e8c55b48476',
+    'kind0': '5021ed33954c6a9d',
+    'kind1': '5abcb4e490c50fd2',
+    'kind2_2d': 'e8bbcee8b3a8b776',
+    'kind2': 'c08c548e08893da2',
+    'kind4': 'd0a9c56839f707b7',
+    'kind5': '7d979debcb430daf',
+    'kind6': '86b4da82ff667a57',
+    'kind7': 'eeb25b7e41f1f7e3',
+}
+
+
+@pytest.mark.parametrize("name", list(PROBLEMS))
+def test_lsqr_directions(rfm, name):
+    assert digest(*run_lsqr(rfm, name)) == LSQR[name]
