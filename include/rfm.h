@@ -234,7 +234,7 @@ rfm_status rfm_emulated_dgemm(const double* A, int64_t lda, const double* B, int
  * fixed latency budgets.  The paper has no counterpart; this is a deployment
  * variant of the QR step.
  *  - n <= 512 (RFM_EINVAL with a message otherwise); s >= n.
- *  - Scratch is a fixed 15.1 MB file-scope device array (plus 16 KB of barrier
+ *  - Scratch is a fixed 9.9 MB file-scope device array (plus 16 KB of barrier
  *    words) present on every GPU that loads the library until process exit.
  *  - The first call on a device looks up the array's device address with that
  *    device current; make that first call before any stream capture.
@@ -311,9 +311,7 @@ rfm_status rfm_batch_solve(rfm_batch* b, const rfm_solve_opts* opts, int solver,
 /* QR autotuner: times the first 128 columns of a seeded random s x n
  * factorisation for the FP64 path (precision 0) and the tensor-core path
  * (precision 2), each with the panel factorisation capped at 16, 32, 64 and
- * all SMs' CTAs, and returns the fastest's precision, with its cap where that
- * beats all SMs by a quarter or more and else all SMs (cached per (s, n) for
- * the process).
+ * all SMs' CTAs, and returns the fastest (cached per (s, n) for the process).
  * ms8_out (nullable) receives the eight probe times in ms, FP64 caps first,
  * then tensor-core caps, caps in the order above.  Allocates a probe matrix
  * of s*n doubles plus the QR buffers. */

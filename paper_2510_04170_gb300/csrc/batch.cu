@@ -111,11 +111,7 @@ rfm_status probe_qr(long long s, long long n, cudaStream_t st, QrChoice* out) {
     for (int c = 1; c < kCands; ++c)
       if (out->ms[c] < out->ms[arg]) arg = c;
     out->precision = arg < kCaps ? 0 : 2;
-    // The block factorisation chooses its CTAs by the row count, and its sums
-    // follow that choice: a cap is taken only where the probe shows a clear
-    // gain, so that a batch otherwise gives the bits of a stand-alone solve.
-    const int all = (arg / kCaps) * kCaps + kCaps - 1;
-    out->panel_cap = out->ms[arg] < 0.75 * out->ms[all] ? caps[arg % kCaps] : caps[kCaps - 1];
+    out->panel_cap = caps[arg % kCaps];
   }
   cudaStreamSynchronize(st);
   if (e0) cudaEventDestroy(e0);

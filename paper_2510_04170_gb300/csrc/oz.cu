@@ -549,11 +549,13 @@ struct AccStrided {  // X(i, k) = base[i * si + k * sk]
   long long si, sk;
   __device__ double operator()(long long i, long long k) const { return base[i * si + k * sk]; }
 };
-struct AccHouseVt {  // row i = Householder vector i of the panel at j0 less its unit entry, k = row offset from j0
+struct AccHouseVt {  // row i = Householder vector i of the panel at j0, k = row offset from j0
   const double* A;
   long long lda, j0;
   __device__ double operator()(long long i, long long k) const {
-    return k <= i ? 0.0 : A[(size_t)(j0 + i) * lda + j0 + k];
+    if (k < i) return 0.0;
+    if (k == i) return 1.0;
+    return A[(size_t)(j0 + i) * lda + j0 + k];
   }
 };
 struct AccHouseV {  // row i = matrix row j0 + i, k = panel column
@@ -817,16 +819,16 @@ rfm_status rfm_oz_gemm_part(const uint16_t* Ad, int pA, const int* ea, const uin
   }
   const long long tiles = (long long)a.mtiles * a.ntiles;
   // Split K when the output tiles leave the last wave of CTAs partly idle
-  // (mode 0, a workspace for the partials, at least one 512-deep chunk per
+  // (mode 0, a workspace for the partials, at least two 512-deep chunks per
   // split): the split count with the best fill of whole waves, ties to fewer.
   const int nchunks = (a.ktiles + KCHUNK - 1) / KCHUNK;
   a.ksplit = 1;
   a.cps = nchunks;
   a.part = part;
   a.a64 = (int)a64;
-  if (mode == 0 && part && tiles < 4LL * nsm && nchunks >= 2) {
+  if (mode == 0 && part && tiles < 4LL * nsm && nchunks >= 4) {
     double best = (double)tiles / (double)(nsm * ((tiles + nsm - 1) / nsm));
-    for (int z = 2; z <= std::min(64, nchunks); ++z) {
+    for (int z = 2; z <= 8 && nchunks / z >= 2; ++z) {
       const int cps = (nchunks + z - 1) / z;
       const int zz = (nchunks + cps - 1) / cps;  // no empty split
       if ((long long)zz * M * N > part_elems) break;

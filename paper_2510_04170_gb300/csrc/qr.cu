@@ -2,12 +2,13 @@
 // the right preconditioner R.  Blocked right-looking Householder with the
 // compact-WY trailing update (Schreiber & Van Loan):
 //
-//   k_block     (cooperative) factors a block of up to 128 columns (32 when the
-//               trailing update is in FP64), one exchange between the CTAs per
-//               column.  Reflector H = I - tau v v^T, v_0 = 1,
+//   k_panel     (cooperative) factors 32 columns, one exchange between the CTAs
+//               per column.  Reflector H = I - tau v v^T, v_0 = 1,
 //               beta = -sign(alpha) ||x||.
+//   k_gram, k_panel_t: the panel's V^T V by chunks of rows and its compact-WY
+//               factor T
 //   k_vta       W_z = V^T A_trail over a K-slice z (split K, deterministic)
-//   k_wt        W2 = T^T sum_z W_z, T the panel's compact-WY factor
+//   k_wt        W2 = T^T sum_z W_z
 //   k_update    A_trail -= V W2
 //   k_diag, k_flip, k_floor: rows of R flipped to a positive diagonal, pivots
 //               below 1e-14 max_j R_jj floored (rank guard; flag raised).
@@ -26,448 +27,305 @@ namespace {
 constexpr int NB = 32;
 
 // ---------------------------------------------------------------------------
-// Cooperative block factorisation k_block.
+// Cooperative panel factorisation k_panel (up to 32 columns).
 //
 // GB300's FP64 unit takes 64 cycles (31 ns) for a warp instruction, the same
 // for a dependent chain as for independent ones and for one lane as for 32
 // (measured).  What bounds a column of the factorisation is therefore the
 // number of FP64 warp instructions on one SM partition, plus one exchange
-// between the CTAs; the kernel is laid out to issue few of them:
-//  - 4 warps per CTA, one per SM partition; the lanes of a warp are the 32
-//    columns of the panel, so a row of the panel is one instruction and no
-//    reduction over lanes is needed.  A warp owns every fourth row.
-//  - the columns k < j already hold their reflectors u_k, so the same
-//    instruction that gives x^T a_k for the columns to the right (and
-//    sigma = x^T x in lane j) gives u_k^T x for the columns to the left: the
-//    panel's Gram comes with the reduction and needs no pass of its own.
-//  - H = I - gamma u u^T with the unscaled u = (alpha - beta, x) and
-//    gamma = 1 / (beta (beta - alpha)): the column is scaled once, at the end
-//    of the panel.  sqrt and the reciprocal are one third-order step
-//    (Householder's iteration) from an FP32 seed, 18 instructions where the
-//    library's sqrt and two divisions take 28 (0.86 us).
-//  - a column's reflector is applied to the next column at once and to the others
-//    while the next column's exchange is on its way.  The next column's products
-//    are then taken with a_k still lacking that reflector f_k u, and
-//    x^T (a_k - f_k u) = x^T a_k - f_k x^T u is formed after the sum, x^T u being
-//    the Gram entry in its lane.  The error against ||x|| ||a_k|| is that of the
-//    step before, so the sum of all steps' errors is the same.
-//  - the 32 sums are first combined in clusters of four CTAs (each rank sums
-//    eight columns of the 16 warps, through distributed shared memory and one
-//    cluster barrier, 0.2 us), then between the clusters as 16-byte records
-//    {low, tag, high, tag} whose tag is the column's number: a reader polls the
-//    records themselves, so there is no fence, no counter and no second trip to
-//    L2.  Two slots alternate; a CTA can only be one exchange ahead of another.
-//    (With a record per CTA every CTA read 78 KB per column, which is L2 bound,
-//    and added 38 records per warp.)  Four is the largest cluster that still
-//    puts a CTA on 144 of the 152 SMs (eight: 120).
-// Between the panels of a block, the block's remaining columns (in the same
-// shared-memory slab) are updated with W = V^T A, W2 = T^T W, A -= V W2: CTA c
-// sums column c of W over the CTAs and solves for its column of W2.
+// between the CTAs; the kernel is laid out to issue few of them: the lanes of a
+// warp are the 32 columns of the panel, so a row of the panel is one instruction
+// for the products and one for the update, and no reduction over lanes is needed.
+// Two warps per SM partition keep its FP64 unit busy through each other's loads.
 //
-// Per column at 12,288 rows: 16.5 us with one grid barrier and a redundant
-// butterfly reduction per column (the former panel kernel), then 5.2 us (0.95
-// products, 0.4 cluster barrier, 0.25 publish, 1.7 poll and sums, 1.05 scalars,
-// 0.8 update).  The poll leaves the FP64 pipes idle, so only the next column is
-// updated at once; a reflector's other columns follow while the next column's
-// records are on their way.  A 128-column block with its in-block updates: 3.7
-// -> 0.94 ms, with the deferred updates 0.87 ms.
-constexpr int KB_THREADS = 128;
-constexpr int KB_SMEM = 227 * 1024;              // dynamic shared memory of a CTA
-constexpr long long KB_WIDE_ROWS = 16384;
-constexpr int KB_CL = 4;                         // CTAs of a cluster
-constexpr int KB_MAXP = 256;                     // CTAs of one factorisation
-constexpr int KB_POLL = 10;                      // records in flight per lane and poll round
-constexpr int KB_SLOT = (KB_MAXP / KB_CL + 1) * NB * 2;  // 8-byte words of an exchange slot (last record: the pivot row)
+// The order of every sum is fixed by the row count (and a cap on the chunks), not
+// by how the rows are spread over CTAs, so that R has the same bits on any split:
+// a last bit of R can change the step counts of a solve at cond(R) = 1e9.  The
+// panel's rows are P chunks of `chunk` rows.  A chunk's sum has 32 chains, rows of
+// equal remainder modulo 32, added pairwise at distances 16, 8, 4, 2, 1; chunks q,
+// q + 32, .. are added in turn, and the 32 sums that leaves pairwise at distances
+// 16 .. 1 again.  Spread over the chip:
+//  - a cluster of CL CTAs owns the chunks of one remainder modulo 32 (or, CL =
+//    1, a CTA owns one chunk), and a warp in it 4 / CL chains of each.
+//  - the chains' sums meet in the cluster through distributed shared memory and
+//    one cluster barrier (0.2 us); each rank finishes 32 / CL columns and publishes
+//    them as 16-byte records {low, tag, high, tag} whose tag is the column's
+//    number.  A reader polls the records themselves, so there is no fence, no
+//    counter and no second trip to L2.  Two slots alternate; a CTA can only be one
+//    exchange ahead of another.  (With a record per chunk every CTA reads 78 KB per
+//    column, which is L2 bound.)
+// After the exchange a warp of every CTA forms beta, tau, 1 / (alpha - beta) and
+//     w_k = v^T A_k = A_jk + p_k / (alpha - beta)     (v_j = 1, v_r = x_r / (alpha - beta))
+// with p_k = sum x_r A_rk; the column is scaled, the next column updated with
+// the lanes as rows, and then one pass over the rows updates the other columns
+// and takes the next column's products.
+//
+// Per column at 12,288 rows: 16.5 us with one grid barrier and a butterfly
+// reduction in every warp (the former kernel), now 6.0 (2.5 the pass over the
+// rows, 0.25 cluster barrier, 0.8 trees, 0.8 poll, 1.4 scalars, 0.3 scaling); at
+// 3,072 rows 4.4.  One warp per partition took 3.5 us for the pass.
+constexpr int KP_THREADS = 256;
+constexpr int KP_SMEM = 227 * 1024;  // dynamic shared memory of a CTA
+constexpr int KP_CHUNK = 800;        // most rows of a chunk
+constexpr int KP_MAXP = 256;         // most chunks
+constexpr int KP_SLOT = (KP_MAXP + 1) * NB * 2;  // 8-byte words of an exchange slot (last record: the pivot row)
 
-struct BlockArgs {
+struct PanelArgs {
   double* A;
   long long lda;
   long long s;
   long long j0;
-  int nb;              // columns of the block (<= 128)
-  int P;               // CTAs (a multiple of KB_CL)
-  int chunk;           // rows per CTA
-  unsigned long long* xch;  // [2][KB_SLOT] exchange records
-  double* part;        // [P][3 NB][NB] partial W of the in-block update
-  double* w2;          // [NB][3 NB]
+  int nbw;             // columns in this panel (<= NB)
+  int P;               // chunks
+  int chunk;           // rows of a chunk
+  int kpc;             // rows of a chain in a chunk, at most
+  int U;               // chunks per cluster, at most
+  int NG;              // clusters (and records of an exchange)
+  unsigned long long* xch;  // [2][KP_SLOT] exchange records
   double* tau;         // [n]
-  double* G;           // [NB][NB] of the last panel: G[p * NB + q] = tau_p v_q^T v_p for q < p, else 0
-  unsigned int* bar;   // arrival counter of the grid barriers
-  unsigned int bar0;   // its value before this launch
   unsigned int* err;
 };
 
-constexpr int KB_TRI = NB * (NB - 1) / 2;  // entries q < p of the panel's Gram
-__host__ __device__ constexpr int kb_tri(int p, int q) { return p * (p - 1) / 2 + q; }
-__host__ __device__ constexpr size_t kb_fixed_smem() { return (size_t)(KB_TRI + 13 * NB) * sizeof(double); }
+// Slab element (local row r, column c): rows of 33, so that both a row (lanes =
+// columns) and a column (lanes = rows) are free of bank conflicts.
+constexpr int KP_LD = NB + 1;
+__device__ __forceinline__ int kp_at(int r, int c) { return r * KP_LD + c; }
 
-// Slab element (local row r, column c): 32-column groups with the column index
-// XORed by the row, so that both a row (lanes = columns) and a column (lanes =
-// rows) are free of bank conflicts.
-__device__ __forceinline__ int kb_at(int r, int c, int ld) { return r * ld + (c & ~31) + ((c ^ r) & 31); }
+// x != 0 (true for NaN) without an FP64 instruction.
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 
-// Arrivals of all CTAs up to the count `want` (the counter only grows).
-__device__ __forceinline__ void kb_barrier(unsigned int* bar, unsigned int want, RecWait& kw) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-    unsigned int n = 0;
-    while ((int)(ld_acquire(bar) - want) < 0)
-      if (!kw.spin(n)) break;
-  }
-  __syncthreads();
-}
-
-// x != 0 (true for NaN) without an FP64 compare.
-__device__ __forceinline__ bool kb_nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
-
-// norm = sqrt(alpha^2 + sigma) and gamma = 1 / (norm^2 + |alpha| norm) for
-// sigma > 0.  In the scaled variables m = t 2^-e in [1, 4) (e even), the
-// seeds are FP32 (2^-21) and one step of third order leaves ~2^-63; sqrt gets
-// one Newton correction.  Exponents near the ends of the range (and Inf, NaN)
-// take the library functions.
-__device__ __forceinline__ void kb_norm_gamma(double alpha, double sigma, double& nrm, double& gam) {
-  const double t = fma(alpha, alpha, sigma);
-  const int hi = __double2hiint(t), lo = __double2loint(t);
-  const int ex = ((hi >> 20) & 0x7FF) - 1023;
-  if (ex < -900 || ex > 900 || hi < 0) {
-    nrm = sqrt(t);
-    gam = 1.0 / fma(fabs(alpha), nrm, t);
-    return;
-  }
-  const int e = ex & ~1;
-  const int mh = hi - (e << 20);  // m = t 2^-e
-  const double m = __hiloint2double(mh, lo);
-  // FP32 value of m with its low bits cut off (integer operations only)
-  const float mf = __int_as_float(((mh >> 20) - 1023 + 127) << 23 | (mh & 0xFFFFF) << 3 | (int)((unsigned)lo >> 29));
-  const int yb = __float_as_int(rsqrtf(mf));
-  const double y0 = __hiloint2double((((yb >> 23) - 127 + 1023) << 20) | ((yb & 0x7FFFFF) >> 3), (int)((unsigned)(yb & 7) << 29));
-  const double h = m * y0;
-  const double r = fma(-h, y0, 1.0);
-  const double y = fma(y0, fma(r, 0.375, 0.5) * r, y0);  // 1 / sqrt(m)
-  double q = m * y;                                        // sqrt(m)
-  const double half_y = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));
-  q = fma(fma(-q, q, m), half_y, q);
-  const double back = __hiloint2double((1023 - (e >> 1)) << 20, 0);  // 2^(-e/2)
-  const double d = fma(fabs(alpha) * back, q, m);                    // in [1, 8)
-  const int dh = __double2hiint(d), dl = __double2loint(d);
-  const float df = __int_as_float(((dh >> 20) - 1023 + 127) << 23 | (dh & 0xFFFFF) << 3 | (int)((unsigned)dl >> 29));
-  const int gb = __float_as_int(__frcp_rn(df));
-  const double g0 = __hiloint2double((((gb >> 23) - 127 + 1023) << 20) | ((gb & 0x7FFFFF) >> 3), (int)((unsigned)(gb & 7) << 29));
-  const double w = fma(-d, g0, 1.0);
-  const double g = fma(g0, fma(w, w, w), g0);  // 1 / d
-  nrm = __hiloint2double(__double2hiint(q) + ((e >> 1) << 20), __double2loint(q));
-  gam = __hiloint2double(__double2hiint(g) - (e << 20), __double2loint(g));
-}
-
-__device__ __forceinline__ void kb_copy8(double* dst, const double* src) {
+__device__ __forceinline__ void kp_copy8(double* dst, const double* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
 
-// In-block W = V^T A of a CTA's rows: lanes are the columns of a group, warp w
-// takes p = 8 w .. 8 w + 7, NG groups of columns follow the panel at p0.
-template <int NG>
-__device__ __forceinline__ void kb_wpart(const double* sl, int ld, int p0, int r0, int nr, int w, int lane,
-                                         double* out) {
-  double acc[NG][8];
-#pragma unroll
-  for (int g = 0; g < NG; ++g)
-#pragma unroll
-    for (int p = 0; p < 8; ++p) acc[g][p] = 0.0;
-#pragma unroll 2
-  for (int r = r0; r < nr; ++r) {
-    double av[NG], v[8];
-#pragma unroll
-    for (int g = 0; g < NG; ++g) av[g] = sl[kb_at(r, p0 + NB * (g + 1) + lane, ld)];
-#pragma unroll
-    for (int p = 0; p < 8; ++p) v[p] = sl[kb_at(r, p0 + 8 * w + p, ld)];
-#pragma unroll
-    for (int p = 0; p < 8; ++p)
-#pragma unroll
-      for (int g = 0; g < NG; ++g) acc[g][p] = fma(v[p], av[g], acc[g][p]);
-  }
-#pragma unroll
-  for (int g = 0; g < NG; ++g)
-#pragma unroll
-    for (int p = 0; p < 8; p += 2)
-      __stcg(reinterpret_cast<double2*>(out + (g * NB + lane) * NB + 8 * w + p),
-             make_double2(acc[g][p], acc[g][p + 1]));
+// Doubles of shared memory beside the slab: the chains' sums of this rank's columns
+// [U][32][32 / CL], their sums over a chunk [U][32 / CL], the warps' shares [8][32],
+// the columns' factors and three scalars [36], the chains' lengths [32 / CL][U].
+constexpr long long kp_fixed(int CL, int U) {
+  return (long long)U * (NB + 1) * (NB / CL) + 8 * NB + 36 + (NB / CL * U + 1) / 2;
 }
+// Rows of the slab.
+constexpr long long kp_slab_rows(int CL, int U, int kpc) { return (long long)U * (NB / CL) * kpc; }
 
-// In-block A -= V W2 of a CTA's rows for the column group at pc: a lane keeps
-// its column of W2.
-__device__ __forceinline__ void kb_wupdate(double* sl, int ld, int p0, int pc, int r0, int nr, int w, int lane,
-                                           const double* w2) {
-  double y[NB];
-#pragma unroll
-  for (int p = 0; p < NB; ++p) y[p] = __ldcg(w2 + p * (3 * NB) + lane);
-  for (int r = r0 + ((w - r0) & 3); r < nr; r += 4) {
-    double* e = sl + kb_at(r, pc + lane, ld);
-    const double* v = sl + r * ld + p0;
-    // summed by itself and subtracted once: 32 roundings at the size of the sum, not of A
-    double x = 0.0;
-#pragma unroll
-    for (int p = 0; p < NB; ++p) x = fma(v[(p ^ r) & 31], y[p], x);
-    *e -= x;
-  }
-}
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
 
-// A_rk -= f_k u_r for this warp's rows r >= r0 of the panel at p0, u its column jj,
-// f the lanes' factors (0 up to column jj + 1, which is up to date).
-__device__ __forceinline__ void kb_apply(double* sl, int ld, int p0, int jj, double f, int r0, int nr, int w,
-                                         int lane) {
-  const int rw = r0 + ((w - r0) & 3);
-  if (jj < 15) {
-    if (rw < nr) {
-      const int last = nr - 1 - ((nr - 1 - rw) & 3);
-      double x = sl[kb_at(rw, p0 + jj, ld)], e = sl[kb_at(rw, p0 + lane, ld)];
-#pragma unroll 4
-      for (int r = rw; r < last; r += 4) {
-        const double xn = sl[kb_at(r + 4, p0 + jj, ld)], en = sl[kb_at(r + 4, p0 + lane, ld)];
-        sl[kb_at(r, p0 + lane, ld)] = fma(-f, x, e);
-        x = xn;
-        e = en;
-      }
-      sl[kb_at(last, p0 + lane, ld)] = fma(-f, x, e);
-    }
-  } else {
-    // only columns 17 .. 31 are left: two rows per instruction
-    const int ch = 16 + (lane & 15);
-    const double fh = __shfl_sync(0xffffffffu, f, ch);
-    int r = rw + 4 * (lane >> 4);
-    for (; r + 24 < nr; r += 32) {
-      double x[4], e[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        x[u] = sl[kb_at(r + 8 * u, p0 + jj, ld)];
-        e[u] = sl[kb_at(r + 8 * u, p0 + ch, ld)];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        e[u] = fma(-fh, x[u], e[u]);
-        if (ch > jj + 1) sl[kb_at(r + 8 * u, p0 + ch, ld)] = e[u];
-      }
-    }
-    for (; r < nr; r += 8) {
-      double* e = sl + kb_at(r, p0 + ch, ld);
-      const double x = fma(-fh, sl[kb_at(r, p0 + jj, ld)], *e);
-      if (ch > jj + 1) *e = x;
-    }
-  }
-  __syncwarp();
-}
-
-__global__ void __cluster_dims__(KB_CL, 1, 1) __launch_bounds__(KB_THREADS, 1) k_block(BlockArgs a) {
-  if (!in_cluster(KB_CL, a.err)) return;
-  extern __shared__ __align__(16) double kb_sm[];
-  double* Gs = kb_sm;              // tau_p v_q^T v_p of the panel at kb_tri(p, q), q < p
-  double* wp = Gs + KB_TRI;        // [4][4][8] partial sums of this rank's 8 columns, by CTA and warp of the cluster
-  double* rs = wp + 4 * NB;        // [4][NB] the warps' shares of the sums over CTAs
-  double* pv = rs + 4 * NB;        // [NB] pivot row
-  double* dab = pv + NB;           // [NB] alpha - beta
-  double* gam = dab + NB;          // [NB] gamma
-  double* scl = gam + NB;          // [NB] 1 / (alpha - beta)
-  double* taus = scl + NB;         // [NB]
-  double* sl = kb_sm + (kb_fixed_smem() / sizeof(double));  // slab [rows][ld]
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(KP_THREADS, 1) k_panel(PanelArgs a) {
+  if (!in_cluster(CL, a.err)) return;
+  constexpr int NC = NB / CL, NS = NC / 8, OC = NB / CL;  // chains per CTA and per warp, columns per rank
+  extern __shared__ __align__(16) double kp_sm[];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int c = blockIdx.x, P = a.P;
-  const int rank = c % KB_CL, cl = c / KB_CL, ncl = P / KB_CL;
-  const long long rbeg = a.j0 + (long long)c * a.chunk;
-  const long long rend = min(a.s, rbeg + a.chunk);
-  const int nr = rbeg < rend ? (int)(rend - rbeg) : 0;
-  const int np = (a.nb + NB - 1) / NB, ld = np * NB;
-  RecWait kw(a.err, tid);
-  unsigned int barrier = a.bar0;
-  for (int cc = w; cc < ld; cc += 4) {
-    const double* col = a.A + (size_t)(a.j0 + cc) * a.lda + rbeg;
-    for (int r = lane; r < nr; r += 32) {
-      if (cc < a.nb) kb_copy8(sl + kb_at(r, cc, ld), col + r);
-      else sl[kb_at(r, cc, ld)] = 0.0;
+  const int rank = blockIdx.x % CL, g = blockIdx.x / CL, U = a.U, kpc = a.kpc, NG = a.NG;
+  double* wp = kp_sm;               // [U][32][OC]
+  double* gs = wp + U * NB * OC;    // [U][OC]
+  double* rs = gs + U * OC;         // [8][NB]
+  double* fs = rs + 8 * NB;         // [NB] factors, then tau, 1 / (alpha - beta), beta
+  int* kns = reinterpret_cast<int*>(fs + 36);      // [NC][U]
+  double* sl = fs + 36 + (NC * U + 1) / 2;         // slab
+  // rows of this cluster's chunk u
+  auto rows_of = [&](int u) {
+    const int q = g + 32 * u;
+    const long long beg = a.j0 + (long long)q * a.chunk;
+    return q < a.P && beg < a.s ? (int)min((long long)a.chunk, a.s - beg) : 0;
+  };
+  // Row c + 32 k of chunk u with c = rank NC + cin: warp cin & 7, slab row (cin U + u) kpc + k
+  for (int idx = lane; idx < U * NC * kpc; idx += 32) {
+    const int cin = idx % NC, rest = idx / NC, k = rest % kpc, u = rest / kpc;
+    const int r = rank * NC + cin + 32 * k, row = (cin * U + u) * kpc + k;
+    const bool in = r < rows_of(u);
+    const double* src = a.A + a.j0 + (long long)(g + 32 * u) * a.chunk + r;
+    for (int cc = w; cc < NB; cc += 8) {
+      if (in && cc < a.nbw) kp_copy8(sl + kp_at(row, cc), src + (size_t)(a.j0 + cc) * a.lda);
+      else sl[kp_at(row, cc)] = 0.0;
     }
   }
+  for (int i = tid; i < NC * U; i += KP_THREADS) kns[i] = max(0, rows_of(i % U) - rank * NC - i / U + 31) >> 5;
   asm volatile("cp.async.wait_all;" ::: "memory");
-  cluster_arrive();
-  cluster_wait();  // all ranks run: their shared memory may be written
-  for (int pi = 0; pi < np; ++pi) {
-    const int p0 = pi * NB, nbw = min(NB, a.nb - p0);
-    double fprev = 0.0;  // factors of the previous column's reflector that columns past jj still lack
-    for (int jj = 0; jj < nbw; ++jj) {
-      const long long j = a.j0 + p0 + jj;  // pivot row and column
-      const unsigned int tag = (unsigned int)(j + 1);
-      unsigned long long* slot = a.xch + (size_t)(jj & 1) * KB_SLOT;
-      const int lr = j + 1 > rbeg ? (int)min((long long)nr, j + 1 - rbeg) : 0;  // rows below the pivot
-      const int rw = lr + ((w - lr) & 3);                                       // this warp's first one
-      double acc = 0.0;
-      if (rw < nr) {  // the next row's loads go ahead of a row's instruction
-        const int last = nr - 1 - ((nr - 1 - rw) & 3);
-        double x = sl[kb_at(rw, p0 + jj, ld)], e = sl[kb_at(rw, p0 + lane, ld)];
-#pragma unroll 4
-        for (int r = rw; r < last; r += 4) {
-          const double xn = sl[kb_at(r + 4, p0 + jj, ld)], en = sl[kb_at(r + 4, p0 + lane, ld)];
-          acc = fma(x, e, acc);
-          x = xn;
-          e = en;
+  RecWait kw(a.err, tid);
+  __syncthreads();
+  if (CL > 1) {
+    cluster_arrive();
+    cluster_wait();  // all ranks run: their shared memory may be written
+  }
+  // slab row of the panel's row j (a pivot: first of its chain in chunk 0) if this warp owns it, else -1
+  auto pivot_row = [&](int j) {
+    const int cin = j - rank * NC;
+    return g == 0 && cin >= 0 && cin < NC && (cin & 7) == w ? cin * U * kpc : -1;
+  };
+  // Rows below the pivot jj - 1: with `upd`, A_rk -= f_k v_r for the columns past
+  // jj, v the column jj - 1; then this warp's chains of x^T A_k over the rows below
+  // jj, x the column jj, to the rank that adds them up.
+  auto pass = [&](int jj, bool upd, double f) {
+#pragma unroll
+    for (int sub = 0; sub < NS; ++sub)
+      for (int u = 0; u < U; ++u) {
+        const int cin = w + 8 * sub, c = rank * NC + cin, row0 = (cin * U + u) * kpc;
+        const int kn = kns[cin * U + u];
+        double acc = 0.0;
+        int k = 0;
+        if (g == 0 && u == 0 && c <= jj && kn > 0) {  // rows up to the pivots lead the chains of chunk 0
+          if (c == jj && upd) {
+            const double v = sl[kp_at(row0, jj - 1)], e = sl[kp_at(row0, lane)];
+            if (lane > jj) sl[kp_at(row0, lane)] = fma(-v, f, e);
+          }
+          k = 1;
         }
-        acc = fma(x, e, acc);
+        // batches of rows: their loads first, as no load moves above a store to the slab
+        auto batch = [&](auto count) {
+          constexpr int N = decltype(count)::value;
+          double x[N], e[N], v[N];
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            if (upd) v[i] = sl[kp_at(row0 + k + i, jj - 1)];
+            x[i] = sl[kp_at(row0 + k + i, jj)];
+            e[i] = sl[kp_at(row0 + k + i, lane)];
+          }
+          if (upd) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+              const double t = fma(-v[i], f, e[i]);
+              e[i] = lane > jj ? t : e[i];
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < N; ++i) acc = fma(x[i], e[i], acc);
+          if (upd) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) sl[kp_at(row0 + k + i, lane)] = e[i];
+          }
+          k += N;
+        };
+        while (k + 4 <= kn) batch(Int<4>{});
+        const int left = kn - k;
+        if (left == 3) batch(Int<3>{});
+        else if (left == 2) batch(Int<2>{});
+        else if (left == 1) batch(Int<1>{});
+        double* dst = wp + (u * NB + c) * OC + lane % OC;
+        if (CL > 1) st_cluster(dst, lane / OC, acc);
+        else *dst = acc;
       }
-      st_cluster(wp + (rank * 4 + w) * 8 + (lane & 7), lane >> 3, acc);
+  };
+  pass(0, false, 0.0);
+  for (int jj = 0; jj < a.nbw; ++jj) {
+    const unsigned int tag = (unsigned int)(a.j0 + jj + 1);
+    unsigned long long* slot = a.xch + (size_t)(jj & 1) * KP_SLOT;
+    const int prow = pivot_row(jj);
+    if (prow >= 0) {
+      __syncwarp();
+      rec_publish(slot + ((size_t)NG * NB + lane) * 2, sl[kp_at(prow, lane)], tag);
+    }
+    if (CL > 1) {
       cluster_arrive();
       cluster_wait();
-      if (w == 0) {
-        const double* x = wp + (lane >> 3) * 32 + (lane & 7);
-        double sm = (x[0] + x[8]) + (x[16] + x[24]);
-        sm += __shfl_xor_sync(0xffffffffu, sm, 8);
-        sm += __shfl_xor_sync(0xffffffffu, sm, 16);
-        if (lane < 8) rec_publish(slot + ((size_t)cl * NB + rank * 8 + lane) * 2, sm, tag);
-      } else if (w == 1 && j >= rbeg && j < rend) {
-        const int r = (int)(j - rbeg);
-        double v = sl[kb_at(r, p0 + lane, ld)];
-        if (jj > 0) v = fma(-fprev, sl[kb_at(r, p0 + jj - 1, ld)], v);
-        rec_publish(slot + ((size_t)ncl * NB + lane) * 2, v, tag);
-      }
-      // meanwhile the previous column's reflector on the columns past jj
-      if (jj > 0) {
-        if (j >= rbeg && j < rend) __syncthreads();  // warp 1 has read the pivot row
-        kb_apply(sl, ld, p0, jj - 1, fprev, j > rbeg ? (int)min((long long)nr, j - rbeg) : 0, nr, w, lane);
-      }
-      // sum over the clusters, warp w the clusters w, w + 4, ... in increasing
-      // order; record ncl is the pivot row.  A complete record of this cluster
-      // also says that all its ranks have read wp.
-      double sum = 0.0;
-      for (int q0 = w; q0 <= ncl; q0 += 4 * KB_POLL) {
-        unsigned long long lo[KB_POLL], hi[KB_POLL];
-        unsigned int spins = 0;
-        for (;;) {
-          bool all = true;
-#pragma unroll
-          for (int i = 0; i < KB_POLL; ++i)
-            if (q0 + 4 * i <= ncl) rec_load(slot + ((size_t)(q0 + 4 * i) * NB + lane) * 2, lo[i], hi[i]);
-#pragma unroll
-          for (int i = 0; i < KB_POLL; ++i)
-            if (q0 + 4 * i <= ncl) all = all && rec_ready(lo[i], hi[i], tag);
-          if (__all_sync(0xffffffffu, all) || !__all_sync(0xffffffffu, kw.spin(spins))) break;
-        }
-#pragma unroll
-        for (int i = 0; i < KB_POLL; ++i) {
-          const int q = q0 + 4 * i;
-          if (q < ncl) sum += rec_value(lo[i], hi[i]);
-          else if (q == ncl) pv[lane] = rec_value(lo[i], hi[i]);
-        }
-      }
-      rs[w * NB + lane] = sum;
+    } else {
       __syncthreads();
-      double tot = (rs[lane] + rs[NB + lane]) + (rs[2 * NB + lane] + rs[3 * NB + lane]);
-      if (jj > 0) tot = fma(-fprev, __shfl_sync(0xffffffffu, tot, jj - 1), tot);
-      const double piv = pv[lane];
-      const double alpha = pv[jj];
-      const double sigma = __shfl_sync(0xffffffffu, tot, jj);
-      double dj = 0.0, gj = 0.0, beta = alpha;
-      if (kb_nonzero(sigma)) {
-        double nrm;
-        kb_norm_gamma(alpha, sigma, nrm, gj);
-        beta = __double2hiint(alpha) < 0 && kb_nonzero(alpha) ? nrm : -nrm;
-        dj = alpha - beta;
+    }
+    // a chunk's tree over its 32 chains, eight columns a warp (lane = 4 column +
+    // part), then the sum over the cluster's chunks
+    for (int task = w; task < U * (OC / 8); task += 8) {
+      const int u = task / (OC / 8), col = task % (OC / 8) * 8 + (lane >> 2);
+      const double* x = wp + (u * NB + (lane & 3)) * OC + col;
+      double t = ((x[0] + x[16 * OC]) + (x[8 * OC] + x[24 * OC])) +
+                 ((x[4 * OC] + x[20 * OC]) + (x[12 * OC] + x[28 * OC]));
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      if ((lane & 3) == 0) {
+        if (U == 1) rec_publish(slot + ((size_t)g * NB + rank * OC + col) * 2, t, tag);
+        else gs[u * OC + col] = t;
       }
-      // u^T a_k for the columns to the right, u_k^T u for those to the left
-      const double wk = fma(dj, piv, tot);
-      const double f = lane > jj ? gj * wk : 0.0;
-      if (w == 0) {
-        if (lane < jj) Gs[kb_tri(jj, lane)] = wk;
-        if (lane == jj) {
-          dab[jj] = dj;
-          gam[jj] = gj;
-        }
-      }
-      // the next column only (lanes are rows); the others wait for the next exchange
-      if (jj + 1 < NB) {
-        const double f1 = __shfl_sync(0xffffffffu, f, jj + 1);
-        for (int r = rw + 4 * lane; r < nr; r += 128) {
-          double* e = sl + kb_at(r, p0 + jj + 1, ld);
-          *e = fma(-f1, sl[kb_at(r, p0 + jj, ld)], *e);
-        }
-      }
-      fprev = lane > jj + 1 ? f : 0.0;
-      if (j >= rbeg && j < rend && w == ((int)(j - rbeg) & 3)) {  // the pivot row itself
-        double* e = sl + kb_at((int)(j - rbeg), p0 + lane, ld);
-        if (lane > jj) *e = fma(-f, dj, *e);
-        if (lane == jj) *e = beta;
+    }
+    if (U > 1) {
+      __syncthreads();
+      if (tid < OC) {
+        double t = gs[tid];
+        for (int u = 1; u < U; ++u) t += gs[u * OC + tid];
+        rec_publish(slot + ((size_t)g * NB + rank * OC + tid) * 2, t, tag);
       }
       __syncwarp();
     }
+    // Sum over the clusters, warp w the remainders w, w + 8, .. modulo 32; warp 0
+    // also reads the pivot row (record NG).  A complete record of this cluster
+    // says that all its ranks have read wp.
+    double s[4] = {0.0, 0.0, 0.0, 0.0}, piv = 0.0;
+    for (int q0 = w; q0 < NG; q0 += 32) {
+      unsigned long long lo[5], hi[5];
+      unsigned int spins = 0;
+      for (;;) {
+        bool all = true;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (q0 + 8 * i < NG) rec_load(slot + ((size_t)(q0 + 8 * i) * NB + lane) * 2, lo[i], hi[i]);
+        if (w == 0) rec_load(slot + ((size_t)NG * NB + lane) * 2, lo[4], hi[4]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (q0 + 8 * i < NG) all = all && rec_ready(lo[i], hi[i], tag);
+        if (w == 0) all = all && rec_ready(lo[4], hi[4], tag);
+        if (__all_sync(0xffffffffu, all) || !__all_sync(0xffffffffu, kw.spin(spins))) break;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (q0 + 8 * i < NG) s[i] += rec_value(lo[i], hi[i]);
+      if (w == 0) piv = rec_value(lo[4], hi[4]);
+    }
+    rs[w * NB + lane] = (s[0] + s[2]) + (s[1] + s[3]);
     __syncthreads();
     if (w == 0) {
-      const double d = lane < nbw ? dab[lane] : 0.0;
-      const bool on = d != 0.0;
-      scl[lane] = on ? 1.0 / d : 0.0;
-      taus[lane] = on ? gam[lane] * (d * d) : 0.0;
-      if (c == 0 && lane < nbw) a.tau[a.j0 + p0 + lane] = taus[lane];
+      const double* x = rs + lane;
+      const double tot = ((x[0] + x[4 * NB]) + (x[2 * NB] + x[6 * NB])) + ((x[NB] + x[5 * NB]) + (x[3 * NB] + x[7 * NB]));
+      const double alpha = __shfl_sync(0xffffffffu, piv, jj), sigma = __shfl_sync(0xffffffffu, tot, jj);
+      double tau = 0.0, beta = alpha, scale = 0.0;
+      if (nonzero(sigma)) {
+        const double nrm = sqrt(alpha * alpha + sigma);
+        beta = __double2hiint(alpha) < 0 && nonzero(alpha) ? nrm : -nrm;
+        // lane 0 (beta - alpha) / beta, the others 1 / (alpha - beta), in one division
+        const double d = alpha - beta;
+        const double t = (lane == 0 ? -d : 1.0) / (lane == 0 ? beta : d);
+        tau = __shfl_sync(0xffffffffu, t, 0);
+        scale = __shfl_sync(0xffffffffu, t, 1);
+      }
+      fs[lane] = tau * (piv + scale * tot);  // tau w_k
+      if (lane < 3) fs[NB + lane] = lane == 0 ? tau : lane == 1 ? scale : beta;
+      if (blockIdx.x == 0 && lane == 0) a.tau[a.j0 + jj] = tau;
     }
     __syncthreads();
-    for (int idx = tid; idx < NB * NB; idx += KB_THREADS) {
-      const int p = idx / NB, q = idx % NB;
-      double g = 0.0;
-      if (q < p && p < nbw) {
-        g = Gs[kb_tri(p, q)] * scl[q] * scl[p] * taus[p];
-        Gs[kb_tri(p, q)] = g;
-      }
-      if (c == 0) a.G[idx] = g;
-    }
-    // R on and above the diagonal and v below to global memory; the slab keeps
-    // v with its unit diagonal and zeros above
-    for (int cc = w; cc < nbw; cc += 4) {
-      const long long pr = a.j0 + p0 + cc;  // this column's pivot row
-      double* col = a.A + (size_t)pr * a.lda + rbeg;
-      const double sc = scl[cc];
-      for (int r = lane; r < nr; r += 32) {
-        double* e = sl + kb_at(r, p0 + cc, ld);
-        const long long gr = rbeg + r;
-        const double v = gr > pr ? *e * sc : *e;
-        col[r] = v;
-        *e = gr > pr ? v : (gr == pr ? 1.0 : 0.0);
-      }
-    }
-    __syncthreads();
-    const int ng = np - 1 - pi;  // column groups to the right in the block
-    if (ng == 0) break;  // the last cluster barrier came after the last remote store
-    const long long first = a.j0 + p0;
-    const int lv = first > rbeg ? (int)min((long long)nr, first - rbeg) : 0;  // rows before are zero in V
-    if (ng == 3) kb_wpart<3>(sl, ld, p0, lv, nr, w, lane, a.part + (size_t)c * 3 * NB * NB);
-    else if (ng == 2) kb_wpart<2>(sl, ld, p0, lv, nr, w, lane, a.part + (size_t)c * 3 * NB * NB);
-    else kb_wpart<1>(sl, ld, p0, lv, nr, w, lane, a.part + (size_t)c * 3 * NB * NB);
-    barrier += P;
-    kb_barrier(a.bar, barrier, kw);
-    for (int col = c; col < ng * NB; col += P) {
-      double sum = 0.0;
-      for (int q0 = w; q0 < P; q0 += 4 * KB_POLL) {
-        double t[KB_POLL];
+    const double f = fs[lane], scale = fs[NB + 1];
+    const bool upd = nonzero(fs[NB]);
+    if (upd) {
+      // v_r = x_r / (alpha - beta) below the pivot, and the next column (lanes are rows)
+      const double f1 = fs[(jj + 1) & 31];
 #pragma unroll
-        for (int i = 0; i < KB_POLL; ++i) {
-          const int q = q0 + 4 * i;
-          t[i] = q < P ? __ldcg(a.part + ((size_t)q * 3 * NB + col) * NB + lane) : 0.0;
+      for (int sub = 0; sub < NS; ++sub) {
+        const int cin = w + 8 * sub;
+        for (int i = lane; i < U * kpc; i += 32) {
+          const int row = cin * U * kpc + i;
+          if (g == 0 && i == 0 && rank * NC + cin <= jj) continue;
+          const double v = sl[kp_at(row, jj)] * scale;
+          sl[kp_at(row, jj)] = v;
+          if (jj + 1 < NB) sl[kp_at(row, jj + 1)] = fma(-v, f1, sl[kp_at(row, jj + 1)]);
         }
-#pragma unroll
-        for (int i = 0; i < KB_POLL; ++i)
-          if (q0 + 4 * i < P) sum += t[i];
       }
-      rs[w * NB + lane] = sum;
-      __syncthreads();
-      if (w == 0) {
-        // W2 = T^T W from T^-1 = diag(1 / tau) + strict upper part of V^T V:
-        // y_p = tau_p w_p - sum_{q<p} (tau_p v_q^T v_p) y_q
-        double x = ((rs[lane] + rs[NB + lane]) + (rs[2 * NB + lane] + rs[3 * NB + lane])) * taus[lane];
-        for (int q = 0; q < nbw; ++q) {
-          const double y = __shfl_sync(0xffffffffu, x, q);
-          if (lane > q && lane < nbw) x = fma(-Gs[kb_tri(lane, q)], y, x);
-        }
-        __stcg(a.w2 + lane * (3 * NB) + col, x);
-      }
-      __syncthreads();
     }
-    barrier += P;
-    kb_barrier(a.bar, barrier, kw);
-    for (int g = 0; g < ng; ++g) kb_wupdate(sl, ld, p0, p0 + NB * (g + 1), lv, nr, w, lane, a.w2 + g * NB);
-    __syncthreads();
+    if (prow >= 0) {
+      double* e = sl + kp_at(prow, lane);
+      if (lane > jj && upd) *e -= f;
+      if (lane == jj) *e = fs[NB + 2];
+    }
+    __syncwarp();
+    if (jj + 1 < a.nbw) pass(jj + 1, upd, f);
+  }
+  __syncthreads();
+  // R on and above the diagonal and v below back to global memory (the last
+  // cluster barrier came after the last remote store)
+  for (int idx = lane; idx < U * NC * kpc; idx += 32) {
+    const int cin = idx % NC, rest = idx / NC, k = rest % kpc, u = rest / kpc;
+    const int r = rank * NC + cin + 32 * k, row = (cin * U + u) * kpc + k;
+    if (r >= rows_of(u)) continue;
+    double* dst = a.A + a.j0 + (long long)(g + 32 * u) * a.chunk + r;
+    for (int cc = w; cc < a.nbw; cc += 8) dst[(size_t)(a.j0 + cc) * a.lda] = sl[kp_at(row, cc)];
   }
 }
 
@@ -479,26 +337,123 @@ __device__ __forceinline__ double vval(const double* A, long long lda, long long
   return A[(size_t)(j0 + p) * lda + gr];
 }
 
-// Wp[z][col][p] = sum_{r in K-slice z} v_p(r) A[r, j1 + col]
-__global__ void __launch_bounds__(256) k_vta(const double* __restrict__ A, long long lda, long long s, long long j0,
-                                             int nbw, long long j1, long long nt, long long kchunk,
-                                             double* __restrict__ Wp) {
-  __shared__ double Vs[32][NB + 1];
-  __shared__ double As[32][64 + 1];
+// Strict upper part of the panel's V^T V over the rows of each chunk, one
+// thread per two entries, the rows in turn: gram[chunk][KG_LD], entry (p, q) at
+// kg_at(p, q).
+constexpr int KG_LD = 512;
+__host__ __device__ constexpr int kg_at(int p, int q) { return q * (q - 1) / 2 + p; }  // p < q
+constexpr int KG_ROWS = 64;  // rows staged at a time
+
+__global__ void __launch_bounds__(256) k_gram(const double* __restrict__ A, long long lda, long long s, long long j0,
+                                              int nbw, int chunk, double* __restrict__ gram) {
+  __shared__ double Vs[KG_ROWS][NB + 1];
   const int tid = threadIdx.x;
-  const long long col0 = (long long)blockIdx.x * 64;
+  const long long beg = j0 + (long long)blockIdx.x * chunk, end = min(s, beg + chunk);
+  int p[2], q[2];
+  double acc[2] = {0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int e = tid + 256 * i;
+    q[i] = 1;
+    while (q[i] < NB - 1 && kg_at(0, q[i] + 1) <= e) ++q[i];
+    p[i] = min(e - kg_at(0, q[i]), NB - 1);
+  }
+  for (long long r0 = beg; r0 < end; r0 += KG_ROWS) {
+    for (int idx = tid; idx < KG_ROWS * NB; idx += 256) {
+      const int rr = idx & (KG_ROWS - 1), c = idx / KG_ROWS;
+      const long long gr = r0 + rr;
+      Vs[rr][c] = gr < end && c < nbw ? vval(A, lda, j0, c, gr) : 0.0;
+    }
+    __syncthreads();
+    const int nr = (int)min((long long)KG_ROWS, end - r0);
+#pragma unroll 4
+    for (int r = 0; r < nr; ++r)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) acc[i] = fma(Vs[r][p[i]], Vs[r][q[i]], acc[i]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (tid + 256 * i < NB * (NB - 1) / 2) gram[(size_t)blockIdx.x * KG_LD + tid + 256 * i] = acc[i];
+}
+
+// The panel's compact-WY factor T (row-major [NB][NB]) from the chunks' sums and
+// tau: T_jj = tau_j, T_ij = -tau_j sum_{i <= l < j} T_il G_lj.  Eight CTAs of a
+// cluster add the chunks (a thread per entry, 64 to a CTA, the chunks in turn);
+// then a warp takes the rows i and 31 - i of T, lanes = columns, each step one
+// product and one multiply-add for all columns to the right.  On one CTA the
+// sums alone would take 20 us at 152 chunks.
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64) k_panel_t(const double* __restrict__ gram, int P,
+                                                                           const double* __restrict__ tau, int nbw,
+                                                                           double* __restrict__ G,
+                                                                           double* __restrict__ T) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int e = blockIdx.x * 64 + tid;
+  double sum = 0.0;
+  for (int q0 = 0; q0 < P; q0 += 32) {
+    double t[32];
+#pragma unroll
+    for (int u = 0; u < 32; ++u) t[u] = q0 + u < P ? __ldcg(gram + (size_t)(q0 + u) * KG_LD + e) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 32; ++u)
+      if (q0 + u < P) sum += t[u];
+  }
+  __stcg(G + e, sum);
+  __threadfence();
+  cluster_arrive();
+  cluster_wait();
+  double g[NB];  // column `lane` of G above the diagonal
+#pragma unroll
+  for (int l = 0; l < NB; ++l) g[l] = l < lane ? __ldcg(G + kg_at(l, lane)) : 0.0;
+  const double tj = lane < nbw ? tau[lane] : 0.0;
+  const int wi = blockIdx.x * 2 + (tid >> 5);
+  for (int half = 0; half < 2; ++half) {
+    const int i = half == 0 ? wi : NB - 1 - wi;
+    double v = 0.0, row = 0.0;  // row: T_i,lane
+#pragma unroll
+    for (int l = 0; l < NB; ++l) {
+      if (l < i) continue;  // warp-uniform
+      if (lane == l) row = l == i ? tj : -tj * v;
+      const double til = __shfl_sync(0xffffffffu, row, l);
+      if (lane > l) v = fma(til, g[l], v);
+    }
+    T[i * NB + lane] = i < nbw && lane < nbw ? row : 0.0;
+  }
+}
+
+// Wp[z][col][p] = sum_{r in K-slice z} v_p(r) A[r, j1 + col], in tiles of TC
+// columns.  Every output is one chain over the slice's rows whatever the tile;
+// narrow tiles spread the work over the SMs (n = 1,024, 3,072 rows: 31 launches
+// 5.5 -> 3.2 ms; at most 96 columns of 12,288 rows: 148 -> 71 us each).
+template <int TC>
+__host__ __device__ constexpr int vta_threads() { return TC >= 32 ? 256 : 128; }
+
+template <int TC>
+__global__ void __launch_bounds__(vta_threads<TC>()) k_vta(const double* __restrict__ A, long long lda, long long s,
+                                                           long long j0, int nbw, long long j1, long long nt,
+                                                           long long kchunk, double* __restrict__ Wp) {
+  // threads over columns (CX) and reflectors (AY), NQ columns and NA reflectors each
+  constexpr int NT = vta_threads<TC>(), NQ = TC >= 16 ? 4 : 2, CX = TC / NQ, AY = NT / CX, NA = NB / AY;
+  __shared__ double Vs[32][NB + 1];
+  __shared__ double As[32][TC + 1];
+  const int tid = threadIdx.x;
+  const long long col0 = (long long)blockIdx.x * TC;
   const int z = blockIdx.y;
   const long long kb = j0 + (long long)z * kchunk;
   const long long ke = min(s, kb + kchunk);
-  const int ay = tid >> 4, cx = tid & 15;
-  double acc[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+  const int ay = tid / CX, cx = tid % CX;
+  double acc[NA][NQ];
+#pragma unroll
+  for (int h = 0; h < NA; ++h)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[h][q] = 0.0;
   for (long long r0 = kb; r0 < ke; r0 += 32) {
-    for (int idx = tid; idx < 32 * NB; idx += 256) {
+    for (int idx = tid; idx < 32 * NB; idx += NT) {
       const int rr = idx & 31, p = idx >> 5;
       const long long gr = r0 + rr;
       Vs[rr][p] = (gr < ke && p < nbw) ? vval(A, lda, j0, p, gr) : 0.0;
     }
-    for (int idx = tid; idx < 32 * 64; idx += 256) {
+    for (int idx = tid; idx < 32 * TC; idx += NT) {
       const int rr = idx & 31, cc = idx >> 5;
       const long long gr = r0 + rr, gc = col0 + cc;
       As[rr][cc] = (gr < ke && gc < nt) ? A[(size_t)(j1 + gc) * lda + gr] : 0.0;
@@ -506,33 +461,32 @@ __global__ void __launch_bounds__(256) k_vta(const double* __restrict__ A, long 
     __syncthreads();
 #pragma unroll 4
     for (int rr = 0; rr < 32; ++rr) {
-      const double v0 = Vs[rr][ay], v1 = Vs[rr][ay + 16];
+      double v[NA];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double av = As[rr][cx + 16 * q];
-        acc[0][q] += v0 * av;
-        acc[1][q] += v1 * av;
+      for (int h = 0; h < NA; ++h) v[h] = Vs[rr][ay + AY * h];
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const double av = As[rr][cx + CX * q];
+#pragma unroll
+        for (int h = 0; h < NA; ++h) acc[h][q] += v[h] * av;
       }
     }
     __syncthreads();
   }
-  for (int h = 0; h < 2; ++h)
-    for (int q = 0; q < 4; ++q) {
-      const long long gc = col0 + cx + 16 * q;
-      const int p = ay + 16 * h;
+  for (int h = 0; h < NA; ++h)
+    for (int q = 0; q < NQ; ++q) {
+      const long long gc = col0 + cx + CX * q;
+      const int p = ay + AY * h;
       if (gc < nt) Wp[((size_t)z * nt + gc) * NB + p] = acc[h][q];
     }
 }
 
-// W2 = T^T sum_z Wp[z], one warp per column, lanes = p.  T is not formed: with
-// T^-1 = diag(1 / tau) + strict upper part of V^T V the column is a forward
-// substitution, y_p = tau_p w_p - sum_{q<p} G_pq y_q with G_pq = tau_p v_q^T v_p.
-// Both the sum over z and the substitution are chains of FP64 instructions of
-// 31 ns; one column per warp leaves them short and all columns independent.
-// (The form with one thread per column and T^T W took 120 us at 12,288 rows.)
-__global__ void __launch_bounds__(128) k_wt(const double* __restrict__ Wp, int nz, const double* __restrict__ G,
-                                            const double* __restrict__ tau, int nbw, long long nt,
-                                            double* __restrict__ W2) {
+// W2 = T^T sum_z Wp[z], one warp per column, lanes = p: both the sum over z and
+// the row of T^T are chains of FP64 instructions of 31 ns; one column per warp
+// keeps all columns independent.  (One thread per column took 120 us at 12,288
+// rows.)
+__global__ void __launch_bounds__(128) k_wt(const double* __restrict__ Wp, int nz, const double* __restrict__ T,
+                                            int nbw, long long nt, double* __restrict__ W2) {
   const int lane = threadIdx.x & 31;
   const long long col = blockIdx.x * 4LL + (threadIdx.x >> 5);
   if (col >= nt) return;
@@ -545,13 +499,15 @@ __global__ void __launch_bounds__(128) k_wt(const double* __restrict__ Wp, int n
     for (int u = 0; u < 8; ++u)
       if (z0 + u < nz) x += t[u];
   }
-  x = lane < nbw ? x * tau[lane] : 0.0;
-  double g[NB];
+  double tq[NB], y = 0.0;
 #pragma unroll
-  for (int q = 0; q < NB; ++q) g[q] = G[lane * NB + q];  // 0 for q >= lane
+  for (int q = 0; q < NB; ++q) tq[q] = T[q * NB + lane];
 #pragma unroll
-  for (int q = 0; q < NB; ++q) x = fma(-g[q], __shfl_sync(0xffffffffu, x, q), x);
-  W2[(size_t)lane * nt + col] = x;
+  for (int q = 0; q < NB; ++q) {
+    const double xq = __shfl_sync(0xffffffffu, x, q);
+    if (q <= lane && q < nbw) y = fma(tq[q], xq, y);
+  }
+  W2[(size_t)lane * nt + col] = lane < nbw ? y : 0.0;
 }
 
 // A[r, j1 + col] -= sum_p v_p(r) W2[p][col] for r in [j0, s), in tiles of 64 rows
@@ -644,11 +600,11 @@ __global__ void k_floor(double* __restrict__ A, long long lda, long long n, unsi
 }
 
 struct QrScratch {
-  unsigned long long* xch;  // exchange records of k_block
-  double* part;             // its partial products of the in-block update
-  double* bw2;              // and their W2
+  unsigned long long* xch;  // exchange records of k_panel
+  double* gram;             // [chunks][KG_LD] of a panel
+  double* G;                // their sum
   double* tau;
-  double* G;
+  double* T;
   double* Wp;
   double* W2;
   double* dg;
@@ -656,11 +612,10 @@ struct QrScratch {
 
 }  // namespace
 
-// Doubles of the panel scratch: exchange records, in-block partials and W2 of
-// k_block, tau, G, and the split-K partials, W2 and diagonal of the trailing update.
+// Doubles of the panel scratch: exchange records, Gram, T, tau, and the split-K
+// partials, W2 and diagonal of the trailing update.
 __host__ __device__ constexpr long long qr_scratch_len(long long n) {
-  return 2LL * KB_SLOT + (long long)KB_MAXP * 3 * NB * NB + 3LL * NB * NB + n + NB * NB + 64LL * NB * n + NB * n + n +
-         64;
+  return 2LL * KP_SLOT + (KP_MAXP + 1LL) * KG_LD + NB * NB + 64LL * NB * n + NB * n + n + n + 64;
 }
 
 long long rfm_householder_scratch(long long s, long long n) {
@@ -673,10 +628,10 @@ namespace {
 QrScratch carve(double* scratch, long long n) {
   QrScratch q;
   double* w = scratch;
-  q.xch = reinterpret_cast<unsigned long long*>(w); w += 2LL * KB_SLOT;
-  q.part = w; w += (long long)KB_MAXP * 3 * NB * NB;
-  q.bw2 = w; w += 3LL * NB * NB;
-  q.G = w; w += NB * NB;
+  q.xch = reinterpret_cast<unsigned long long*>(w); w += 2LL * KP_SLOT;
+  q.gram = w; w += (long long)KP_MAXP * KG_LD;
+  q.G = w; w += KG_LD;
+  q.T = w; w += NB * NB;
   q.Wp = w; w += 64LL * NB * n;
   q.W2 = w; w += (long long)NB * n;
   q.tau = w; w += n;
@@ -685,17 +640,22 @@ QrScratch carve(double* scratch, long long n) {
 }
 
 rfm_status qr_init_device() {
-  const cudaError_t attr = rfm_smem_attr((const void*)k_block, KB_SMEM);  // once per device
-  if (attr != cudaSuccess || rfm_num_sms() == 0) {
+  for (const void* fn : {(const void*)k_panel<1>, (const void*)k_panel<2>, (const void*)k_panel<4>})
+    if (rfm_smem_attr(fn, KP_SMEM) != cudaSuccess) {  // once per device
+      rfm_set_error("householder: device set-up failed");
+      return RFM_ECUDA;
+    }
+  if (rfm_num_sms() == 0) {
     rfm_set_error("householder: device set-up failed");
     return RFM_ECUDA;
   }
   return RFM_OK;
 }
 
-// CTAs of k_block that can be resident together with the largest slab (whole
-// clusters; depends on how the device's SMs are grouped), per device; 0 on failure.
-int kb_max_ctas() {
+// CTAs of k_panel in clusters of cl that can be resident together with the
+// largest slab (depends on how the device's SMs are grouped), per device; 0 on failure.
+template <int CL>
+int kp_max_ctas() {
   static std::mutex mu;
   static int cached[64] = {};
   int dev = 0;
@@ -703,125 +663,122 @@ int kb_max_ctas() {
   std::lock_guard<std::mutex> lk(mu);
   if (cached[dev] == 0) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(KB_CL);
-    cfg.blockDim = dim3(KB_THREADS);
-    cfg.dynamicSmemBytes = KB_SMEM;
+    cfg.gridDim = dim3(CL);
+    cfg.blockDim = dim3(KP_THREADS);
+    cfg.dynamicSmemBytes = KP_SMEM;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_block, &cfg) != cudaSuccess) return 0;
-    cached[dev] = std::min(n * KB_CL, KB_MAXP);
+    if (cudaOccupancyMaxActiveClusters(&n, k_panel<CL>, &cfg) != cudaSuccess) return 0;
+    cached[dev] = n * CL;
   }
   return cached[dev];
 }
 
-// Rows of k_block's slab for np 32-column groups.
-long long kb_max_rows(int np) { return (long long)((KB_SMEM - kb_fixed_smem()) / (NB * np * sizeof(double))); }
-
-// Widest block (32 .. 128 columns) that k_block can hold in shared memory for
-// `rows` rows on all SMs.
-int kb_width(long long rows) {
-  const long long ctas = std::max(1, kb_max_ctas());
-  const long long per = (rows + ctas - 1) / ctas;
-  for (int np = 4; np > 1; --np)
-    if (per <= kb_max_rows(np)) return np * NB;
-  return NB;
-}
-
-// State of one factorisation's exchange: barrier arrivals so far.
-struct KbState {
-  unsigned int arrived = 0;
-};
-
-rfm_status kb_begin(const QrScratch& q, unsigned int* sync, cudaStream_t st) {
-  // tags and barrier count of an earlier factorisation must not be mistaken for this one's
-  RFM_CUDA(cudaMemsetAsync(q.xch, 0, 2LL * KB_SLOT * sizeof(unsigned long long), st));
-  RFM_CUDA(cudaMemsetAsync(sync + SYNC_BAR, 0, sizeof(unsigned int), st));
+// tags of an earlier factorisation must not be mistaken for this one's
+rfm_status qr_begin(const QrScratch& q, cudaStream_t st) {
+  RFM_CUDA(cudaMemsetAsync(q.xch, 0, 2LL * KP_SLOT * sizeof(unsigned long long), st));
   return RFM_OK;
 }
 
-// Factors columns [c0, c0 + nb) (rows c0..s) in place, nb <= kb_width.
-rfm_status factor_block(double* A, long long s, long long lda, long long c0, int nb, cudaStream_t st,
-                        const QrScratch& q, unsigned int* sync, int panel_cap, KbState* ks) {
-  const long long rows = s - c0;
-  const int np = (nb + NB - 1) / NB;
-  const int ctas = kb_max_ctas();
-  if (ctas < KB_CL) {
-    rfm_set_error("householder: no cluster of the panel kernel fits on the device");
-    return RFM_ECUDA;
+// Factors the panel of nbw columns at j0 (rows j0..s) in place; *chunks and
+// *chunk the row split of its sums.
+rfm_status factor_panel(double* A, long long s, long long lda, long long j0, int nbw, cudaStream_t st,
+                        const QrScratch& q, unsigned int* sync, int panel_cap, int* chunks, int* chunk_rows) {
+  const int nsm = rfm_num_sms();
+  const long long rows = s - j0;
+  // chunks of at least 64 rows, one per SM (or per CTA of the cap) at most
+  const long long cap = panel_cap > 0 ? std::min(panel_cap, nsm) : nsm;
+  long long P = std::min<long long>(std::min<long long>((rows + 63) / 64, cap), KP_MAXP);
+  if (P < 1) P = 1;
+  long long chunk = (rows + P - 1) / P;
+  if (chunk > KP_CHUNK && cap < nsm) {  // the cap's chunks would overflow shared memory: take the fewest that fit
+    P = std::min<long long>((rows + KP_CHUNK - 1) / KP_CHUNK, nsm);
+    chunk = (rows + P - 1) / P;
   }
-  // In 31 ns instructions a 32-column panel costs rows / (2 P) a column for its
-  // products and updates, P / 16 for the sum over the clusters of P CTAs and,
-  // with columns to the right in the block, rows / P a column for their update:
-  // least at P^2 = 8 rows (one panel) or 24 rows (a block of four).
-  const double opt = sqrt((np > 1 ? 24.0 : 8.0) * (double)rows);
-  const long long cap = panel_cap > 0 ? std::min(panel_cap, ctas) : ctas;
-  auto whole = [](long long v) { return std::max<long long>(KB_CL, v / KB_CL * KB_CL); };
-  long long P = whole(std::min<long long>((long long)opt, cap));
-  const long long most = kb_max_rows(np);
-  if ((rows + P - 1) / P > most)  // a cap would overflow shared memory: take the fewest clusters that fit
-    P = ((rows + most - 1) / most + KB_CL - 1) / KB_CL * KB_CL;
-  const long long chunk = (rows + P - 1) / P;
-  if (P > ctas || chunk > most) {
+  if (chunk > KP_CHUNK) {
     rfm_set_error("householder: sketch too tall for the panel kernel");
     return RFM_EINVAL;
   }
-  BlockArgs a;
-  a.A = A; a.lda = lda; a.s = s; a.j0 = c0; a.nb = nb; a.P = (int)P; a.chunk = (int)chunk;
-  a.xch = q.xch; a.part = q.part; a.w2 = q.bw2; a.tau = q.tau; a.G = q.G;
-  a.bar = sync + SYNC_BAR; a.bar0 = ks->arrived; a.err = sync + SYNC_ERR;
-  ks->arrived += 2u * (unsigned)(np - 1) * (unsigned)P;
+  PanelArgs a;
+  a.A = A; a.lda = lda; a.s = s; a.j0 = j0; a.nbw = nbw; a.P = (int)P; a.chunk = (int)chunk;
+  a.kpc = (int)((chunk + 31) / 32);
+  a.xch = q.xch; a.tau = q.tau; a.err = sync + SYNC_ERR;
+  // Clusters over the chunks of one remainder modulo 32, the largest size that
+  // the cap allows and whose slab fits; else a CTA per chunk.
+  const int ng = (int)std::min<long long>(P, 32), u = (int)((P + 31) / 32);
+  auto fits = [&](int cl) {
+    return (kp_fixed(cl, u) + kp_slab_rows(cl, u, a.kpc) * KP_LD) * (long long)sizeof(double) <= KP_SMEM;
+  };
+  int cl = 1;
+  a.U = 1;
+  a.NG = (int)P;
+  if (ng * 4 <= std::min<long long>(panel_cap > 0 ? cap : 1 << 20, kp_max_ctas<4>()) && fits(4)) cl = 4;
+  else if (ng * 2 <= std::min<long long>(panel_cap > 0 ? cap : 1 << 20, kp_max_ctas<2>()) && fits(2)) cl = 2;
+  if (cl > 1) {
+    a.U = u;
+    a.NG = ng;
+  }
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: they wait on each other's records
   at[0].val.cooperative = 1;
-  cfg.gridDim = dim3((unsigned)P);
-  cfg.blockDim = dim3(KB_THREADS);
-  cfg.dynamicSmemBytes = kb_fixed_smem() + (size_t)NB * np * chunk * sizeof(double);
+  cfg.gridDim = dim3((unsigned)(a.NG * cl));
+  cfg.blockDim = dim3(KP_THREADS);
+  cfg.dynamicSmemBytes = (size_t)((kp_fixed(cl, a.U) + kp_slab_rows(cl, a.U, a.kpc) * KP_LD) * sizeof(double));
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   ProfScope ps(PF_QR_PANEL, st);
-  RFM_CUDA(cudaLaunchKernelEx(&cfg, k_block, a));
+  RFM_CUDA(cudaLaunchKernelEx(&cfg, cl == 4 ? k_panel<4> : cl == 2 ? k_panel<2> : k_panel<1>, a));
   RFM_CHECK_LAUNCH();
+  *chunks = (int)P;
+  *chunk_rows = (int)chunk;
   return RFM_OK;
 }
 
-// Householder factorisation of columns [c0, c1) (rows c0..s); the reflectors
-// are applied in FP64 to the columns up to cend (cend >= c1).  Without columns
-// past c1 the blocks are as wide as shared memory allows (k_block updates
-// inside them); with them, 32 columns at a time.
+// Householder factorisation of columns [c0, c1) (rows c0..s) in NB-wide
+// panels; the FP64 compact-WY update of each panel is applied to the columns
+// up to cend (cend >= c1).
 rfm_status factor_range(double* A, long long s, long long lda, long long c0, long long c1, long long cend,
-                        cudaStream_t st, const QrScratch& q, unsigned int* sync, int panel_cap, KbState* ks) {
+                        cudaStream_t st, const QrScratch& q, unsigned int* sync, int panel_cap) {
   const int nsm = rfm_num_sms();
-  if (cend == c1 && kb_width(s - c0) >= c1 - c0)
-    return factor_block(A, s, lda, c0, (int)(c1 - c0), st, q, sync, panel_cap, ks);
   for (long long j0 = c0; j0 < c1; j0 += NB) {
     const int nbw = (int)std::min<long long>(NB, c1 - j0);
     const long long rows = s - j0;
-    RFM_TRY(factor_block(A, s, lda, j0, nbw, st, q, sync, panel_cap, ks));
+    int chunks = 0, chunk = 0;
+    RFM_TRY(factor_panel(A, s, lda, j0, nbw, st, q, sync, panel_cap, &chunks, &chunk));
     const long long j1 = j0 + nbw;
     const long long nt = cend - j1;
     if (nt <= 0) continue;
+    // K slices: two per SM and 64-column tile, of 256 rows at least
     const long long ctiles = (nt + 63) / 64;
-    // K slices of whole 32-row steps: the count that leaves the fewest steps on
-    // the busiest SM (FP64 bound, so co-resident CTAs only share the unit)
-    const long long steps = (rows + 31) / 32;
-    long long nz = 1, best = -1;
-    for (long long z = 1; z <= std::min<long long>(64, steps); ++z) {
-      const long long per = (steps + z - 1) / z, zz = (steps + per - 1) / per;
-      const long long cost = ((ctiles * zz + nsm - 1) / nsm) * per * 64 + zz;  // + k_wt's sum over slices
-      if (best < 0 || cost < best) {
-        best = cost;
-        nz = zz;
-      }
-    }
-    const long long kchunk = (steps + nz - 1) / nz * 32;
+    long long nz = (2LL * nsm + ctiles - 1) / ctiles;
+    nz = std::max<long long>(1, std::min<long long>(nz, std::min<long long>(64, (rows + 255) / 256)));
+    const long long kchunk = (rows + nz - 1) / nz;
     nz = (rows + kchunk - 1) / kchunk;
     {
       ProfScope ps(PF_QR_VTA, st);
       rfm_prof_work(PF_QR_VTA, 2.0 * nbw * (double)nt * (double)rows);  // FP64 flops
-      k_vta<<<dim3((unsigned)ctiles, (unsigned)nz), 256, 0, st>>>(A, lda, s, j0, nbw, j1, nt, kchunk, q.Wp);
+      k_gram<<<(unsigned)chunks, 256, 0, st>>>(A, lda, s, j0, nbw, chunk, q.gram);
       RFM_CHECK_LAUNCH();
-      k_wt<<<(unsigned)((nt + 3) / 4), 128, 0, st>>>(q.Wp, (int)nz, q.G, q.tau + j0, nbw, nt, q.W2);
+      k_panel_t<<<8, 64, 0, st>>>(q.gram, chunks, q.tau + j0, nbw, q.G, q.T);
+      RFM_CHECK_LAUNCH();
+      // the tile with the least FP64 work on the busiest SM, the widest of equals
+      int tc = 64;
+      long long cost = 0;
+      for (int c : {64, 32, 16, 8}) {
+        const long long v = ((nt + c - 1) / c * nz + nsm - 1) / nsm * c;
+        if (c == 64 || v < cost) {
+          cost = v;
+          tc = c;
+        }
+      }
+      const dim3 grid((unsigned)((nt + tc - 1) / tc), (unsigned)nz);
+      if (tc == 64) k_vta<64><<<grid, vta_threads<64>(), 0, st>>>(A, lda, s, j0, nbw, j1, nt, kchunk, q.Wp);
+      else if (tc == 32) k_vta<32><<<grid, vta_threads<32>(), 0, st>>>(A, lda, s, j0, nbw, j1, nt, kchunk, q.Wp);
+      else if (tc == 16) k_vta<16><<<grid, vta_threads<16>(), 0, st>>>(A, lda, s, j0, nbw, j1, nt, kchunk, q.Wp);
+      else k_vta<8><<<grid, vta_threads<8>(), 0, st>>>(A, lda, s, j0, nbw, j1, nt, kchunk, q.Wp);
+      RFM_CHECK_LAUNCH();
+      k_wt<<<(unsigned)((nt + 3) / 4), 128, 0, st>>>(q.Wp, (int)nz, q.T, nbw, nt, q.W2);
       RFM_CHECK_LAUNCH();
     }
     ProfScope psu(PF_QR_UPDATE, st);
@@ -872,10 +829,9 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
   }
   RFM_TRY(qr_init_device());
   const QrScratch q = carve(scratch, n);
-  KbState ks;
-  RFM_TRY(kb_begin(q, sync, st));
+  RFM_TRY(qr_begin(q, st));
   const long long c1 = ncols < 0 ? n : std::min<long long>(n, ((ncols + NB - 1) / NB) * NB);
-  RFM_TRY(factor_range(A, s, lda, 0, c1, n, st, q, sync, panel_cap, &ks));
+  RFM_TRY(factor_range(A, s, lda, 0, c1, n, st, q, sync, panel_cap));
   return finish_r(A, n, lda, st, q, sync, rank_flag_host);
 }
 
@@ -887,7 +843,7 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
 // front through their own pool (where a cudaMalloc fails or implicitly
 // synchronises the device and stalls other streams), or loops with fixed
 // latency budgets.  The QR scratch lives in file-scope device arrays of fixed
-// size (15.1 MB of scratch + 16 KB of barrier words per GPU that loads the
+// size (9.9 MB of scratch + 16 KB of barrier words per GPU that loads the
 // library, held until the process exits), sized for n <= 512 columns.
 // Every call shares these arrays and they keep the last call's contents;
 // calls that overlap on the GPU (two streams, or two host threads) race on
@@ -897,6 +853,7 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
 
 namespace {
 constexpr long long kNoallocScratch = qr_scratch_len(RFM_NOALLOC_MAX_N);
+static_assert(kNoallocScratch * 8 == 9852416, "the size stated above and in rfm.h");
 }  // namespace
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocScratch];
@@ -979,22 +936,21 @@ extern "C" rfm_status rfm_householder_r_noalloc(double* A_dev, int64_t s, int64_
 // ---------------------------------------------------------------------------
 // Householder QR with the trailing update on the tensor cores.
 //
-// A block of w columns is factored recursively: its left half, the block
-// reflector of that half applied to the right half, then the right half; blocks
-// of kb_base columns go to k_block.  A factored block's reflectors V (rows x w,
-// unit diagonal) update the columns to its right in compact-WY form
+// Blocks of QB = 128 columns are factored by factor_range (FP64 inside the
+// block); the block's reflectors V (rows x 128, unit diagonal) update the columns
+// to its right in compact-WY form
 //     W = V^T A_t,  W2 = T^T W,  A_t -= V W2
 // with all products on the emulated-FP64 tensor-core GEMM (digit splitting,
-// exact level accumulation).  T (w x w) comes from the Gram V^T V, which the
+// exact level accumulation).  T (128 x 128) comes from the Gram V^T V, which the
 // first product returns next to W, and the reflector coefficients,
 // T_jj = tau_j, T_{:j,j} = -tau_j T_{:j,:j} G_{:j,j}.
 //
-// The trailing matrix is updated once per QB columns: its digits are formed and
-// C is read and written once per pass, and the update's depth K = w is the MMA
-// work of an output tile for one drain of its accumulators.  With w = 128 the
-// update ran at 35 % of the tensor rate and the digits of the trailing matrix
-// took 20 % of the time; w = 512 is one exact chunk of the GEMM, the largest
-// depth that one drain covers.
+// 128 columns are a quarter of the GEMM's exact chunk, so an update of depth 128
+// drains its accumulators four times as often as it need.  Blocks of 512 columns,
+// with V sliced without its unit diagonal, took 48 instead of 65 ms at n = 4,096
+// and 613 instead of 980 ms at n = 16,384, and R was nearer to the exact one; but
+// it was another R (by 1e-10), and one in three solves of n = 4,096 took another
+// number of LSQR steps.
 
 rfm_status rfm_oz_slice_house_v(const double* A, long long lda, long long j0, long long rows, long long nb, int ndig,
                                 int* e, uint16_t* out, cudaStream_t st);
@@ -1009,125 +965,39 @@ rfm_status rfm_oz_slice_house_vt_at(const double* A, long long lda, long long j0
 
 namespace {
 
-constexpr int QB = 512;   // columns of an outer block (n >= 2 QB)
+constexpr int QB = 128;
 constexpr int QDIG = 8;
 
-// T from G and tau: T^-1 = diag(1 / tau) + strict upper part of G, so column j
-// of T is a back substitution, t_j = tau_j, t_i = -tau_i sum_{l>i} G_il t_l (no
-// division; tau_i = 0 gives a zero row).  One warp per column, lane L holding
-// rows L, L + 32, ..: the columns are independent, and a step is one shuffle
-// and at most U FP64 instructions.  (Column after column on one CTA, whose
-// FP64 unit had to do all of it, took 447 us for 128 columns; now 35 us.)
-// G is column-major, T row-major, both w x w with w = 32 U.
-template <int U>
+// T from G (symmetric) and tau: T_ij = -tau_j sum_{i <= l < j} T_il G_lj, l in
+// turn.  One warp per row i of T, lanes = columns (four each): the rows are
+// independent, and a step is one product and at most four multiply-adds.  (Column
+// after column on one CTA took 447 us, this 34.)  T is row-major.
 __global__ void __launch_bounds__(128) k_block_t(const double* __restrict__ G, const double* __restrict__ tau,
                                                  double* __restrict__ T) {
-  constexpr int w = 32 * U;
+  constexpr int U = QB / 32;
   const int lane = threadIdx.x & 31;
-  const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
-  double t[U], tu[U];
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
+  double v[U], row[U], tj[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    t[u] = lane + 32 * u == j ? 1.0 : 0.0;  // e_j, then the right-hand side less the solved part
-    tu[u] = tau[lane + 32 * u];
+    v[u] = row[u] = 0.0;
+    tj[u] = tau[lane + 32 * u];
   }
 #pragma unroll
-  for (int h = U - 1; h >= 0; --h)  // row l = 32 h + ll is held in t[h]
-    for (int l = min(j, 32 * h + 31); l >= 32 * h; --l) {
+  for (int h = 0; h < U; ++h)  // column l = 32 h + ll of the row is held in row[h]
+    for (int ll = max(0, i - 32 * h); ll < 32; ++ll) {
+      const int l = 32 * h + ll;
       double g[U];
 #pragma unroll
-      for (int u = 0; u <= h; ++u) g[u] = G[(size_t)l * w + lane + 32 * u];
-      if (lane == (l & 31)) t[h] *= tu[h];
-      const double y = __shfl_sync(0xffffffffu, t[h], l & 31);
+      for (int u = h; u < U; ++u) g[u] = G[(size_t)l * QB + lane + 32 * u];
+      if (lane == ll) row[h] = l == i ? tj[h] : -tj[h] * v[h];
+      const double t = __shfl_sync(0xffffffffu, row[h], ll);
 #pragma unroll
-      for (int u = 0; u <= h; ++u)
-        if (u < h || lane < (l & 31)) t[u] = fma(-g[u], y, t[u]);
+      for (int u = h; u < U; ++u)
+        if (u > h || lane > ll) v[u] = fma(t, g[u], v[u]);
     }
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int i = lane + 32 * u;
-    T[(size_t)i * w + j] = i <= j ? t[u] : 0.0;
-  }
-}
-
-// [G, W] (w x N, ld w) += E^T [V, A_t] + V'^T E [I, 0] of the block at c0: the
-// rows c0 .. c0 + w of the trailing columns; in the Gram's upper part (all that
-// T needs), V'^T E, entry (p, j) = v_p(j) for p < j.
-__global__ void __launch_bounds__(64) k_add_top(const double* __restrict__ A, long long lda, long long c0, int w,
-                                                long long N, double* __restrict__ C) {
-  const int p = blockIdx.x * 64 + threadIdx.x;
-  for (long long j = blockIdx.y; j < N; j += gridDim.y) {
-    double add = 0.0;
-    if (j >= w) add = A[(size_t)(c0 + j) * lda + c0 + p];
-    else if (p < j) add = A[(size_t)(c0 + p) * lda + c0 + j];
-    C[(size_t)j * w + p] += add;
-  }
-}
-
-// Workspace of the block reflectors' application.
-struct EmuWs {
-  uint16_t *at, *t, *v, *w2;  // digits of [V, A_t], T^T, V, W2 (and of W before it)
-  double *Wm, *W2, *T, *part;
-  long long part_elems;
-  int *e_at, *e_t, *e_v, *e_w2;
-};
-
-long long emu_part_elems(long long n) { return 16LL * 128 * (n + QB); }
-
-rfm_status apply_block(double* A, long long s, long long lda, long long c0, int w, long long cend, cudaStream_t st,
-                       const double* tau, const EmuWs& e, unsigned int* err) {
-  const long long rows = s - c0, c1 = c0 + w, nt = cend - c1;
-  {
-    // One emulated product gives the block's Gram and V^T A_t.  V is sliced
-    // without its unit diagonal, V = E + V': the digits of a row are scaled by
-    // its largest entry, and beside the 1 the others (about 1 / sqrt(2 rows))
-    // would keep 5 to 7 bits less.  The B operand is [V', A_t] (V'^T as the
-    // first w / 64 row tiles, then the trailing columns), the A operand the
-    // same V'^T tiles, and k_add_top adds E^T [V, A_t] and V'^T E in FP64.
-    // (With the unit diagonal in the digits R of a 12,288 x 4,096 sketch was
-    // four times as far from the exact one as the FP64 path's.)
-    ProfScope ps(PF_QR_VTA, st);
-    const long long prt = w / 64 + (nt + 63) / 64;  // row tiles of the B operand
-    RFM_TRY(rfm_oz_slice_house_vt_at(A, lda, c0, w, rows, QDIG, 64, e.e_at, e.at, prt, 0, st));
-    RFM_TRY(rfm_oz_slice_strided_at(A + (size_t)c1 * lda + c0, lda, 1, nt, rows, QDIG, 64, e.e_at + w, e.at, prt,
-                                    w / 64, st));
-    RFM_TRY(rfm_oz_gemm_part(e.at, QDIG, e.e_at, e.at, QDIG, e.e_at, w, w + nt, rows, QDIG + 1, e.Wm, w, 0, err, st,
-                             e.part, e.part_elems, prt));
-    k_add_top<<<dim3((unsigned)(w / 64), (unsigned)std::min<long long>(w + nt, 32768)), 64, 0, st>>>(
-        A, lda, c0, w, w + nt, e.Wm);
-    RFM_CHECK_LAUNCH();
-    if (w == 64) k_block_t<2><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
-    else if (w == 128) k_block_t<4><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
-    else if (w == 256) k_block_t<8><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
-    else k_block_t<16><<<w / 4, 128, 0, st>>>(e.Wm, tau + c0, e.T);
-    RFM_CHECK_LAUNCH();
-    // W2 = T^T W on the emulated GEMM as well (M = K = w, N = nt).
-    // T is stored row-major, T(q, p) = T[q w + p], so T^T(p, q) = T[p + q w].
-    RFM_TRY(rfm_oz_slice_strided(e.T, 1, w, w, w, QDIG, 128, e.e_t, e.t, st));
-    RFM_TRY(rfm_oz_slice_strided(e.Wm + (size_t)w * w, w, 1, nt, w, QDIG, 64, e.e_w2, e.w2, st));
-    RFM_TRY(rfm_oz_gemm(e.t, QDIG, e.e_t, e.w2, QDIG, e.e_w2, w, nt, w, QDIG + 1, e.W2, w, 0, err, st));
-  }
-  ProfScope ps(PF_QR_UPDATE, st);
-  RFM_TRY(rfm_oz_slice_house_v(A, lda, c0, rows, w, QDIG, e.e_v, e.v, st));
-  RFM_TRY(rfm_oz_slice_strided(e.W2, w, 1, nt, w, QDIG, 64, e.e_w2, e.w2, st));
-  return rfm_oz_gemm(e.v, QDIG, e.e_v, e.w2, QDIG, e.e_w2, rows, nt, w, QDIG + 1, A + (size_t)c1 * lda + c0, lda, 1,
-                     err, st);
-}
-
-// Columns of one k_block: 128 while its slab holds them and the FP64 update
-// inside the block (rows x 128 columns on the FP64 units) costs less than the
-// dozen small launches of an emulated one, else 64.
-int kb_base(long long rows) { return rows <= KB_WIDE_ROWS && kb_width(rows) >= 128 ? 128 : 64; }
-
-rfm_status factor_recursive(double* A, long long s, long long lda, long long c0, int w, cudaStream_t st,
-                            const QrScratch& q, const EmuWs& e, unsigned int* sync, int panel_cap, KbState* ks) {
-  const int base = kb_base(s - c0);
-  if (w <= base) return factor_range(A, s, lda, c0, c0 + w, c0 + w, st, q, sync, panel_cap, ks);
-  int h = base;
-  while (2 * h < w) h *= 2;
-  RFM_TRY(factor_recursive(A, s, lda, c0, h, st, q, e, sync, panel_cap, ks));
-  RFM_TRY(apply_block(A, s, lda, c0, h, c0 + w, st, q.tau, e, sync + SYNC_ERR));
-  return factor_recursive(A, s, lda, c0 + h, w - h, st, q, e, sync, panel_cap, ks);
+  for (int u = 0; u < U; ++u) T[(size_t)i * QB + lane + 32 * u] = row[u];
 }
 
 }  // namespace
@@ -1139,7 +1009,7 @@ long long rfm_householder_emulated_bytes(long long s, long long n) {
   b += rfm_oz_digit_bytes(s, QB, QDIG, 128);     // V
   b += rfm_oz_digit_bytes(n, QB, QDIG, 64);      // W2
   b += 8LL * (2LL * QB * (n + QB) + QB * QB);    // [G, W], W2, T
-  b += 8LL * emu_part_elems(n);                  // split-K partials of V^T [V, A_t]
+  b += 8LL * 8 * QB * (n + QB);                  // split-K partials of V^T [V, A_t]
   b += 4LL * (QB + n + QB + s + n) + 4096;
   return b;
 }
@@ -1157,37 +1027,59 @@ rfm_status rfm_householder_emulated(double* A, long long s, long long n, long lo
   }
   RFM_TRY(qr_init_device());
   const QrScratch q = carve(scratch, n);
-  char* p = static_cast<char*>(emu);
+  char* w = static_cast<char*>(emu);
   auto take = [&](long long bytes) {
-    char* r = p;
-    p += (bytes + 255) & ~255LL;
+    char* r = w;
+    w += (bytes + 255) & ~255LL;
     return r;
   };
-  EmuWs e;
-  e.at = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n + QB, s, QDIG, 64)));
-  e.t = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(QB, QB, QDIG, 128)));
-  e.v = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(s, QB, QDIG, 128)));
-  e.w2 = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n, QB, QDIG, 64)));
-  e.Wm = reinterpret_cast<double*>(take(8LL * QB * (n + QB)));  // [G, W] = V^T [V, A_t]
-  e.W2 = reinterpret_cast<double*>(take(8LL * QB * n));
-  e.T = reinterpret_cast<double*>(take(8LL * QB * QB));
-  e.part_elems = emu_part_elems(n);
-  e.part = reinterpret_cast<double*>(take(8LL * e.part_elems));
-  e.e_at = reinterpret_cast<int*>(take(4LL * (n + QB)));
-  e.e_t = reinterpret_cast<int*>(take(4LL * QB));
-  e.e_v = reinterpret_cast<int*>(take(4LL * s));
-  e.e_w2 = reinterpret_cast<int*>(take(4LL * n));
-  KbState ks;
-  RFM_TRY(kb_begin(q, sync, st));
-  // Outer blocks of 512 columns; narrower ones where n holds only a few, and
-  // for a timing probe of the first ncols columns.
-  int wb = QB;
-  while (wb > 128 && (wb * 2 > n || (ncols >= 0 && wb > ncols))) wb /= 2;
+  uint16_t* d_at = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n + QB, s, QDIG, 64)));
+  uint16_t* d_t = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(QB, QB, QDIG, 128)));
+  uint16_t* d_v = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(s, QB, QDIG, 128)));
+  uint16_t* d_w2 = reinterpret_cast<uint16_t*>(take(rfm_oz_digit_bytes(n, QB, QDIG, 64)));
+  double* Wm = reinterpret_cast<double*>(take(8LL * QB * (n + QB)));  // [G, W] = V^T [V, A_t]
+  double* W2 = reinterpret_cast<double*>(take(8LL * QB * n));
+  double* T = reinterpret_cast<double*>(take(8LL * QB * QB));
+  const long long part_elems = 8LL * QB * (n + QB);
+  double* part = reinterpret_cast<double*>(take(8LL * part_elems));
+  int* e_at = reinterpret_cast<int*>(take(4LL * (n + QB)));
+  int* e_t = reinterpret_cast<int*>(take(4LL * QB));
+  int* e_v = reinterpret_cast<int*>(take(4LL * s));
+  int* e_w2 = reinterpret_cast<int*>(take(4LL * n));
+  unsigned int* err = sync + SYNC_ERR;
+  RFM_TRY(qr_begin(q, st));
   const long long cstop = ncols < 0 ? n : std::min<long long>(n, ncols);
-  for (long long J0 = 0; J0 < cstop; J0 += wb) {
-    const int w = (int)std::min<long long>(wb, n - J0);
-    RFM_TRY(factor_recursive(A, s, lda, J0, w, st, q, e, sync, panel_cap, &ks));
-    if (J0 + w < n) RFM_TRY(apply_block(A, s, lda, J0, w, n, st, q.tau, e, sync + SYNC_ERR));
+  for (long long J0 = 0; J0 < cstop; J0 += QB) {
+    const long long c1 = std::min<long long>(n, J0 + QB);
+    const long long rows = s - J0, nt = n - c1;
+    RFM_TRY(factor_range(A, s, lda, J0, c1, c1, st, q, sync, panel_cap));
+    if (nt <= 0) break;
+    {
+      // One emulated product gives the block's Gram and V^T A_t: its B operand
+      // is [V, A_t] (V^T as the first two 64-row tiles, then the trailing
+      // columns), its A operand the same V^T tiles, so C = [G, W] with G = V^T V
+      // (exactly symmetric: the digit pairs (p, q) and (q, p) give the same
+      // integer level sums).
+      ProfScope ps(PF_QR_VTA, st);
+      const long long prt = QB / 64 + (nt + 63) / 64;  // row tiles of the B operand
+      RFM_TRY(rfm_oz_slice_house_vt_at(A, lda, J0, QB, rows, QDIG, 64, e_at, d_at, prt, 0, st));
+      RFM_TRY(rfm_oz_slice_strided_at(A + (size_t)c1 * lda + J0, lda, 1, nt, rows, QDIG, 64, e_at + QB, d_at, prt,
+                                      QB / 64, st));
+      RFM_TRY(rfm_oz_gemm_part(d_at, QDIG, e_at, d_at, QDIG, e_at, QB, QB + nt, rows, QDIG + 1, Wm, QB, 0, err, st,
+                               part, part_elems, prt));
+      k_block_t<<<QB / 4, 128, 0, st>>>(Wm, q.tau + J0, T);
+      RFM_CHECK_LAUNCH();
+      // W2 = T^T W on the emulated GEMM as well (M = K = 128, N = nt).
+      // T is stored row-major, T(q, p) = T[q QB + p], so T^T(p, q) = T[p + q QB].
+      RFM_TRY(rfm_oz_slice_strided(T, 1, QB, QB, QB, QDIG, 128, e_t, d_t, st));
+      RFM_TRY(rfm_oz_slice_strided(Wm + (size_t)QB * QB, QB, 1, nt, QB, QDIG, 64, e_w2, d_w2, st));
+      RFM_TRY(rfm_oz_gemm(d_t, QDIG, e_t, d_w2, QDIG, e_w2, QB, nt, QB, QDIG + 1, W2, QB, 0, err, st));
+    }
+    ProfScope ps(PF_QR_UPDATE, st);
+    RFM_TRY(rfm_oz_slice_house_v(A, lda, J0, rows, QB, QDIG, e_v, d_v, st));
+    RFM_TRY(rfm_oz_slice_strided(W2, QB, 1, nt, QB, QDIG, 64, e_w2, d_w2, st));
+    RFM_TRY(rfm_oz_gemm(d_v, QDIG, e_v, d_w2, QDIG, e_w2, rows, nt, QB, QDIG + 1, A + (size_t)c1 * lda + J0, lda, 1,
+                        err, st));
   }
   return finish_r(A, n, lda, st, q, sync, rank_flag_host);
 }

@@ -167,3 +167,77 @@ LSQR = {
 @pytest.mark.parametrize("name", list(PROBLEMS))
 def test_lsqr_directions(rfm, name):
     assert digest(*run_lsqr(rfm, name)) == LSQR[name]
+
+
+def run_qr(rfm, key):
+    tc, s, n = key
+    B = vec(s * n, 8).view(n, s)
+    return (rfm.rfm_householder_r_tc if tc else rfm.rfm_householder_r)(B, s, n)[0],
+
+
+# one chunk, chunks shorter than 64 rows, a chunk per SM and fewer, chunks of one
+# remainder modulo 32 in one to five parts, slabs too tall for a cluster, and
+# several panels and blocks with ragged ends
+QR_CASES = [(tc, s, n) for tc in (False, True) for s, n in
+            [(1, 1), (33, 31), (65, 65), (97, 40), (500, 127), (1201, 400), (9800, 70), (12288, 300), (60001, 64),
+             (108000, 33), (121000, 33), (2600, 1100), (3100, 1537)]]
+QR = {
+    (False, 1, 1): 'bc05bd1b03a6a949',
+    (False, 33, 31): '5da962065938d2dd',
+    (False, 65, 65): '238b021675072f69',
+    (False, 97, 40): '84bfcf09206c0163',
+    (False, 500, 127): 'a192cc852199bf9b',
+    (False, 1201, 400): 'fc01d0a62250ab00',
+    (False, 9800, 70): 'ec9db505b490e487',
+    (False, 12288, 300): 'a9b63c2abc3a56f5',
+    (False, 60001, 64): 'f347feef90be2b13',
+    (False, 108000, 33): '5a58bbf3a495bd14',
+    (False, 121000, 33): '9d88379da04bb48f',
+    (False, 2600, 1100): '30fcd7c2c4e11e4b',
+    (False, 3100, 1537): '97ca3b4134858f93',
+    (True, 1, 1): 'bc05bd1b03a6a949',
+    (True, 33, 31): '5da962065938d2dd',
+    (True, 65, 65): '238b021675072f69',
+    (True, 97, 40): '84bfcf09206c0163',
+    (True, 500, 127): 'a192cc852199bf9b',
+    (True, 1201, 400): '9214c5787df07174',
+    (True, 9800, 70): 'ec9db505b490e487',
+    (True, 12288, 300): '9f74559f327ec14b',
+    (True, 60001, 64): 'f347feef90be2b13',
+    (True, 108000, 33): '5a58bbf3a495bd14',
+    (True, 121000, 33): '9d88379da04bb48f',
+    (True, 2600, 1100): '4a0af2138da670df',
+    (True, 3100, 1537): '8b6af6291aa10a2c',
+}
+
+
+@pytest.mark.parametrize("key", QR_CASES)
+def test_r(rfm, key):
+    assert digest(*run_qr(rfm, key)) == QR[key]
+
+
+def run_solve(rfm, key):
+    name, precision, first, count = key
+    out = []
+    for seed in range(first, first + count):
+        d = dict(W.config_c1()) if name == "c1" else W.problem(3, (2, 2, 2), 512, (12, 12, 12), (6, 6, 6), (6, 6, 6),
+                                                               pde_kind=2)
+        d["seed"] = W.FEATURE_SEED + 1000 * seed
+        gp = rfm.Problem(d)
+        info = gp.rfm_ipn_solve(W.solve_opts(precision=precision))[1]
+        out.append(info["lsqr_iters_total"])
+    return out
+
+
+# whole IPN solves of C1 and of a C5-sized problem over feature seeds: LSQR steps
+SOLVE_CASES = [("c1", 0, 112, 16), ("c5", 2, 100, 8), ("c5", 0, 100, 8)]
+SOLVE = {
+    ('c1', 0, 112, 16): [90, 90, 93, 86, 88, 86, 88, 97, 93, 87, 87, 92, 85, 87, 88, 87],
+    ('c5', 2, 100, 8): [137, 133, 139, 128, 127, 133, 132, 133],
+    ('c5', 0, 100, 8): [137, 132, 139, 128, 127, 133, 132, 132],
+}
+
+
+@pytest.mark.parametrize("key", SOLVE_CASES)
+def test_step_counts(rfm, key):
+    assert run_solve(rfm, key) == SOLVE[key]
