@@ -281,11 +281,14 @@ __global__ void __launch_bounds__(GD_THREADS) k_gauss_digits(long long s, const 
       ts[rfm_swz128(2 * pr + 1, k64) >> 1] = (uint16_t)(__float_as_uint(d1) >> 16);
     }
     __syncthreads();
+    // The queue's length for every thread's decision below: read between the two
+    // barriers, where the tile's additions are done and no thread has begun the
+    // next tile's.
+    const int nq = min(queued, GD_QUEUE);
     uint4* dst = reinterpret_cast<uint4*>(out + (size_t)tile * (128 * 64));
 #pragma unroll
     for (int u = 0; u < 4; ++u) dst[tid + GD_THREADS * u] = tile_s[tid + GD_THREADS * u];
     __syncthreads();  // the tile is written; ts and the queue may change again
-    const int nq = min(queued, GD_QUEUE);
     if (nq >= GD_THREADS || tile + gridDim.x >= tiles) {
       for (int at = tid; at < nq; at += GD_THREADS) redo(queue[at]);
       __syncthreads();
