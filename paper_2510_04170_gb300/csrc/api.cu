@@ -287,8 +287,25 @@ rfm_status read_scalars(rfm_problem* p, const double* dev, int count, double* ho
 
 // Clears the device error word at the start of a public call, so a wait that
 // gave up in an earlier call is not reported again.
+// 8-byte words of the records of the line search and of the triangular solve.
+long long record_words(long long n) { return 2 * LS_BLOCKS * 2 + (n + 63) / 64 * 64 * 4; }
+
+// Error word back to zero.  If it was set, a wait gave up and the CTAs of that
+// launch went on without each other: one may have read the next epoch and left
+// records under the tags of the next solve or search.  All records are dropped
+// then (tag 0 is never asked for).
+__global__ void __launch_bounds__(256) k_clear_err(unsigned int* __restrict__ err, unsigned long long* __restrict__ rec,
+                                                   long long words) {
+  const bool failed = __ldcg(err) != 0u;
+  __syncthreads();
+  if (!failed) return;
+  for (long long i = threadIdx.x; i < words; i += 256) rec[i] = 0ull;
+  if (threadIdx.x == 0) *err = 0u;
+}
+
 rfm_status clear_err(rfm_problem* p) {
-  RFM_CUDA(cudaMemsetAsync(p->sync + SYNC_ERR, 0, sizeof(unsigned int), p->stream));
+  k_clear_err<<<1, 256, 0, p->stream>>>(p->sync + SYNC_ERR, p->ls_rec, record_words(p->n));
+  RFM_CHECK_LAUNCH();
   return RFM_OK;
 }
 
@@ -948,7 +965,7 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->red, 4096));
     // one allocation for the smaller solver buffers; the records, which start at
     // zero, come first
-    const long long nrec = 2 * LS_BLOCKS * 2 + (p->n + 63) / 64 * 64 * 4;
+    const long long nrec = record_words(p->n);
     TRYA(dalloc(&p->slab, (size_t)(nrec + 8 * nfeat + JT_SLICES * p->n + rfm_trsv_tiles_len(p->n))));
     p->ls_rec = reinterpret_cast<unsigned long long*>(p->slab);
     p->trsv_rec = p->ls_rec + 2 * LS_BLOCKS * 2;

@@ -719,7 +719,8 @@ __global__ void __launch_bounds__(256, 2) k_ls_search(LsArgs a) {
   const bool down = fbest < a.f0;
   a.out[0] = down ? best : 0.0;
   a.out[1] = down ? fbest : a.f0;
-  // every other CTA has read the epoch: this one has seen its records
+  // every other CTA has read the epoch: this one has seen its records (or a wait gave
+  // up, and k_clear_err drops what a late CTA leaves)
   *a.epoch = base + (unsigned int)evals;
 }
 

@@ -674,7 +674,8 @@ __global__ void __cluster_dims__(CHAIN_CL, 1, 1) __launch_bounds__(256, 1) k_trs
   RecWait wait(a.err, threadIdx.x);
   if (blockIdx.x < CHAIN_CL) {
     trsv_chain<TRANS>(a, tag, wait, csm);
-    // every helper whose records the chain used has read the epoch; the others use no tag
+    // every helper whose records the chain used has read the epoch; the others use no
+    // tag (after a wait that gave up, k_clear_err drops what a late one leaves)
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.epoch = tag;
   } else {
     trsv_helper<TRANS, NT>(a, tag, wait, csm);
