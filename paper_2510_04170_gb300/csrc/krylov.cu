@@ -19,7 +19,7 @@
 //             flags of the blocks it needs, accumulates their contribution
 //             with coalesced column reads of R, solves its diagonal block in
 //             one warp and publishes its part of x with a release flag.
-//  * k_partial_* / k_finish_*: deterministic two-stage norms and dots.
+//  * k_partial_norm2, k_finish: deterministic two-stage norms.
 #include <algorithm>
 #include <mutex>
 
@@ -691,11 +691,10 @@ __global__ void k_trsv_prep(unsigned int* __restrict__ epoch, unsigned int* __re
   *ticket = 0u;
 }
 
-__global__ void k_partial_dot(const double* __restrict__ a, const double* __restrict__ b, long long n,
-                              double* __restrict__ partial) {
+__global__ void k_partial_norm2(const double* __restrict__ x, long long n, double* __restrict__ partial) {
   double acc = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    acc += a[i] * b[i];
+    acc += x[i] * x[i];
   __shared__ double sh[32];
   acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -707,11 +706,11 @@ __global__ void k_partial_dot(const double* __restrict__ a, const double* __rest
   }
 }
 
-__global__ void k_finish(const double* __restrict__ partial, int np, int take_sqrt, double* __restrict__ out) {
+__global__ void k_finish(const double* __restrict__ partial, int np, double* __restrict__ out) {
   double acc = 0.0;
   for (int i = threadIdx.x; i < np; i += 32) acc += partial[i];
   acc = warp_sum(acc);
-  if (threadIdx.x == 0) out[0] = take_sqrt ? sqrt(acc) : acc;
+  if (threadIdx.x == 0) out[0] = sqrt(acc);
 }
 
 constexpr int kRedBlocks = 304;
@@ -719,18 +718,9 @@ constexpr int kRedBlocks = 304;
 }  // namespace
 
 rfm_status rfm_norm2(cudaStream_t st, const double* x, long long n, double* partial, double* out_dev) {
-  k_partial_dot<<<kRedBlocks, 256, 0, st>>>(x, x, n, partial);
+  k_partial_norm2<<<kRedBlocks, 256, 0, st>>>(x, n, partial);
   RFM_CHECK_LAUNCH();
-  k_finish<<<1, 32, 0, st>>>(partial, kRedBlocks, 1, out_dev);
-  RFM_CHECK_LAUNCH();
-  return RFM_OK;
-}
-
-rfm_status rfm_dot(cudaStream_t st, const double* x, const double* y, long long n, double* partial,
-                   double* out_dev) {
-  k_partial_dot<<<kRedBlocks, 256, 0, st>>>(x, y, n, partial);
-  RFM_CHECK_LAUNCH();
-  k_finish<<<1, 32, 0, st>>>(partial, kRedBlocks, 0, out_dev);
+  k_finish<<<1, 32, 0, st>>>(partial, kRedBlocks, out_dev);
   RFM_CHECK_LAUNCH();
   return RFM_OK;
 }

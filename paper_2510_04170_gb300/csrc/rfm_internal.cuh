@@ -212,10 +212,8 @@ rfm_status rfm_householder_inplace(double* A, long long s, long long n, long lon
 // panel_cap: most CTAs of one panel factorisation (0: one per SM); ncols >= 0
 // stops after the blocks that cover the first ncols columns (timing probes).
 long long rfm_householder_scratch(long long s, long long n);
-// deterministic norms / dots: result written to out_dev[0]
+// deterministic norm: result written to out_dev[0]
 rfm_status rfm_norm2(cudaStream_t st, const double* x, long long n, double* partial, double* out_dev);
-rfm_status rfm_dot(cudaStream_t st, const double* x, const double* y, long long n, double* partial,
-                   double* out_dev);
 
 #define RFM_SYNC_WORDS 4096
 // layout of p->sync
@@ -256,10 +254,8 @@ __device__ __forceinline__ void st_release(unsigned int* p, unsigned int v) {
 // SYNC_WAITLIM holds the limit: 0 the default of 2^22 polls (well under a
 // second of sleeping), a positive count that many polls, a negative value
 // "give up at once" (a host-side test setting, rfm_set_wait_limit).
-// `pause_ns` > 0 sleeps that long between polls from the start (many waiters
-// on one line leave the L2 slice free for the write they wait for).
 __device__ __forceinline__ bool wait_flag(const unsigned int* flag, unsigned int want,
-                                          unsigned int* err, unsigned int pause_ns = 0) {
+                                          unsigned int* err) {
   const int lim = (int)__ldcg(err + (SYNC_WAITLIM - SYNC_ERR));
   if (lim < 0) {
     atomicExch(err, 1u);
@@ -272,8 +268,7 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* flag, unsigned int
       atomicExch(err, 1u);
       return false;
     }
-    if (pause_ns) __nanosleep(pause_ns);
-    else if (spins > (1u << 16)) __nanosleep(128);
+    if (spins > (1u << 16)) __nanosleep(128);
   }
   return true;
 }
