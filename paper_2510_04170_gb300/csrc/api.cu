@@ -956,26 +956,36 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     TRYA(dalloc(&p->rhs, p->m));
     TRYA(dalloc(&p->Jp, (size_t)p->m * p->W));
     TRYA(dalloc(&p->Js, (size_t)std::max(1LL, p->m_iface) * p->W));
-    TRYA(dalloc(&p->lam, p->m));
-    TRYA(dalloc(&p->F, p->m));
     TRYA(dalloc(&p->colptr, colptr.size()));
     TRYA(dalloc(&p->colrows, colrows.size()));
     TRYA(dalloc(&p->hbuck, p->m));
     TRYA(dalloc(&p->hsign, p->m));
-    TRYA(dalloc(&p->red, 4096));
-    // one allocation for the smaller solver buffers; the records, which start at
-    // zero, come first
-    const long long nrec = record_words(p->n);
-    TRYA(dalloc(&p->slab, (size_t)(nrec + 8 * nfeat + JT_SLICES * p->n + rfm_trsv_tiles_len(p->n))));
-    p->ls_rec = reinterpret_cast<unsigned long long*>(p->slab);
-    p->trsv_rec = p->ls_rec + 2 * LS_BLOCKS * 2;
-    p->slopes = p->slab + nrec;
-    p->jt_part = p->slopes + 8 * nfeat;
-    p->chain_tiles = p->jt_part + JT_SLICES * p->n;
-    TRYA(dalloc(&p->dinv, (size_t)((p->n + 63) / 64) * 64 * 64));
-    TRYA(dalloc(&p->sync, RFM_SYNC_WORDS));
+    // One allocation for the vectors and the solvers' smaller buffers, each on a
+    // 256-byte boundary: an allocation takes about as long as a kernel launch.  What
+    // starts at zero (records, synchronisation words) comes first.
+    long long words = 0;
+    auto place = [&](long long count) {
+      const long long at = words;
+      words += (count + 31) / 32 * 32;
+      return at;
+    };
     p->work_cap = vec_stride(p) * WV_COUNT;
-    TRYA(dalloc(&p->work, p->work_cap));
+    const long long a_rec = place(record_words(p->n)), a_sync = place(RFM_SYNC_WORDS / 2), zeroed = words;
+    const long long a_slopes = place(8 * nfeat), a_jt = place(JT_SLICES * p->n), a_tiles = place(rfm_trsv_tiles_len(p->n));
+    const long long a_dinv = place((p->n + 63) / 64 * 64 * 64), a_work = place(p->work_cap), a_lam = place(p->m);
+    const long long a_f = place(p->m), a_red = place(4096);
+    TRYA(dalloc(&p->slab, (size_t)words));
+    p->ls_rec = reinterpret_cast<unsigned long long*>(p->slab + a_rec);
+    p->trsv_rec = p->ls_rec + 2 * LS_BLOCKS * 2;
+    p->sync = reinterpret_cast<unsigned int*>(p->slab + a_sync);
+    p->slopes = p->slab + a_slopes;
+    p->jt_part = p->slab + a_jt;
+    p->chain_tiles = p->slab + a_tiles;
+    p->dinv = p->slab + a_dinv;
+    p->work = p->slab + a_work;
+    p->lam = p->slab + a_lam;
+    p->F = p->slab + a_f;
+    p->red = p->slab + a_red;
     if (cudaMallocHost((void**)&p->hostbuf, 64 * sizeof(double)) != cudaSuccess) {
       g_err = "cudaMallocHost failed";
       st = RFM_ENOMEM;
@@ -999,8 +1009,7 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
       CPY(p->rmeta, ball_meta.data(), ball_meta.size());
     }
 #undef CPY
-    if (cudaMemsetAsync(p->sync, 0, RFM_SYNC_WORDS * sizeof(unsigned int), s0) != cudaSuccess ||
-        cudaMemsetAsync(p->slab, 0, (size_t)nrec * sizeof(double), s0) != cudaSuccess) {
+    if (cudaMemsetAsync(p->slab, 0, (size_t)zeroed * sizeof(double), s0) != cudaSuccess) {
       st = RFM_ECUDA;
       goto fail;
     }
@@ -1023,10 +1032,9 @@ rfm_status rfm_problem_destroy(rfm_problem* p) {
   if (!p) return RFM_OK;
   if (p->stream) cudaStreamSynchronize(p->stream);
   else cudaDeviceSynchronize();
-  void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slab, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js, p->lam, p->F,
-                  p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->work,
-                  p->red, p->sync, p->sdig, p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch,
-                  p->dinv};
+  void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slab, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js,
+                  p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->sdig,
+                  p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch};
   drop_lsqr_graph(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   for (void* b : bufs) dfree(b);

@@ -42,7 +42,7 @@ struct rfm_problem {
   double* X = nullptr;      // breakpoints [3][nmaxbp]
   double* mu = nullptr;     // [G][4]
   double* sig = nullptr;    // [G][4]
-  double* slab = nullptr;   // allocation of slopes, jt_part, ls_rec, trsv_rec and chain_tiles
+  double* slab = nullptr;   // allocation of lam, F, work, red, sync, slopes, jt_part, dinv, chain_tiles and the records
   double* feat = nullptr;   // [G*fields*M][4]
   double* slopes = nullptr; // [G*fields*M][8]: k_b / sigma_b and their squares
   RowSeg* segs = nullptr;
