@@ -60,12 +60,14 @@ __device__ __forceinline__ void gauss_pair_q16_exact(const uint32_t c[4], float*
 // The same integers from FP32 with the hardware's log2, square root, sine and
 // cosine; false where 16 z lies too near a rounding tie to be sure (0.2 % of
 // the pairs) or w is below 2^-12.  No FP64 instruction (31 ns each on GB300).
-// Errors of 16 z: w from its top 32 bits, 2^-20 relative or less; log2 2^-22
-// absolute on [0.5, 2], 2 ulp elsewhere, so L = r^2 is within 5e-7 (L <= 1.4) or
-// 4e-7 L, and 16 r within 8 dL / r <= 4e-4 for r >= 0.01; sine and cosine on
-// [-pi, pi] within 6e-7 and their argument within 4e-7, times 16 r <= 66 (w >=
-// 2^-12): 7e-5 where the first term is below 4e-5.  Below 5e-4 in all.  For r <
-// 0.01 the computed r^2 is off by 5e-7 at most, |16 z| < 0.2 and both are 0.
+// A tie needs |16 z| near 1/2 or more, so r >= 1/32 (below, 16 r < 1/2).  Errors of
+// 16 z there: w from its top 32 bits, 1.2e-7 relative for w >= 1/2 and 6e-7 at most;
+// log2 2^-22 absolute on [0.5, 2], 2 ulp elsewhere; so L = r^2 is within 8e-7 (L <=
+// 1.4) or 5e-7 L, and 16 r within 8 dL / r <= 2.1e-4; the square root adds 16 r
+// 2^-22; sine and cosine on [-pi, pi] within 6e-7 and their argument within 4e-7,
+// times 16 r <= 66 (w >= 2^-12): 7e-5 where the first term is below 2e-5.  Below
+// 2.5e-4 in all, half the margin of 5e-4.  For computed r < 0.01, r^2 is off by 8e-7
+// at most, |16 z| < 0.2 and both are 0.
 __device__ __forceinline__ bool gauss_pair_q16_fast(const uint32_t c[4], float* d0, float* d1) {
   const uint32_t wt = ~(((c[0] >> 5) << 5) | (c[1] >> 27));  // top 32 bits of 2^53 - (53 bits of u1), less one unit
   const float w = fmaf((float)wt, 0x1p-32f, 0x1p-33f);
