@@ -213,12 +213,12 @@ def read_dominant(lib, rfm, names, dom_fams):
 
 # DRAM traffic per launch of a dominant kernel family, from an ncu capture of the
 # same workload (dram__bytes_read.sum + dram__bytes_write.sum), keyed by
-# (workload, precision, family).  c2 / 2 / oz_gemm: the first 495 k_oz_gemm
-# launches of one c2 solve (the sketch and the larger early blocks of the first
-# factorisation) moved 1,026 GB/s of their device time.  That rate times the
-# solve's mean launch duration (1.63 ms) gives the mean launch's bytes.  Taken
-# with the 512-deep products; it must be measured again whenever those change.
-MEASURED_TRAFFIC = {("c2", 2, "oz_gemm"): 1.67e9}
+# (workload, precision, family).  c2 / 2 / oz_gemm: the first 300 k_oz_gemm
+# launches of the QR of a 65,536 x 32,768 sketch (the larger early blocks) moved
+# 2,053 GB/s of their device time.  That rate times the solve's mean launch
+# duration (5.12 ms) gives the mean launch's bytes.  Taken with the 128-deep
+# products; it must be measured again whenever those change.
+MEASURED_TRAFFIC = {("c2", 2, "oz_gemm"): 1.05e10}
 
 
 def roofline(dom_fams, dom_ms, dom_cnt, dom_work, key=None):
