@@ -799,8 +799,10 @@ int chain_max_ctas() {
         int c = 0;
         const ChainKernel fn = chain_kernel(trans, nt);
         if (rfm_smem_attr((const void*)fn, (int)chain_smem_bytes()) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&c, fn, &cfg) != cudaSuccess)
+            cudaOccupancyMaxActiveClusters(&c, fn, &cfg) != cudaSuccess) {
+          cudaGetLastError();  // the caller takes k_trsv; no later check may find this error
           return 0;
+        }
         least = std::min(least, c * CHAIN_CL);
       }
     // one CTA per SM: two would share the FP64 units the chain depends on

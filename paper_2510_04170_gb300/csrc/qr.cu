@@ -667,7 +667,10 @@ int kp_max_ctas() {
     cfg.blockDim = dim3(KP_THREADS);
     cfg.dynamicSmemBytes = KP_SMEM;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_panel<CL>, &cfg) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_panel<CL>, &cfg) != cudaSuccess) {
+      cudaGetLastError();  // the caller takes a form without clusters; no later check may find this error
+      return 0;
+    }
     cached[dev] = n * CL;
   }
   return cached[dev];
