@@ -971,17 +971,14 @@ rfm_status rfm_problem_create(const rfm_problem_desc* desc, void* cuda_stream, r
     };
     p->work_cap = vec_stride(p) * WV_COUNT;
     const long long a_rec = place(record_words(p->n)), a_sync = place(RFM_SYNC_WORDS / 2), zeroed = words;
-    const long long a_slopes = place(8 * nfeat), a_jt = place(JT_SLICES * p->n), a_tiles = place(rfm_trsv_tiles_len(p->n));
-    const long long a_dinv = place((p->n + 63) / 64 * 64 * 64), a_work = place(p->work_cap), a_lam = place(p->m);
-    const long long a_f = place(p->m), a_red = place(4096);
+    const long long a_slopes = place(8 * nfeat), a_jt = place(JT_SLICES * p->n), a_work = place(p->work_cap);
+    const long long a_lam = place(p->m), a_f = place(p->m), a_red = place(4096);
     TRYA(dalloc(&p->slab, (size_t)words));
     p->ls_rec = reinterpret_cast<unsigned long long*>(p->slab + a_rec);
     p->trsv_rec = p->ls_rec + 2 * LS_BLOCKS * 2;
     p->sync = reinterpret_cast<unsigned int*>(p->slab + a_sync);
     p->slopes = p->slab + a_slopes;
     p->jt_part = p->slab + a_jt;
-    p->chain_tiles = p->slab + a_tiles;
-    p->dinv = p->slab + a_dinv;
     p->work = p->slab + a_work;
     p->lam = p->slab + a_lam;
     p->F = p->slab + a_f;
@@ -1033,7 +1030,7 @@ rfm_status rfm_problem_destroy(rfm_problem* p) {
   if (p->stream) cudaStreamSynchronize(p->stream);
   else cudaDeviceSynchronize();
   void* bufs[] = {p->X, p->mu, p->sig, p->feat, p->slab, p->segs, p->pts, p->rmeta, p->rhs, p->Jp, p->Js,
-                  p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->sdig,
+                  p->colptr, p->colrows, p->B, p->Sg, p->hbuck, p->hsign, p->bptr, p->brows, p->Rown, p->dinv, p->sdig,
                   p->jdig, p->oz_e, p->oz_toff, p->qr_emu, p->qr_scratch};
   drop_lsqr_graph(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);

@@ -22,6 +22,7 @@
 //  * k_partial_norm2, k_finish: deterministic two-stage norms.
 #include <algorithm>
 #include <mutex>
+#include <string>
 
 #include "rfm_internal.cuh"
 
@@ -758,19 +759,6 @@ rfm_status rfm_launch_jtmv(rfm_problem* p, const double* x, double* y) {
   return RFM_OK;
 }
 
-rfm_status rfm_trsv_prepare(rfm_problem* p) {
-  if (!p->dinv || !p->R) return RFM_OK;
-  const int n = (int)p->n, nblk = (n + TB - 1) / TB;
-  k_trsv_dinv<<<dim3(nblk, 16), 128, 0, p->stream>>>(p->R, p->ldr, n, p->dinv);
-  RFM_CHECK_LAUNCH();
-  k_trsv_pack<<<dim3(nblk, CHAIN_D + 1, 2), 256, 0, p->stream>>>(p->R, p->ldr, n, nblk, p->dinv, p->chain_tiles);
-  RFM_CHECK_LAUNCH();
-  p->dinv_of = p->R;
-  return RFM_OK;
-}
-
-long long rfm_trsv_tiles_len(long long n) { return 2LL * ((n + TB - 1) / TB) * (CHAIN_D + 1) * TB * TB; }
-
 namespace {
 using ChainKernel = void (*)(ChainArgs);
 ChainKernel chain_kernel(int trans, int nt) {
@@ -812,6 +800,39 @@ int chain_max_ctas() {
 }
 }  // namespace
 
+// Helper CTAs of the chain for nblk blocks; 0 where k_trsv solves instead.  Chain
+// and helpers up to four blocks per SM (n = 38,800), a rule on n alone so that the
+// solution's bits are those of one form; the helpers, fewer than the SMs, take a
+// fifth target at the end of that range.
+static int chain_helpers(int nblk) {
+  const int H = std::min(chain_max_ctas() - CHAIN_CL, (nblk + CHAIN_CL - 1) / CHAIN_CL * CHAIN_CL);
+  return H > 0 && nblk <= HMAXT * H && nblk - CHAIN_D - 1 <= 4 * (rfm_num_sms() - 1) ? H : 0;
+}
+
+// Inverses and tiles of R for the chain; their buffer comes with the first R, like
+// the sketch's and the QR's.
+rfm_status rfm_trsv_prepare(rfm_problem* p) {
+  const int n = (int)p->n, nblk = (n + TB - 1) / TB;
+  if (!p->R || chain_helpers(nblk) == 0) return RFM_OK;
+  if (!p->dinv) {
+    const size_t inv = (size_t)nblk * TB * TB, tiles = 2 * inv * (CHAIN_D + 1);
+    double* buf = nullptr;
+    if (cudaMalloc(&buf, (inv + tiles) * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      rfm_set_error("triangular solve: allocation of " + std::to_string((inv + tiles) * sizeof(double)) + " bytes failed");
+      return RFM_ENOMEM;
+    }
+    p->dinv = buf;
+    p->chain_tiles = buf + inv;
+  }
+  k_trsv_dinv<<<dim3(nblk, 16), 128, 0, p->stream>>>(p->R, p->ldr, n, p->dinv);
+  RFM_CHECK_LAUNCH();
+  k_trsv_pack<<<dim3(nblk, CHAIN_D + 1, 2), 256, 0, p->stream>>>(p->R, p->ldr, n, nblk, p->dinv, p->chain_tiles);
+  RFM_CHECK_LAUNCH();
+  p->dinv_of = p->R;
+  return RFM_OK;
+}
+
 rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x) {
   const int n = (int)p->n;
   const int nblk = (n + TB - 1) / TB;
@@ -819,17 +840,13 @@ rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x
     rfm_set_error("trsv: too many blocks");
     return RFM_EINVAL;
   }
-  if (p->dinv && p->dinv_of != p->R) RFM_TRY(rfm_trsv_prepare(p));
+  const int H = chain_helpers(nblk);
+  if (H > 0 && p->dinv_of != p->R) RFM_TRY(rfm_trsv_prepare(p));
   ProfScope ps(PF_TRSV, p->stream);
   rfm_prof_work(PF_TRSV, 8.0 * (double)n * (n + 1) / 2 + 16.0 * n);  // R read once, b and x
-  // Chain + helpers up to four blocks per SM (n = 38,800), a rule on n alone so
-  // that the solution's bits are those of one form; the helpers, fewer than the
-  // SMs, take a fifth target at the end of that range.
-  const int H = std::min(chain_max_ctas() - CHAIN_CL, (nblk + CHAIN_CL - 1) / CHAIN_CL * CHAIN_CL);
-  if (p->trsv_rec && p->dinv && p->chain_tiles && H > 0 && nblk <= HMAXT * H &&
-      nblk - CHAIN_D - 1 <= 4 * (rfm_num_sms() - 1)) {
+  if (H > 0) {
     ChainArgs a;
-    a.R = p->R; a.P = p->chain_tiles + (trans ? rfm_trsv_tiles_len(n) / 2 : 0);
+    a.R = p->R; a.P = p->chain_tiles + (trans ? (size_t)nblk * (CHAIN_D + 1) * TB * TB : 0);
     a.ldr = p->ldr; a.n = n; a.nblk = nblk; a.H = H; a.rhs = b; a.x = x;
     a.hrec = p->trsv_rec; a.xrec = p->trsv_rec + (size_t)nblk * TB * 2;
     a.epoch = p->sync + SYNC_EPOCH; a.err = p->sync + SYNC_ERR; a.skip = p->skip;

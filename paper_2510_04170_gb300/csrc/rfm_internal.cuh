@@ -42,7 +42,7 @@ struct rfm_problem {
   double* X = nullptr;      // breakpoints [3][nmaxbp]
   double* mu = nullptr;     // [G][4]
   double* sig = nullptr;    // [G][4]
-  double* slab = nullptr;   // allocation of lam, F, work, red, sync, slopes, jt_part, dinv, chain_tiles and the records
+  double* slab = nullptr;   // allocation of lam, F, work, red, sync, slopes, jt_part and the records
   double* feat = nullptr;   // [G*fields*M][4]
   double* slopes = nullptr; // [G*fields*M][8]: k_b / sigma_b and their squares
   RowSeg* segs = nullptr;
@@ -104,7 +104,7 @@ struct rfm_problem {
   unsigned long long* ls_rec = nullptr;  // [2][LS_BLOCKS] 16-byte records of the line search
   double* jt_part = nullptr;      // [JT_SLICES][n] partial sums of J^T x
   unsigned long long* trsv_rec = nullptr;  // [2][ceil(n/64)][64] 16-byte records: the triangular solve's sums and x
-  double* chain_tiles = nullptr;  // dinv and R's near off-diagonal blocks in the chain's order (rfm_trsv_tiles_len)
+  double* chain_tiles = nullptr;  // dinv and R's near off-diagonal blocks in the chain's order (rfm_trsv_prepare)
   double* dinv = nullptr;         // [ceil(n/64)][64 x 64] inverses of R's diagonal blocks (column-major)
   const double* dinv_of = nullptr;  // the R that dinv was computed from (nullptr: stale)
   // per-problem QR scratch (FP64 panel buffers)
@@ -180,7 +180,6 @@ rfm_status rfm_launch_jmv(rfm_problem* p, const double* x, double* y);
 rfm_status rfm_launch_jtmv(rfm_problem* p, const double* x, double* y);
 rfm_status rfm_launch_trsv(rfm_problem* p, int trans, const double* b, double* x);
 rfm_status rfm_trsv_prepare(rfm_problem* p);  // inverts R's diagonal blocks (after every change of R)
-long long rfm_trsv_tiles_len(long long n);    // doubles of rfm_problem::chain_tiles
 rfm_status rfm_launch_count_sketch(rfm_problem* p, long long s, int kJ);
 rfm_status rfm_launch_gauss_sketch(rfm_problem* p, long long s, int kJ);
 rfm_status rfm_launch_gauss_sketch_tc(rfm_problem* p, long long s, int kJ);
